@@ -161,7 +161,7 @@ tc_gemm_f32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   unsigned char* epi_stage = reinterpret_cast<unsigned char*>(bars) + 1024;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp-uniform
   constexpr int kTr = (EPI == kTcEpiF32) ? 3 : 2;           // trace builds: kernel id of the stamps
   constexpr int kTrKb = 8;                                  // the k-block whose conversion and MMAs are stamped
 
@@ -187,7 +187,7 @@ tc_gemm_f32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
   // As in tc_gemm_kernel: with `early_b` (GEMM-2: the tile list is final long before its CTAs start) the producer
   // requests the weight boxes of its first stages before the dependent-launch wait; only the activations have to wait.
   int pre = 0;
-  if (warp == 0 && lane == 0 && a.early_b) {
+  if (warp == 0 && a.early_b) {
     const int n_rt = __ldcg(a.n_tiles);
     const int per = n_rt * a.n_col_tiles;
     if ((int)blockIdx.x < per * a.n_split) {
@@ -198,15 +198,18 @@ tc_gemm_f32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
       const int brow = td.phys * a.b_rows_per_phys + ct * kBoxRows;
       pre = a.k_blocks < kStages ? a.k_blocks : kStages;
       for (int kb = 0; kb < pre; ++kb) {
-        ptx::mbar_expect_tx(&full[kb], (uint32_t)(kF32ABytes + kBBytesK));
-        if (kSwap) {
-          ptx::tma_load_2d(raw + kb * kStageBytes, &tmA, &full[kb], (z * a.k_blocks + kb) * kF32BK, brow);
-        } else {
+        if (ptx::elect_one()) {
+          ptx::mbar_expect_tx(&full[kb], (uint32_t)(kF32ABytes + kBBytesK));
+          if (kSwap) {
+            ptx::tma_load_2d(raw + kb * kStageBytes, &tmA, &full[kb], (z * a.k_blocks + kb) * kF32BK, brow);
+          } else {
 #pragma unroll
-          for (int j = 0; j < kNB; ++j)
-            ptx::tma_load_2d(raw + kb * kStageBytes + kF32ABytes + j * kBoxRows * kF32BK * 4, &tmB, &full[kb],
-                             (z * a.k_blocks + kb) * kF32BK, brow + j * a.b_rows_gate);
+            for (int j = 0; j < kNB; ++j)
+              ptx::tma_load_2d(raw + kb * kStageBytes + kF32ABytes + j * kBoxRows * kF32BK * 4, &tmB, &full[kb],
+                               (z * a.k_blocks + kb) * kF32BK, brow + j * a.b_rows_gate);
+          }
         }
+        __syncwarp();
       }
     }
   }
@@ -219,25 +222,25 @@ tc_gemm_f32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
   const int total = per_slice * a.n_split;        // item = slice * per_slice + (col tile * n_row_tiles + row tile)
 
   if (warp == 0) {
-    if (lane == 0) {
-      // ------------------------------------------------------------------ TMA producer
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
-        const int z = t / per_slice, u = t - z * per_slice;
-        const int ct = u / n_row_tiles, rt = u - ct * n_row_tiles;
-        const TileDesc td = a.tiles[rt];
-        const int brow = td.phys * a.b_rows_per_phys + ct * kBoxRows;
-        const int kb0 = z * a.k_blocks;
-        for (int kb = 0; kb < a.k_blocks; ++kb) {
-          const bool early = t == (int)blockIdx.x && kb < pre;   // armed and weights requested above
-          unsigned char* sA = raw + stage * kStageBytes;
-          if (!early) {
-            ok = bounded_wait(&empty[stage], phase ^ 1u, abort_flag, a.status, 31);
-            if (!ok) break;
-            ptx::mbar_expect_tx(&full[stage], (uint32_t)(kF32ABytes + kBBytesK));
-          }
+    // ------------------------------------------------------------------ TMA producer
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
+      const int z = t / per_slice, u = t - z * per_slice;
+      const int ct = u / n_row_tiles, rt = u - ct * n_row_tiles;
+      const TileDesc td = a.tiles[rt];
+      const int brow = td.phys * a.b_rows_per_phys + ct * kBoxRows;
+      const int kb0 = z * a.k_blocks;
+      for (int kb = 0; kb < a.k_blocks; ++kb) {
+        const bool early = t == (int)blockIdx.x && kb < pre;   // armed and weights requested above
+        unsigned char* sA = raw + stage * kStageBytes;
+        if (!early) {
+          ok = warp_wait(&empty[stage], phase ^ 1u, abort_flag, a.status, 31);
+          if (!ok) break;
+        }
+        if (ptx::elect_one()) {
+          if (!early) ptx::mbar_expect_tx(&full[stage], (uint32_t)(kF32ABytes + kBBytesK));
           if (kSwap) {
             // tokens are the B operand, weights the A operand (the one that may have been requested early)
             ptx::tma_load_2d(sA + kF32ABytes, &tmB, &full[stage], (kb0 + kb) * kF32BK, td.row0);
@@ -251,36 +254,37 @@ tc_gemm_f32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
                                  brow + j * a.b_rows_gate);
             }
           }
-          if (++stage == kStages) { stage = 0; phase ^= 1u; }
         }
-        SWAPMOE_STAMP(kTr, 3);
+        __syncwarp();
+        if (++stage == kStages) { stage = 0; phase ^= 1u; }
       }
-      if (!ok) {
-        // Give copies that are still in flight time to land before shared memory is released.
-        const uint64_t t0 = ptx::globaltimer_ns();
-        while (ptx::globaltimer_ns() - t0 < 2000000ull) __nanosleep(1000);
-      }
+      if (lane == 0) SWAPMOE_STAMP(kTr, 3);
+    }
+    if (!ok) {
+      // Give copies that are still in flight time to land before shared memory is released.
+      const uint64_t t0 = ptx::globaltimer_ns();
+      while (ptx::globaltimer_ns() - t0 < 2000000ull) __nanosleep(1000);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ------------------------------------------------------------------ MMA issuer
-      int stage = 0, slot = 0, acc = 0;
-      uint32_t slot_phase = 0, acc_phase = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
-        ok = bounded_wait(&acc_empty[acc], acc_phase ^ 1u, abort_flag, a.status, 32);
+    // ------------------------------------------------------------------ MMA issuer
+    int stage = 0, slot = 0, acc = 0;
+    uint32_t slot_phase = 0, acc_phase = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
+      ok = warp_wait(&acc_empty[acc], acc_phase ^ 1u, abort_flag, a.status, 32);
+      if (!ok) break;
+      ptx::tc_fence_after();
+      const uint32_t tmem_d = tmem_base + (uint32_t)(acc * kAccStride);
+      for (int kb = 0; kb < a.k_blocks; ++kb) {
+        ok = warp_wait(&conv_done[slot], slot_phase, abort_flag, a.status, 33);
         if (!ok) break;
         ptx::tc_fence_after();
-        const uint32_t tmem_d = tmem_base + (uint32_t)(acc * kAccStride);
-        for (int kb = 0; kb < a.k_blocks; ++kb) {
-          ok = bounded_wait(&conv_done[slot], slot_phase, abort_flag, a.status, 33);
-          if (!ok) break;
-          ptx::tc_fence_after();
-          if (kb == kTrKb && t == (int)blockIdx.x) SWAPMOE_STAMP(kTr, 14);
-          // B row = [b1 of the 32 elements | b2 of them]: 16 elements = 32 bytes = +2 in the address field;
-          // A slot = [8 columns b1 (k 0-15) | 8 b1 (k 16-31) | 8 b2 | 8 b2]; small terms first
-          const uint64_t db = make_kmajor_sw128_desc(ptx::smem_u32(raw + stage * kStageBytes + kF32ABytes));
-          const uint32_t a1 = tmem_base + (uint32_t)(kASlotBase + slot * kASlotCols), a2 = a1 + 16;
+        if (lane == 0 && kb == kTrKb && t == (int)blockIdx.x) SWAPMOE_STAMP(kTr, 14);
+        // B row = [b1 of the 32 elements | b2 of them]: 16 elements = 32 bytes = +2 in the address field;
+        // A slot = [8 columns b1 (k 0-15) | 8 b1 (k 16-31) | 8 b2 | 8 b2]; small terms first
+        const uint64_t db = make_kmajor_sw128_desc(ptx::smem_u32(raw + stage * kStageBytes + kF32ABytes));
+        const uint32_t a1 = tmem_base + (uint32_t)(kASlotBase + slot * kASlotCols), a2 = a1 + 16;
+        if (ptx::elect_one()) {
           ptx::umma_bf16_ts(tmem_d, a2, db, kIdesc, kb > 0 ? 1u : 0u);
           ptx::umma_bf16_ts(tmem_d, a2 + 8, db + 2, kIdesc, 1u);
           ptx::umma_bf16_ts(tmem_d, a1, db + 4, kIdesc, 1u);
@@ -289,15 +293,16 @@ tc_gemm_f32_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constan
           ptx::umma_bf16_ts(tmem_d, a1 + 8, db + 2, kIdesc, 1u);
           ptx::umma_commit(&empty[stage]);       // the raw stage may be refilled
           ptx::umma_commit(&lo_empty[slot]);     // the TMEM slot may be rewritten
-          if (kb == kTrKb && t == (int)blockIdx.x) SWAPMOE_STAMP(kTr, 15);
-          if (++stage == kStages) stage = 0;
-          if (++slot == kSlots) { slot = 0; slot_phase ^= 1u; }
+          if (kb + 1 == a.k_blocks) ptx::umma_commit(&acc_full[acc]);
         }
-        if (!ok) break;
-        ptx::umma_commit(&acc_full[acc]);
-        SWAPMOE_STAMP(kTr, 5);
-        if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+        __syncwarp();
+        if (lane == 0 && kb == kTrKb && t == (int)blockIdx.x) SWAPMOE_STAMP(kTr, 15);
+        if (++stage == kStages) stage = 0;
+        if (++slot == kSlots) { slot = 0; slot_phase ^= 1u; }
       }
+      if (!ok) break;
+      if (lane == 0) SWAPMOE_STAMP(kTr, 5);
+      if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
     }
   } else if (warp >= 8) {
     // ---------------------------------------------------------------------- converters

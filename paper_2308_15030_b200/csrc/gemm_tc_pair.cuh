@@ -115,7 +115,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   unsigned char* epi_stage = smem + kStages * kPairStageBytes + 1024;   // [4 warps][32 rows][128 bytes]
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp-uniform
   const uint32_t rank = ptx::cluster_ctarank();               // 0: issues the MMAs
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
 
@@ -143,7 +143,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   // As in tc_gemm_kernel: with `early_b` each producer requests the weight boxes of its first stages before the
   // dependent-launch wait.
   int pre = 0;
-  if (warp == 0 && lane == 0 && a.early_b) {
+  if (warp == 0 && a.early_b) {
     const int n_rt = __ldcg(a.n_tiles);
     if (pair < n_rt * a.n_col_tiles) {
       int rt, ct;
@@ -154,10 +154,14 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
                        (EPI == kTcEpiSwigluBf16 ? ct * kPairHalfRows + (int)rank * a.b_rows_gate
                                                 : ct * kPairBN + (int)rank * kPairHalfRows);
       pre = a.k_blocks < kStages ? a.k_blocks : kStages;
+      const uint32_t full0 = ptx::map_to_cta(ptx::smem_u32(full), 0u);
       for (int kb = 0; kb < pre; ++kb) {
-        if (rank == 0)
-          ptx::mbar_expect_tx(&full[kb], (uint32_t)((td.rows > kTcBM ? 2 : 1) * kPairABytes + 2 * kPairBBytes));
-        ptx::tma_load_2d_pair(sB + kb * kPairBBytes, &tmB, ptx::map_to_cta(ptx::smem_u32(&full[kb]), 0u), kb * kTcBK, brow);
+        if (ptx::elect_one()) {
+          if (rank == 0)
+            ptx::mbar_expect_tx(&full[kb], (uint32_t)((td.rows > kTcBM ? 2 : 1) * kPairABytes + 2 * kPairBBytes));
+          ptx::tma_load_2d_pair(sB + kb * kPairBBytes, &tmB, full0 + 8u * (uint32_t)kb, kb * kTcBK, brow);
+        }
+        __syncwarp();
       }
     }
   }
@@ -169,71 +173,76 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   const int total = n_row_tiles * a.n_col_tiles;
 
   if (warp == 0) {
-    if (lane == 0) {
-      // ------------------------------------------------------------------ TMA producer (both CTAs)
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      for (int t = pair; t < total && ok; t += n_pairs) {
-        int rt, ct;
-        decode_tile(t, n_row_tiles, a.n_col_tiles, a.row_group, &rt, &ct);
-        const TileDesc td = a.tiles[rt];
-        const bool two_halves = td.rows > kTcBM;
-        // ReLU / plain: the pair's 256 weight rows are consecutive; SwiGLU: 128 rows of W1 (even CTA) and the
-        // same 128 rows of W3 (odd CTA)
-        const int brow = td.phys * a.b_rows_per_phys +
-                         (EPI == kTcEpiSwigluBf16 ? ct * kPairHalfRows + (int)rank * a.b_rows_gate
-                                                  : ct * kPairBN + (int)rank * kPairHalfRows);
-        const bool load_a = rank == 0 || two_halves;
-        for (int kb = 0; kb < a.k_blocks; ++kb) {
-          const bool early = t == pair && kb < pre;          // armed and weights requested above
-          if (!early) {
-            ok = bounded_wait(&empty[stage], phase ^ 1u, abort_flag, a.status, 11);
-            if (!ok) break;
-          }
-          const uint32_t full_addr = ptx::map_to_cta(ptx::smem_u32(&full[stage]), 0u);
-          if (rank == 0 && !early)
-            ptx::mbar_expect_tx(&full[stage], (uint32_t)((two_halves ? 2 : 1) * kPairABytes + 2 * kPairBBytes));
-          if (load_a)
-            ptx::tma_load_2d_pair(sA + stage * kPairABytes, &tmA, full_addr, kb * kTcBK, td.row0 + (int)rank * kTcBM);
-          if (!early) ptx::tma_load_2d_pair(sB + stage * kPairBBytes, &tmB, full_addr, kb * kTcBK, brow);
-          if (++stage == kStages) { stage = 0; phase ^= 1u; }
+    // ------------------------------------------------------------------ TMA producer (both CTAs)
+    const uint32_t full0 = ptx::map_to_cta(ptx::smem_u32(full), 0u);
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int t = pair; t < total && ok; t += n_pairs) {
+      int rt, ct;
+      decode_tile(t, n_row_tiles, a.n_col_tiles, a.row_group, &rt, &ct);
+      const TileDesc td = a.tiles[rt];
+      const bool two_halves = td.rows > kTcBM;
+      // ReLU / plain: the pair's 256 weight rows are consecutive; SwiGLU: 128 rows of W1 (even CTA) and the
+      // same 128 rows of W3 (odd CTA)
+      const int brow = td.phys * a.b_rows_per_phys +
+                       (EPI == kTcEpiSwigluBf16 ? ct * kPairHalfRows + (int)rank * a.b_rows_gate
+                                                : ct * kPairBN + (int)rank * kPairHalfRows);
+      const int arow = td.row0 + (int)rank * kTcBM;
+      const bool load_a = rank == 0 || two_halves;
+      const uint32_t bytes = (uint32_t)((two_halves ? 2 : 1) * kPairABytes + 2 * kPairBBytes);
+      for (int kb = 0; kb < a.k_blocks; ++kb) {
+        const bool early = t == pair && kb < pre;          // armed and weights requested above
+        if (!early) {
+          ok = warp_wait(&empty[stage], phase ^ 1u, abort_flag, a.status, 11);
+          if (!ok) break;
         }
-        SWAPMOE_STAMP(kTr, 3);
+        const uint32_t bar = full0 + 8u * (uint32_t)stage;
+        if (ptx::elect_one()) {
+          if (rank == 0 && !early) ptx::mbar_expect_tx(&full[stage], bytes);
+          if (load_a) ptx::tma_load_2d_pair(sA + stage * kPairABytes, &tmA, bar, kb * kTcBK, arow);
+          if (!early) ptx::tma_load_2d_pair(sB + stage * kPairBBytes, &tmB, bar, kb * kTcBK, brow);
+        }
+        __syncwarp();
+        if (++stage == kStages) { stage = 0; phase ^= 1u; }
       }
-      if (!ok) {
-        // Give copies that are still in flight time to land before shared memory is released.
-        const uint64_t t0 = ptx::globaltimer_ns();
-        while (ptx::globaltimer_ns() - t0 < 2000000ull) __nanosleep(1000);
-      }
+      if (lane == 0) SWAPMOE_STAMP(kTr, 3);
+    }
+    if (!ok) {
+      // Give copies that are still in flight time to land before shared memory is released.
+      const uint64_t t0 = ptx::globaltimer_ns();
+      while (ptx::globaltimer_ns() - t0 < 2000000ull) __nanosleep(1000);
     }
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
       // ------------------------------------------------------------------ MMA issuer (even CTA, for the pair)
       int stage = 0, acc = 0;
       uint32_t phase = 0, acc_phase = 0;
       bool ok = true;
       for (int t = pair; t < total && ok; t += n_pairs) {
-        ok = bounded_wait(&acc_empty[acc], acc_phase ^ 1u, abort_flag, a.status, 12);
+        ok = warp_wait(&acc_empty[acc], acc_phase ^ 1u, abort_flag, a.status, 12);
         if (!ok) break;
         ptx::tc_fence_after();
         const uint32_t tmem_d = tmem_base + (uint32_t)(acc * kPairBN);
         for (int kb = 0; kb < a.k_blocks; ++kb) {
-          ok = bounded_wait(&full[stage], phase, abort_flag, a.status, 13);
+          ok = warp_wait(&full[stage], phase, abort_flag, a.status, 13);
           if (!ok) break;
           ptx::tc_fence_after();
-          if (t == pair && kb == 0) SWAPMOE_STAMP(kTr, 4);
+          if (lane == 0 && t == pair && kb == 0) SWAPMOE_STAMP(kTr, 4);
           const uint64_t da = make_kmajor_sw128_desc(ptx::smem_u32(sA + stage * kPairABytes));
           const uint64_t db = make_kmajor_sw128_desc(ptx::smem_u32(sB + stage * kPairBBytes));
+          if (ptx::elect_one()) {
 #pragma unroll
-          for (int k = 0; k < kTcBK / kTcUmmaK; ++k)
-            ptx::umma_bf16_pair(tmem_d, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), kIdesc, (kb > 0 || k > 0) ? 1u : 0u);
-          ptx::umma_commit_pair(&empty[stage]);   // frees the stage in both CTAs once these MMAs have read it
+            for (int k = 0; k < kTcBK / kTcUmmaK; ++k)
+              ptx::umma_bf16_pair(tmem_d, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), kIdesc, (kb > 0 || k > 0) ? 1u : 0u);
+            ptx::umma_commit_pair(&empty[stage]);   // frees the stage in both CTAs once these MMAs have read it
+            if (kb + 1 == a.k_blocks) ptx::umma_commit_pair(&acc_full[acc]);    // accumulator complete, in both CTAs
+          }
+          __syncwarp();
           if (++stage == kStages) { stage = 0; phase ^= 1u; }
         }
         if (!ok) break;
-        ptx::umma_commit_pair(&acc_full[acc]);    // accumulator complete, in both CTAs
-        SWAPMOE_STAMP(kTr, 5);
+        if (lane == 0) SWAPMOE_STAMP(kTr, 5);
         if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
       }
     }

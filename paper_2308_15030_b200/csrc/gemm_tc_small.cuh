@@ -62,7 +62,7 @@ tc_gemm_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp-uniform
   if (threadIdx.x == 0) {
     for (int s = 0; s < n_stages; ++s) { ptx::mbar_init(&full[s], 1); ptx::mbar_init(&empty[s], 1); }
     for (int b = 0; b < 2; ++b) { ptx::mbar_init(&acc_full[b], 1); ptx::mbar_init(&acc_empty[b], 128); }
@@ -84,7 +84,7 @@ tc_gemm_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
   // As in tc_gemm_kernel: with `early_b` the producer requests the weight boxes of its first stages before the
   // dependent-launch wait.
   int pre = 0;
-  if (warp == 0 && lane == 0 && a.early_b) {
+  if (warp == 0 && a.early_b) {
     const int n_rt = __ldcg(a.n_tiles);
     if ((int)blockIdx.x < n_rt * a.n_col_tiles) {
       const int ct = (int)blockIdx.x / n_rt, rt = (int)blockIdx.x - ct * n_rt;
@@ -93,8 +93,11 @@ tc_gemm_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
       const int brow = td.phys * a.b_rows_per_phys + ct * BN;
       pre = n_chunks < n_stages ? n_chunks : n_stages;
       for (int c = 0; c < pre; ++c) {
-        ptx::mbar_expect_tx(&full[c], (uint32_t)(stage_a + stage_b));
-        tma_load_3d(sB + c * stage_b, &tmB, &full[c], 0, brow, c * kps);
+        if (ptx::elect_one()) {
+          ptx::mbar_expect_tx(&full[c], (uint32_t)(stage_a + stage_b));
+          tma_load_3d(sB + c * stage_b, &tmB, &full[c], 0, brow, c * kps);
+        }
+        __syncwarp();
       }
     }
   }
@@ -104,62 +107,65 @@ tc_gemm_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
   const int total = n_row_tiles * a.n_col_tiles;
 
   if (warp == 0) {
-    if (lane == 0) {
-      // ------------------------------------------------------------------ TMA producer
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
-        const int ct = t / n_row_tiles, rt = t - ct * n_row_tiles;
-        const TileDesc td = a.tiles[rt];
-        const int brow = td.phys * a.b_rows_per_phys + ct * BN;
-        for (int c = 0; c < n_chunks; ++c) {
-          const bool early = t == (int)blockIdx.x && c < pre;    // armed and weights requested above
-          if (!early) {
-            ok = bounded_wait(&empty[stage], phase ^ 1u, abort_flag, a.status, 31);
-            if (!ok) break;
-            ptx::mbar_expect_tx(&full[stage], (uint32_t)(stage_a + stage_b));
-          }
+    // ------------------------------------------------------------------ TMA producer
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
+      const int ct = t / n_row_tiles, rt = t - ct * n_row_tiles;
+      const TileDesc td = a.tiles[rt];
+      const int brow = td.phys * a.b_rows_per_phys + ct * BN;
+      for (int c = 0; c < n_chunks; ++c) {
+        const bool early = t == (int)blockIdx.x && c < pre;    // armed and weights requested above
+        if (!early) {
+          ok = warp_wait(&empty[stage], phase ^ 1u, abort_flag, a.status, 31);
+          if (!ok) break;
+        }
+        if (ptx::elect_one()) {
+          if (!early) ptx::mbar_expect_tx(&full[stage], (uint32_t)(stage_a + stage_b));
           tma_load_3d(sA + stage * stage_a, &tmA, &full[stage], 0, td.row0, c * kps);
           if (!early) tma_load_3d(sB + stage * stage_b, &tmB, &full[stage], 0, brow, c * kps);
-          if (++stage == n_stages) { stage = 0; phase ^= 1u; }
         }
-      }
-      if (!ok) {
-        const uint64_t t0 = ptx::globaltimer_ns();
-        while (ptx::globaltimer_ns() - t0 < 2000000ull) __nanosleep(1000);
+        __syncwarp();
+        if (++stage == n_stages) { stage = 0; phase ^= 1u; }
       }
     }
+    if (!ok) {
+      const uint64_t t0 = ptx::globaltimer_ns();
+      while (ptx::globaltimer_ns() - t0 < 2000000ull) __nanosleep(1000);
+    }
   } else if (warp == 1) {
-    if (lane == 0) {
-      // ------------------------------------------------------------------ MMA issuer
-      int stage = 0, acc = 0;
-      uint32_t phase = 0, acc_phase = 0;
-      bool ok = true;
-      for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
-        ok = bounded_wait(&acc_empty[acc], acc_phase ^ 1u, abort_flag, a.status, 32);
+    // ------------------------------------------------------------------ MMA issuer
+    int stage = 0, acc = 0;
+    uint32_t phase = 0, acc_phase = 0;
+    bool ok = true;
+    for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
+      ok = warp_wait(&acc_empty[acc], acc_phase ^ 1u, abort_flag, a.status, 32);
+      if (!ok) break;
+      ptx::tc_fence_after();
+      const uint32_t tmem_d = tmem_base + (uint32_t)(acc * BN);
+      for (int c = 0; c < n_chunks; ++c) {
+        ok = warp_wait(&full[stage], phase, abort_flag, a.status, 33);
         if (!ok) break;
         ptx::tc_fence_after();
-        const uint32_t tmem_d = tmem_base + (uint32_t)(acc * BN);
-        for (int c = 0; c < n_chunks; ++c) {
-          ok = bounded_wait(&full[stage], phase, abort_flag, a.status, 33);
-          if (!ok) break;
-          ptx::tc_fence_after();
+        const uint64_t da0 = make_kmajor_sw128_desc(ptx::smem_u32(sA + stage * stage_a));
+        const uint64_t db0 = make_kmajor_sw128_desc(ptx::smem_u32(sB + stage * stage_b));
+        if (ptx::elect_one()) {
           for (int kk = 0; kk < kps; ++kk) {
-            const uint64_t da = make_kmajor_sw128_desc(ptx::smem_u32(sA + stage * stage_a + kk * a_tile));
-            const uint64_t db = make_kmajor_sw128_desc(ptx::smem_u32(sB + stage * stage_b + kk * kBTile));
+            const uint64_t da = da0 + (uint64_t)(kk * (a_tile >> 4)), db = db0 + (uint64_t)(kk * (kBTile >> 4));
 #pragma unroll
             for (int k = 0; k < kTcBK / kTcUmmaK; ++k)
               ptx::umma_bf16(tmem_d, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), kIdesc,
                              (c > 0 || kk > 0 || k > 0) ? 1u : 0u);
           }
           ptx::umma_commit(&empty[stage]);
-          if (++stage == n_stages) { stage = 0; phase ^= 1u; }
+          if (c + 1 == n_chunks) ptx::umma_commit(&acc_full[acc]);
         }
-        if (!ok) break;
-        ptx::umma_commit(&acc_full[acc]);
-        if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+        __syncwarp();
+        if (++stage == n_stages) { stage = 0; phase ^= 1u; }
       }
+      if (!ok) break;
+      if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
     }
   } else if (warp >= 4) {
     // -------------------------------------------------------------------- epilogue

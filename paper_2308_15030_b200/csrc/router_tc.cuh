@@ -90,7 +90,7 @@ router_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant_
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   const GateSmem g = gate_smem_carve(bars + 2 * kRtMaxStages + 8);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // warp: warp-uniform
   const int tok0 = blockIdx.x * tok;
   const int k_blocks = a.d / kTcBK;
   uint32_t tmem_cols = 32;
@@ -138,43 +138,45 @@ router_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant_
   const uint32_t tmem_base = *tmem_slot;
 
   if (warp == 0) {
-    if (lane == 0) {
-      // the first `pre` stages were requested above; the ring continues behind them
-      int stage = pre == n_stages ? 0 : pre; uint32_t phase = pre == n_stages ? 1u : 0u;
-      for (int kb = pre; kb < k_blocks; ++kb) {
-        if (!bounded_wait(&empty[stage], phase ^ 1u, abort_flag, status, 11)) break;
+    // the first `pre` stages were requested above; the ring continues behind them
+    int stage = pre == n_stages ? 0 : pre; uint32_t phase = pre == n_stages ? 1u : 0u;
+    for (int kb = pre; kb < k_blocks; ++kb) {
+      if (!warp_wait(&empty[stage], phase ^ 1u, abort_flag, status, 11)) break;
+      if (ptx::elect_one()) {
         ptx::mbar_expect_tx(&full[stage], (uint32_t)(a_box_bytes + b_bytes));
         ptx::tma_load_2d(sA + stage * a_bytes, &tmX, &full[stage], kb * kTcBK, tok0);
         ptx::tma_load_2d(sB + stage * b_bytes, &tmW, &full[stage], kb * kTcBK, 0);
-        if (++stage == n_stages) { stage = 0; phase ^= 1u; }
       }
-      if (*abort_flag) {
-        const uint64_t t0 = ptx::globaltimer_ns();
-        while (ptx::globaltimer_ns() - t0 < 2000000ull) __nanosleep(1000);
-      }
+      __syncwarp();
+      if (++stage == n_stages) { stage = 0; phase ^= 1u; }
+    }
+    if (*abort_flag) {
+      const uint64_t t0 = ptx::globaltimer_ns();
+      while (ptx::globaltimer_ns() - t0 < 2000000ull) __nanosleep(1000);
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      const uint32_t idesc = make_idesc_bf16(kRtTok, Epad);
-      int stage = 0; uint32_t phase = 0;
-      bool ok = true;
-      for (int kb = 0; kb < k_blocks; ++kb) {
-        ok = bounded_wait(&full[stage], phase, abort_flag, status, 12);
-        if (!ok) break;
-        ptx::tc_fence_after();
-        if (kb == 0) SWAPMOE_STAMP(0, 2);
-        const uint64_t da = make_kmajor_sw128_desc(ptx::smem_u32(sA + stage * a_bytes));
-        const uint64_t db = make_kmajor_sw128_desc(ptx::smem_u32(sB + stage * b_bytes));
+    const uint32_t idesc = make_idesc_bf16(kRtTok, Epad);
+    int stage = 0; uint32_t phase = 0;
+    bool ok = true;
+    for (int kb = 0; kb < k_blocks; ++kb) {
+      ok = warp_wait(&full[stage], phase, abort_flag, status, 12);
+      if (!ok) break;
+      ptx::tc_fence_after();
+      if (lane == 0 && kb == 0) SWAPMOE_STAMP(0, 2);
+      const uint64_t da = make_kmajor_sw128_desc(ptx::smem_u32(sA + stage * a_bytes));
+      const uint64_t db = make_kmajor_sw128_desc(ptx::smem_u32(sB + stage * b_bytes));
+      if (ptx::elect_one()) {
 #pragma unroll
         for (int kk = 0; kk < kTcBK / kTcUmmaK; ++kk)
           ptx::umma_bf16(tmem_base, da + (uint64_t)(2 * kk), db + (uint64_t)(2 * kk), idesc,
                          (kb > 0 || kk > 0) ? 1u : 0u);
         ptx::umma_commit(&empty[stage]);
-        if (++stage == n_stages) { stage = 0; phase ^= 1u; }
+        if (kb + 1 == k_blocks) ptx::umma_commit(acc_full);
       }
-      if (ok) ptx::umma_commit(acc_full);
-      SWAPMOE_STAMP(0, 3);
+      __syncwarp();
+      if (++stage == n_stages) { stage = 0; phase ^= 1u; }
     }
+    if (lane == 0) SWAPMOE_STAMP(0, 3);
   } else if (warp >= 4) {
     // ------------------------------------------------ ||x||^2 while the tiles stream through
     const int q = warp - 4, r = q * 32 + lane;
