@@ -52,6 +52,16 @@ __device__ __forceinline__ void store8(bf16* p, const float v[8]) {
                                             pack_bf16x2(v[4], v[5]), pack_bf16x2(v[6], v[7]));
 }
 
+// Order-preserving integer key of a logit: a > b  <=>  key(a) > key(b), equal logits (-0 and +0 included) have
+// equal keys, and no finite or infinite logit maps to 0, which stands for "nothing available".
+__device__ __forceinline__ uint32_t gate_key(float x) {
+  const uint32_t b = __float_as_uint(x + 0.f);              // -0 becomes +0
+  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+}
+__device__ __forceinline__ float gate_key_value(uint32_t key) {
+  return __uint_as_float((key & 0x80000000u) ? (key & 0x7fffffffu) : ~key);
+}
+
 // Programmatic dependent launch: a kernel launched with the stream-serialization attribute may
 // start while its predecessor is still running; it must execute pdl_wait() before it reads or
 // writes any global memory the predecessors touch.  pdl_trigger() lets the NEXT kernel's

@@ -91,16 +91,6 @@ __host__ __device__ inline int decode_rows_per_wave(int d) {
   return rp;
 }
 
-// Order-preserving integer key of a logit: a > b  <=>  key(a) > key(b), equal logits (-0 and +0 included) have
-// equal keys, and no finite or infinite logit maps to 0, which stands for "nothing available".
-__device__ __forceinline__ uint32_t gate_key(float x) {
-  const uint32_t b = __float_as_uint(x + 0.f);              // -0 becomes +0
-  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-}
-__device__ __forceinline__ float gate_key_value(uint32_t key) {
-  return __uint_as_float((key & 0x80000000u) ? (key & 0x7fffffffu) : ~key);
-}
-
 // Top-k of one token's logits by a whole warp: row[e] is the logit of expert e (shared memory), lane l looks
 // at experts l, l + 32, ... of the `ei` 32-expert groups that exist; allow bit i says whether expert l + 32 i
 // may be chosen; ties go to the lowest expert index.  Gate values are the softmax over the allowed experts (or

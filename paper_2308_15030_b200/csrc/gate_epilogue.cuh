@@ -12,28 +12,58 @@ namespace swapmoe {
 constexpr int kGateTokMax = 128;   // largest token tile
 constexpr int kGateThreads = 256;
 
-// Running top-k list, descending by value; a candidate is inserted below every entry
-// that is >= it, so equal values stay in arrival (= expert index) order.
+// Running list of the N best logits, descending, as order-preserving keys (gate_key; 0 = nothing).  A candidate goes
+// below every entry that is >= it, so equal values stay in arrival (= expert index) order.  Without branches: on a warp of
+// 32 tokens some token takes nearly every candidate, so a branch only adds its own cost (256 experts, top-4, 64
+// tokens per CTA: logits copy and this scan 23 -> 9.2 us).
+template <int N>
 struct TopK {
-  float v[kMaxTopK];
-  int e[kMaxTopK];
+  uint32_t v[N];
+  int e[N];
   __device__ __forceinline__ void init() {
 #pragma unroll
-    for (int j = 0; j < kMaxTopK; ++j) { v[j] = -INFINITY; e[j] = -1; }
+    for (int j = 0; j < N; ++j) { v[j] = 0u; e[j] = -1; }
   }
-  __device__ __forceinline__ void push(float cv, int ce, int k) {
-    bool shifting = false;
+  __device__ __forceinline__ void push(uint32_t cv, int ce) {
+    bool beats[N];
 #pragma unroll
-    for (int j = 0; j < kMaxTopK; ++j) {
-      if (j < k && (shifting || e[j] < 0 || cv > v[j])) {
-        const float tv = v[j]; const int te = e[j];
-        v[j] = cv; e[j] = ce;
-        cv = tv; ce = te;
-        shifting = true;
-      }
+    for (int j = 0; j < N; ++j) beats[j] = cv > v[j];
+#pragma unroll
+    for (int j = N - 1; j > 0; --j) {
+      v[j] = beats[j - 1] ? v[j - 1] : (beats[j] ? cv : v[j]);
+      e[j] = beats[j - 1] ? e[j - 1] : (beats[j] ? ce : e[j]);
     }
+    v[0] = beats[0] ? cv : v[0];
+    e[0] = beats[0] ? ce : e[0];
   }
 };
+
+// The logit behind a list entry (an empty one, possible with fewer allowed experts than k, weighs nothing).
+__device__ __forceinline__ float gate_entry_value(uint32_t key) { return key ? gate_key_value(key) : -INFINITY; }
+
+// The best N of the allowed experts [e_lo, e_hi) (e_lo a multiple of 32) of one logits row; at most seven floats
+// behind the row's end are read.
+template <int N>
+__device__ __forceinline__ void gate_scan(const float* row, const uint32_t* allow, int e_lo, int e_hi, uint32_t* cand_v,
+                                          int* cand_e) {
+  TopK<N> tk;
+  tk.init();
+#pragma unroll 1
+  for (int e0 = e_lo; e0 < e_hi; e0 += 8) {
+    const uint32_t w = (allow[e0 >> 5] >> (e0 & 31)) & 0xffu;
+    if (w == 0u) continue;                         // the same for all threads of a warp
+    float l[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) l[i] = row[e0 + i];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) tk.push((w >> i) & 1u ? gate_key(l[i]) : 0u, e0 + i);
+  }
+#pragma unroll
+  for (int j = 0; j < kMaxTopK; ++j) {
+    cand_v[j] = j < N ? tk.v[j < N ? j : 0] : 0u;
+    cand_e[j] = j < N ? tk.e[j < N ? j : 0] : -1;
+  }
+}
 
 // Shared-memory arrays of the gate, carved from one block by gate_smem_carve().
 struct GateSmem {
@@ -45,15 +75,14 @@ struct GateSmem {
   int* s_e2s;          // [256] expert -> slot
   float* s_enorm;      // [256] ||E_e||
   uint32_t* s_mask;    // [2][8] valid / resident expert bits
-  uint32_t* s_present; // [8] experts selected (unmasked) in this tile
-  float* cand_v;       // [256 threads][kMaxTopK] per-thread top-k values
+  uint32_t* cand_v;    // [256 threads][kMaxTopK] per-thread top-k keys
   int* cand_e;         //  ... and experts
   float* part_den;     // [256] partial softmax denominators
   float* s_m;          // [tok][2] row maximum per gate
 };
 
 __host__ __device__ constexpr size_t gate_smem_bytes() {
-  return (size_t)4 * (4 * kGateTokMax * kMaxTopK + kGateTokMax + 2 * kMaxE + 24 +
+  return (size_t)4 * (4 * kGateTokMax * kMaxTopK + kGateTokMax + 2 * kMaxE + 16 +
                       2 * kGateThreads * kMaxTopK + kGateThreads + 2 * kGateTokMax);
 }
 
@@ -67,8 +96,7 @@ __device__ __forceinline__ GateSmem gate_smem_carve(void* base) {
   g.s_e2s = reinterpret_cast<int*>(g.snorm + kGateTokMax);
   g.s_enorm = reinterpret_cast<float*>(g.s_e2s + kMaxE);
   g.s_mask = reinterpret_cast<uint32_t*>(g.s_enorm + kMaxE);
-  g.s_present = g.s_mask + 16;
-  g.cand_v = reinterpret_cast<float*>(g.s_present + 8);
+  g.cand_v = g.s_mask + 16;
   g.cand_e = reinterpret_cast<int*>(g.cand_v + kGateThreads * kMaxTopK);
   g.part_den = reinterpret_cast<float*>(g.cand_e + kGateThreads * kMaxTopK);
   g.s_m = g.part_den + kGateThreads;
@@ -91,7 +119,7 @@ __device__ __forceinline__ void gate_load_tables(const RouterArgs& a, const Gate
   int sl = e < a.E ? a.e2s[e] : -1;
   if (sl >= a.K) sl = -1;
   const uint32_t wv = __ballot_sync(0xffffffffu, e < a.E), wr = __ballot_sync(0xffffffffu, sl >= 0);
-  if (lane == 0) { g.s_mask[warp] = wv; g.s_mask[8 + warp] = wr; g.s_present[warp] = 0u; }
+  if (lane == 0) { g.s_mask[warp] = wv; g.s_mask[8 + warp] = wr; }
 }
 
 // The gate proper.  slog holds the tile's logits, row stride E + 1 floats (with at least 8
@@ -136,52 +164,26 @@ __device__ __forceinline__ void gate_epilogue(const RouterArgs& a, const GateSme
   const int n_chunks = (E + 31) >> 5, cpp = (n_chunks + parts - 1) >> (parts == 4 ? 2 : parts - 1);
   const int e_lo = min(E, part * cpp * 32), e_hi = min(E, (part + 1) * cpp * 32);
   {
-    // The loops below run once per CTA, so they are kept rolled (short bodies that stay in the
-    // instruction cache) rather than unrolled over the whole expert range.
-    TopK tk;
-    tk.init();
-    if (k == 1) {
-      float best = -INFINITY;
-      int bi = -1;
-#pragma unroll 4
-      for (int e = e_lo; e < e_hi; ++e) {
-        const float l = row[e];
-        const bool take = ((allow[e >> 5] >> (e & 31)) & 1u) && (bi < 0 || l > best);
-        best = take ? l : best;
-        bi = take ? e : bi;
-      }
-      tk.v[0] = best;
-      tk.e[0] = bi;
-    } else {
-      float thr = -INFINITY;
-      int filled = 0;
-#pragma unroll 1
-      for (int e = e_lo; e < e_hi; ++e) {
-        const float l = row[e];
-        if (((allow[e >> 5] >> (e & 31)) & 1u) && (filled < k || l > thr)) {
-          tk.push(l, e, k);
-          ++filled;
-          thr = (k == 2) ? tk.v[1] : (k == 3) ? tk.v[2] : tk.v[3];
-        }
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < kMaxTopK; ++j) { g.cand_v[tid * kMaxTopK + j] = tk.v[j]; g.cand_e[tid * kMaxTopK + j] = tk.e[j]; }
+    uint32_t* cv = g.cand_v + tid * kMaxTopK;
+    int* ce = g.cand_e + tid * kMaxTopK;
+    if (k == 1) gate_scan<1>(row, allow, e_lo, e_hi, cv, ce);
+    else if (k == 2) gate_scan<2>(row, allow, e_lo, e_hi, cv, ce);
+    else gate_scan<kMaxTopK>(row, allow, e_lo, e_hi, cv, ce);
   }
   __syncthreads();
   if (threadIdx.x == 0) SWAPMOE_STAMP(0, 6);
   // merge the shares of one (token, gate) in ascending expert order: a candidate only displaces
   // an entry it strictly beats, so equal logits keep the lowest expert index
-  TopK fin;
+  TopK<kMaxTopK> fin;
   fin.init();
   if (part == 0) {
     for (int pp = 0; pp < parts; ++pp) {
-      const int src = ((masked ? parts : 0) + pp) * tok + tl;
+      const int src = (((masked ? parts : 0) + pp) * tok + tl) * kMaxTopK;
 #pragma unroll
       for (int j = 0; j < kMaxTopK; ++j)
-        if (j < k && g.cand_e[src * kMaxTopK + j] >= 0) fin.push(g.cand_v[src * kMaxTopK + j], g.cand_e[src * kMaxTopK + j], k);
+        if (j < k) fin.push(g.cand_v[src + j], g.cand_e[src + j]);      // (key 0, nothing there, displaces nothing)
     }
-    g.s_m[tl * 2 + (masked ? 1 : 0)] = fin.v[0];
+    g.s_m[tl * 2 + (masked ? 1 : 0)] = gate_entry_value(fin.v[0]);
   }
   __syncthreads();
   if (threadIdx.x == 0) SWAPMOE_STAMP(0, 7);
@@ -207,12 +209,12 @@ __device__ __forceinline__ void gate_epilogue(const RouterArgs& a, const GateSme
   __syncthreads();
   if (threadIdx.x == 0) SWAPMOE_STAMP(0, 8);
   if (part == 0) {
-    const float m = fin.v[0];
+    const float m = gate_entry_value(fin.v[0]);
     float den = 0.f;
     if (a.renorm) {
 #pragma unroll
       for (int j = 0; j < kMaxTopK; ++j)
-        if (j < k) den += expf(fin.v[j] - m);
+        if (j < k) den += expf(gate_entry_value(fin.v[j]) - m);
     } else {
       for (int pp = 0; pp < parts; ++pp) den += g.part_den[((masked ? parts : 0) + pp) * tok + tl];
     }
@@ -222,13 +224,12 @@ __device__ __forceinline__ void gate_epilogue(const RouterArgs& a, const GateSme
       if (j < k) {
         const int pl = tl * k + j;
         const size_t p = (size_t)token * k + j;
-        const float gv = failed ? 0.f : expf(fin.v[j] - m) / den;
+        const float gv = failed ? 0.f : expf(gate_entry_value(fin.v[j]) - m) / den;
         const int e = fin.e[j];
         if (!masked) {
           if (token < a.T) {
             a.uidx[p] = e; a.ugate[p] = gv;
             g.pe[pl] = e; g.pt[pl] = xn * fabsf(gv) * g.s_enorm[e];   // one term of Eq. (1)
-            atomicOr(&g.s_present[e >> 5], 1u << (e & 31));
           } else {
             g.pe[pl] = -1; g.pt[pl] = 0.f;
           }
@@ -252,44 +253,33 @@ __device__ __forceinline__ void gate_epilogue(const RouterArgs& a, const GateSme
   }
   __syncthreads();
   if (threadIdx.x == 0) SWAPMOE_STAMP(0, 9);
-  // Per-CTA partial sums with a fixed association (lane-strided partials, then the
-  // shuffle tree), so the result does not depend on scheduling.  Only experts that some
-  // token of this tile selected are visited; the others get an exact zero.
-  const int npair = tok * k;
-  for (int e = tid; e < E; e += kGateThreads) {
-    a.cta_imp[(size_t)blockIdx.x * E + e] = 0.f;
-    if (a.cta_cnt) a.cta_cnt[(size_t)blockIdx.x * E + e] = 0.f;
-  }
-  for (int sl = tid; sl < a.K; sl += kGateThreads) a.cta_hist[(size_t)blockIdx.x * a.K + sl] = 0;
-  __syncthreads();
-  if (threadIdx.x == 0) SWAPMOE_STAMP(0, 10);
-  for (int c = 0; c * 32 < E; ++c) {
-    uint32_t present = g.s_present[c];
-    for (int n = 0; present; ++n) {
-      const int bit = __ffs(present) - 1;
-      present &= present - 1;
-      if ((n & 7) != warp) continue;                    // experts dealt round-robin to the warps
-      const int e = c * 32 + bit;
-      float sum = 0.f;
-      int hits = 0;
-      for (int p = lane; p < npair; p += 32) { sum += (g.pe[p] == e) ? g.pt[p] : 0.f; hits += (g.pe[p] == e); }
-      sum = warp_sum(sum);
-      hits = __reduce_add_sync(0xffffffffu, hits);
-      if (lane == 0) {
-        a.cta_imp[(size_t)blockIdx.x * E + e] = sum;
-        if (a.cta_cnt) a.cta_cnt[(size_t)blockIdx.x * E + e] = (float)hits;
-      }
+  // Per-CTA partial sums: a thread owns an expert (or a slot) and walks the tile's pairs in order, four per shared-memory
+  // load that all threads share - the same association as the small-batch routers, whatever the scheduling.  (A warp per
+  // selected expert, lanes over the pairs and a shuffle tree, took 14 us at 256 experts, 64 slots and 256 pairs, this takes 4.3; 3.3 -> 1.0 us at 128, 32 and 64.)
+  const int nq = tok * k >> 2;                             // tok is a multiple of 32
+  const int n_cols = E + a.K;
+  for (int c = tid; c < n_cols; c += kGateThreads) {
+    const bool by_slot = c >= E;
+    const int id = by_slot ? c - E : c;
+    const int4* ids = reinterpret_cast<const int4*>(by_slot ? g.ps : g.pe);
+    const float4* terms = reinterpret_cast<const float4*>(by_slot ? g.pm : g.pt);
+    float sum = 0.f;
+    int n = 0;
+#pragma unroll 4
+    for (int q = 0; q < nq; ++q) {
+      const int4 i4 = ids[q];
+      const float4 t4 = terms[q];
+      if (i4.x == id) { sum += t4.x; ++n; }
+      if (i4.y == id) { sum += t4.y; ++n; }
+      if (i4.z == id) { sum += t4.z; ++n; }
+      if (i4.w == id) { sum += t4.w; ++n; }
     }
-  }
-  for (int sl = warp; sl < a.K; sl += kGateThreads / 32) {
-    int c = 0;
-    float m = 0.f;
-    for (int p = lane; p < npair; p += 32) { c += (g.ps[p] == sl); m += (g.ps[p] == sl) ? g.pm[p] : 0.f; }
-    c = __reduce_add_sync(0xffffffffu, c);
-    m = warp_sum(m);
-    if (lane == 0) {
-      if (c) a.cta_hist[(size_t)blockIdx.x * a.K + sl] = c;
-      if (a.cta_mimp) a.cta_mimp[(size_t)blockIdx.x * a.K + sl] = m;
+    if (by_slot) {
+      a.cta_hist[(size_t)blockIdx.x * a.K + id] = n;
+      if (a.cta_mimp) a.cta_mimp[(size_t)blockIdx.x * a.K + id] = sum;
+    } else {
+      a.cta_imp[(size_t)blockIdx.x * E + id] = sum;
+      if (a.cta_cnt) a.cta_cnt[(size_t)blockIdx.x * E + id] = (float)n;
     }
   }
   if (threadIdx.x == 0) SWAPMOE_STAMP(0, 11);

@@ -647,3 +647,21 @@ def test_fp32_router_long_contraction(T, E, k, K):
     from harness import Case, check_against_oracle
     case = Case(_cfg(T=T, dtype=I.F32, d=4096, f=128, E=E, k=k, K=K, renorm=1, zipf_s=1.0, seed=43))
     check_against_oracle(case, case.run())
+
+
+@pytest.mark.parametrize("T,E,K,k,ext", [(70, 13, 5, 3, True), (33, 256, 64, 4, True), (45, 40, 40, 2, True),
+                                         (2400, 40, 9, 3, False), (9500, 33, 7, 1, False), (2500, 256, 5, 4, False)])
+def test_general_gate_selects_in_expert_order(T, E, K, k, ext):
+    """The gate of the routers for large batches and external logits: every length of the running list, expert counts
+    that end inside a group of eight or 32, token tiles of 32, 64 and 128 with one, two and four shares of the expert
+    range, and (external logits) complete ties, equal values on both sides of a share's edge, and +0 against -0."""
+    from harness import Case, check_against_oracle
+    cfg = _cfg(T=T, E=E, K=K, k=k, d=64, f=256, renorm=k > 1, zipf_s=1.1)
+    case = Case(cfg, s2e=np.random.default_rng(E).permutation(E)[:K])
+    lg = None
+    if ext:
+        lg = np.random.default_rng(T).integers(-2, 3, size=(T, E)).astype(np.float32)      # many equal values
+        lg[5:9] = 0.0
+        lg[6, ::2] = -0.0
+        lg[8] = -0.0
+    check_against_oracle(case, case.run(ext_logits=lg), check_logits=not ext)
