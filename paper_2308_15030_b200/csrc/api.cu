@@ -312,7 +312,7 @@ int32_t forward_impl(swapmoe_layer* L, const void* x, const float* ext_logits, v
       rc = tc_ffn_small(L->tc, L->small, c, L->xp, L->h, L->y, out, L->rows_pad_max, L->arena_in, L->arena_out,
                         L->tiles, L->n_tiles, L->row_pair, L->mgate, max_tiles, T, L->status, st, pdl,
                         &L->launches, &combined, mid);
-    } else if (mt == 2 && L->gemm_pairs > 0 && c.d_ff % 256 == 0) {
+    } else if (mt == 2 && L->gemm_pairs > 0 && tc_wide_ok(c.d_ff)) {
       // 256-row tiles: GEMM-1 always on CTA pairs (its one-CTA form pulls 48 KB per k-block); GEMM-2 on pairs for
       // very large slots, else on one CTA with two row sub-tiles (same bytes per flop, and a tile whose second
       // half is empty costs half; cfg3: 128.6 -> 126.8 us)

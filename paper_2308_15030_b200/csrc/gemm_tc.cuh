@@ -312,15 +312,18 @@ __device__ __forceinline__ void epi_load_pieces(uint32_t taddr, int c0, int gate
   }
 }
 
-// One accumulator (kOutCols output columns of this thread's row) -> global memory, 128 bytes per row and chunk.
+// One accumulator (kOutCols output columns of this thread's row) -> global memory, 128 bytes per row and chunk.  `cols` =
+// columns of the matrix from this tile's first one on: the last tile of a matrix whose width is no multiple of kOutCols
+// (but of a chunk: widths are multiples of 64) holds products with the rows of whatever lies behind the slot's weights,
+// which are not stored.
 template <int EPI, int kOutCols>
 __device__ __forceinline__ void epi_store_tile(uint32_t taddr, unsigned char* stg, int lane, float gate,
-                                               unsigned char* const (&dst)[8]) {
+                                               unsigned char* const (&dst)[8], int cols) {
   constexpr int kElem = (EPI == kTcEpiF32) ? 4 : 2;
   constexpr int kChunkCols = 128 / kElem;                  // 32 fp32 or 64 bf16 columns
   static_assert(kOutCols % kChunkCols == 0, "whole 128-byte chunks");
 #pragma unroll 1
-  for (int c0 = 0; c0 < kOutCols; c0 += kChunkCols) {
+  for (int c0 = 0; c0 < min(kOutCols, cols); c0 += kChunkCols) {
     uint4 pc[8];
     epi_load_pieces<EPI>(taddr, c0, kOutCols, gate, pc);
     if (EPI != kTcEpiF32) epi_load_pieces<EPI>(taddr, c0 + 32, kOutCols, gate, pc + 4);
@@ -567,7 +570,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           if constexpr ((kOutCols * kElem) % 128 == 0) {
             unsigned char* dst[8];
             epi_row_pointers(dst, drow_h[hf], lane, a.C, (size_t)a.ldc, (size_t)ct * kOutCols, kElem);
-            epi_store_tile<EPI, kOutCols>(taddr, epi_stage + q * kTcEpiWarpStage, lane, gate_h[hf], dst);
+            epi_store_tile<EPI, kOutCols>(taddr, epi_stage + q * kTcEpiWarpStage, lane, gate_h[hf], dst, a.ldc - ct * kOutCols);
           } else {
             // 64 bytes per row (the narrowest bf16 tiles): every thread stores its own row
             uint4 pc[4];
@@ -619,9 +622,15 @@ struct TcState {
   int only;                           // 0: both grouped GEMMs; 1 / 2: launch only GEMM-1 / GEMM-2 (measurement re-runs)
 };
 
+// Every bf16 layer: d_model and d_ff are multiples of 64, so k-blocks are whole, and the last column tile may be ragged.
+// Layers with d_model no multiple of 128 or d_ff of 256 used to run on gemm_tf32x3_kernel: d_model 704, d_ff 2240,
+// 16 slots, us per forward there / here at 9, 300, 9000 tokens: 93 / 23, 180 / 42, 1142 / 90.
 inline bool tc_supported(const swapmoe_config_t& c) {
-  return c.dtype == SWAPMOE_BF16 && c.d_model % 128 == 0 && c.d_ff % 256 == 0;
+  return c.dtype == SWAPMOE_BF16;
 }
+
+// Whether 256-column tiles suit a matrix of n columns: at most a fifth of the last tiles' width empty.
+inline bool tc_wide_ok(int n) { return (long long)(n + 255) / 256 * 256 * 4 <= 5ll * n; }
 
 // Row sub-tiles per CTA for a forward of T tokens: two when the average slot has well over
 // 128 rows (weight tiles are then shared by two sub-tiles), one for small slots (nothing to
@@ -629,13 +638,13 @@ inline bool tc_supported(const swapmoe_config_t& c) {
 inline int tc_row_subtiles(const swapmoe_config_t& c, int T, bool cta_pairs = false) {
   const long long rows_per_slot = (long long)T * c.top_k / c.K;
   // CTA pairs (tc_gemm_pair_kernel) keep two accumulator sets, so they take the very large slots
-  if (cta_pairs && rows_per_slot >= 1024 && c.d_model % 256 == 0) return 2;
-  return (rows_per_slot >= 160 && rows_per_slot < 1024 && c.d_model % 256 == 0) ? 2 : 1;
+  if (cta_pairs && rows_per_slot >= 1024) return 2;
+  return (rows_per_slot >= 160 && rows_per_slot < 1024 && tc_wide_ok(c.d_model)) ? 2 : 1;
 }
 // Whether a forward with 256-row tiles runs on CTA pairs: slots of at least `min_rows` rows on average (a
 // 256-row tile with <= 128 valid rows leaves one SM of the pair idle, so ragged small slots stay with one CTA per tile).
 inline bool tc_use_pairs(const swapmoe_config_t& c, int T, int n_pairs, int min_rows) {
-  return n_pairs > 0 && (long long)T * c.top_k / c.K >= min_rows && c.d_model % 256 == 0 && c.d_ff % 256 == 0;
+  return n_pairs > 0 && (long long)T * c.top_k / c.K >= min_rows && tc_wide_ok(c.d_model) && tc_wide_ok(c.d_ff);
 }
 
 // Automatic choice: tensor cores whenever the shape allows it.
@@ -742,14 +751,15 @@ inline cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block
 
 // Column-tile width (index into `options`) that minimises the bytes the busiest SM has to pull:
 // (tiles per SM) x (k-blocks) x (activation box + weight box).  Wide tiles amortise the
-// activation box, narrow ones give every SM work when there are few row tiles.
+// activation box, narrow ones give every SM work when there are few row tiles.  n = weight rows of a slot's matrix (both
+// matrices of SwiGLU together); the last tile may be ragged and counts in full.
 inline int tc_pick_bn(const int* options, int n_options, int n, long long row_tiles, int sm_count, int a_box_bytes,
                       int min_bn) {
   int pick = -1;
   long long best = 0;
   for (int i = 0; i < n_options; ++i) {
-    if (n % options[i] || options[i] < min_bn) continue;
-    const long long tiles = row_tiles * (n / options[i]);
+    if (options[i] < min_bn) continue;
+    const long long tiles = row_tiles * ((n + options[i] - 1) / options[i]);
     const long long per_sm = (tiles + sm_count - 1) / sm_count;
     const long long cost = per_sm * (a_box_bytes + (long long)options[i] * kTcBK * 2);
     if (pick < 0 || cost < best) { pick = i; best = cost; }

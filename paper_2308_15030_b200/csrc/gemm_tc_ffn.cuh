@@ -31,11 +31,13 @@ inline bool tc_plan_gemm1(const TcState& s, const swapmoe_config_t& c, int n_tok
   p->row_group = 1 << 30;
   if (row_group_forced > 0) p->row_group = row_group_forced;
   else if (pairs * (long long)c.d_model * 2 > (48ll << 20)) p->row_group = 32;
-  p->i1 = tc_pick_bn(kBn1Options, 3, c.d_ff, p->row_tiles_est * mt, s.sm_count, p->a_box_bytes, swiglu ? 64 : 32);
+  // (SwiGLU counts the rows of both matrices; with one matrix's the model saw half the tiles: 13 tokens, d_model 4096,
+  // d_ff 14336, four slots, GEMM-1 alone 187 us at 448 tiles on 148 SMs, 174 at 896 narrower ones)
+  p->i1 = tc_pick_bn(kBn1Options, 3, swiglu ? 2 * c.d_ff : c.d_ff, p->row_tiles_est * mt, s.sm_count, p->a_box_bytes, swiglu ? 64 : 32);
   if (p->i1 < 0) return false;
   p->bn1 = kBn1Options[p->i1];
   p->out1 = swiglu ? p->bn1 / 2 : p->bn1;
-  p->n_col_tiles = c.d_ff / p->out1;
+  p->n_col_tiles = (c.d_ff + p->out1 - 1) / p->out1;
   const long long work = (long long)max_tiles * mt * p->n_col_tiles;
   p->grid = work > s.sm_count ? s.sm_count : (int)work;
   p->stages = (kTcSmemBudget - 2048) / (kTcBM * kTcBK * 2 + p->bn1 * kTcBK * 2);
@@ -63,7 +65,7 @@ inline int32_t tc_ffn(TcState& s, const swapmoe_config_t& c, void* h, float* y, 
   g1.C = h; g1.status = status; g1.ldc = c.d_ff;
   g1.tiles = mt == 2 ? tiles128 : tiles;          // always a list of 128-row tiles
   g1.n_tiles = mt == 2 ? n_tiles128 : n_tiles;
-  g1.n_col_tiles = c.d_ff / out1;
+  g1.n_col_tiles = plan.n_col_tiles;
   g1.k_blocks = c.d_model / kTcBK;
   g1.b_rows_per_phys = swiglu ? 2 * c.d_ff : c.d_ff;
   g1.b_rows_gate = swiglu ? c.d_ff : 0;
@@ -89,12 +91,12 @@ inline int32_t tc_ffn(TcState& s, const swapmoe_config_t& c, void* h, float* y, 
 
   // ---- GEMM-2: y = h * W_out^T (or out = gate * y for top-1)
   const int i2 = mt == 2 ? 0 : tc_pick_bn(kBn2Options, 4, c.d_model, row_tiles_est, s.sm_count, a_box_bytes, 32);
-  if (i2 < 0 || c.d_model % kBn2Options[i2]) return SWAPMOE_ERR_UNSUPPORTED;
+  if (i2 < 0) return SWAPMOE_ERR_UNSUPPORTED;
   const int bn2 = kBn2Options[i2];
   TcGemmArgs g2;
   g2.C = scatter ? out : static_cast<void*>(y);
   g2.tiles = tiles; g2.n_tiles = n_tiles; g2.status = status; g2.ldc = c.d_model;
-  g2.n_col_tiles = c.d_model / bn2;
+  g2.n_col_tiles = (c.d_model + bn2 - 1) / bn2;
   g2.k_blocks = c.d_ff / kTcBK;
   g2.b_rows_per_phys = c.d_model;
   g2.b_rows_gate = 0;

@@ -275,7 +275,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * kPairBN);
         unsigned char* dst[8];
         epi_row_pointers(dst, drow, lane, a.C, (size_t)a.ldc, (size_t)ct * kOutCols, EPI == kTcEpiF32 ? 4 : 2);
-        epi_store_tile<EPI, kOutCols>(taddr, epi_stage + q * kTcEpiWarpStage, lane, gate, dst);
+        epi_store_tile<EPI, kOutCols>(taddr, epi_stage + q * kTcEpiWarpStage, lane, gate, dst, a.ldc - ct * kOutCols);
       }
       ptx::tc_fence_before();
       __syncwarp();
@@ -332,7 +332,6 @@ inline int32_t tc_ffn_pair(TcState& s, int n_pairs, const swapmoe_config_t& c, v
   const bool swiglu = c.act == SWAPMOE_ACT_SWIGLU;
   const bool scatter = c.top_k == 1;
   const int out1 = swiglu ? kPairBN / 2 : kPairBN;
-  if (c.d_ff % out1 || c.d_model % kPairBN) return SWAPMOE_ERR_UNSUPPORTED;
   const long long pairs = (long long)n_tokens * c.top_k;
   int row_group = 1 << 30;
   if (row_group_forced > 0) row_group = row_group_forced;
@@ -345,7 +344,7 @@ inline int32_t tc_ffn_pair(TcState& s, int n_pairs, const swapmoe_config_t& c, v
   TcGemmArgs g1;
   g1.C = h; g1.status = status; g1.ldc = c.d_ff;
   g1.tiles = tiles; g1.n_tiles = n_tiles;
-  g1.n_col_tiles = c.d_ff / out1;
+  g1.n_col_tiles = (c.d_ff + out1 - 1) / out1;
   g1.k_blocks = c.d_model / kTcBK;
   g1.b_rows_per_phys = swiglu ? 2 * c.d_ff : c.d_ff;
   g1.b_rows_gate = swiglu ? c.d_ff : 0;
@@ -369,7 +368,7 @@ inline int32_t tc_ffn_pair(TcState& s, int n_pairs, const swapmoe_config_t& c, v
   TcGemmArgs g2;
   g2.C = scatter ? out : static_cast<void*>(y);
   g2.tiles = tiles; g2.n_tiles = n_tiles; g2.status = status; g2.ldc = c.d_model;
-  g2.n_col_tiles = c.d_model / kPairBN;
+  g2.n_col_tiles = (c.d_model + kPairBN - 1) / kPairBN;
   g2.k_blocks = c.d_ff / kTcBK;
   g2.b_rows_per_phys = c.d_model;
   g2.b_rows_gate = 0;

@@ -25,7 +25,7 @@ constexpr int kSmSmemBudget = 196 * 1024;
 
 struct TcSmallArgs {
   TcGemmArgs g;          // C, tiles, n_tiles, status, ldc, n_col_tiles, k_blocks, b_rows_per_phys, row_pair, gate, top_k
-  int32_t kps;           // k-blocks per stage (k_blocks % kps == 0)
+  int32_t kps;           // k-blocks per stage; the last stage of a tile may reach beyond the contraction (boxes are zero-filled there)
   int32_t n_stages;
   int32_t a_tile_bytes;  // a_rows * 128: one k-block of the activation box
 };
@@ -80,7 +80,7 @@ tc_gemm_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
   ptx::tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
-  const int n_chunks = a.k_blocks / kps;
+  const int n_chunks = (a.k_blocks + kps - 1) / kps;
   // As in tc_gemm_kernel: with `early_b` the producer requests the weight boxes of its first stages before the
   // dependent-launch wait.
   int pre = 0;
@@ -192,7 +192,7 @@ tc_gemm_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
       ptx::tc_fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN);
 #pragma unroll 1
-      for (int c0 = 0; c0 < BN; c0 += 32) {
+      for (int c0 = 0; c0 < min(BN, a.ldc - ct * BN); c0 += 32) {
         uint32_t v[32];
         ptx::tmem_ld32(taddr + (uint32_t)c0, v);
         ptx::tmem_ld_wait();
@@ -257,12 +257,13 @@ inline bool tc_small_geometry(int n, int k_blocks, long long row_tiles, int sm_c
   g->bn = kBn2Options[g->bn_index];
   const int per_kb = a_tile_bytes + g->bn * kTcBK * 2;
   g->kps = 1;
-  for (int kps = 8; kps > 1; kps >>= 1)
-    if (k_blocks % kps == 0 && kps * per_kb <= 48 * 1024) { g->kps = kps; break; }
+  for (int kps = 8; kps > 1; --kps)      // the most that fits, with at most an eighth of a tile's k-blocks empty
+    if ((k_blocks + kps - 1) / kps * kps * 8 <= 9 * k_blocks && kps * per_kb <= 48 * 1024) { g->kps = kps; break; }
   const int stage = g->kps * per_kb;
   int ns = (kSmSmemBudget - kTcBM * kTcBK * 2 - 2048) / stage;
   if (ns > kSmMaxStages) ns = kSmMaxStages;
-  if (ns > k_blocks / g->kps) ns = k_blocks / g->kps > 1 ? k_blocks / g->kps : 2;
+  const int chunks = (k_blocks + g->kps - 1) / g->kps;
+  if (ns > chunks) ns = chunks > 1 ? chunks : 2;
   if (ns < 2) return false;
   g->n_stages = ns;
   g->smem_bytes = ns * stage + kTcBM * kTcBK * 2 + 2048;
@@ -333,7 +334,7 @@ inline int32_t tc_ffn_small(TcState& s, TcSmallCache& cache, const swapmoe_confi
   const bool scatter = c.top_k == 1;
   TcSmallArgs a1;
   a1.g.C = h; a1.g.tiles = tiles; a1.g.n_tiles = n_tiles; a1.g.status = status; a1.g.ldc = c.d_ff;
-  a1.g.n_col_tiles = c.d_ff / cache.g1.bn; a1.g.k_blocks = c.d_model / kTcBK;
+  a1.g.n_col_tiles = (c.d_ff + cache.g1.bn - 1) / cache.g1.bn; a1.g.k_blocks = c.d_model / kTcBK;
   a1.g.b_rows_per_phys = c.d_ff; a1.g.b_rows_gate = 0; a1.g.a_box_bytes = a_tile; a1.g.row_group = 1 << 30;
   a1.g.row_pair = nullptr; a1.g.gate = nullptr; a1.g.top_k = c.top_k; a1.g.early_b = 0;
   a1.kps = cache.g1.kps; a1.n_stages = cache.g1.n_stages; a1.a_tile_bytes = a_tile;
@@ -348,7 +349,7 @@ inline int32_t tc_ffn_small(TcState& s, TcSmallCache& cache, const swapmoe_confi
   TcSmallArgs a2;
   a2.g.C = scatter ? out : static_cast<void*>(y);
   a2.g.tiles = tiles; a2.g.n_tiles = n_tiles; a2.g.status = status; a2.g.ldc = c.d_model;
-  a2.g.n_col_tiles = c.d_model / cache.g2.bn; a2.g.k_blocks = c.d_ff / kTcBK;
+  a2.g.n_col_tiles = (c.d_model + cache.g2.bn - 1) / cache.g2.bn; a2.g.k_blocks = c.d_ff / kTcBK;
   a2.g.b_rows_per_phys = c.d_model; a2.g.b_rows_gate = 0; a2.g.a_box_bytes = a_tile; a2.g.row_group = 1 << 30;
   a2.g.row_pair = row_pair; a2.g.gate = mgate; a2.g.top_k = c.top_k; a2.g.early_b = 1;
   a2.kps = cache.g2.kps; a2.n_stages = cache.g2.n_stages; a2.a_tile_bytes = a_tile;

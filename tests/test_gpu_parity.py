@@ -665,3 +665,26 @@ def test_general_gate_selects_in_expert_order(T, E, K, k, ext):
         lg[6, ::2] = -0.0
         lg[8] = -0.0
     check_against_oracle(case, case.run(ext_logits=lg), check_logits=not ext)
+
+
+@pytest.mark.parametrize("dtype,T,d,f,K,k,act", [
+    (I.BF16, 40, 704, 448, 5, 1, I.ACT_RELU),       # small-batch kernels: ragged column tiles, 11 and 7 k-blocks
+    (I.BF16, 7, 64, 64, 3, 1, I.ACT_RELU),          # one k-block, one tile wider than the matrix
+    (I.BF16, 300, 320, 832, 5, 1, I.ACT_RELU),      # one CTA per 128-row tile, both widths ragged
+    (I.BF16, 90, 192, 320, 4, 2, I.ACT_SWIGLU),
+    (I.BF16, 1500, 704, 448, 5, 1, I.ACT_RELU),     # 256-row tiles: GEMM-1 on CTA pairs, GEMM-2 on two row sub-tiles
+    (I.BF16, 900, 448, 704, 5, 2, I.ACT_SWIGLU),
+    (I.BF16, 900, 448, 320, 5, 2, I.ACT_RELU),      # 256-row tiles with a d_ff too narrow for wide column tiles
+    (I.BF16, 3000, 448, 960, 2, 1, I.ACT_RELU),     # both GEMMs on CTA pairs
+    (I.BF16, 1600, 960, 448, 2, 2, I.ACT_SWIGLU),
+    (I.F32, 100, 192, 448, 5, 1, I.ACT_RELU),       # fp32, weights on the MMA rows
+    (I.F32, 900, 320, 704, 4, 1, I.ACT_RELU),       # fp32, tokens on the MMA rows
+    (I.F32, 150, 64, 192, 3, 2, I.ACT_SWIGLU),
+])
+def test_ragged_column_tiles(dtype, T, d, f, K, k, act):
+    """d_model and d_ff that are multiples of 64 but not of a tile's width: the last column tile of every matrix is
+    multiplied with what lies behind the slot's weights and must not store it."""
+    from harness import Case, check_against_oracle
+    cfg = _cfg(T=T, dtype=dtype, d=d, f=f, E=8, K=K, k=k, act=act, renorm=k > 1)
+    case = Case(cfg, phys=list(range(1, K)) + [0])
+    check_against_oracle(case, case.run())
