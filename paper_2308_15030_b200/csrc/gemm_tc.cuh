@@ -288,7 +288,7 @@ __device__ __forceinline__ void epi_load_pieces(uint32_t taddr, int c0, int gate
 #pragma unroll
     for (int i = 0; i < 32; ++i) {
       const float x1 = __uint_as_float(v[i]);
-      v[i] = __float_as_uint(x1 / (1.f + __expf(-x1)) * __uint_as_float(g[i]));
+      v[i] = __float_as_uint(silu_from_exp(x1, __expf(-x1)) * __uint_as_float(g[i]));
     }
   } else {
     ptx::tmem_ld_wait();
