@@ -647,6 +647,17 @@ inline bool tc_use_pairs(const swapmoe_config_t& c, int T, int n_pairs, int min_
   return n_pairs > 0 && (long long)T * c.top_k / c.K >= min_rows && tc_wide_ok(c.d_model) && tc_wide_ok(c.d_ff);
 }
 
+// Whether GEMM-2 of such a forward runs on CTA pairs although its slots are smaller than that.  One CTA with two row
+// sub-tiles fills tensor memory with one accumulator set, so a tile's epilogue is not overlapped, but a tile whose second
+// half is empty costs it half.  Alone, one CTA / pairs, us: short contractions, d_ff 512 59 / 49, 768 22.5 / 20.9,
+// 1024 117 / 95, 2048 29 / 24.5; long ones, 3072 46 / 51, 4096 113 / 123; and where the tiles fit one round of pairs two
+// SMs work on each instead of one: d_ff 3584, 32 tiles 44 / 27.
+inline bool tc_gemm2_on_pairs(const swapmoe_config_t& c, int T, int n_pairs) {
+  const long long rows = (long long)T * c.top_k;
+  const long long tiles = (rows / (2 * kTcBM) + (rows < c.K ? rows : c.K) / 2 + 1) * ((c.d_model + 255) / 256);
+  return c.d_ff <= 2048 || tiles <= n_pairs;
+}
+
 // Automatic choice: tensor cores whenever the shape allows it.
 inline bool tc_selected(int path, const swapmoe_config_t& c, int /*T*/) {
   if (path == 1) return false;
