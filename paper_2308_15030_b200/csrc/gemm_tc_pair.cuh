@@ -55,8 +55,12 @@ __device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* m
       ::"r"(smem_u32(dst)), "l"(map), "r"(bar_cluster_addr), "r"(c0), "r"(c1)
       : "memory");
 }
+// Relaxed: the arrival says that the accumulator has been READ (tcgen05.wait::ld has returned), nothing about the stores
+// that follow from it.  With .release every epilogue warp waited here until its tile's global stores had been performed,
+// behind the operand loads in flight (24044 rows,
+// d_model 1024, d_ff 512, y in fp32: GEMM-2 alone 49 -> 42 us; 8192 rows 768 x 3072: GEMM-1 49.5 -> 46.0).
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster_addr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr) : "memory");
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr) : "memory");
 }
 __device__ __forceinline__ void tmem_alloc_pair(uint32_t* dst_smem, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst_smem)),
