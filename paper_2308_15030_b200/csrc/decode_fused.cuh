@@ -244,6 +244,14 @@ __device__ __forceinline__ void mma_bf16_16x8x16(float (&c)[4], uint32_t a0, uin
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
       : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
+// Draws a ticket: what this thread has seen written (its own CTA's partial rows, behind a block barrier) is released with
+// it, and what the earlier holders released may be read by whoever it orders next.
+__device__ __forceinline__ unsigned dec_draw_ticket(unsigned* t) {
+  unsigned v;
+  asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(v) : "l"(t) : "memory");
+  return v;
+}
+
 __device__ __forceinline__ uint32_t lds32(const unsigned char* p) { return *reinterpret_cast<const uint32_t*>(p); }
 
 // Waits for wave w (buffer w & 1, its barrier's phase (w >> 1) & 1): thread 0 polls (bounded), the
@@ -304,6 +312,67 @@ __device__ __noinline__ void dec_wave_dots(const unsigned char* st, int rows, in
 #pragma unroll
     for (int w = 0; w < kDecWarps; ++w) s += red[(w * 32 + r) * 8 + n];
     if (r < rows && n < nn) dst[n * dst_stride + r] = s;
+  }
+  __syncthreads();
+}
+
+// All logits of the CTA in ONE pass when the router matrix fits the two wave buffers (E <= 2 waves of rows):
+// a warp owns a tile of 16 experts (all NT token tiles of it: the router-matrix fragments are read once and
+// feed NT mma) and a contiguous share of the contraction; the 16 / tiles shares of a tile are added in order.
+// Per CTA that is one pair of barriers and a 4-way sum for 64 experts x 16 tokens, where the wave-by-wave form
+// (every wave's contraction split over all 16 warps) pays a 16-way sum and two barriers per wave.
+// slog[token * (kMaxE + 1) + expert] receives the logits.
+template <int NT>
+__device__ __forceinline__ void rs_dots_resident(const unsigned char* ring, int E, int RW, int d, const unsigned char* xs,
+                                                 int n_tok, float* red, float* slog) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  const int pitch = d * 2 + kDecRowPad;
+  const int MT = (E + 15) >> 4;                 // 16-expert row tiles (<= 4)
+  int tiles_p2 = 1;
+  while (tiles_p2 < MT) tiles_p2 <<= 1;
+  const int S = kDecWarps / tiles_p2;           // shares of the contraction per tile (>= 4)
+  const int m = warp & (tiles_p2 - 1), part = warp / tiles_p2;
+  if (m < MT) {
+    const int row0 = m * 16;                    // first expert of the tile; wave row0 / RW, row row0 % RW inside it
+    const unsigned char* ap0 = ring + (row0 / RW) * kDecHalfBytes + ((row0 % RW) + g) * pitch + t * 4;
+    const unsigned char* xrow[NT];
+#pragma unroll
+    for (int j = 0; j < NT; ++j) xrow[j] = xs + min(8 * j + g, n_tok - 1) * pitch + t * 4;
+    const int nks = d / 16, ks0 = part * nks / S, ks1 = (part + 1) * nks / S;
+    float acc[NT][4];
+#pragma unroll
+    for (int j = 0; j < NT; ++j)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[j][q] = 0.f;
+#pragma unroll 4
+    for (int ks = ks0; ks < ks1; ++ks) {
+      const int kb = ks * 32;
+      const uint32_t a0 = lds32(ap0 + kb), a1 = lds32(ap0 + 8 * pitch + kb), a2 = lds32(ap0 + kb + 16),
+                     a3 = lds32(ap0 + 8 * pitch + kb + 16);
+#pragma unroll
+      for (int j = 0; j < NT; ++j) {            // NT independent accumulators: NT chains of dependent mma
+        const uint32_t b0 = lds32(xrow[j] + kb), b1 = lds32(xrow[j] + kb + 16);
+        mma_bf16_16x8x16(acc[j], a0, a1, a2, a3, b0, b1);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < NT; ++j) {
+      float* rp = red + (((part * MT + m) * NT + j) * 16 + g) * 8 + 2 * t;
+      *reinterpret_cast<float2*>(rp) = make_float2(acc[j][0], acc[j][1]);
+      *reinterpret_cast<float2*>(rp + 8 * 8) = make_float2(acc[j][2], acc[j][3]);
+    }
+  }
+  if (tid == 0) SWAPMOE_STAMP(0, 12);
+  __syncthreads();
+  if (tid == 0) SWAPMOE_STAMP(0, 13);
+  const int n_tiles = MT * NT;
+  for (int o = tid; o < n_tiles * 128; o += kDecThreads) {
+    const int tl = o >> 7, r = (o >> 3) & 15, c = o & 7;      // tl = m * NT + j
+    float sum = 0.f;
+    for (int p = 0; p < S; ++p) sum += red[((p * n_tiles + tl) * 16 + r) * 8 + c];
+    const int mm = tl / NT, j = tl - mm * NT;
+    const int e = mm * 16 + r, tok = 8 * j + c;
+    if (e < E && tok < n_tok) slog[tok * (kMaxE + 1) + e] = sum;
   }
   __syncthreads();
 }
@@ -427,6 +496,13 @@ decode_fused_kernel(const __grid_constant__ CUtensorMap tmWo, const DecodeArgs a
     }
   }
   bool alive = true;
+  if (n_rw > 0 && n_rw <= 2 && RW % 16 == 0) {
+    // the whole router matrix sits in the two wave buffers: one pass over all experts (wave by wave, every wave's
+    // contraction over all sixteen warps, costs a 16-way sum and two barriers per wave: twelve layers at one token 224.5
+    // us per step, in one pass and with one fence per ticket less 210.6)
+    for (int w = 0; w < n_rw && alive; ++w) alive = dec_wait_wave(bars, w, R, a.status, 21);
+    if (alive) rs_dots_resident<1>(ring, E, RW, d, xs, T, red, slog);
+  } else {
 #pragma unroll 1
   for (int w = 0; w < n_rw; ++w) {
     // router wave w holds rows w*RW .. of Wr
@@ -436,6 +512,7 @@ decode_fused_kernel(const __grid_constant__ CUtensorMap tmWo, const DecodeArgs a
       ptx::fence_proxy_async();
       issue_rows(w + 2, a.Wr + (size_t)(w + 2) * RW * d, min(RW, E - (w + 2) * RW));
     }
+  }
   }
   __syncthreads();
   if (tid == 0) SWAPMOE_STAMP(0, 3);
@@ -725,10 +802,7 @@ decode_fused_kernel(const __grid_constant__ CUtensorMap tmWo, const DecodeArgs a
     // before its fence (fences are cumulative), and its second fence orders the ticket before the
     // reads of the other CTAs' rows (L2 loads below).
     if (tid == 0) {
-      __threadfence();
-      const bool last = atomicAdd(&a.tickets[s * n_groups + grp], 1u) == (unsigned)(n_sets - 1);
-      __threadfence();
-      R->last = last;
+      R->last = dec_draw_ticket(&a.tickets[s * n_groups + grp]) == (unsigned)(n_sets - 1);
     }
     __syncthreads();
     if (tid == 0) SWAPMOE_STAMP(0, 11);
@@ -771,10 +845,7 @@ decode_fused_kernel(const __grid_constant__ CUtensorMap tmWo, const DecodeArgs a
       if (tid == 0) {
         SWAPMOE_STAMP(0, 12);
         a.tickets[s * n_groups + grp] = 0u;
-        __threadfence();
-        const bool last = atomicAdd(&a.tickets[K * n_groups], 1u) == (unsigned)(R->n_touched * n_groups - 1);
-        __threadfence();
-        R->last = last;
+        R->last = dec_draw_ticket(&a.tickets[K * n_groups]) == (unsigned)(R->n_touched * n_groups - 1);
       }
       __syncthreads();
       if (R->last) {
