@@ -17,6 +17,7 @@
 #include "gemm_tc.cuh"
 #include "gemm_tc_f32.cuh"
 #include "gemm_tc_pair.cuh"
+#include "gemm_tc_f32_pair.cuh"
 #include "gemm_tc_ffn.cuh"
 #include "gemm_tc_small.cuh"
 #include "permute.cuh"
@@ -80,6 +81,7 @@ struct swapmoe_layer {
   int32_t router_tok;          // 0 = automatic token-tile size of the tensor-core router, else 32/64/128
   bool prefetch;               // pull resident weights into L2 from the router kernel
   long long l2_prefetch_bytes; // how much of them (L2 capacity minus head room)
+  int pair32_min_rows;         // fp32 layers on CTA pairs: 0 = tc_f32_use_pairs decides, else from this many rows per slot
   bool fp32_swap;              // fp32 layers: swapped-operand GEMM for small slots
   int prefetch_min_pairs;      // ... when the batch has at least this many HALF pairs per slot (SWAPMOE_PREFETCH_MIN_PAIRS)
   void* const* stage_events;   // 7 cudaEvent_t of the forward being enqueued, or nullptr
@@ -188,7 +190,11 @@ int32_t forward_impl(swapmoe_layer* L, const void* x, const float* ext_logits, v
   // fp32 layers whose slots hold well under 128 rows on average: weights on the MMA's rows, the slot's tokens on its
   // columns (64-token tiles), so that no tensor time goes to empty rows (SWAPMOE_FP32_SWAP=0: never)
   const bool swap32 = use_tc32 && L->tc32.swap_ok && L->fp32_swap && (long long)n_pairs < 96ll * c.K;
-  const int tile_rows = use_tc ? kTcBM * mt : (use_tc32 ? (swap32 ? kF32SwapTok : kTcBM) : kMmaBM);
+  // ... and whose slots hold well over 128 rows: 256-row tiles on CTA pairs (fewer operand bytes per product)
+  const bool pair32 = use_tc32 && !swap32 && L->tc32.n_pairs > 0 &&
+                      (L->pair32_min_rows > 0 ? (long long)n_pairs >= (long long)L->pair32_min_rows * c.K
+                                              : tc_f32_use_pairs(c, L->tc32.n_pairs, L->sm_count, n_pairs, L->y_copies));
+  const int tile_rows = use_tc ? kTcBM * mt : (use_tc32 ? (swap32 ? kF32SwapTok : pair32 ? 2 * kTcBM : kTcBM) : kMmaBM);
   const int max_tiles = (n_pairs + tile_rows - 1) / tile_rows + c.K;
 
   RouterArgs ra;
@@ -329,7 +335,10 @@ int32_t forward_impl(swapmoe_layer* L, const void* x, const float* ext_logits, v
   } else if (use_tc32) {
     cudaEvent_t mid = L->stage_events ? static_cast<cudaEvent_t>(L->stage_events[4]) : nullptr;
     L->tc32.only = rerun;
-    const int32_t rc = tc_ffn_f32(L->tc32, c, L->h, L->y, (long long)L->rows_pad_max * c.d_model, L->y_copies, L->tiles,
+    const int32_t rc = pair32
+        ? tc_ffn_f32_pair(L->tc32, c, L->h, L->y, (long long)L->rows_pad_max * c.d_model, L->y_copies, L->tiles, L->n_tiles,
+                          max_tiles, T, L->status, st, pdl, &L->launches, &y_split, mid)
+        : tc_ffn_f32(L->tc32, c, L->h, L->y, (long long)L->rows_pad_max * c.d_model, L->y_copies, L->tiles,
                                   L->n_tiles, max_tiles, T, L->status, st, pdl, &L->launches, &y_split, mid, swap32);
     L->tc32.only = 0;
     if (rc != SWAPMOE_OK) return rc;
@@ -479,6 +488,8 @@ int32_t swapmoe_create(swapmoe_layer_t** out, const swapmoe_config_t* cfg) {
     L->prefetch = L->l2_prefetch_bytes > 0;
     env = std::getenv("SWAPMOE_FP32_SWAP");             // SWAPMOE_FP32_SWAP=0: fp32 layers always on 128-token tiles
     L->fp32_swap = !(env && env[0] == '0');
+    env = std::getenv("SWAPMOE_PAIR32_MIN_ROWS");       // rows per slot from which fp32 layers run on CTA pairs (0: automatic)
+    L->pair32_min_rows = env ? std::max(0, std::atoi(env)) : 0;
     env = std::getenv("SWAPMOE_PREFETCH_MIN_PAIRS");
     L->prefetch_min_pairs = env ? std::max(1, std::atoi(env)) : 1;
   }
@@ -602,6 +613,8 @@ int32_t swapmoe_create(swapmoe_layer_t** out, const swapmoe_config_t* cfg) {
     if (ok && c.dtype == SWAPMOE_F32 && !(env && env[0] == '0')) {
       L->encode32 = tc_get_encoder();
       ok = tc_f32_init(L->tc32, L->encode32, c, L->xp, L->h, L->rows_pad_max, L->sm_count) == SWAPMOE_OK;
+      const char* envp = std::getenv("SWAPMOE_PAIR_GEMM");
+      if (ok && L->tc32.enabled && !(envp && envp[0] == '0')) L->tc32.n_pairs = tc_f32_pair_init(L->sm_count);
     }
   }
   if (L->tc.encode == nullptr) L->decode_path = false;     // its W_out loads need a tensor map

@@ -103,26 +103,29 @@ __device__ __forceinline__ void split_bf16_pair(uint32_t x0, uint32_t x1, uint32
 // accumulator columns [c0, c0 + 32) of this thread's TMEM lane -> activation -> eight 16-byte pieces of fp32
 template <int EPI>
 __device__ __forceinline__ void epi_load_pieces_f32(uint32_t taddr, int c0, int gate_cols, uint4* pc) {
-  uint32_t v[32];
-  ptx::tmem_ld32(taddr + (uint32_t)c0, v);
-  if (EPI == kTcEpiSwigluF32) {
-    uint32_t g[32];
-    ptx::tmem_ld32(taddr + (uint32_t)(c0 + gate_cols), g);
-    ptx::tmem_ld_wait();
 #pragma unroll
-    for (int i = 0; i < 32; ++i) {
-      const float x1 = __uint_as_float(v[i]);
-      v[i] = __float_as_uint(silu_from_exp(x1, expf(-x1)) * __uint_as_float(g[i]));
-    }
-  } else {
-    ptx::tmem_ld_wait();
-    if (EPI == kTcEpiReluF32) {
+  for (int hb = 0; hb < 2; ++hb) {                 // sixteen columns at a time: both matrices' of SwiGLU fit the registers
+    uint32_t v[16];
+    ptx::tmem_ld16(taddr + (uint32_t)(c0 + 16 * hb), v);
+    if (EPI == kTcEpiSwigluF32) {
+      uint32_t g[16];
+      ptx::tmem_ld16(taddr + (uint32_t)(c0 + 16 * hb + gate_cols), g);
+      ptx::tmem_ld_wait();
 #pragma unroll
-      for (int i = 0; i < 32; ++i) v[i] = __float_as_uint(fmaxf(__uint_as_float(v[i]), 0.f));
+      for (int i = 0; i < 16; ++i) {
+        const float x1 = __uint_as_float(v[i]);
+        v[i] = __float_as_uint(silu_from_exp(x1, expf(-x1)) * __uint_as_float(g[i]));
+      }
+    } else {
+      ptx::tmem_ld_wait();
+      if (EPI == kTcEpiReluF32) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = __float_as_uint(fmaxf(__uint_as_float(v[i]), 0.f));
+      }
     }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) pc[4 * hb + i] = make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
   }
-#pragma unroll
-  for (int i = 0; i < 8; ++i) pc[i] = make_uint4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
 }
 
 // kSwap = false: A (128 rows, split into tensor memory) = token rows of a slot tile, B (shared memory) = 128 weight
@@ -443,6 +446,8 @@ struct TcF32State {
   CUtensorMap map_xp, map_h;          // activations, box 32 x 128
   CUtensorMap map_win, map_wout;      // weights flattened to 2D; box 32 x 128 (64 for SwiGLU's W1 / W3)
   CUtensorMap map_xp_tok, map_h_tok;  // activations, box 32 x kF32SwapTok (swapped form)
+  CUtensorMap map_win_pair, map_wout_pair;   // weights, box 32 x 96 (CTA-pair kernel)
+  int n_pairs;                        // CTA pairs available to it (0: not used)
   bool swap_ok;                       // the swapped form is available (ReLU layers)
   int only;                           // 0: both grouped GEMMs; 1 / 2: launch only GEMM-1 / GEMM-2 (measurement re-runs)
 };
@@ -481,6 +486,7 @@ inline int32_t tc_f32_init(TcF32State& s, PFN_encodeTiled enc, const swapmoe_con
   s.enabled = false;
   s.arena_bound = false;
   s.only = 0;
+  s.n_pairs = 0;
   s.sm_count = sm_count;
   if (!enc || !tc_f32_supported(c)) return SWAPMOE_OK;
   if (!tc_encode_2d_f32(enc, &s.map_xp, xp, (uint64_t)rows_pad, (uint64_t)c.d_model, kTcBM) ||
@@ -514,6 +520,9 @@ inline int32_t tc_f32_bind_arena(TcF32State& s, PFN_encodeTiled enc, const swapm
   if (!tc_encode_2d_f32(enc, &s.map_win, arena_in, (uint64_t)P * nin * c.d_ff, (uint64_t)c.d_model,
                         (uint32_t)(kF32BN / nin)) ||
       !tc_encode_2d_f32(enc, &s.map_wout, arena_out, (uint64_t)P * c.d_model, (uint64_t)c.d_ff, (uint32_t)kF32BN))
+    return SWAPMOE_ERR_CUDA;
+  if (!tc_encode_2d_f32(enc, &s.map_win_pair, arena_in, (uint64_t)P * nin * c.d_ff, (uint64_t)c.d_model, 96u) ||
+      !tc_encode_2d_f32(enc, &s.map_wout_pair, arena_out, (uint64_t)P * c.d_model, (uint64_t)c.d_ff, 96u))
     return SWAPMOE_ERR_CUDA;
   s.arena_bound = true;
   return SWAPMOE_OK;

@@ -688,3 +688,24 @@ def test_ragged_column_tiles(dtype, T, d, f, K, k, act):
     cfg = _cfg(T=T, dtype=dtype, d=d, f=f, E=8, K=K, k=k, act=act, renorm=k > 1)
     case = Case(cfg, phys=list(range(1, K)) + [0])
     check_against_oracle(case, case.run())
+
+
+@pytest.mark.parametrize("T,d,f,K,k,act,min_rows", [
+    (1500, 256, 512, 5, 1, I.ACT_RELU, "1"),        # sliced contraction of GEMM-2, ragged halves and absent ones
+    (700, 64, 64, 3, 1, I.ACT_RELU, "1"),           # two k-blocks, one column tile wider than the matrix
+    (800, 192, 384, 5, 2, I.ACT_SWIGLU, "1"),       # whole column tiles
+    (1300, 448, 704, 4, 2, I.ACT_SWIGLU, "1"),      # ragged ones, SwiGLU's narrower last tile
+    (6, 128, 256, 3, 2, I.ACT_SWIGLU, "1"),         # tiles of a row or two: the odd CTA has nothing to store
+    (9000, 128, 320, 6, 1, I.ACT_RELU, None),       # the default rule; more items than pairs
+])
+def test_fp32_cta_pairs(monkeypatch, T, d, f, K, k, act, min_rows):
+    """fp32 layers with well over 128 rows per slot: 256 x 192 tiles on CTA pairs, both operands split by both CTAs."""
+    from harness import Case, check_against_oracle
+    if min_rows:
+        monkeypatch.setenv("SWAPMOE_PAIR32_MIN_ROWS", min_rows)
+        monkeypatch.setenv("SWAPMOE_FP32_SWAP", "0")
+    cfg = _cfg(T=T, dtype=I.F32, d=d, f=f, E=12, K=K, k=k, act=act, renorm=k > 1, zipf_s=1.3)
+    case = Case(cfg)
+    res = check_against_oracle(case, case.run())
+    assert res["out_rel_err"] <= 1e-4
+    assert np.array_equal(case.run(), case.run())
