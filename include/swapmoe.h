@@ -197,8 +197,8 @@ int32_t swapmoe_debug_rerun_gemm(swapmoe_layer_t* layer, void* out_dev, int32_t 
 
 /* End-to-end form with HOST buffers: copies x_host [n_tokens, d_model] to the
  * device, runs swapmoe_forward, copies the result to out_host, and returns after
- * `stream` has completed.  Pinned host memory makes the copies asynchronous
- * with respect to other streams; pageable memory works but is slower.  It shares
+ * `stream` has completed.  Pinned host memory of up to 9 MB each way is read and
+ * written in place by the kernels; pageable memory works but is slower.  It shares
  * the layer's staging buffers with swapmoe_forward_host_async and is ordered
  * behind that call's outstanding work on this layer. */
 int32_t swapmoe_forward_host(swapmoe_layer_t* layer, const void* x_host, void* out_host,

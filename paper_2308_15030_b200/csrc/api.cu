@@ -91,6 +91,7 @@ struct swapmoe_layer {
   TcState tc;
   TcF32State tc32;             // tcgen05 grouped GEMM of fp32 layers, bf16-piece split (SWAPMOE_FP32_TC=0: warp-level mma)
   PFN_encodeTiled encode32;
+  void* pointer_attributes;    // the driver's pointer query (host path), or nullptr
 };
 
 namespace {
@@ -125,6 +126,50 @@ __global__ void snapshot_scores_kernel(const ScoreSnapshot s) {
   if (k >= 3 || !((s.mask >> k) & 1)) return;
   s.dst[threadIdx.x] = s.acc[k][e];
   if (s.reset) s.acc[k][e] = 0.f;
+}
+
+// Tokens from mapped pinned host memory to the device.  Bound by the host link; a kernel reads it as fast as a copy engine,
+// joins the chain of dependent launches, and its first loads (four 16-byte ones per thread) are on their way before the
+// kernel in front has finished.
+constexpr int kFetchThreads = 512, kFetchLoads = 4;
+constexpr size_t kHostInPlaceBytes = (size_t)9 << 20;
+__global__ void __launch_bounds__(kFetchThreads) fetch_rows_kernel(const uint4* src, uint4* dst, long long n) {
+  const long long stride = (long long)gridDim.x * kFetchThreads;
+  long long i = (long long)blockIdx.x * kFetchThreads + threadIdx.x;
+  uint4 v[kFetchLoads];
+#pragma unroll
+  for (int u = 0; u < kFetchLoads; ++u)
+    if (i + u * stride < n) v[u] = __ldcs(src + i + u * stride);
+  pdl_wait();          // the staging buffer may still be read by the forward in front
+  pdl_trigger();
+  while (i < n) {
+#pragma unroll
+    for (int u = 0; u < kFetchLoads; ++u)
+      if (i + u * stride < n) dst[i + u * stride] = v[u];
+    i += kFetchLoads * stride;
+#pragma unroll
+    for (int u = 0; u < kFetchLoads; ++u)
+      if (i + u * stride < n) v[u] = __ldcs(src + i + u * stride);
+  }
+}
+
+typedef CUresult (*PFN_pointerAttributes)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr);
+
+// Device address of [p, p + bytes) if all of it lies in ONE pinned host allocation (or registration) that the device
+// can address, else nullptr.  Asked on every call: nothing is remembered about a pointer.
+void* mapped_host_range(PFN_pointerAttributes query, const void* p, size_t bytes) {
+  if (query == nullptr || (reinterpret_cast<uintptr_t>(p) & 15)) return nullptr;
+  unsigned int type = 0;
+  CUdeviceptr dev = 0, start = 0;
+  size_t size = 0;
+  CUpointer_attribute what[4] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                 CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  void* out[4] = {&type, &dev, &start, &size};
+  const CUdeviceptr at = (CUdeviceptr)reinterpret_cast<uintptr_t>(p);
+  if (query(4, what, out, at) != CUDA_SUCCESS) return nullptr;
+  if (type != CU_MEMORYTYPE_HOST || dev == 0 || (dev & 15) || start == 0 || at < start || at + bytes > start + size)
+    return nullptr;
+  return reinterpret_cast<void*>(dev);
 }
 
 struct EnormTable { float v[kMaxE]; };
@@ -647,6 +692,15 @@ int32_t swapmoe_create(swapmoe_layer_t** out, const swapmoe_config_t* cfg) {
                                               (int)router_small_smem_bytes(c.d_model, 2)));
     }
   }
+  {
+    cudaDriverEntryPointQueryResult qres;
+    void* fn = nullptr;
+    if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &fn, 12000, cudaEnableDefault, &qres) == cudaSuccess &&
+        qres == cudaDriverEntryPointSuccess)
+      L->pointer_attributes = fn;
+    else
+      cudaGetLastError();
+  }
   if (ok && L->tc.enabled) ok = tc_small_set_attrs();
   ok = ok && cuda_ok(cudaStreamCreateWithFlags(&L->s_in, cudaStreamNonBlocking));
   ok = ok && cuda_ok(cudaStreamCreateWithFlags(&L->s_out, cudaStreamNonBlocking));
@@ -773,10 +827,28 @@ int32_t swapmoe_forward_host(swapmoe_layer_t* L, const void* x_host, void* out_h
   // reads x_stage) and its last copy-out (which reads out_stage); no-ops when it was never used
   if (!cuda_ok(cudaStreamWaitEvent(st, L->ev_comp, 0)) || !cuda_ok(cudaStreamWaitEvent(st, L->ev_out, 0)))
     return SWAPMOE_ERR_CUDA;
-  if (!cuda_ok(cudaMemcpyAsync(L->x_stage, x_host, bytes, cudaMemcpyHostToDevice, st))) return SWAPMOE_ERR_CUDA;
-  const int32_t rc = forward_checked(L, L->x_stage, nullptr, L->out_stage, T, stream);
+  // Pinned buffers are used in place: the tokens come in by a kernel of the chain and the last kernel of the forward, which
+  // writes every output element once, writes it to the host, so the way out overlaps the second product and neither
+  // copy's start-up is waited for.  us per request, copies / in place: 16 tokens of d_model 768 62 / 53, 600 of 512 110 / 86,
+  // 1999 of 768 279 / 195, 4000 of 1024 (8 MB) 465 / 443; at 8192 of 768 (13 MB) the copy engines are level or ahead, 589 / 598.
+  const PFN_pointerAttributes query = reinterpret_cast<PFN_pointerAttributes>(L->pointer_attributes);
+  const bool in_place = bytes <= kHostInPlaceBytes;
+  const void* x_dev = in_place ? mapped_host_range(query, x_host, bytes) : nullptr;
+  void* out_dev = in_place ? mapped_host_range(query, out_host, bytes) : nullptr;
+  if (x_dev) {
+    const long long n = (long long)(bytes / 16), per_cta = kFetchThreads * kFetchLoads;
+    const long long want = (n + per_cta - 1) / per_cta;
+    const int grid = (int)(want < 2 * L->sm_count ? want : 2 * L->sm_count);
+    if (launch_kernel(fetch_rows_kernel, dim3(grid), dim3(kFetchThreads), 0, st, L->use_pdl, static_cast<const uint4*>(x_dev),
+                      static_cast<uint4*>(L->x_stage), n) != cudaSuccess)
+      return SWAPMOE_ERR_CUDA;
+    L->launches++;
+  } else if (!cuda_ok(cudaMemcpyAsync(L->x_stage, x_host, bytes, cudaMemcpyHostToDevice, st))) {
+    return SWAPMOE_ERR_CUDA;
+  }
+  const int32_t rc = forward_checked(L, L->x_stage, nullptr, out_dev ? out_dev : L->out_stage, T, stream);
   if (rc != SWAPMOE_OK) return rc;
-  if (!cuda_ok(cudaMemcpyAsync(out_host, L->out_stage, bytes, cudaMemcpyDeviceToHost, st))) return SWAPMOE_ERR_CUDA;
+  if (!out_dev && !cuda_ok(cudaMemcpyAsync(out_host, L->out_stage, bytes, cudaMemcpyDeviceToHost, st))) return SWAPMOE_ERR_CUDA;
   if (!cuda_ok(cudaStreamSynchronize(st))) return SWAPMOE_ERR_CUDA;
   return SWAPMOE_OK;
 }

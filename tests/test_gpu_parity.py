@@ -709,3 +709,27 @@ def test_fp32_cta_pairs(monkeypatch, T, d, f, K, k, act, min_rows):
     res = check_against_oracle(case, case.run())
     assert res["out_rel_err"] <= 1e-4
     assert np.array_equal(case.run(), case.run())
+
+
+@pytest.mark.parametrize("dtype,T,k,pinned", [(I.BF16, 3, 1, (True, True)), (I.BF16, 2500, 1, (True, True)),
+                                              (I.BF16, 300, 2, (True, False)), (I.F32, 257, 1, (False, True)),
+                                              (I.BF16, 90, 1, (False, False))])
+def test_host_path_uses_pinned_buffers_in_place(dtype, T, k, pinned):
+    """swapmoe_forward_host with every mixture of pinned and pageable buffers, one of them a slice of a larger
+    allocation, from one row to more than a grid of the fetching kernel holds at once; and with one buffer for both."""
+    import torch
+    from harness import Case, to_host_f32
+    case = Case(_cfg(T=T, dtype=dtype, d=1024 if T > 2000 else 128, f=256, E=16, K=5, k=k, renorm=k > 1))
+    ref = case.run().copy()
+    x = case.d_x.cpu()
+    pad = torch.zeros(4, x.shape[1], dtype=x.dtype)
+    xh = torch.cat([pad, x, pad]).contiguous()
+    oh = torch.full_like(xh, -1.0)
+    xh, oh = (t.pin_memory() if p else t for t, p in zip((xh, oh), pinned))
+    for _ in range(2):
+        oh[4:-4] = -1.0
+        case.layer.forward_host(xh[4:-4], oh[4:-4])
+        assert np.array_equal(to_host_f32(oh[4:-4]), ref)
+        assert torch.all(oh[:4] == -1.0) and torch.all(oh[-4:] == -1.0)
+    case.layer.forward_host(xh[4:-4], xh[4:-4])
+    assert np.array_equal(to_host_f32(xh[4:-4]), ref)
