@@ -346,8 +346,8 @@ int32_t forward_impl(swapmoe_layer* L, const void* x, const float* ext_logits, v
   const int groups = groups_planned;
   // own_scan: three extra columns of CTAs, whose first CTAs reduce the three per-expert scores
   if (!rerun) {
-    if (launch_kernel(permute_gather_kernel<DT>, dim3(n_cta + (own_scan ? 3 : 0), groups), dim3(kPermThreads), 0, st, pdl,
-                      pa) != cudaSuccess)
+    if (launch_kernel(c.top_k == 1 ? permute_gather_kernel<DT, true> : permute_gather_kernel<DT, false>,
+                      dim3(n_cta + (own_scan ? 3 : 0), groups), dim3(kPermThreads), 0, st, pdl, pa) != cudaSuccess)
       return SWAPMOE_ERR_CUDA;
     L->launches++;
   }

@@ -60,7 +60,7 @@ inline int32_t tc_ffn(TcState& s, const swapmoe_config_t& c, void* h, float* y, 
   if (!tc_plan_gemm1(s, c, n_tokens, mt, max_tiles, row_group_forced, &plan)) return SWAPMOE_ERR_UNSUPPORTED;
   const long long row_tiles_est = plan.row_tiles_est;
   const int ia = plan.ia, a_box_bytes = plan.a_box_bytes, row_group = plan.row_group;
-  const int i1 = plan.i1, out1 = plan.out1;     // output columns per tile
+  const int i1 = plan.i1;
   TcGemmArgs g1;
   g1.C = h; g1.status = status; g1.ldc = c.d_ff;
   g1.tiles = mt == 2 ? tiles128 : tiles;          // always a list of 128-row tiles

@@ -293,7 +293,9 @@ __device__ __forceinline__ float reduce_columns_parallel(const float* src, int n
 // tile (its base counts): thread (share, slot) adds a contiguous share of the rows, thread `slot` adds
 // the shares.  That is 8 KB of L2 reads per CTA at 2048 tokens, in place of a serial scan by the last
 // router CTA that kept every other SM waiting for a third of the router's duration.
-template <typename T>
+// kTop1: one pair per token, in code of its own: the kernel runs once through cold code, and the loops of the general form
+// cost a twelve-layer step of 29 tokens 2 %.
+template <typename T, bool kTop1>
 __global__ void __launch_bounds__(kPermThreads) permute_gather_kernel(const PermuteArgs a) {
   // 11 KB of shared memory, so that these CTAs fit beside a router CTA (over 210 KB) and are already
   // waiting when the router finishes.  The reducing CTAs use the same bytes for their shares.
@@ -341,23 +343,26 @@ __global__ void __launch_bounds__(kPermThreads) permute_gather_kernel(const Perm
 
   for (int i = lane; i < kMaxSlots; i += 32) wcount[warp][i] = 0;     // each warp clears (and later fills) its own row
   __syncwarp();
-  // this CTA's rows: local pair pl = ri * gridDim.y + blockIdx.y; the first kPre 16-byte pieces per
-  // thread are fetched now
+  // this CTA's tokens: local token tl = ti * gridDim.y + blockIdx.y.  A piece of 16 bytes is read once and stored to the
+  // rows of all k pairs of its token (one read per PAIR: 6011 tokens of 2 KB, top-4 25.1 us
+  // between stage events, now 20.9; 4096 of 8 KB, top-2 36 -> 27); the first kPre pieces per thread are fetched now
   constexpr int kPre = 4;
   const int vec_per_row = a.d * (int)sizeof(T) / 16;
   const uint4* src = static_cast<const uint4*>(a.x);
-  const int my_rows = (npair - (int)blockIdx.y + (int)gridDim.y - 1) / (int)gridDim.y;
+  const int t0 = (int)blockIdx.x * a.tok_tile;
+  const int my_toks = (a.tok_tile - (int)blockIdx.y + (int)gridDim.y - 1) / (int)gridDim.y;
+  const int n_pieces = my_toks * vec_per_row;
+  auto load_piece = [&](int i) -> uint4 {
+    if (i < n_pieces) {
+      const int ti = i / vec_per_row, v = i - ti * vec_per_row;
+      const int tg = t0 + ti * (int)gridDim.y + (int)blockIdx.y;
+      if (tg < a.T) return src[(size_t)tg * vec_per_row + v];
+    }
+    return make_uint4(0u, 0u, 0u, 0u);
+  };
   uint4 pre[kPre];
 #pragma unroll
-  for (int u = 0; u < kPre; ++u) {
-    const int i = tid + u * kPermThreads;
-    pre[u] = make_uint4(0u, 0u, 0u, 0u);
-    if (i < my_rows * vec_per_row) {
-      const int ri = i / vec_per_row, v = i - ri * vec_per_row;
-      const int pg = p0 + ri * (int)gridDim.y + (int)blockIdx.y;
-      if (pg < n_total) pre[u] = src[(size_t)(pg / a.k) * vec_per_row + v];
-    }
-  }
+  for (int u = 0; u < kPre; ++u) pre[u] = load_piece(tid + u * kPermThreads);
   pdl_wait();
   if (tid == 0 && blockIdx.y == 0) SWAPMOE_STAMP(1, 1);
   int s = -1, rank = 0;
@@ -428,24 +433,32 @@ __global__ void __launch_bounds__(kPermThreads) permute_gather_kernel(const Perm
   }
   __syncthreads();
   if (tid == 0 && blockIdx.y == 0) SWAPMOE_STAMP(1, 2);
-  // Gather: copy each pair's token row into its slot segment, 16 bytes per access.
+  // Gather: copy each token row into the slot segments of its pairs, 16 bytes per access, kPre loads in flight.
   uint4* dst = static_cast<uint4*>(a.xp);
-#pragma unroll
-  for (int u = 0; u < kPre; ++u) {
-    const int i = tid + u * kPermThreads;
-    if (i < my_rows * vec_per_row) {
-      const int ri = i / vec_per_row, v = i - ri * vec_per_row;
-      const int row = dst_row[ri * gridDim.y + blockIdx.y];
-      if (row >= 0) dst[(size_t)row * vec_per_row + v] = pre[u];
+  auto store_piece = [&](int i, const uint4& piece) {
+    if (i >= n_pieces) return;
+    const int ti = i / vec_per_row, v = i - ti * vec_per_row;
+    const int tl = ti * (int)gridDim.y + (int)blockIdx.y;
+    if constexpr (kTop1) {
+      const int row = dst_row[tl];
+      if (row >= 0) dst[(size_t)row * vec_per_row + v] = piece;
+    } else {
+      for (int j = 0; j < a.k; ++j) {
+        const int row = dst_row[tl * a.k + j];
+        if (row >= 0) dst[(size_t)row * vec_per_row + v] = piece;
+      }
     }
-  }
-  for (int i = tid + kPre * kPermThreads; i < my_rows * vec_per_row; i += kPermThreads) {
-    const int ri = i / vec_per_row, v = i - ri * vec_per_row;
-    const int pl = ri * gridDim.y + blockIdx.y;
-    const int row = dst_row[pl];
-    if (row >= 0) {
-      const int t = (p0 + pl) / a.k;
-      dst[(size_t)row * vec_per_row + v] = src[(size_t)t * vec_per_row + v];
+  };
+#pragma unroll
+  for (int u = 0; u < kPre; ++u) store_piece(tid + u * kPermThreads, pre[u]);
+  if constexpr (kTop1) {
+    for (int i = tid + kPre * kPermThreads; i < n_pieces; i += kPermThreads) store_piece(i, load_piece(i));
+  } else {
+    for (int i0 = tid + kPre * kPermThreads; i0 < n_pieces; i0 += kPre * kPermThreads) {
+#pragma unroll
+      for (int u = 0; u < kPre; ++u) pre[u] = load_piece(i0 + u * kPermThreads);
+#pragma unroll
+      for (int u = 0; u < kPre; ++u) store_piece(i0 + u * kPermThreads, pre[u]);
     }
   }
   if (tid == 0 && blockIdx.y == 0) SWAPMOE_STAMP(1, 3);
