@@ -79,8 +79,7 @@ struct swapmoe_layer {
   cudaStream_t s_in, s_out;    // private copy streams of the asynchronous host path
   cudaEvent_t ev_in, ev_comp, ev_out, ev_load;
   int32_t router_tok;          // 0 = automatic token-tile size of the tensor-core router, else 32/64/128
-  bool prefetch;               // pull resident weights into L2 from the router kernel
-  long long l2_prefetch_bytes; // how much of them (L2 capacity minus head room)
+  long long l2_prefetch_bytes; // resident weights to pull into L2 from the router kernel; -1: automatic (see forward_impl)
   int pair32_min_rows;         // fp32 layers on CTA pairs: 0 = tc_f32_use_pairs decides, else from this many rows per slot
   bool fp32_swap;              // fp32 layers: swapped-operand GEMM for small slots
   int prefetch_min_pairs;      // ... when the batch has at least this many HALF pairs per slot (SWAPMOE_PREFETCH_MIN_PAIRS)
@@ -269,17 +268,25 @@ int32_t forward_impl(swapmoe_layer* L, const void* x, const float* ext_logits, v
   ra.pf_total_bytes[0] = ra.pf_total_bytes[1] = 0;
   ra.pf_phys = L->phys;
   int pf_ctas = 0;
-  if (tc_router && use_tc && L->prefetch && 2 * n_pairs >= L->prefetch_min_pairs * c.K &&
+  // Automatic: 16 MB for batches of up to 64 tokens, whose few router CTAs leave over 140 SMs and HBM idle for the length
+  // of the routing (eight layers of 768 x 3072, 12 slots, us per step without / with at 12, 29, 64 tokens: 267 / 255, 294 /
+  // 280, 301 / 289; of 1024 x 4096, 16 slots: 365 / 356, 493 / 488, 509 / 504; 8, 24 and 48 MB gain less).  Larger batches
+  // none: their router fills the chip, and every megabyte slows it by about what the first product gains (one layer of
+  // 768 x 3072 at 130 tokens 52.0 / 52.9, at 400 54.0 / 52.8, at 2048 54.7 / 54.9).
+  const long long pf_budget = L->l2_prefetch_bytes >= 0 ? L->l2_prefetch_bytes : (rs_nt == 1 ? 16ll << 20 : 0);
+  if (tc_router && use_tc && pf_budget > 0 && 2 * n_pairs >= L->prefetch_min_pairs * c.K &&
       (long long)c.K * (L->nin + 1) * c.d_ff * c.d_model * (long long)L->elem <= (320ll << 20)) {
     // Most slots will be touched (at least half a pair per slot): pull the resident weights towards L2 now,
     // while the router and the permutation leave HBM idle (a slot that stays untouched costs idle bandwidth only).  GEMM-1's matrices first, then as much of GEMM-2's
     // as the L2 budget allows.
     const long long in_slot = (long long)L->nin * c.d_ff * c.d_model * L->elem;
     const long long out_slot = (long long)c.d_ff * c.d_model * L->elem;
-    const long long budget = L->l2_prefetch_bytes;
-    long long in_total = in_slot * c.K, out_total = out_slot * c.K;
-    if (in_total > budget) in_total = budget / 16384 * 16384;
-    if (out_total > budget - in_total) out_total = (budget - in_total) / 16384 * 16384;
+    // In whole chunks of whole slots: chunk c belongs to slot c / (chunks per slot), so the total must not exceed K slots'
+    // chunks (a slot's last partial chunk is left out, and a slot smaller than a chunk altogether).
+    const long long in_chunks = in_slot / kPrefetchChunk * c.K, out_chunks = out_slot / kPrefetchChunk * c.K;
+    const long long budget = pf_budget / kPrefetchChunk;
+    const long long in_total = std::min(in_chunks, budget) * kPrefetchChunk;
+    const long long out_total = std::min(out_chunks, budget - in_total / kPrefetchChunk) * kPrefetchChunk;
     ra.pf_base[0] = static_cast<const char*>(L->arena_in);
     ra.pf_base[1] = static_cast<const char*>(L->arena_out);
     ra.pf_slot_bytes[0] = in_slot; ra.pf_slot_bytes[1] = out_slot;
@@ -525,12 +532,9 @@ int32_t swapmoe_create(swapmoe_layer_t** out, const swapmoe_config_t* cfg) {
     L->small_path = !(env && env[0] == '0');
     env = std::getenv("SWAPMOE_ROW_GROUP");             // row tiles per scheduling group of the grouped GEMMs
     L->row_group = env && std::atoi(env) > 0 ? std::atoi(env) : 0;
-    // L2 weight prefetch from the router's idle blocks (SWAPMOE_PREFETCH_MB=<MB> switches it on).  Off by default:
-    // since the slot scan left the router, the router is too short to hide it - every megabyte prefetched slows
-    // the router by about as much as it speeds GEMM-1 up (B200, 2048 tokens: 0 / 24 / 56 MB -> 54.7 / 54.9 / 56.4 us).
+    // L2 weight prefetch from the router's idle blocks: budget in MB, 0 = off (default: by batch size, see forward_impl)
     env = std::getenv("SWAPMOE_PREFETCH_MB");
-    L->l2_prefetch_bytes = env ? std::atoll(env) << 20 : 0;
-    L->prefetch = L->l2_prefetch_bytes > 0;
+    L->l2_prefetch_bytes = env ? std::max(0ll, std::atoll(env)) << 20 : -1;
     env = std::getenv("SWAPMOE_FP32_SWAP");             // SWAPMOE_FP32_SWAP=0: fp32 layers always on 128-token tiles
     L->fp32_swap = !(env && env[0] == '0');
     env = std::getenv("SWAPMOE_PAIR32_MIN_ROWS");       // rows per slot from which fp32 layers run on CTA pairs (0: automatic)

@@ -28,14 +28,16 @@ struct RouterArgs {
   // experts' matrices into L2 while the router runs, when HBM is otherwise idle.
   const char* pf_base[2];       // arena_in, arena_out
   long long pf_slot_bytes[2];   // bytes of one arena entry
-  long long pf_total_bytes[2];  // bytes to prefetch, counted over logical slots 0..K-1 in order
+  long long pf_total_bytes[2];  // bytes to prefetch, in whole chunks of the logical slots 0..K-1 in order
   const int32_t* pf_phys;       // [K] arena entry of each logical slot
 };
+
+constexpr long long kPrefetchChunk = 16384;
 
 // Role of the blocks beyond the router's token tiles: pull the resident experts' matrices towards
 // L2 (GEMM-1's first, in slot order) while the router leaves HBM idle.
 __device__ __forceinline__ void router_prefetch_role(const RouterArgs& a, int n_router_ctas) {
-  constexpr long long kChunk = 16384;
+  constexpr long long kChunk = kPrefetchChunk;
   // chunks are dealt round-robin over the prefetch blocks: an SM sustains only about 200 GB/s of
   // prefetch requests, so the budget must be spread over enough of them to drain while the router runs
   const long long n_blk = (long long)gridDim.x - n_router_ctas;

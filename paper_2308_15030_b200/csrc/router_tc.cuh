@@ -53,7 +53,7 @@ router_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant_
     // ---------------------------------------------------- weight-prefetch blocks
     pdl_wait();
     pdl_trigger();
-    constexpr long long kChunk = 16384;
+    constexpr long long kChunk = kPrefetchChunk;
     const long long n_pf = (long long)(gridDim.x - a.scan.n_cta) * kRtThreads;
     const long long me = (long long)(blockIdx.x - a.scan.n_cta) * kRtThreads + threadIdx.x;
 #pragma unroll 1
