@@ -677,7 +677,7 @@ int32_t swapmoe_create(swapmoe_layer_t** out, const swapmoe_config_t* cfg) {
   {
     const char* env = std::getenv("SWAPMOE_SMALL_ROUTER");   // SWAPMOE_SMALL_ROUTER=0: tcgen05 router for small batches too
     L->small_router = c.dtype == SWAPMOE_BF16 && !(env && env[0] == '0') &&
-                      router_small_smem_bytes(c.d_model, 1) <= (size_t)(226 << 10);
+                      router_small_smem_bytes(c.d_model, 1) <= (size_t)(226 << 10) + 512;   // (static memory beside it: 272 bytes)
     if (L->small_router)
       ok = ok && cuda_ok(cudaFuncSetAttribute(router_small_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)router_small_smem_bytes(c.d_model, 1)));

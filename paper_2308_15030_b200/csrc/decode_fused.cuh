@@ -39,8 +39,8 @@ constexpr int kDecThreads = 512;
 constexpr int kDecWarps = kDecThreads / 32;
 constexpr int kDecJB = 32;            // hidden units per work item
 constexpr int kDecGroup = 16;         // work items per first-step sum
-constexpr int kDecRowPad = 16;        // bytes added to a row's pitch in shared memory
-constexpr int kDecHalfBytes = 66048;  // one wave buffer (32 rows of 2064 bytes; a multiple of 512); there are two
+constexpr int kDecRowPad = 64;        // bytes added to a row's pitch in shared memory: neighbouring rows in different halves of the banks
+constexpr int kDecHalfBytes = 67584;  // one wave buffer (32 rows of 2112 bytes; a multiple of 512); there are two
 constexpr int kDecRecent = 4;         // recently served experts remembered per layer
 constexpr int kDecOutRows = 256;      // rows of W_out per TMA box
 constexpr int kDecOutBoxes = 4;       // boxes per W_out wave: 1024 rows
@@ -252,8 +252,21 @@ __device__ __forceinline__ unsigned dec_draw_ticket(unsigned* t) {
   return v;
 }
 
-__device__ __forceinline__ uint32_t lds32(const unsigned char* p) { return *reinterpret_cast<const uint32_t*>(p); }
-
+// Fragments of 64 contraction elements (128 bytes of a row) for four m16n8k16 products, as two 16-byte loads: a dot product
+// may take its elements in any order as long as both operands agree, so thread t of a row's four holds the elements of
+// 16-byte pieces t and t + 4 instead of the pairs the instruction's own order would scatter over eight 4-byte loads.
+// Eight lanes (two rows) of a load cover all banks once.  us per pass, 4-byte / 16-byte loads: twelve layers at one token
+// 210.9 / 207.8, eight layers of 1536 x 1088 at four 252.5 / 238.1.
+struct Frag64 { uint4 lo, hi; };
+__device__ __forceinline__ Frag64 lds_frag(const unsigned char* p) {      // p = row + block of 128 bytes + 16 t
+  return {*reinterpret_cast<const uint4*>(p), *reinterpret_cast<const uint4*>(p + 64)};
+}
+__device__ __forceinline__ void mma_frag(float (&c)[4], const Frag64& a0, const Frag64& a1, const Frag64& b) {
+  mma_bf16_16x8x16(c, a0.lo.x, a1.lo.x, a0.hi.x, a1.hi.x, b.lo.x, b.hi.x);
+  mma_bf16_16x8x16(c, a0.lo.y, a1.lo.y, a0.hi.y, a1.hi.y, b.lo.y, b.hi.y);
+  mma_bf16_16x8x16(c, a0.lo.z, a1.lo.z, a0.hi.z, a1.hi.z, b.lo.z, b.hi.z);
+  mma_bf16_16x8x16(c, a0.lo.w, a1.lo.w, a0.hi.w, a1.hi.w, b.lo.w, b.hi.w);
+}
 // Waits for wave w (buffer w & 1, its barrier's phase (w >> 1) & 1): thread 0 polls (bounded), the
 // block barrier releases the others, and every thread then observes the completed phase itself.
 // Returns false when a wait gave up.
@@ -268,8 +281,8 @@ __device__ __noinline__ bool dec_wait_wave(uint64_t* bars, int w, DecRoute* R, i
 }
 
 // dst[n * dst_stride + r] = <row r of the wave buffer, token R->tok[n]> for r < rows <= 32,
-// n < nn <= 8.  The contraction is split over the warps in steps of 16; a warp multiplies its
-// steps for both 16-row tiles, the per-warp partial products meet in `red` and are added in warp
+// n < nn <= 8.  The contraction is split over the warps in blocks of 64; a warp multiplies its
+// blocks for both 16-row tiles, the per-warp partial products meet in `red` and are added in warp
 // order.  Rows of the buffer beyond `rows` hold stale data whose products are dropped; row indices beyond what
 // a wave buffer holds at this row length (fewer than 32 rows from d_model 2048 on) are clamped to its last row,
 // so that no read leaves the buffer.
@@ -283,21 +296,18 @@ __device__ __noinline__ void dec_wave_dots(const unsigned char* st, int rows, in
   for (int i = 0; i < 2; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-  const unsigned char* xrow = xs + R->tok[g] * pitch + t * 4;
+  const unsigned char* xrow = xs + R->tok[g] * pitch + t * 16;
   const int rmax = rows_held - 1;              // rows_held = decode_rows_per_wave(d): what a wave buffer holds
   const unsigned char* ar[2][2];               // rows 16 i + 8 h + g of the buffer
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int h = 0; h < 2; ++h) ar[i][h] = st + min(16 * i + 8 * h + g, rmax) * pitch + t * 4;
-#pragma unroll 2
-  for (int ks = warp; ks < d / 16; ks += kDecWarps) {
-    const int kb = ks * 32;                    // byte offset of the step inside a row
-    const uint32_t b0 = lds32(xrow + kb), b1 = lds32(xrow + kb + 16);
+    for (int h = 0; h < 2; ++h) ar[i][h] = st + min(16 * i + 8 * h + g, rmax) * pitch + t * 16;
+#pragma unroll 1
+  for (int kb = warp; kb < d / 64; kb += kDecWarps) {
+    const Frag64 b = lds_frag(xrow + kb * 128);
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
-      mma_bf16_16x8x16(acc[i], lds32(ar[i][0] + kb), lds32(ar[i][1] + kb), lds32(ar[i][0] + kb + 16),
-                       lds32(ar[i][1] + kb + 16), b0, b1);
+    for (int i = 0; i < 2; ++i) mma_frag(acc[i], lds_frag(ar[i][0] + kb * 128), lds_frag(ar[i][1] + kb * 128), b);
   }
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
@@ -334,26 +344,21 @@ __device__ __forceinline__ void rs_dots_resident(const unsigned char* ring, int 
   const int m = warp & (tiles_p2 - 1), part = warp / tiles_p2;
   if (m < MT) {
     const int row0 = m * 16;                    // first expert of the tile; wave row0 / RW, row row0 % RW inside it
-    const unsigned char* ap0 = ring + (row0 / RW) * kDecHalfBytes + ((row0 % RW) + g) * pitch + t * 4;
+    const unsigned char* ap0 = ring + (row0 / RW) * kDecHalfBytes + ((row0 % RW) + g) * pitch + t * 16;
     const unsigned char* xrow[NT];
 #pragma unroll
-    for (int j = 0; j < NT; ++j) xrow[j] = xs + min(8 * j + g, n_tok - 1) * pitch + t * 4;
-    const int nks = d / 16, ks0 = part * nks / S, ks1 = (part + 1) * nks / S;
+    for (int j = 0; j < NT; ++j) xrow[j] = xs + min(8 * j + g, n_tok - 1) * pitch + t * 16;
+    const int nkb = d / 64, kb0 = part * nkb / S, kb1 = (part + 1) * nkb / S;
     float acc[NT][4];
 #pragma unroll
     for (int j = 0; j < NT; ++j)
 #pragma unroll
       for (int q = 0; q < 4; ++q) acc[j][q] = 0.f;
-#pragma unroll 4
-    for (int ks = ks0; ks < ks1; ++ks) {
-      const int kb = ks * 32;
-      const uint32_t a0 = lds32(ap0 + kb), a1 = lds32(ap0 + 8 * pitch + kb), a2 = lds32(ap0 + kb + 16),
-                     a3 = lds32(ap0 + 8 * pitch + kb + 16);
+#pragma unroll 2
+    for (int kb = kb0; kb < kb1; ++kb) {
+      const Frag64 a0 = lds_frag(ap0 + kb * 128), a1 = lds_frag(ap0 + 8 * pitch + kb * 128);
 #pragma unroll
-      for (int j = 0; j < NT; ++j) {            // NT independent accumulators: NT chains of dependent mma
-        const uint32_t b0 = lds32(xrow[j] + kb), b1 = lds32(xrow[j] + kb + 16);
-        mma_bf16_16x8x16(acc[j], a0, a1, a2, a3, b0, b1);
-      }
+      for (int j = 0; j < NT; ++j) mma_frag(acc[j], a0, a1, lds_frag(xrow[j] + kb * 128));
     }
 #pragma unroll
     for (int j = 0; j < NT; ++j) {
@@ -394,18 +399,29 @@ decode_fused_kernel(const __grid_constant__ CUtensorMap tmWo, const DecodeArgs a
   float* red = reinterpret_cast<float*>(smem + lay.red);
   DecRoute* R = reinterpret_cast<DecRoute*>(smem + lay.route);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + lay.bars);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // warp-uniform
 
   const int RW = decode_rows_per_wave(d);            // rows of Wr / W_in per wave
   const bool have_ext = a.ext_logits != nullptr;
   const int n_rw = have_ext ? 0 : (E + RW - 1) / RW; // router waves
   // Rows of a row-major matrix -> padded rows of buffer (w & 1): lane r of warp 0 copies row r.
-  auto issue_rows = [&](int w, const bf16* src, int rows) {
+  auto issue_rows = [&](int w, const bf16* src, int rows) {          // all of warp 0
     uint64_t* bar = &bars[w & 1];
     if (lane == 0) ptx::mbar_expect_tx(bar, (uint32_t)(rows * d * 2));
     __syncwarp();
     if (lane < rows)
       ptx::bulk_load_1d(ring + (w & 1) * kDecHalfBytes + lane * pitch, src + (size_t)lane * d, (uint32_t)(d * 2), bar);
+  };
+  // Waves of the router matrix: warp v copies rows v, v + 16 (a bulk copy takes its operands from uniform registers, so
+  // the lanes of one warp issue theirs one after the other; eight waves, 256 experts, one token: 30.7 -> 26.5 us).  The
+  // experts' waves stay with warp 0: requested by all warps they measured 210.8 -> 218.8 us per twelve-layer step, by one 207.2.
+  auto issue_router_rows = [&](int w, const bf16* src, int rows) {   // all warps, converged
+    uint64_t* bar = &bars[w & 1];
+    if (tid == 0) ptx::mbar_expect_tx(bar, (uint32_t)(rows * d * 2));  // (copies may complete before it: the arrival is pending)
+    for (int r = warp; r < rows; r += kDecWarps)
+      if (ptx::elect_one())
+        ptx::bulk_load_1d(ring + (w & 1) * kDecHalfBytes + r * pitch, src + (size_t)r * d, (uint32_t)(d * 2), bar);
+    __syncwarp();
   };
 
   if (tid == 0) {
@@ -418,10 +434,8 @@ decode_fused_kernel(const __grid_constant__ CUtensorMap tmWo, const DecodeArgs a
   }
   __syncthreads();
   // the router matrix is a constant of the layer: request it before waiting for the predecessor
-  if (warp == 0) {
-    if (n_rw > 0) issue_rows(0, a.Wr, min(RW, E));
-    if (n_rw > 1) issue_rows(1, a.Wr + (size_t)RW * d, min(RW, E - RW));
-  }
+  if (n_rw > 0) issue_router_rows(0, a.Wr, min(RW, E));
+  if (n_rw > 1) issue_router_rows(1, a.Wr + (size_t)RW * d, min(RW, E - RW));
   // The list of recently served experts was written by this layer's previous forward, which is long complete
   // (every kernel of the stream waits for the one in front of it): it may be read before the wait.
   int recent_e = -1;
@@ -508,9 +522,9 @@ decode_fused_kernel(const __grid_constant__ CUtensorMap tmWo, const DecodeArgs a
     // router wave w holds rows w*RW .. of Wr
     if (!dec_wait_wave(bars, w, R, a.status, 21)) { alive = false; break; }
     dec_wave_dots(ring + (w & 1) * kDecHalfBytes, min(RW, E - w * RW), d, xs, R, T, red, slog + w * RW, kMaxE + 1, RW);
-    if (warp == 0 && w + 2 < n_rw) {               // dec_wave_dots ends with a block barrier: the buffer is free
+    if (w + 2 < n_rw) {                            // dec_wave_dots ends with a block barrier: the buffer is free
       ptx::fence_proxy_async();
-      issue_rows(w + 2, a.Wr + (size_t)(w + 2) * RW * d, min(RW, E - (w + 2) * RW));
+      issue_router_rows(w + 2, a.Wr + (size_t)(w + 2) * RW * d, min(RW, E - (w + 2) * RW));
     }
   }
   }
@@ -612,6 +626,7 @@ decode_fused_kernel(const __grid_constant__ CUtensorMap tmWo, const DecodeArgs a
       if (lane < boxes)
         ptx::tma_load_2d(ring + (w & 1) * kDecHalfBytes + lane * (kDecOutRows * kDecJB * 2), &tmWo, bar, jb * kDecJB,
                          ph * d + ow * out_rows + lane * kDecOutRows);
+      __syncwarp();
     }
   };
   if (warp == 0) {
@@ -741,8 +756,8 @@ decode_fused_kernel(const __grid_constant__ CUtensorMap tmWo, const DecodeArgs a
 #pragma unroll 1
       for (int nb = 0; nb < n_s; nb += 8) {
         const int nn = min(8, n_s - nb);
-        const unsigned char* hrow = reinterpret_cast<const unsigned char*>(hsb) + (nb + min(g, nn - 1)) * (kDecHPitch * 2) + t * 4;
-        const uint32_t b00 = lds32(hrow), b01 = lds32(hrow + 16), b10 = lds32(hrow + 32), b11 = lds32(hrow + 48);
+        const unsigned char* hrow = reinterpret_cast<const unsigned char*>(hsb) + (nb + min(g, nn - 1)) * (kDecHPitch * 2) + t * 16;
+        const uint4 b = *reinterpret_cast<const uint4*>(hrow);       // hidden units 8 t .. 8 t + 7 (any order: see lds_frag)
         if (!runs || run_jb < 0) {              // a new run (without runs: every item, batch and wave)
           run_jb = jb;
 #pragma unroll
@@ -754,13 +769,10 @@ decode_fused_kernel(const __grid_constant__ CUtensorMap tmWo, const DecodeArgs a
         for (int i = 0; i < kDecOutBoxes; ++i) {
           const int r0 = (warp + kDecWarps * i) * 16 + g, r1 = r0 + 8;      // rows of the wave
           // 16-byte chunk j of row r sits at chunk j ^ ((r >> 1) & 3)
-          const unsigned char* p0 = st + r0 * 64 + t * 4;
-          const unsigned char* p1 = st + r1 * 64 + t * 4;
-          const int x0 = (r0 >> 1) & 3, x1 = (r1 >> 1) & 3;
-          mma_bf16_16x8x16(yacc[i], lds32(p0 + ((0 ^ x0) << 4)), lds32(p1 + ((0 ^ x1) << 4)), lds32(p0 + ((1 ^ x0) << 4)),
-                           lds32(p1 + ((1 ^ x1) << 4)), b00, b01);
-          mma_bf16_16x8x16(yacc[i], lds32(p0 + ((2 ^ x0) << 4)), lds32(p1 + ((2 ^ x1) << 4)), lds32(p0 + ((3 ^ x0) << 4)),
-                           lds32(p1 + ((3 ^ x1) << 4)), b10, b11);
+          const uint4 a0 = *reinterpret_cast<const uint4*>(st + r0 * 64 + ((t ^ ((r0 >> 1) & 3)) << 4));
+          const uint4 a1 = *reinterpret_cast<const uint4*>(st + r1 * 64 + ((t ^ ((r1 >> 1) & 3)) << 4));
+          mma_bf16_16x8x16(yacc[i], a0.x, a1.x, a0.y, a1.y, b.x, b.y);
+          mma_bf16_16x8x16(yacc[i], a0.z, a1.z, a0.w, a1.w, b.z, b.w);
         }
         if (run_ends) {
           // partial rows of the run go out under the run's first hidden block

@@ -69,23 +69,17 @@ __device__ __forceinline__ void rs_wave_dots(const unsigned char* st, int rows, 
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int h = 0; h < 2; ++h) ar[i][h] = st + min(16 * i + 8 * h + g, rmax) * pitch + t * 4;
-#pragma unroll 2
-  for (int ks = warp; ks < d / 16; ks += kDecWarps) {
-    const int kb = ks * 32;
-    uint32_t b0[NT], b1[NT];
+    for (int h = 0; h < 2; ++h) ar[i][h] = st + min(16 * i + 8 * h + g, rmax) * pitch + t * 16;
+#pragma unroll 1
+  for (int kb = warp; kb < d / 64; kb += kDecWarps) {
+    Frag64 b[NT];
 #pragma unroll
-    for (int j = 0; j < NT; ++j) {
-      const unsigned char* xrow = xs + min(8 * j + g, n_tok - 1) * pitch + t * 4 + kb;
-      b0[j] = lds32(xrow);
-      b1[j] = lds32(xrow + 16);
-    }
+    for (int j = 0; j < NT; ++j) b[j] = lds_frag(xs + min(8 * j + g, n_tok - 1) * pitch + t * 16 + kb * 128);
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-      const uint32_t a0 = lds32(ar[i][0] + kb), a1 = lds32(ar[i][1] + kb), a2 = lds32(ar[i][0] + kb + 16),
-                     a3 = lds32(ar[i][1] + kb + 16);
+      const Frag64 a0 = lds_frag(ar[i][0] + kb * 128), a1 = lds_frag(ar[i][1] + kb * 128);
 #pragma unroll
-      for (int j = 0; j < NT; ++j) mma_bf16_16x8x16(acc[i][j], a0, a1, a2, a3, b0[j], b1[j]);
+      for (int j = 0; j < NT; ++j) mma_frag(acc[i][j], a0, a1, b[j]);
     }
   }
 #pragma unroll
@@ -130,7 +124,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) router_small_kernel(const Rout
   DecRoute* R = reinterpret_cast<DecRoute*>(smem + lay.route);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + lay.bars);
   RsRoute* Q = reinterpret_cast<RsRoute*>(smem + lay.pairs);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // warp-uniform
   const int tok0 = blockIdx.x * TOK;
   const int T = min(TOK, a.T - tok0);                       // tokens of this CTA
   const int P = T * k;
@@ -139,13 +133,14 @@ __global__ void __launch_bounds__(kDecThreads, 1) router_small_kernel(const Rout
 
   const int RW = decode_rows_per_wave(d);
   const int n_rw = (E + RW - 1) / RW;
-  auto issue_router_wave = [&](int w) {                     // all of warp 0
+  auto issue_router_wave = [&](int w) {                     // all warps (see issue_rows of the decode kernel)
     const int rows = min(RW, E - w * RW);
     uint64_t* bar = &bars[w & 1];
-    if (lane == 0) ptx::mbar_expect_tx(bar, (uint32_t)(rows * d * 2));
+    if (tid == 0) ptx::mbar_expect_tx(bar, (uint32_t)(rows * d * 2));
+    for (int r = warp; r < rows; r += kDecWarps)
+      if (ptx::elect_one())
+        ptx::bulk_load_1d(ring + (w & 1) * kDecHalfBytes + r * pitch, Wr + ((size_t)w * RW + r) * d, (uint32_t)(d * 2), bar);
     __syncwarp();
-    if (lane < rows)
-      ptx::bulk_load_1d(ring + (w & 1) * kDecHalfBytes + lane * pitch, Wr + ((size_t)w * RW + lane) * d, (uint32_t)(d * 2), bar);
   };
   if (tid == 0) {
     ptx::mbar_init(&bars[0], 1);
@@ -154,10 +149,8 @@ __global__ void __launch_bounds__(kDecThreads, 1) router_small_kernel(const Rout
     ptx::fence_barrier_init();
   }
   __syncthreads();
-  if (warp == 0) {                                          // the router matrix is a constant of the layer
-    issue_router_wave(0);
-    if (n_rw > 1) issue_router_wave(1);
-  }
+  issue_router_wave(0);                                     // the router matrix is a constant of the layer
+  if (n_rw > 1) issue_router_wave(1);
   if (warp == 1 && lane == 0) {
     // The CTA's token rows (one contiguous range) are pulled towards L2 while the kernel in front still runs.
     // A prefetch only moves what DRAM holds into L2, where any later write of the producer lands too, so it
@@ -218,7 +211,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) router_small_kernel(const Rout
     for (int w = 0; w < n_rw; ++w) {
       if (!dec_wait_wave(bars, w, R, status, 23)) { alive = false; break; }
       rs_wave_dots<NT>(ring + (w & 1) * kDecHalfBytes, min(RW, E - w * RW), d, xs, T, red, slog + w * RW, kMaxE + 1);
-      if (warp == 0 && w + 2 < n_rw) {
+      if (w + 2 < n_rw) {
         ptx::fence_proxy_async();
         issue_router_wave(w + 2);
       }

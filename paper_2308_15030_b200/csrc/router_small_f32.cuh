@@ -15,15 +15,16 @@
 namespace swapmoe {
 
 // rows of an fp32 row-contiguous matrix (row length d) per wave: a power of two, at most 32
+constexpr int kRsfRowPad = 16;            // bytes added to a row's pitch in shared memory
 __host__ __device__ inline int rsf_rows_per_wave(int d) {
   int rp = 32;
-  while (rp > 1 && rp * (d * 4 + kDecRowPad) > kDecHalfBytes) rp >>= 1;
+  while (rp > 1 && rp * (d * 4 + kRsfRowPad) > kDecHalfBytes) rp >>= 1;
   return rp;
 }
 __host__ __device__ inline RsSmem router_small_f32_layout(int d) {
   RsSmem m;
   int o = 2 * kDecHalfBytes;
-  m.xs = o;    o += kRsTok * (d * 4 + kDecRowPad);
+  m.xs = o;    o += kRsTok * (d * 4 + kRsfRowPad);
   m.slog = o;  o += kRsTok * (kMaxE + 1) * 4;
   o = (o + 15) & ~15;
   m.red = o;   o += kDecWarps * 32 * 8 * 4;
@@ -41,7 +42,7 @@ inline size_t router_small_f32_smem_bytes(int d) { return (size_t)router_small_f
 __device__ __forceinline__ void rsf_wave_dots(const unsigned char* st, int rows, int d, const unsigned char* xs,
                                               int n_tok, float* red, float* dst, int dst_stride) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
-  const int pitch = d * 4 + kDecRowPad;
+  const int pitch = d * 4 + kRsfRowPad;
   float acc[2][4];
 #pragma unroll
   for (int i = 0; i < 2; ++i)
@@ -103,7 +104,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) router_small_f32_kernel(const 
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~static_cast<uintptr_t>(1023));
   const int d = a.d, E = a.E, k = a.k, K = a.K;
-  const int chunks = d / 4, pitch = d * 4 + kDecRowPad;
+  const int chunks = d / 4, pitch = d * 4 + kRsfRowPad;
   const RsSmem lay = router_small_f32_layout(d);
   unsigned char* ring = smem;
   unsigned char* xs = smem + lay.xs;
