@@ -321,6 +321,36 @@ __device__ __forceinline__ void epi_load_pieces(uint32_t taddr, int c0, int gate
   }
 }
 
+// The accumulator columns [c0, c0 + 16) -> two 16-byte pieces of bf16 output.
+template <int EPI>
+__device__ __forceinline__ void epi_load_pieces16(uint32_t taddr, int c0, int gate_cols, float gate, uint4 (&pc)[2]) {
+  uint32_t v[16];
+  ptx::tmem_ld16(taddr + (uint32_t)c0, v);
+  float f[16];
+  if (EPI == kTcEpiSwigluBf16) {
+    uint32_t g[16];
+    ptx::tmem_ld16(taddr + (uint32_t)(c0 + gate_cols), g);
+    ptx::tmem_ld_wait();
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const float x1 = __uint_as_float(v[i]);
+      f[i] = silu_from_exp(x1, __expf(-x1)) * __uint_as_float(g[i]);
+    }
+  } else {
+    ptx::tmem_ld_wait();
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      f[i] = __uint_as_float(v[i]);
+      if (EPI == kTcEpiReluBf16) f[i] = fmaxf(f[i], 0.f);
+      if (EPI == kTcEpiScatterBf16) f[i] *= gate;
+    }
+  }
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+    pc[h] = make_uint4(pack_bf16x2(f[8 * h], f[8 * h + 1]), pack_bf16x2(f[8 * h + 2], f[8 * h + 3]),
+                       pack_bf16x2(f[8 * h + 4], f[8 * h + 5]), pack_bf16x2(f[8 * h + 6], f[8 * h + 7]));
+}
+
 // One accumulator (kOutCols output columns of this thread's row) -> global memory, 128 bytes per row and chunk.  `cols` =
 // columns of the matrix from this tile's first one on: the last tile of a matrix whose width is no multiple of kOutCols
 // (but of a chunk: widths are multiples of 64) holds products with the rows of whatever lies behind the slot's weights,
@@ -366,7 +396,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   constexpr int kNB = (EPI == kTcEpiSwigluBf16) ? 2 : 1;   // weight boxes per stage
   constexpr int kBoxRows = BN / kNB;
   constexpr int kOutCols = BN / kNB;                        // output columns per tile
-  constexpr uint32_t kTmemCols = kAccBufs * MT * BN;
+  constexpr uint32_t kTmemCols = kAccBufs * MT * BN <= 64 ? 64 : kAccBufs * MT * BN <= 128 ? 128
+                                 : kAccBufs * MT * BN <= 256 ? 256 : 512;      // a power of two
   constexpr uint32_t kIdesc = make_idesc_bf16(kTcBM, BN);
 
   extern __shared__ unsigned char smem_raw[];
@@ -581,14 +612,17 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             epi_row_pointers(dst, drow_h[hf], lane, a.C, (size_t)a.ldc, (size_t)ct * kOutCols, kElem);
             epi_store_tile<EPI, kOutCols>(taddr, epi_stage + q * kTcEpiWarpStage, lane, gate_h[hf], dst, a.ldc - ct * kOutCols);
           } else {
-            // 64 bytes per row (the narrowest bf16 tiles): every thread stores its own row
-            uint4 pc[4];
-            epi_load_pieces<EPI>(taddr, 0, kOutCols, gate_h[hf], pc);
-            if (drow_h[hf] >= 0) {
-              uint4* dst = reinterpret_cast<uint4*>(static_cast<bf16*>(a.C) + (size_t)drow_h[hf] * a.ldc +
-                                                    (size_t)ct * kOutCols);
-#pragma unroll
-              for (int i = 0; i < 4; ++i) dst[i] = pc[i];
+            // tiles whose rows are no whole 128-byte chunks (the narrowest, and 80 columns): every thread stores its own
+            // row, sixteen columns at a time
+            bf16* dst = drow_h[hf] < 0 ? nullptr : static_cast<bf16*>(a.C) + (size_t)drow_h[hf] * a.ldc + (size_t)ct * kOutCols;
+#pragma unroll 1
+            for (int c0 = 0; c0 < min(kOutCols, a.ldc - ct * kOutCols); c0 += 16) {
+              uint4 pc[2];
+              epi_load_pieces16<EPI>(taddr, c0, kOutCols, gate_h[hf], pc);
+              if (dst != nullptr) {
+                reinterpret_cast<uint4*>(dst + c0)[0] = pc[0];
+                reinterpret_cast<uint4*>(dst + c0)[1] = pc[1];
+              }
             }
           }
         }
@@ -615,7 +649,8 @@ typedef CUresult (*PFN_encodeTiled)(CUtensorMap*, CUtensorMapDataType, cuuint32_
 
 // Column-tile widths the kernels are built for.  Narrow tiles exist for small batches
 // (decode): with few row tiles, wide column tiles would leave most SMs without work.
-constexpr int kBn1Options[3] = {256, 128, 64};
+// (the last of GEMM-1's: SwiGLU layers at up to 64 pairs, see tc_plan_gemm1)
+constexpr int kBn1Options[4] = {256, 128, 64, 160};
 constexpr int kBn2Options[4] = {256, 128, 64, 32};
 
 struct TcState {
@@ -623,7 +658,7 @@ struct TcState {
   int sm_count;
   PFN_encodeTiled encode;
   CUtensorMap map_xp[4], map_h[4];    // activations [rows_pad, d] / [rows_pad, f]; box rows 128, 64, 32, 16
-  CUtensorMap map_win[3];             // W_in flattened to 2D, one map per entry of kBn1Options
+  CUtensorMap map_win[4];             // W_in flattened to 2D, one map per entry of kBn1Options
   CUtensorMap map_wout[4];            // W_out flattened to 2D, one map per entry of kBn2Options
   CUtensorMap map_wr;                 // router matrix [E, d], box 64 x Epad
   bool arena_bound;
@@ -727,7 +762,7 @@ inline int32_t tc_init(TcState& s, const swapmoe_config_t& c, void* xp, void* h,
   }
   bool ok = tc_set_smem_attr<256, kTcEpiReluBf16>() && tc_set_smem_attr<128, kTcEpiReluBf16>() &&
             tc_set_smem_attr<64, kTcEpiReluBf16>() && tc_set_smem_attr<256, kTcEpiSwigluBf16>() &&
-            tc_set_smem_attr<128, kTcEpiSwigluBf16>() && tc_set_smem_attr<64, kTcEpiSwigluBf16>() &&
+            tc_set_smem_attr<128, kTcEpiSwigluBf16>() && tc_set_smem_attr<64, kTcEpiSwigluBf16>() && tc_set_smem_attr<160, kTcEpiSwigluBf16>() &&
             tc_set_smem_attr<256, kTcEpiF32>() && tc_set_smem_attr<128, kTcEpiF32>() &&
             tc_set_smem_attr<64, kTcEpiF32>() && tc_set_smem_attr<32, kTcEpiF32>() &&
             tc_set_smem_attr<256, kTcEpiScatterBf16>() && tc_set_smem_attr<128, kTcEpiScatterBf16>() &&
@@ -742,7 +777,7 @@ inline int32_t tc_bind_arena(TcState& s, const swapmoe_config_t& c, const void* 
   if (!s.enabled) return SWAPMOE_OK;
   const int P = c.K + c.spare_slots;
   const int nin = c.act == SWAPMOE_ACT_SWIGLU ? 2 : 1;
-  for (int i = 0; i < 3; ++i)     // SwiGLU loads W1 and W3 as two boxes of half the tile width
+  for (int i = 0; i < 4; ++i)     // SwiGLU loads W1 and W3 as two boxes of half the tile width
     if (!tc_encode_2d(s.encode, &s.map_win[i], arena_in, (uint64_t)P * nin * c.d_ff, (uint64_t)c.d_model,
                       (uint32_t)(kBn1Options[i] / nin)))
       return SWAPMOE_ERR_CUDA;

@@ -33,7 +33,11 @@ inline bool tc_plan_gemm1(const TcState& s, const swapmoe_config_t& c, int n_tok
   else if (pairs * (long long)c.d_model * 2 > (48ll << 20)) p->row_group = 32;
   // (SwiGLU counts the rows of both matrices; with one matrix's the model saw half the tiles: 13 tokens, d_model 4096,
   // d_ff 14336, four slots, GEMM-1 alone 187 us at 448 tiles on 148 SMs, 174 at 896 narrower ones)
-  p->i1 = tc_pick_bn(kBn1Options, 3, swiglu ? 2 * c.d_ff : c.d_ff, p->row_tiles_est * mt, s.sm_count, p->a_box_bytes, swiglu ? 64 : 32);
+  // With few rows the weights are all there is to pull, and what counts is how evenly the column tiles fill the last round:
+  // SwiGLU at up to 64 pairs may also take 160 weight rows (80 outputs), whose epilogue is only good for few rows.
+  // us per forward without / with, four slots: 4096 x 14336 at 13 tokens 258 / 245, 2048 x 5632 at 6 85 / 72, 960 x 2624 at
+  // 20 41 / 36; 1024 x 3584, where 256 rows are one round, keeps them.
+  p->i1 = tc_pick_bn(kBn1Options, swiglu && pairs <= 64 ? 4 : 3, swiglu ? 2 * c.d_ff : c.d_ff, p->row_tiles_est * mt, s.sm_count, p->a_box_bytes, swiglu ? 64 : 32);
   if (p->i1 < 0) return false;
   p->bn1 = kBn1Options[p->i1];
   p->out1 = swiglu ? p->bn1 / 2 : p->bn1;
@@ -75,11 +79,11 @@ inline int32_t tc_ffn(TcState& s, const swapmoe_config_t& c, void* h, float* y, 
   g1.early_b = 0;
   long long work = (long long)max_tiles * mt * g1.n_col_tiles;
   int grid = plan.grid;
-  static const TcGemmKernel k1[2][3] = {
-      {tc_gemm_kernel<256, kTcEpiReluBf16>, tc_gemm_kernel<128, kTcEpiReluBf16>, tc_gemm_kernel<64, kTcEpiReluBf16>},
+  static const TcGemmKernel k1[2][4] = {
+      {tc_gemm_kernel<256, kTcEpiReluBf16>, tc_gemm_kernel<128, kTcEpiReluBf16>, tc_gemm_kernel<64, kTcEpiReluBf16>, nullptr},
       {tc_gemm_kernel<256, kTcEpiSwigluBf16>, tc_gemm_kernel<128, kTcEpiSwigluBf16>,
-       tc_gemm_kernel<64, kTcEpiSwigluBf16>}};
-  static const int smem1[3] = {TcSmem<256>::kBytes, TcSmem<128>::kBytes, TcSmem<64>::kBytes};
+       tc_gemm_kernel<64, kTcEpiSwigluBf16>, tc_gemm_kernel<160, kTcEpiSwigluBf16>}};
+  static const int smem1[4] = {TcSmem<256>::kBytes, TcSmem<128>::kBytes, TcSmem<64>::kBytes, TcSmem<160>::kBytes};
   if (s.only != 2) {
     if (launch_kernel(k1[swiglu ? 1 : 0][i1], dim3(grid), dim3(kTcThreads), smem1[i1], st, pdl, s.map_xp[ia], s.map_win[i1],
                       g1) != cudaSuccess)
