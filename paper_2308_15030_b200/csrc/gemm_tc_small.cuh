@@ -43,7 +43,7 @@ tc_gemm_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
                      const TcSmallArgs sa) {
   const TcGemmArgs& a = sa.g;
   constexpr int kBTile = BN * kTcBK * 2;                    // one k-block of the weight box
-  constexpr uint32_t kTmemCols = 2 * BN < 32 ? 32 : 2 * BN;
+  constexpr uint32_t kTmemCols = 2 * BN <= 64 ? 64 : 2 * BN <= 128 ? 128 : 2 * BN <= 256 ? 256 : 512;   // a power of two
   constexpr uint32_t kIdesc = make_idesc_bf16(kTcBM, BN);
   const int kps = sa.kps, n_stages = sa.n_stages, a_tile = sa.a_tile_bytes;
   const int stage_a = kps * a_tile, stage_b = kps * kBTile;
@@ -245,6 +245,27 @@ inline bool tc_encode_3d(PFN_encodeTiled enc, CUtensorMap* m, const void* base, 
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Tile widths of the small-batch kernels.  Few rows, so the weights are all there is to pull, and the widths between the
+// powers of two let the column tiles fill the last round.  us, powers of two
+// only / all: 768 x 3072, 16 slots, 12 tokens 29.3 / 27.8, 40 tokens 36.4 / 34.2; 704 x 2240 at 40 31.5 / 30.5; twelve layers
+// of 1024 x 4096 at 29 726 / 715; 1536 x 1088, 48 slots, 60 tokens 80.6 / 81.1.
+constexpr int kSmallBn[8] = {256, 224, 192, 160, 128, 96, 64, 32};
+
+// As tc_pick_bn (bytes the busiest SM pulls over all k-blocks), plus the epilogue of its last tile, which nothing overlaps:
+// about 300 clocks per 32 columns, the time of 13 KB.  Without that term eight tokens of 768 x 3072 took 192 columns in one
+// round where 64 in three are 1.5 % faster.
+inline int tc_small_pick_bn(int n, int k_blocks, long long row_tiles, int sm_count, int a_tile_bytes) {
+  int pick = 0;
+  long long best = 0;
+  for (int i = 0; i < 8; ++i) {
+    const long long tiles = row_tiles * ((n + kSmallBn[i] - 1) / kSmallBn[i]);
+    const long long cost = (tiles + sm_count - 1) / sm_count * k_blocks * (a_tile_bytes + (long long)kSmallBn[i] * kTcBK * 2) +
+                           kSmallBn[i] * 422ll;
+    if (i == 0 || cost < best) { pick = i; best = cost; }
+  }
+  return pick;
+}
+
 struct TcSmallGeom {
   int bn_index, bn, kps, n_stages, smem_bytes;
 };
@@ -252,9 +273,8 @@ struct TcSmallGeom {
 // Tile width, k-blocks per stage and stage count of one small-batch GEMM.
 inline bool tc_small_geometry(int n, int k_blocks, long long row_tiles, int sm_count, int a_tile_bytes,
                               TcSmallGeom* g) {
-  g->bn_index = tc_pick_bn(kBn2Options, 4, n, row_tiles, sm_count, a_tile_bytes, 32);
-  if (g->bn_index < 0) return false;
-  g->bn = kBn2Options[g->bn_index];
+  g->bn_index = tc_small_pick_bn(n, k_blocks, row_tiles, sm_count, a_tile_bytes);
+  g->bn = kSmallBn[g->bn_index];
   const int per_kb = a_tile_bytes + g->bn * kTcBK * 2;
   g->kps = 1;
   for (int kps = 8; kps > 1; --kps)      // the most that fits, with at most an eighth of a tile's k-blocks empty
@@ -284,15 +304,19 @@ template <int EPI>
 inline TcSmallKernel tc_small_kernel_for(int bn_index) {
   switch (bn_index) {
     case 0: return tc_gemm_small_kernel<256, EPI>;
-    case 1: return tc_gemm_small_kernel<128, EPI>;
-    case 2: return tc_gemm_small_kernel<64, EPI>;
+    case 1: return tc_gemm_small_kernel<224, EPI>;
+    case 2: return tc_gemm_small_kernel<192, EPI>;
+    case 3: return tc_gemm_small_kernel<160, EPI>;
+    case 4: return tc_gemm_small_kernel<128, EPI>;
+    case 5: return tc_gemm_small_kernel<96, EPI>;
+    case 6: return tc_gemm_small_kernel<64, EPI>;
     default: return tc_gemm_small_kernel<32, EPI>;
   }
 }
 
 inline bool tc_small_set_attrs() {
   bool ok = true;
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < 8; ++i) {
     ok = ok && cudaFuncSetAttribute(tc_small_kernel_for<kTcEpiReluBf16>(i), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     kSmSmemBudget) == cudaSuccess;
     ok = ok && cudaFuncSetAttribute(tc_small_kernel_for<kTcEpiF32>(i), cudaFuncAttributeMaxDynamicSharedMemorySize,

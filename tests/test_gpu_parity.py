@@ -672,6 +672,8 @@ def test_general_gate_selects_in_expert_order(T, E, K, k, ext):
     (I.BF16, 7, 64, 64, 3, 1, I.ACT_RELU),          # one k-block, one tile wider than the matrix
     (I.BF16, 300, 320, 832, 5, 1, I.ACT_RELU),      # one CTA per 128-row tile, both widths ragged
     (I.BF16, 90, 192, 320, 4, 2, I.ACT_SWIGLU),
+    (I.BF16, 24, 704, 2240, 6, 1, I.ACT_RELU),      # small-batch kernels' widths between the powers of two
+    (I.BF16, 20, 512, 3072, 8, 1, I.ACT_RELU),
     (I.BF16, 20, 64, 2624, 4, 2, I.ACT_SWIGLU),     # few rows of a gated layer: 80-column tiles, the last one ragged
     (I.BF16, 32, 128, 2560, 4, 2, I.ACT_SWIGLU),    # ... and whole ones, at the most pairs they take
     (I.BF16, 1500, 704, 448, 5, 1, I.ACT_RELU),     # 256-row tiles: GEMM-1 on CTA pairs, GEMM-2 on two row sub-tiles
