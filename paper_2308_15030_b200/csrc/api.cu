@@ -127,29 +127,24 @@ __global__ void snapshot_scores_kernel(const ScoreSnapshot s) {
   if (s.reset) s.acc[k][e] = 0.f;
 }
 
-// Tokens from mapped pinned host memory to the device.  Bound by the host link; a kernel reads it as fast as a copy engine,
-// joins the chain of dependent launches, and its first loads (four 16-byte ones per thread) are on their way before the
-// kernel in front has finished.
+// Tokens from mapped pinned host memory to the device, four 16-byte pieces per thread.  Bound by the host link; a kernel reads
+// it as fast as a copy engine and joins the chain of dependent launches.  Nothing is read before the wait: what is in
+// front on the stream may be writing the rows (a forward whose `out` is this buffer lets its dependents start early), and a
+// copy in this place would be ordered behind it.
 constexpr int kFetchThreads = 512, kFetchLoads = 4;
 constexpr size_t kHostInPlaceBytes = (size_t)9 << 20;
 __global__ void __launch_bounds__(kFetchThreads) fetch_rows_kernel(const uint4* src, uint4* dst, long long n) {
-  const long long stride = (long long)gridDim.x * kFetchThreads;
-  long long i = (long long)blockIdx.x * kFetchThreads + threadIdx.x;
+  pdl_wait();
+  pdl_trigger();
+  const long long stride = (long long)gridDim.x * kFetchThreads;       // gridDim.x * kFetchThreads * kFetchLoads >= n
+  const long long i = (long long)blockIdx.x * kFetchThreads + threadIdx.x;
   uint4 v[kFetchLoads];
 #pragma unroll
   for (int u = 0; u < kFetchLoads; ++u)
     if (i + u * stride < n) v[u] = __ldcs(src + i + u * stride);
-  pdl_wait();          // the staging buffer may still be read by the forward in front
-  pdl_trigger();
-  while (i < n) {
 #pragma unroll
-    for (int u = 0; u < kFetchLoads; ++u)
-      if (i + u * stride < n) dst[i + u * stride] = v[u];
-    i += kFetchLoads * stride;
-#pragma unroll
-    for (int u = 0; u < kFetchLoads; ++u)
-      if (i + u * stride < n) v[u] = __ldcs(src + i + u * stride);
-  }
+  for (int u = 0; u < kFetchLoads; ++u)
+    if (i + u * stride < n) dst[i + u * stride] = v[u];
 }
 
 typedef CUresult (*PFN_pointerAttributes)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr);
@@ -833,16 +828,17 @@ int32_t swapmoe_forward_host(swapmoe_layer_t* L, const void* x_host, void* out_h
     return SWAPMOE_ERR_CUDA;
   // Pinned buffers are used in place: the tokens come in by a kernel of the chain and the last kernel of the forward, which
   // writes every output element once, writes it to the host, so the way out overlaps the second product and neither
-  // copy's start-up is waited for.  us per request, copies / in place: 16 tokens of d_model 768 62 / 53, 600 of 512 110 / 86,
-  // 1999 of 768 279 / 195, 4000 of 1024 (8 MB) 465 / 443; at 8192 of 768 (13 MB) the copy engines are level or ahead, 589 / 598.
+  // copy's start-up is waited for.  us per request, copies / in place, in a loop of requests on three pairs of buffers: 16
+  // tokens of d_model 768 57 / 57, 600 of 512 82 / 76, 1999 of 768 192 / 189, 4000 of 1024 (8 MB) 432 / 434, 8192 of 768
+  // (13 MB) 585 / 597; single requests on buffers the device has not seen: 63 / 61, 101 / 88, 273 / 214, 570 / 463, 740 / 642.
+  // The line lies where the loop starts to lose.
   const PFN_pointerAttributes query = reinterpret_cast<PFN_pointerAttributes>(L->pointer_attributes);
   const bool in_place = bytes <= kHostInPlaceBytes;
   const void* x_dev = in_place ? mapped_host_range(query, x_host, bytes) : nullptr;
   void* out_dev = in_place ? mapped_host_range(query, out_host, bytes) : nullptr;
   if (x_dev) {
     const long long n = (long long)(bytes / 16), per_cta = kFetchThreads * kFetchLoads;
-    const long long want = (n + per_cta - 1) / per_cta;
-    const int grid = (int)(want < 2 * L->sm_count ? want : 2 * L->sm_count);
+    const int grid = (int)((n + per_cta - 1) / per_cta);
     if (launch_kernel(fetch_rows_kernel, dim3(grid), dim3(kFetchThreads), 0, st, L->use_pdl, static_cast<const uint4*>(x_dev),
                       static_cast<uint4*>(L->x_stage), n) != cudaSuccess)
       return SWAPMOE_ERR_CUDA;

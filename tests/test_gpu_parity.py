@@ -737,3 +737,26 @@ def test_host_path_uses_pinned_buffers_in_place(dtype, T, k, pinned):
         assert torch.all(oh[:4] == -1.0) and torch.all(oh[-4:] == -1.0)
     case.layer.forward_host(xh[4:-4], xh[4:-4])
     assert np.array_equal(to_host_f32(xh[4:-4]), ref)
+
+
+@pytest.mark.parametrize("T,d,k", [(1500, 512, 1), (700, 768, 2), (4, 512, 1), (40, 1024, 1)])
+def test_host_path_reads_behind_the_kernel_in_front(T, d, k):
+    """A forward writes its result into a pinned buffer, and a host request on the same stream takes that buffer as its
+    tokens at once: the request must see all of it, however early the kernels in front let their dependents start."""
+    import torch
+    from harness import Case, to_host_f32
+    a = Case(_cfg(T=T, d=d, f=1024, E=16, K=5, k=k, renorm=k > 1))
+    b = Case(_cfg(T=T, d=d, f=256, E=16, K=5, seed=9))
+    xs = [torch.randn_like(a.d_x) for _ in range(3)]
+    refs = []
+    for x in xs:
+        mid, ref = torch.empty_like(x), torch.empty_like(x)
+        a.layer.forward(x, mid)
+        b.layer.forward(mid, ref)
+        refs.append(to_host_f32(ref))
+    torch.cuda.synchronize()
+    pinned, out = torch.zeros_like(a.d_x, device="cpu").pin_memory(), torch.zeros_like(a.d_x, device="cpu").pin_memory()
+    for i in range(30):
+        a.layer.forward(xs[i % 3], pinned)
+        b.layer.forward_host(pinned, out)
+        assert np.array_equal(to_host_f32(out), refs[i % 3]), i
