@@ -653,10 +653,12 @@ int32_t swapmoe_create(swapmoe_layer_t** out, const swapmoe_config_t* cfg) {
   L->tc32.enabled = L->tc32.arena_bound = false;
   L->encode32 = nullptr;
   {
-    const char* env = std::getenv("SWAPMOE_FP32_TC");        // SWAPMOE_FP32_TC=0: warp-level mma (or FFMA) for fp32 layers
+    // SWAPMOE_FP32_TC=0: warp-level mma for every fp32 layer, 1: tcgen05 for every one (default: tc_f32_supported decides)
+    const char* env = std::getenv("SWAPMOE_FP32_TC");
     if (ok && c.dtype == SWAPMOE_F32 && !(env && env[0] == '0')) {
       L->encode32 = tc_get_encoder();
-      ok = tc_f32_init(L->tc32, L->encode32, c, L->xp, L->h, L->rows_pad_max, L->sm_count) == SWAPMOE_OK;
+      ok = tc_f32_init(L->tc32, L->encode32, c, L->xp, L->h, L->rows_pad_max, L->sm_count,
+                       env && env[0] == '1') == SWAPMOE_OK;
       const char* envp = std::getenv("SWAPMOE_PAIR_GEMM");
       if (ok && L->tc32.enabled && !(envp && envp[0] == '0')) L->tc32.n_pairs = tc_f32_pair_init(L->sm_count);
     }

@@ -464,10 +464,18 @@ inline PFN_encodeTiled tc_get_encoder() {
   return reinterpret_cast<PFN_encodeTiled>(fn);
 }
 
-// Every fp32 layer (see tc_supported).  d_model 704, d_ff 2240, top-1 of 6 slots, us per forward on gemm_tf32x3_kernel /
-// here at 20, 700, 3000 tokens: 93 / 47, 144 / 58, 371 / 140.
-inline bool tc_f32_supported(const swapmoe_config_t& c) {
-  return c.dtype == SWAPMOE_F32;
+// Which fp32 layers run here rather than on gemm_tf32x3_kernel.  Both leave about the same error, from different sources: two
+// bf16 pieces per operand drop 2^-17 of every product (6.3e-6 of the result whatever the widths), while the warp-level
+// kernel's products are good to 2^-20 but its tensor core truncates at each of the many small steps of its sums, which grows
+// with the contraction.  Layers of whole 128-wide tiles always run here.  The others (704 x 2240, top-1 of 6 slots, us per
+// forward there / here at 20, 700, 3000 tokens: 93 / 47, 144 / 58, 371 / 140) do where the error against 64 bits is no larger:
+// ratio of the two errors, here over there, normally distributed operands, ReLU: 64 x 64 4.0, 320 x 320 1.6, 576 x 576 1.04,
+// 704 x 448 1.02, 704 x 1088 0.80, 960 x 704 0.77, 704 x 2240 0.64, 1536 x 1088 0.55; SwiGLU 64 x 2240 0.92 but 1.5 with
+// heavy-tailed operands, 640 x 1344 0.68 and 0.96.
+inline bool tc_f32_supported(const swapmoe_config_t& c, bool every_width) {
+  if (c.dtype != SWAPMOE_F32) return false;
+  if (every_width || (c.d_model % kF32BN == 0 && c.d_ff % kF32BN == 0)) return true;
+  return c.d_model >= 640 && 2ll * c.d_model + c.d_ff >= 2560;
 }
 
 inline bool tc_encode_2d_f32(PFN_encodeTiled enc, CUtensorMap* m, const void* base, uint64_t rows, uint64_t cols,
@@ -482,13 +490,13 @@ inline bool tc_encode_2d_f32(PFN_encodeTiled enc, CUtensorMap* m, const void* ba
 }
 
 inline int32_t tc_f32_init(TcF32State& s, PFN_encodeTiled enc, const swapmoe_config_t& c, void* xp, void* h,
-                           int rows_pad, int sm_count) {
+                           int rows_pad, int sm_count, bool every_width) {
   s.enabled = false;
   s.arena_bound = false;
   s.only = 0;
   s.n_pairs = 0;
   s.sm_count = sm_count;
-  if (!enc || !tc_f32_supported(c)) return SWAPMOE_OK;
+  if (!enc || !tc_f32_supported(c, every_width)) return SWAPMOE_OK;
   if (!tc_encode_2d_f32(enc, &s.map_xp, xp, (uint64_t)rows_pad, (uint64_t)c.d_model, kTcBM) ||
       !tc_encode_2d_f32(enc, &s.map_h, h, (uint64_t)rows_pad, (uint64_t)c.d_ff, kTcBM) ||
       !tc_encode_2d_f32(enc, &s.map_xp_tok, xp, (uint64_t)rows_pad, (uint64_t)c.d_model, kF32SwapTok) ||

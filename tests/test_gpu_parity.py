@@ -684,11 +684,15 @@ def test_general_gate_selects_in_expert_order(T, E, K, k, ext):
     (I.F32, 100, 192, 448, 5, 1, I.ACT_RELU),       # fp32, weights on the MMA rows
     (I.F32, 900, 320, 704, 4, 1, I.ACT_RELU),       # fp32, tokens on the MMA rows
     (I.F32, 150, 64, 192, 3, 2, I.ACT_SWIGLU),
+    (I.F32, 40, 704, 1216, 5, 1, I.ACT_RELU),       # fp32 widths that come here by themselves
+    (I.F32, 300, 832, 960, 4, 2, I.ACT_SWIGLU),
 ])
-def test_ragged_column_tiles(dtype, T, d, f, K, k, act):
+def test_ragged_column_tiles(monkeypatch, dtype, T, d, f, K, k, act):
     """d_model and d_ff that are multiples of 64 but not of a tile's width: the last column tile of every matrix is
     multiplied with what lies behind the slot's weights and must not store it."""
     from harness import Case, check_against_oracle
+    if dtype == I.F32 and d < 640:
+        monkeypatch.setenv("SWAPMOE_FP32_TC", "1")  # short contractions run on the warp-level kernel otherwise
     cfg = _cfg(T=T, dtype=dtype, d=d, f=f, E=8, K=K, k=k, act=act, renorm=k > 1)
     case = Case(cfg, phys=list(range(1, K)) + [0])
     check_against_oracle(case, case.run())
@@ -705,6 +709,7 @@ def test_ragged_column_tiles(dtype, T, d, f, K, k, act):
 def test_fp32_cta_pairs(monkeypatch, T, d, f, K, k, act, min_rows):
     """fp32 layers with well over 128 rows per slot: 256 x 192 tiles on CTA pairs, both operands split by both CTAs."""
     from harness import Case, check_against_oracle
+    monkeypatch.setenv("SWAPMOE_FP32_TC", "1")
     if min_rows:
         monkeypatch.setenv("SWAPMOE_PAIR32_MIN_ROWS", min_rows)
         monkeypatch.setenv("SWAPMOE_FP32_SWAP", "0")
@@ -760,3 +765,42 @@ def test_host_path_reads_behind_the_kernel_in_front(T, d, k):
         a.layer.forward(xs[i % 3], pinned)
         b.layer.forward_host(pinned, out)
         assert np.array_equal(to_host_f32(out), refs[i % 3]), i
+
+
+@pytest.mark.parametrize("d,f,act", [(64, 64, I.ACT_RELU), (192, 192, I.ACT_RELU), (320, 64, I.ACT_RELU),
+                                     (64, 192, I.ACT_SWIGLU), (704, 1216, I.ACT_RELU), (1088, 704, I.ACT_SWIGLU)])
+@pytest.mark.parametrize("T", [40, 1200])
+def test_fp32_ragged_layers_keep_their_precision(monkeypatch, T, d, f, act):
+    """fp32 layers whose widths are no multiple of 128 may only leave the warp-level kernel where that costs no precision
+    against 64 bits.  An operand of two bf16 pieces has a relative error spread over +-2^-17, so a product of two of them
+    2^-17 sqrt(2/3) = 6.2e-6 of its size, which is also what a sum of many keeps; on short contractions the warp-level
+    kernel stays well under that."""
+    import torch
+    from paper_2308_15030_b200 import binding
+    g = torch.Generator(device="cuda").manual_seed(d + f)
+    E, K, nin = 8, 4, 2 if act else 1
+    Wr = 0.1 * torch.randn(E, d, device="cuda", generator=g)
+    x = torch.randn(T, d, device="cuda", generator=g)
+    a_in = torch.randn(K, nin, f, d, device="cuda", generator=g) / d ** 0.5
+    a_out = torch.randn(K, d, f, device="cuda", generator=g) / f ** 0.5
+    errs = []
+    xd, lg = x.double(), x.double() @ Wr.double().T[:, :K]
+    slot, gate = lg.argmax(1), torch.softmax(lg, 1).amax(1, keepdim=True)
+    ref = torch.zeros_like(xd)
+    for s in range(K):
+        t = (slot == s).nonzero()[:, 0]
+        h = xd[t] @ a_in[s, 0].double().T
+        h = torch.nn.functional.silu(h) * (xd[t] @ a_in[s, 1].double().T) if act else torch.relu(h)
+        ref[t] = gate[t] * (h @ a_out[s].double().T)
+    for path in (None, "0"):
+        if path:
+            monkeypatch.setenv("SWAPMOE_FP32_TC", path)
+        layer = binding.Layer(E, d, f, 1, K, I.F32, act, 0, max_tokens=T)
+        layer.set_router(Wr, np.ones(E, np.float32))
+        layer.set_resident(np.arange(K, dtype=np.int32), a_in, a_out)
+        out = torch.empty_like(x)
+        layer.forward(x, out)
+        errs.append(float((out.double() - ref).norm() / ref.norm()))
+    assert errs[0] <= errs[1] * 1.001, errs        # by itself / on the warp-level kernel
+    if d + f < 600:
+        assert errs[0] <= 5.5e-6, errs
