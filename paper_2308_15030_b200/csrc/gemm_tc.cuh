@@ -81,6 +81,16 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
+// The same for a barrier that the other CTA of a cluster signals: what it released is to be seen too.
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
 __device__ __forceinline__ uint64_t globaltimer_ns() {
   uint64_t t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -183,13 +193,16 @@ __host__ __device__ constexpr uint32_t make_idesc_bf16(int M, int N) {
 }
 
 // Bounded wait: polls the barrier, and every 256 polls checks a 2-second deadline.
-// Returns false (after recording `code`) when the wait gave up or another role aborted.
+// Returns false (after recording `code`) when the wait gave up or another role aborted.  kPeer: the other CTA of the
+// cluster signals the barrier.
+template <bool kPeer = false>
 __device__ __forceinline__ bool bounded_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
                                              int32_t* status, int code, uint64_t limit_ns = 2000000000ull) {
-  if (ptx::mbar_try_wait(bar, parity)) return true;
+  auto arrived = [&]() { return kPeer ? ptx::mbar_try_wait_cluster(bar, parity) : ptx::mbar_try_wait(bar, parity); };
+  if (arrived()) return true;
   const uint64_t t0 = ptx::globaltimer_ns();
   for (uint32_t spin = 1;; ++spin) {
-    if (ptx::mbar_try_wait(bar, parity)) return true;
+    if (arrived()) return true;
     if ((spin & 255u) == 0) {
       if (*abort_flag) return false;
       if (ptx::globaltimer_ns() - t0 > limit_ns) {
@@ -202,11 +215,12 @@ __device__ __forceinline__ bool bounded_wait(uint64_t* bar, uint32_t parity, vol
 }
 
 // The same by a whole converged warp: true when the phase has completed for every lane.
+template <bool kPeer = false>
 __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int32_t* status,
                                           int code) {
-  bool ok = ptx::mbar_try_wait(bar, parity);
+  bool ok = kPeer ? ptx::mbar_try_wait_cluster(bar, parity) : ptx::mbar_try_wait(bar, parity);
   if (!__all_sync(0xffffffffu, ok)) {
-    if (!ok) ok = bounded_wait(bar, parity, abort_flag, status, code);
+    if (!ok) ok = bounded_wait<kPeer>(bar, parity, abort_flag, status, code);
     ok = __all_sync(0xffffffffu, ok);
   }
   return ok;

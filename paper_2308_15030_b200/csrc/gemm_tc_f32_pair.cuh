@@ -41,12 +41,14 @@ __device__ __forceinline__ void umma_bf16_ts_pair(uint32_t tmem_d, uint32_t tmem
       "r"(tmem_a), "l"(desc_b), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-// Arrival of a converter warp on the even CTA's barrier.  Its writes to shared and tensor memory are complete before it
-// (every writer has executed its proxy fence and tcgen05 wait and fence), and the tensor core of its own SM reads them, so
-// a CTA-scope release is what it needs; a cluster-scope one is a full memory fence behind the loads in flight
-// (0.86 us per k-block instead of 0.58).
-__device__ __forceinline__ void mbar_arrive_remote(uint32_t bar_cluster_addr) {
-  asm volatile("mbarrier.arrive.release.cta.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr) : "memory");
+// Arrival of a converter warp on the even CTA's barrier, whose waiter issues MMAs that read what the warp has written: tensor
+// memory, ordered by the tcgen05 fences on either side, and shared memory, for which the release has to reach the cluster.
+// It is restricted to this CTA's shared memory: an unrestricted one is a full memory fence behind the loads in flight (us per
+// forward, 3062 rows of 1024 x 2816 SwiGLU 386 against 256, 6400 of 768 x 3072 ReLU 380 against 260; with no release beyond the
+// CTA, which the waiter's SM is not bound to see, 254 and 256).
+__device__ __forceinline__ void mbar_arrive_converted(uint32_t bar_cluster_addr) {
+  asm volatile("fence.release.sync_restrict::shared::cta.cluster;" ::: "memory");
+  mbar_arrive_cluster(bar_cluster_addr);
 }
 }  // namespace ptx
 
@@ -138,7 +140,7 @@ tc_gemm_f32_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
       for (int kb = 0; kb < a.k_blocks; ++kb) {
         const bool early = t == pair && kb < pre;
         if (!early) {
-          ok = warp_wait(&empty[stage], phase ^ 1u, abort_flag, a.status, 51);
+          ok = warp_wait<true>(&empty[stage], phase ^ 1u, abort_flag, a.status, 51);
           if (!ok) break;
         }
         if (ptx::elect_one()) {
@@ -166,12 +168,12 @@ tc_gemm_f32_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
       uint32_t slot_phase = 0, acc_phase = 0;
       bool ok = true;
       for (int t = pair; t < total && ok; t += n_pairs) {
-        ok = warp_wait(&acc_empty[acc], acc_phase ^ 1u, abort_flag, a.status, 52);
+        ok = warp_wait<true>(&acc_empty[acc], acc_phase ^ 1u, abort_flag, a.status, 52);
         if (!ok) break;
         ptx::tc_fence_after();
         const uint32_t tmem_d = tmem_base + (uint32_t)(acc * kF32PairBN);
         for (int kb = 0; kb < a.k_blocks; ++kb) {
-          ok = warp_wait(&conv_done[slot], slot_phase, abort_flag, a.status, 53);
+          ok = warp_wait<true>(&conv_done[slot], slot_phase, abort_flag, a.status, 53);
           if (!ok) break;
           ptx::tc_fence_after();
           // layouts of a converted stage and slot: see tc_gemm_f32_kernel; small terms first
@@ -209,7 +211,7 @@ tc_gemm_f32_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
       for (int kb = 0; kb < a.k_blocks; ++kb) {
         if ((slot & 1) == grp) {
           ok = warp_wait(&full[stage], phase, abort_flag, a.status, 54);
-          if (ok) ok = warp_wait(&lo_empty[slot], slot_phase ^ 1u, abort_flag, a.status, 55);
+          if (ok) ok = warp_wait<true>(&lo_empty[slot], slot_phase ^ 1u, abort_flag, a.status, 55);
           if (!ok) break;
           ptx::tc_fence_after();
           if (!does_b) {
@@ -246,7 +248,7 @@ tc_gemm_f32_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
           ptx::tc_fence_before();
           ptx::fence_proxy_async();                    // these writes are read by the tensor cores (async proxy)
           __syncwarp();
-          if (lane == 0) ptx::mbar_arrive_remote(done0 + 8u * (uint32_t)slot);
+          if (lane == 0) ptx::mbar_arrive_converted(done0 + 8u * (uint32_t)slot);
         }
         if (++stage == kStages) { stage = 0; phase ^= 1u; }
         if (++slot == kSlots) { slot = 0; slot_phase ^= 1u; }
@@ -263,7 +265,7 @@ tc_gemm_f32_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
       const int z = t / per_slice, u = t - z * per_slice;
       const int ct = u / n_row_tiles;
       const TileDesc td = a.tiles[u - ct * n_row_tiles];
-      ok = warp_wait(&acc_full[acc], acc_phase, abort_flag, a.status, 56);
+      ok = warp_wait<true>(&acc_full[acc], acc_phase, abort_flag, a.status, 56);
       if (!ok) break;
       ptx::tc_fence_after();
       if (rank == 0 || td.rows > kTcBM) {              // the odd CTA has nothing to store for a tile of <= 128 rows

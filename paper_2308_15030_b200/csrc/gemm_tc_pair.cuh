@@ -55,10 +55,11 @@ __device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* m
       ::"r"(smem_u32(dst)), "l"(map), "r"(bar_cluster_addr), "r"(c0), "r"(c1)
       : "memory");
 }
-// Relaxed: the arrival says that the accumulator has been READ (tcgen05.wait::ld has returned), nothing about the stores
-// that follow from it.  With .release every epilogue warp waited here until its tile's global stores had been performed,
-// behind the operand loads in flight (24044 rows,
-// d_model 1024, d_ff 512, y in fp32: GEMM-2 alone 49 -> 42 us; 8192 rows 768 x 3072: GEMM-1 49.5 -> 46.0).
+// Arrival on a barrier that the peer CTA's threads wait on (mbar_try_wait_cluster).  Relaxed at cluster scope: with the tcgen05
+// fences on either side it orders this warp's tcgen05 accesses (the accumulator has been read, tcgen05.wait::ld has
+// returned) before the waiter's, and nothing else is handed over: nobody in this kernel reads the stores of the epilogue.  With
+// .release every epilogue warp waited here until its tile's global stores had been performed, behind the operand loads in
+// flight (24044 rows, d_model 1024, d_ff 512, y in fp32: GEMM-2 alone 49 -> 42 us; 8192 rows 768 x 3072: GEMM-1 49.5 -> 46.0).
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster_addr) {
   asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr) : "memory");
 }
@@ -198,7 +199,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       for (int kb = 0; kb < a.k_blocks; ++kb) {
         const bool early = t == pair && kb < pre;          // armed and weights requested above
         if (!early) {
-          ok = warp_wait(&empty[stage], phase ^ 1u, abort_flag, a.status, 11);
+          ok = warp_wait<true>(&empty[stage], phase ^ 1u, abort_flag, a.status, 11);
           if (!ok) break;
         }
         const uint32_t bar = full0 + 8u * (uint32_t)stage;
@@ -224,12 +225,12 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       uint32_t phase = 0, acc_phase = 0;
       bool ok = true;
       for (int t = pair; t < total && ok; t += n_pairs) {
-        ok = warp_wait(&acc_empty[acc], acc_phase ^ 1u, abort_flag, a.status, 12);
+        ok = warp_wait<true>(&acc_empty[acc], acc_phase ^ 1u, abort_flag, a.status, 12);
         if (!ok) break;
         ptx::tc_fence_after();
         const uint32_t tmem_d = tmem_base + (uint32_t)(acc * kPairBN);
         for (int kb = 0; kb < a.k_blocks; ++kb) {
-          ok = warp_wait(&full[stage], phase, abort_flag, a.status, 13);
+          ok = warp_wait<true>(&full[stage], phase, abort_flag, a.status, 13);
           if (!ok) break;
           ptx::tc_fence_after();
           if (lane == 0 && t == pair && kb == 0) SWAPMOE_STAMP(kTr, 4);
@@ -272,7 +273,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
         gate = a.gate[p];
         drow = p / a.top_k;
       }
-      ok = bounded_wait(&acc_full[acc], acc_phase, abort_flag, a.status, 14);
+      ok = bounded_wait<true>(&acc_full[acc], acc_phase, abort_flag, a.status, 14);
       if (!ok) break;
       ptx::tc_fence_after();
       if (rank == 0 || td.rows > kTcBM) {      // the odd CTA has nothing to read for a tile of <= 128 rows

@@ -804,3 +804,25 @@ def test_fp32_ragged_layers_keep_their_precision(monkeypatch, T, d, f, act):
     assert errs[0] <= errs[1] * 1.001, errs        # by itself / on the warp-level kernel
     if d + f < 600:
         assert errs[0] <= 5.5e-6, errs
+
+
+@pytest.mark.parametrize("dtype,T,d,f,K,k,act", [(I.F32, 3000, 448, 1024, 5, 1, I.ACT_RELU), (I.F32, 1800, 512, 768, 4, 2, I.ACT_SWIGLU),
+                                                 (I.BF16, 6000, 512, 512, 4, 1, I.ACT_RELU), (I.BF16, 3000, 512, 768, 4, 2, I.ACT_SWIGLU)])
+def test_cta_pairs_repeat_bit_for_bit(monkeypatch, dtype, T, d, f, K, k, act):
+    """Forty forwards over two alternating batches on the CTA-pair kernels, nothing waited for in between: a tile that was
+    multiplied before its operands had been converted, or an accumulator overwritten before it had been read, would show
+    as a result that differs from the first of its batch."""
+    import torch
+    from harness import Case, check_against_oracle
+    monkeypatch.setenv("SWAPMOE_FP32_TC", "1")
+    monkeypatch.setenv("SWAPMOE_PAIR32_MIN_ROWS", "1")
+    case = Case(_cfg(T=T, dtype=dtype, d=d, f=f, E=8, K=K, k=k, act=act, renorm=k > 1))
+    check_against_oracle(case, case.run(), token_subset=range(0, T, 37))
+    xs = [case.d_x, torch.randn_like(case.d_x)]
+    outs = [torch.empty_like(case.d_x) for _ in range(40)]
+    for i, o in enumerate(outs):
+        case.layer.forward(xs[i & 1], o)
+    torch.cuda.synchronize()
+    for i, o in enumerate(outs[2:]):
+        assert torch.equal(o, outs[i & 1]), i
+    assert case.layer.device_status() == (0, 0)
