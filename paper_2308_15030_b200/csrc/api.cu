@@ -243,6 +243,7 @@ int32_t forward_impl(swapmoe_layer* L, const void* x, const float* ext_logits, v
   ra.cta_imp = L->cta_imp;
   ra.cta_cnt = L->cta_cnt; ra.cta_mimp = L->cta_mimp;
   ra.T = T; ra.d = c.d_model; ra.E = c.E; ra.k = c.top_k; ra.K = c.K; ra.renorm = c.renorm_topk;
+  ra.wave_rows = rs_wide_rows(c.d_model * 2 + kDecRowPad); ra.wave_bytes = rs_wide_bytes(c.d_model * 2 + kDecRowPad);
   ScanArgs& sa = ra.scan;
   sa.cta_hist = L->cta_hist; sa.cta_imp = L->cta_imp; sa.phys_slot = L->phys;
   // Up to 256 router CTAs the router only leaves its per-CTA histograms and the permute kernel sums them itself
@@ -294,10 +295,8 @@ int32_t forward_impl(swapmoe_layer* L, const void* x, const float* ext_logits, v
   if (rerun) {
     // measurement re-run: routing, permutation and tile list are those of the last forward
   } else if (small_router) {
-    if ((rs_nt == 1 ? launch_kernel(router_small_kernel<1>, dim3(n_cta + pf_ctas), dim3(kDecThreads),
-                                    router_small_smem_bytes(c.d_model, 1), st, pdl, ra, L->status)
-                    : launch_kernel(router_small_kernel<2>, dim3(n_cta + pf_ctas), dim3(kDecThreads),
-                                    router_small_smem_bytes(c.d_model, 2), st, pdl, ra, L->status)) != cudaSuccess)
+    if (launch_kernel(router_small_fn(c.d_model, rs_nt), dim3(n_cta + pf_ctas), dim3(kDecThreads),
+                      router_small_smem_bytes(c.d_model, rs_nt), st, pdl, ra, L->status) != cudaSuccess)
       return SWAPMOE_ERR_CUDA;
   } else if (tc_router) {
     if (x != L->map_x_ptr || T != L->map_x_T) {   // the token map is re-encoded only when x or T changes
@@ -593,7 +592,7 @@ int32_t swapmoe_create(swapmoe_layer_t** out, const swapmoe_config_t* cfg) {
     if (envt && std::atoi(envt) >= 1 && std::atoi(envt) <= kDecMaxPairs) L->decode_max_pairs = std::atoi(envt);
     const char* env = std::getenv("SWAPMOE_DECODE_PATH");   // SWAPMOE_DECODE_PATH=0: general kernels for tiny batches too
     L->decode_path = c.dtype == SWAPMOE_BF16 && !(env && env[0] == '0') &&
-                     decode_smem_bytes(c.d_model) <= (size_t)(226 << 10) &&
+                     c.d_model <= kDecMaxModel &&
                      decode_ws_floats(c.d_model, c.d_ff, c.top_k) * sizeof(float) <= ((size_t)64 << 20);
   }
   const size_t o_dec_ws = cv.take<float>(L->decode_path ? decode_ws_floats(c.d_model, c.d_ff, c.top_k) : 1);
@@ -673,23 +672,22 @@ int32_t swapmoe_create(swapmoe_layer_t** out, const swapmoe_config_t* cfg) {
   }
   {
     const char* env = std::getenv("SWAPMOE_SMALL_ROUTER");   // SWAPMOE_SMALL_ROUTER=0: tcgen05 router for small batches too
-    L->small_router = c.dtype == SWAPMOE_BF16 && !(env && env[0] == '0') &&
-                      router_small_smem_bytes(c.d_model, 1) <= (size_t)(226 << 10) + 512;   // (static memory beside it: 272 bytes)
+    L->small_router = c.dtype == SWAPMOE_BF16 && !(env && env[0] == '0') && router_small_takes(c.d_model, c.E, 1);
     if (L->small_router)
-      ok = ok && cuda_ok(cudaFuncSetAttribute(router_small_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      ok = ok && cuda_ok(cudaFuncSetAttribute(router_small_fn(c.d_model, 1), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)router_small_smem_bytes(c.d_model, 1)));
     L->small_router_f32 = c.dtype == SWAPMOE_F32 && !(env && env[0] == '0') &&
-                          router_small_f32_smem_bytes(c.d_model) <= (size_t)(226 << 10);
+                          router_small_f32_smem_bytes(c.d_model) <= kDecSmemLimit;
     if (L->small_router_f32)
       ok = ok && cuda_ok(cudaFuncSetAttribute(router_small_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)router_small_f32_smem_bytes(c.d_model)));
     // sixteen-token CTAs: while the grid stays within one wave of CTAs and the shared memory fits
     L->small_router_max_t = 0;
-    if (L->small_router && router_small_smem_bytes(c.d_model, 2) <= (size_t)(226 << 10)) {
+    if (L->small_router && router_small_takes(c.d_model, c.E, 2)) {
       L->small_router_max_t = 2 * kRsTok * L->sm_count;
       const char* envm = std::getenv("SWAPMOE_SMALL_ROUTER_MAX_T");
       if (envm) L->small_router_max_t = std::min(std::atoi(envm), 2 * kRsTok * 256);
-      ok = ok && cuda_ok(cudaFuncSetAttribute(router_small_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+      ok = ok && cuda_ok(cudaFuncSetAttribute(router_small_fn(c.d_model, 2), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)router_small_smem_bytes(c.d_model, 2)));
     }
   }

@@ -41,6 +41,7 @@ constexpr int kDecJB = 32;            // hidden units per work item
 constexpr int kDecGroup = 16;         // work items per first-step sum
 constexpr int kDecRowPad = 64;        // bytes added to a row's pitch in shared memory: neighbouring rows in different halves of the banks
 constexpr int kDecHalfBytes = 67584;  // one wave buffer (32 rows of 2112 bytes; a multiple of 512); there are two
+constexpr size_t kDecSmemLimit = 226 << 10;
 constexpr int kDecRecent = 4;         // recently served experts remembered per layer
 constexpr int kDecOutRows = 256;      // rows of W_out per TMA box
 constexpr int kDecOutBoxes = 4;       // boxes per W_out wave: 1024 rows
@@ -85,7 +86,7 @@ inline size_t decode_ticket_count(int f, int K) {
   return (size_t)K * groups + 1;
 }
 // rows of a row-contiguous matrix (row length d) per wave: a power of two, at most 32
-__host__ __device__ inline int decode_rows_per_wave(int d) {
+__host__ __device__ constexpr int decode_rows_per_wave(int d) {
   int rp = 32;
   while (rp > 1 && rp * (d * 2 + kDecRowPad) > kDecHalfBytes) rp >>= 1;
   return rp;
@@ -218,8 +219,8 @@ struct DecRoute {
 struct DecSmem {
   int xs, slog, hraw, hraw3, hsb, red, route, bars, total;
 };
-__host__ __device__ inline DecSmem decode_smem_layout(int d) {
-  DecSmem m;
+__host__ __device__ constexpr DecSmem decode_smem_layout(int d) {
+  DecSmem m{};
   int o = 2 * kDecHalfBytes;
   m.xs = o;    o += kDecMaxTokens * (d * 2 + kDecRowPad);
   m.slog = o;  o += kDecMaxTokens * (kMaxE + 1) * 4;
@@ -234,7 +235,12 @@ __host__ __device__ inline DecSmem decode_smem_layout(int d) {
   m.total = o;
   return m;
 }
-inline size_t decode_smem_bytes(int d) { return (size_t)decode_smem_layout(d).total + 1024; }
+constexpr size_t decode_smem_bytes(int d) { return (size_t)decode_smem_layout(d).total + 1024; }
+// Wider layers would fit up to 3776 with wave buffers of their own size, but the general kernels are faster there (3584 x 1792 at
+// one token 45 us in one launch, 28 in four; 3584 x 7168 at three 186 and 71), and a size that is no constant costs this
+// kernel 6 % (twelve layers of one token 207 / 220 us).
+constexpr int kDecMaxModel = 3520;
+static_assert(decode_smem_bytes(kDecMaxModel) <= kDecSmemLimit, "shared memory per CTA");
 
 __device__ __forceinline__ void mma_bf16_16x8x16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
                                                  uint32_t b0, uint32_t b1) {
@@ -331,9 +337,9 @@ __device__ __noinline__ void dec_wave_dots(const unsigned char* st, int rows, in
 // feed NT mma) and a contiguous share of the contraction; the 16 / tiles shares of a tile are added in order.
 // Per CTA that is one pair of barriers and a 4-way sum for 64 experts x 16 tokens, where the wave-by-wave form
 // (every wave's contraction split over all 16 warps) pays a 16-way sum and two barriers per wave.
-// slog[token * (kMaxE + 1) + expert] receives the logits.
+// slog[token * (kMaxE + 1) + expert] receives the logits.  half: bytes of a wave buffer.
 template <int NT>
-__device__ __forceinline__ void rs_dots_resident(const unsigned char* ring, int E, int RW, int d, const unsigned char* xs,
+__device__ __forceinline__ void rs_dots_resident(const unsigned char* ring, int half, int E, int RW, int d, const unsigned char* xs,
                                                  int n_tok, float* red, float* slog) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
   const int pitch = d * 2 + kDecRowPad;
@@ -344,7 +350,7 @@ __device__ __forceinline__ void rs_dots_resident(const unsigned char* ring, int 
   const int m = warp & (tiles_p2 - 1), part = warp / tiles_p2;
   if (m < MT) {
     const int row0 = m * 16;                    // first expert of the tile; wave row0 / RW, row row0 % RW inside it
-    const unsigned char* ap0 = ring + (row0 / RW) * kDecHalfBytes + ((row0 % RW) + g) * pitch + t * 16;
+    const unsigned char* ap0 = ring + (row0 / RW) * half + ((row0 % RW) + g) * pitch + t * 16;
     const unsigned char* xrow[NT];
 #pragma unroll
     for (int j = 0; j < NT; ++j) xrow[j] = xs + min(8 * j + g, n_tok - 1) * pitch + t * 16;
@@ -515,7 +521,7 @@ decode_fused_kernel(const __grid_constant__ CUtensorMap tmWo, const DecodeArgs a
     // contraction over all sixteen warps, costs a 16-way sum and two barriers per wave: twelve layers at one token 224.5
     // us per step, in one pass and with one fence per ticket less 210.6)
     for (int w = 0; w < n_rw && alive; ++w) alive = dec_wait_wave(bars, w, R, a.status, 21);
-    if (alive) rs_dots_resident<1>(ring, E, RW, d, xs, T, red, slog);
+    if (alive) rs_dots_resident<1>(ring, kDecHalfBytes, E, RW, d, xs, T, red, slog);
   } else {
 #pragma unroll 1
   for (int w = 0; w < n_rw; ++w) {

@@ -23,6 +23,7 @@ struct RouterArgs {
   float* cta_cnt;           // [n_cta, E] or nullptr
   float* cta_mimp;          // [n_cta, K] or nullptr
   int32_t T, d, E, k, K, renorm;
+  int32_t wave_rows, wave_bytes;   // small-batch bf16 router of wide layers: experts per wave, bytes of a wave buffer
   ScanArgs scan;            // work of the last CTA to finish
   // Weight prefetch (tensor-core router only): blocks beyond the token tiles pull the resident
   // experts' matrices into L2 while the router runs, when HBM is otherwise idle.

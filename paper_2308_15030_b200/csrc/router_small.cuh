@@ -29,12 +29,21 @@ struct RsRoute {
   float enorm[kMaxE];                      // ||E_e|| of every expert (the gate tasks would otherwise wait for a global load each)
 };
 
+// Layers whose token rows leave no room for two wave buffers of kDecHalfBytes (router_small_wide) have buffers of their own
+// size: the rows that fit in 66048 bytes, and no more bytes than those take.  In code of its own (kWide): sizes that are no
+// constants cost a twelve-layer step of 29 tokens 0.5 %.
+__host__ __device__ constexpr int rs_wide_rows(int pitch) {
+  int rp = 32;
+  while (rp > 1 && rp * pitch > 66048) rp >>= 1;
+  return rp;
+}
+__host__ __device__ constexpr int rs_wide_bytes(int pitch) { return (rs_wide_rows(pitch) * pitch + 511) & ~511; }
 struct RsSmem {
   int xs, slog, red, route, bars, pairs, total;
 };
-__host__ __device__ inline RsSmem router_small_layout(int d, int nt) {
-  RsSmem m;
-  int o = 2 * kDecHalfBytes;
+__host__ __device__ constexpr RsSmem router_small_layout(int d, int nt, int half) {
+  RsSmem m{};
+  int o = 2 * half;
   m.xs = o;    o += kRsTok * nt * (d * 2 + kDecRowPad);
   m.slog = o;  o += kRsTok * nt * (kMaxE + 1) * 4;
   o = (o + 15) & ~15;
@@ -46,13 +55,30 @@ __host__ __device__ inline RsSmem router_small_layout(int d, int nt) {
   m.total = o;
   return m;
 }
-inline size_t router_small_smem_bytes(int d, int nt) { return (size_t)router_small_layout(d, nt).total + 1024; }
+constexpr bool router_small_wide(int d, int nt) {
+  return (size_t)router_small_layout(d, nt, kDecHalfBytes).total + 1024 > kDecSmemLimit;
+}
+constexpr size_t router_small_smem_bytes(int d, int nt) {
+  return (size_t)router_small_layout(d, nt, router_small_wide(d, nt) ? rs_wide_bytes(d * 2 + kDecRowPad) : kDecHalfBytes).total +
+         1024;
+}
+// Layers that route here: with eight-token CTAs d_model up to 4096, with sixteen-token ones up to 1216, and somewhat wider ones
+// while their router matrix is at most four waves.  us per forward here / with the tcgen05 router: d_model 4160, eight
+// tokens 16 experts 48.7 / 56.7, 30 tokens 64 experts 94 / 78; sixteen-token CTAs, d_model 1280, 1200 tokens 16 experts
+// 68 / 74, 600 tokens 64 experts 106.3 / 106.7, 96 experts 52.2 / 49.6.
+constexpr bool router_small_takes(int d, int E, int nt) {
+  const int rows = rs_wide_rows(d * 2 + kDecRowPad);
+  return d <= (nt == 1 ? 4096 : 1216) || (d <= (nt == 1 ? 4288 : 1344) && (E + rows - 1) / rows <= 4);
+}
+static_assert(router_small_smem_bytes(4096, 1) <= kDecSmemLimit && router_small_smem_bytes(4288, 1) <= kDecSmemLimit &&
+              router_small_smem_bytes(1344, 2) <= kDecSmemLimit, "shared memory per CTA");
+static_assert(!router_small_wide(4032, 1) && !router_small_wide(1216, 2), "all but the widest use constant sizes");
 
 // dst[(8 j + n) * dst_stride + r] = <row r of the wave buffer, token 8 j + n> for r < rows <= 32, j < NT,
 // 8 j + n < n_tok: dec_wave_dots for NT column tiles at once (the weight fragments are loaded once).
 template <int NT>
 __device__ __forceinline__ void rs_wave_dots(const unsigned char* st, int rows, int d, const unsigned char* xs,
-                                             int n_tok, float* red, float* dst, int dst_stride) {
+                                             int n_tok, float* red, float* dst, int dst_stride, int rows_held) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
   const int pitch = d * 2 + kDecRowPad;
   float acc[2][NT][4];
@@ -64,7 +90,7 @@ __device__ __forceinline__ void rs_wave_dots(const unsigned char* st, int rows, 
       for (int q = 0; q < 4; ++q) acc[i][j][q] = 0.f;
   // (row indices beyond what a wave buffer holds at this row length are clamped to its last row: their products
   // are dropped, and no read leaves the buffer)
-  const int rmax = decode_rows_per_wave(d) - 1;
+  const int rmax = rows_held - 1;                            // what a wave buffer holds
   const unsigned char* ar[2][2];               // rows 16 i + 8 h + g of the buffer
 #pragma unroll
   for (int i = 0; i < 2; ++i)
@@ -101,7 +127,7 @@ __device__ __forceinline__ void rs_wave_dots(const unsigned char* st, int rows, 
   __syncthreads();
 }
 
-template <int NT>
+template <int NT, bool kWide>
 __global__ void __launch_bounds__(kDecThreads, 1) router_small_kernel(const RouterArgs a, int32_t* status) {
   constexpr int TOK = kRsTok * NT;                          // tokens per CTA
   if ((int)blockIdx.x >= a.scan.n_cta) {                    // blocks beyond the token tiles prefetch weights
@@ -116,7 +142,8 @@ __global__ void __launch_bounds__(kDecThreads, 1) router_small_kernel(const Rout
       (reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~static_cast<uintptr_t>(1023));
   const int d = a.d, E = a.E, k = a.k, K = a.K;
   const int chunks = d / 8, pitch = d * 2 + kDecRowPad;
-  const RsSmem lay = router_small_layout(d, NT);
+  const int half = kWide ? a.wave_bytes : kDecHalfBytes;
+  const RsSmem lay = router_small_layout(d, NT, half);
   unsigned char* ring = smem;
   unsigned char* xs = smem + lay.xs;
   float* slog = reinterpret_cast<float*>(smem + lay.slog);
@@ -131,15 +158,15 @@ __global__ void __launch_bounds__(kDecThreads, 1) router_small_kernel(const Rout
   const bf16* x = static_cast<const bf16*>(a.x) + (size_t)tok0 * d;
   const bf16* Wr = static_cast<const bf16*>(a.Wr);
 
-  const int RW = decode_rows_per_wave(d);
+  const int RW = kWide ? a.wave_rows : decode_rows_per_wave(d);
   const int n_rw = (E + RW - 1) / RW;
-  auto issue_router_wave = [&](int w) {                     // all warps (see issue_rows of the decode kernel)
+  auto issue_router_wave = [&](int w) {                     // all warps (see issue_router_rows of the decode kernel)
     const int rows = min(RW, E - w * RW);
     uint64_t* bar = &bars[w & 1];
     if (tid == 0) ptx::mbar_expect_tx(bar, (uint32_t)(rows * d * 2));
     for (int r = warp; r < rows; r += kDecWarps)
       if (ptx::elect_one())
-        ptx::bulk_load_1d(ring + (w & 1) * kDecHalfBytes + r * pitch, Wr + ((size_t)w * RW + r) * d, (uint32_t)(d * 2), bar);
+        ptx::bulk_load_1d(ring + (w & 1) * half + r * pitch, Wr + ((size_t)w * RW + r) * d, (uint32_t)(d * 2), bar);
     __syncwarp();
   };
   if (tid == 0) {
@@ -205,12 +232,12 @@ __global__ void __launch_bounds__(kDecThreads, 1) router_small_kernel(const Rout
     // the whole router matrix is resident in the two wave buffers: one pass over all experts
     for (int w = 0; w < n_rw && alive; ++w) alive = dec_wait_wave(bars, w, R, status, 23);
     if (tid == 0) SWAPMOE_STAMP(0, 11);
-    if (alive) rs_dots_resident<NT>(ring, E, RW, d, xs, T, red, slog);
+    if (alive) rs_dots_resident<NT>(ring, half, E, RW, d, xs, T, red, slog);
   } else {
 #pragma unroll 1
     for (int w = 0; w < n_rw; ++w) {
       if (!dec_wait_wave(bars, w, R, status, 23)) { alive = false; break; }
-      rs_wave_dots<NT>(ring + (w & 1) * kDecHalfBytes, min(RW, E - w * RW), d, xs, T, red, slog + w * RW, kMaxE + 1);
+      rs_wave_dots<NT>(ring + (w & 1) * half, min(RW, E - w * RW), d, xs, T, red, slog + w * RW, kMaxE + 1, RW);
       if (w + 2 < n_rw) {
         ptx::fence_proxy_async();
         issue_router_wave(w + 2);
@@ -332,8 +359,14 @@ __global__ void __launch_bounds__(kDecThreads, 1) router_small_kernel(const Rout
     while (ptx::globaltimer_ns() - t0 < 2000000ull) __nanosleep(1000);
   }
   if (tid == 0) SWAPMOE_STAMP(0, 6);
-  finish_router_cta(a.scan, ring, 2 * kDecHalfBytes);       // the wave buffers are free: stage the scan inputs there
+  finish_router_cta(a.scan, ring, 2 * half);                // the wave buffers are free: stage the scan inputs there
   if (tid == 0) SWAPMOE_STAMP(0, 10);
+}
+
+typedef void (*RouterSmallKernel)(const RouterArgs, int32_t*);
+inline RouterSmallKernel router_small_fn(int d, int nt) {
+  if (nt == 1) return router_small_wide(d, 1) ? router_small_kernel<1, true> : router_small_kernel<1, false>;
+  return router_small_wide(d, 2) ? router_small_kernel<2, true> : router_small_kernel<2, false>;
 }
 
 }  // namespace swapmoe

@@ -16,14 +16,15 @@ namespace swapmoe {
 
 // rows of an fp32 row-contiguous matrix (row length d) per wave: a power of two, at most 32
 constexpr int kRsfRowPad = 16;            // bytes added to a row's pitch in shared memory
-__host__ __device__ inline int rsf_rows_per_wave(int d) {
+constexpr int kRsfHalfBytes = 66048;      // one wave buffer (32 rows of 2064 bytes; a multiple of 512); there are two
+__host__ __device__ constexpr int rsf_rows_per_wave(int d) {
   int rp = 32;
-  while (rp > 1 && rp * (d * 4 + kRsfRowPad) > kDecHalfBytes) rp >>= 1;
+  while (rp > 1 && rp * (d * 4 + kRsfRowPad) > kRsfHalfBytes) rp >>= 1;
   return rp;
 }
-__host__ __device__ inline RsSmem router_small_f32_layout(int d) {
-  RsSmem m;
-  int o = 2 * kDecHalfBytes;
+__host__ __device__ constexpr RsSmem router_small_f32_layout(int d) {
+  RsSmem m{};
+  int o = 2 * kRsfHalfBytes;
   m.xs = o;    o += kRsTok * (d * 4 + kRsfRowPad);
   m.slog = o;  o += kRsTok * (kMaxE + 1) * 4;
   o = (o + 15) & ~15;
@@ -35,7 +36,8 @@ __host__ __device__ inline RsSmem router_small_f32_layout(int d) {
   m.total = o;
   return m;
 }
-inline size_t router_small_f32_smem_bytes(int d) { return (size_t)router_small_f32_layout(d).total + 1024; }
+constexpr size_t router_small_f32_smem_bytes(int d) { return (size_t)router_small_f32_layout(d).total + 1024; }
+static_assert(router_small_f32_smem_bytes(2112) <= kDecSmemLimit, "the small-batch fp32 router takes every d_model up to 2112");
 
 // dst[n * dst_stride + r] = <row r of the wave buffer, token n> for r < rows <= 32, n < n_tok <= 8 (fp32 rows,
 // split-TF32 products; the contraction is split over the warps in steps of 8 and added in warp order).
@@ -128,7 +130,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) router_small_f32_kernel(const 
     if (lane == 0) ptx::mbar_expect_tx(bar, (uint32_t)(rows * d * 4));
     __syncwarp();
     if (lane < rows)
-      ptx::bulk_load_1d(ring + (w & 1) * kDecHalfBytes + lane * pitch, Wr + ((size_t)w * RW + lane) * d, (uint32_t)(d * 4), bar);
+      ptx::bulk_load_1d(ring + (w & 1) * kRsfHalfBytes + lane * pitch, Wr + ((size_t)w * RW + lane) * d, (uint32_t)(d * 4), bar);
   };
   if (tid == 0) {
     ptx::mbar_init(&bars[0], 1);
@@ -179,7 +181,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) router_small_f32_kernel(const 
 #pragma unroll 1
   for (int w = 0; w < n_rw; ++w) {
     if (!dec_wait_wave(bars, w, R, status, 25)) { alive = false; break; }
-    rsf_wave_dots(ring + (w & 1) * kDecHalfBytes, min(RW, E - w * RW), d, xs, T, red, slog + w * RW, kMaxE + 1);
+    rsf_wave_dots(ring + (w & 1) * kRsfHalfBytes, min(RW, E - w * RW), d, xs, T, red, slog + w * RW, kMaxE + 1);
     if (warp == 0 && w + 2 < n_rw) {
       ptx::fence_proxy_async();
       issue_router_wave(w + 2);
@@ -257,7 +259,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) router_small_f32_kernel(const 
     const uint64_t t0 = ptx::globaltimer_ns();
     while (ptx::globaltimer_ns() - t0 < 2000000ull) __nanosleep(1000);
   }
-  finish_router_cta(a.scan, ring, 2 * kDecHalfBytes);       // the wave buffers are free: stage the scan inputs there
+  finish_router_cta(a.scan, ring, 2 * kRsfHalfBytes);       // the wave buffers are free: stage the scan inputs there
 }
 
 }  // namespace swapmoe

@@ -826,3 +826,27 @@ def test_cta_pairs_repeat_bit_for_bit(monkeypatch, dtype, T, d, f, K, k, act):
     for i, o in enumerate(outs[2:]):
         assert torch.equal(o, outs[i & 1]), i
     assert case.layer.device_status() == (0, 0)
+
+
+@pytest.mark.parametrize("dtype,T,d,E,k,K,launches", [
+    (I.BF16, 100, 1280, 64, 1, 8, 4),       # sixteen-token router CTAs: the widest layers they take, four waves of 16 experts
+    (I.BF16, 333, 1344, 50, 2, 9, 5),
+    (I.BF16, 70, 1344, 72, 1, 8, 4),        # ... five waves: the tcgen05 router
+    (I.BF16, 30, 4288, 16, 1, 5, 4),        # eight-token ones: four experts to a wave
+    (I.BF16, 9, 4160, 14, 2, 4, 5),
+    (I.BF16, 17, 2048, 40, 1, 6, 4),        # the widest with sixteen experts to a wave, and the first with eight
+    (I.BF16, 17, 2112, 40, 1, 6, 4),
+    (I.BF16, 3, 3520, 16, 1, 4, 1),         # one-launch decode kernel: the widest layer it takes, and the next width
+    (I.BF16, 3, 3584, 16, 1, 4, 4),
+    (I.F32, 50, 2112, 12, 1, 4, 5),         # fp32 small-batch router: the widest layers it takes, and the next width
+    (I.F32, 13, 2176, 9, 2, 4, 5),
+    (I.F32, 13, 2240, 9, 2, 4, 5),
+])
+def test_widest_layers_of_the_small_batch_kernels(dtype, T, d, E, k, K, launches):
+    """The wave buffers are sized by the layer's width: the widest layers that each small-batch kernel takes, where shared
+    memory is full, and the first ones behind them."""
+    from harness import Case, check_against_oracle
+    case = Case(_cfg(T=T, dtype=dtype, d=d, f=128, E=E, k=k, K=K, renorm=k > 1, zipf_s=1.0))
+    n0 = case.layer.launch_count
+    check_against_oracle(case, case.run())
+    assert case.layer.launch_count - n0 == launches
