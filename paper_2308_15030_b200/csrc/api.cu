@@ -264,21 +264,23 @@ int32_t forward_impl(swapmoe_layer* L, const void* x, const float* ext_logits, v
   ra.pf_total_bytes[0] = ra.pf_total_bytes[1] = 0;
   ra.pf_phys = L->phys;
   int pf_ctas = 0;
-  // Automatic: 16 MB for batches of up to 64 tokens, whose few router CTAs leave over 140 SMs and HBM idle for the length
-  // of the routing (eight layers of 768 x 3072, 12 slots, us per step without / with at 12, 29, 64 tokens: 267 / 255, 294 /
-  // 280, 301 / 289; of 1024 x 4096, 16 slots: 365 / 356, 493 / 488, 509 / 504; 8, 24 and 48 MB gain less).  Larger batches
-  // none: their router fills the chip, and every megabyte slows it by about what the first product gains (one layer of
-  // 768 x 3072 at 130 tokens 52.0 / 52.9, at 400 54.0 / 52.8, at 2048 54.7 / 54.9).
-  const long long pf_budget = L->l2_prefetch_bytes >= 0 ? L->l2_prefetch_bytes : (rs_nt == 1 ? 16ll << 20 : 0);
+  // Automatic: 16 MB for batches of up to 64 tokens, whose few router CTAs leave over 140 SMs and HBM idle for the length of the
+  // routing, the same part of every slot, so that it does not matter which ones are busy.  us per step of eight layers,
+  // without / with, tokens over all slots: 768 x 3072, 12 slots, 29 tokens 268 / 262, 64 295 / 283; 1024 x 4096, 16 slots, 29 436 /
+  // 429; 704 x 2240 at 64 278 / 264; tokens on four slots only, first or last ones: level (768 x 3072 at 29 216 / 215, 704 x
+  // 2240 at 64 221 / 222).  (The first slots whole gained 2 % more where those were the busy ones and lost 1 to 2 % where they
+  // were not.)  Not for small slots, whose router is as long as their products: 256 x 1024 at 29 125 / 138, 384 x 1536 150 / 157.
+  // Larger batches none: their router fills the chip, and every megabyte slows it by about what the first product gains (one
+  // layer of 768 x 3072 at 130 tokens 52.0 / 52.9, at 400 54.0 / 52.8, at 2048 54.7 / 54.9).
+  const long long in_slot = (long long)L->nin * c.d_ff * c.d_model * L->elem;
+  const long long out_slot = (long long)c.d_ff * c.d_model * L->elem;
+  const long long pf_budget = L->l2_prefetch_bytes >= 0 ? L->l2_prefetch_bytes
+                              : rs_nt == 1 && in_slot >= ((n_pairs >= c.K ? 2ll : 3ll) << 20) ? 16ll << 20 : 0;
   if (tc_router && use_tc && pf_budget > 0 && 2 * n_pairs >= L->prefetch_min_pairs * c.K &&
-      (long long)c.K * (L->nin + 1) * c.d_ff * c.d_model * (long long)L->elem <= (320ll << 20)) {
-    // Most slots will be touched (at least half a pair per slot): pull the resident weights towards L2 now,
-    // while the router and the permutation leave HBM idle (a slot that stays untouched costs idle bandwidth only).  GEMM-1's matrices first, then as much of GEMM-2's
-    // as the L2 budget allows.
-    const long long in_slot = (long long)L->nin * c.d_ff * c.d_model * L->elem;
-    const long long out_slot = (long long)c.d_ff * c.d_model * L->elem;
-    // In whole chunks of whole slots: chunk c belongs to slot c / (chunks per slot), so the total must not exceed K slots'
-    // chunks (a slot's last partial chunk is left out, and a slot smaller than a chunk altogether).
+      (in_slot + out_slot) * c.K <= (320ll << 20)) {
+    // Pull the resident weights towards L2 now, while the router and the permutation leave HBM idle: GEMM-1's matrices first,
+    // then as much of GEMM-2's as the budget allows.  In whole chunks (a slot's last partial chunk is left out, and a slot
+    // smaller than a chunk altogether).
     const long long in_chunks = in_slot / kPrefetchChunk * c.K, out_chunks = out_slot / kPrefetchChunk * c.K;
     const long long budget = pf_budget / kPrefetchChunk;
     const long long in_total = std::min(in_chunks, budget) * kPrefetchChunk;

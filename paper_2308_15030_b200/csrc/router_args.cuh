@@ -29,14 +29,14 @@ struct RouterArgs {
   // experts' matrices into L2 while the router runs, when HBM is otherwise idle.
   const char* pf_base[2];       // arena_in, arena_out
   long long pf_slot_bytes[2];   // bytes of one arena entry
-  long long pf_total_bytes[2];  // bytes to prefetch, in whole chunks of the logical slots 0..K-1 in order
+  long long pf_total_bytes[2];  // bytes to prefetch, in whole chunks: the first of every slot, then the second ...
   const int32_t* pf_phys;       // [K] arena entry of each logical slot
 };
 
 constexpr long long kPrefetchChunk = 16384;
 
 // Role of the blocks beyond the router's token tiles: pull the resident experts' matrices towards
-// L2 (GEMM-1's first, in slot order) while the router leaves HBM idle.
+// L2 (GEMM-1's first, all slots alike, first rows first) while the router leaves HBM idle.
 __device__ __forceinline__ void router_prefetch_role(const RouterArgs& a, int n_router_ctas) {
   constexpr long long kChunk = kPrefetchChunk;
   // chunks are dealt round-robin over the prefetch blocks: an SM sustains only about 200 GB/s of
@@ -46,10 +46,9 @@ __device__ __forceinline__ void router_prefetch_role(const RouterArgs& a, int n_
   const long long me = (long long)threadIdx.x * n_blk + (blockIdx.x - n_router_ctas);
 #pragma unroll 1
   for (int m = 0; m < 2; ++m) {
-    const long long per_slot = a.pf_slot_bytes[m] / kChunk;
     const long long n_chunks = a.pf_total_bytes[m] / kChunk;
     for (long long c = me; c < n_chunks; c += n_pf) {
-      const long long s = c / per_slot, o = c - s * per_slot;
+      const long long o = c / a.K, s = c - o * a.K;
       const char* src = a.pf_base[m] + (long long)a.pf_phys[s] * a.pf_slot_bytes[m] + o * kChunk;
       asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"((unsigned)kChunk) : "memory");
     }

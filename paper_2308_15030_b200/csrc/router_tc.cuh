@@ -53,19 +53,7 @@ router_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant_
     // ---------------------------------------------------- weight-prefetch blocks
     pdl_wait();
     pdl_trigger();
-    constexpr long long kChunk = kPrefetchChunk;
-    const long long n_pf = (long long)(gridDim.x - a.scan.n_cta) * kRtThreads;
-    const long long me = (long long)(blockIdx.x - a.scan.n_cta) * kRtThreads + threadIdx.x;
-#pragma unroll 1
-    for (int m = 0; m < 2; ++m) {
-      const long long per_slot = a.pf_slot_bytes[m] / kChunk;
-      const long long n_chunks = a.pf_total_bytes[m] / kChunk;
-      for (long long c = me; c < n_chunks; c += n_pf) {
-        const long long s = c / per_slot, o = c - s * per_slot;
-        const char* src = a.pf_base[m] + (long long)a.pf_phys[s] * a.pf_slot_bytes[m] + o * kChunk;
-        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"((unsigned)kChunk) : "memory");
-      }
-    }
+    router_prefetch_role(a, a.scan.n_cta);
     return;
   }
   const int E = a.E;

@@ -850,3 +850,17 @@ def test_widest_layers_of_the_small_batch_kernels(dtype, T, d, E, k, K, launches
     n0 = case.layer.launch_count
     check_against_oracle(case, case.run())
     assert case.layer.launch_count - n0 == launches
+
+
+@pytest.mark.parametrize("T,d,f,K,mb", [(20, 192, 320, 5, "64"), (300, 192, 320, 5, "1"), (20, 64, 64, 3, "1"), (40, 512, 2112, 6, None)])
+def test_weight_prefetch_changes_nothing(monkeypatch, T, d, f, K, mb):
+    """Weights pulled towards L2 beside both routers: slots of no whole number of chunks, slots smaller than one, budgets
+    that end inside a round over the slots and beyond everything there is."""
+    from harness import Case, check_against_oracle
+    if mb:
+        monkeypatch.setenv("SWAPMOE_PREFETCH_MB", mb)
+    case = Case(_cfg(T=T, d=d, f=f, E=8, K=K), phys=list(range(1, K)) + [0])
+    out = case.run()
+    check_against_oracle(case, out)
+    monkeypatch.setenv("SWAPMOE_PREFETCH_MB", "0")
+    assert np.array_equal(Case(_cfg(T=T, d=d, f=f, E=8, K=K), phys=list(range(1, K)) + [0]).run(), out)
