@@ -12,7 +12,15 @@ namespace swapmoe {
 constexpr int kGateTokMax = 128;   // largest token tile
 constexpr int kGateThreads = 256;
 
-// Running list of the N best logits, descending, as order-preserving keys (gate_key; 0 = nothing).  A candidate goes
+// Order-preserving key of a logit, as gate_key (equal for -0 and +0, never 0), with NaN as -inf: a logit that is NaN is chosen
+// only if no number is left.  (gate_key promises nothing about NaN: the sign of the sum it starts from is the compiler's
+// choice, and NaN came out above the negative logits.)
+__device__ __forceinline__ uint32_t gate_scan_key(float x) {
+  const uint32_t b = __float_as_uint(fmaxf(x, -INFINITY));
+  return (b & 0x80000000u) ? 0u - b : b + 0x80000000u;
+}
+
+// Running list of the N best logits, descending, as order-preserving keys (gate_scan_key; 0 = nothing).  A candidate goes
 // below every entry that is >= it, so equal values stay in arrival (= expert index) order.  Without branches: on a warp of
 // 32 tokens some token takes nearly every candidate, so a branch only adds its own cost (256 experts, top-4, 64
 // tokens per CTA: logits copy and this scan 23 -> 9.2 us).
@@ -39,7 +47,7 @@ struct TopK {
 };
 
 // The logit behind a list entry (an empty one, possible with fewer allowed experts than k, weighs nothing).
-__device__ __forceinline__ float gate_entry_value(uint32_t key) { return key ? gate_key_value(key) : -INFINITY; }
+__device__ __forceinline__ float gate_entry_value(const float* row, int e) { return e >= 0 ? row[e] : -INFINITY; }
 
 // The best N of the allowed experts [e_lo, e_hi) (e_lo a multiple of 32) of one logits row; at most seven floats
 // behind the row's end are read.
@@ -56,7 +64,7 @@ __device__ __forceinline__ void gate_scan(const float* row, const uint32_t* allo
 #pragma unroll
     for (int i = 0; i < 8; ++i) l[i] = row[e0 + i];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) tk.push((w >> i) & 1u ? gate_key(l[i]) : 0u, e0 + i);
+    for (int i = 0; i < 8; ++i) tk.push((w >> i) & 1u ? gate_scan_key(l[i]) : 0u, e0 + i);
   }
 #pragma unroll
   for (int j = 0; j < kMaxTopK; ++j) {
@@ -183,7 +191,7 @@ __device__ __forceinline__ void gate_epilogue(const RouterArgs& a, const GateSme
       for (int j = 0; j < kMaxTopK; ++j)
         if (j < k) fin.push(g.cand_v[src + j], g.cand_e[src + j]);      // (key 0, nothing there, displaces nothing)
     }
-    g.s_m[tl * 2 + (masked ? 1 : 0)] = gate_entry_value(fin.v[0]);
+    g.s_m[tl * 2 + (masked ? 1 : 0)] = gate_entry_value(row, fin.e[0]);
   }
   __syncthreads();
   if (threadIdx.x == 0) SWAPMOE_STAMP(0, 7);
@@ -209,12 +217,12 @@ __device__ __forceinline__ void gate_epilogue(const RouterArgs& a, const GateSme
   __syncthreads();
   if (threadIdx.x == 0) SWAPMOE_STAMP(0, 8);
   if (part == 0) {
-    const float m = gate_entry_value(fin.v[0]);
+    const float m = gate_entry_value(row, fin.e[0]);
     float den = 0.f;
     if (a.renorm) {
 #pragma unroll
       for (int j = 0; j < kMaxTopK; ++j)
-        if (j < k) den += expf(gate_entry_value(fin.v[j]) - m);
+        if (j < k) den += expf(gate_entry_value(row, fin.e[j]) - m);
     } else {
       for (int pp = 0; pp < parts; ++pp) den += g.part_den[((masked ? parts : 0) + pp) * tok + tl];
     }
@@ -224,7 +232,7 @@ __device__ __forceinline__ void gate_epilogue(const RouterArgs& a, const GateSme
       if (j < k) {
         const int pl = tl * k + j;
         const size_t p = (size_t)token * k + j;
-        const float gv = failed ? 0.f : expf(gate_entry_value(fin.v[j]) - m) / den;
+        const float gv = failed ? 0.f : expf(gate_entry_value(row, fin.e[j]) - m) / den;
         const int e = fin.e[j];
         if (!masked) {
           if (token < a.T) {

@@ -864,3 +864,20 @@ def test_weight_prefetch_changes_nothing(monkeypatch, T, d, f, K, mb):
     check_against_oracle(case, out)
     monkeypatch.setenv("SWAPMOE_PREFETCH_MB", "0")
     assert np.array_equal(Case(_cfg(T=T, d=d, f=f, E=8, K=K), phys=list(range(1, K)) + [0]).run(), out)
+
+
+@pytest.mark.parametrize("T,E,k", [(70, 40, 2), (33, 256, 4), (200, 13, 1)])
+def test_general_gate_passes_over_nan_logits(T, E, k):
+    """External logits with NaN (of either sign and payload) behind the first experts: as in the oracle's comparisons a NaN
+    never beats a number, so the tokens are routed, and weighted over their selection, by the others."""
+    from harness import Case, check_against_oracle
+    cfg = _cfg(T=T, E=E, K=6, k=k, d=64, f=256, renorm=1)
+    case = Case(cfg, s2e=[0, 1, 2, 3, 4, E - 1])
+    rng = np.random.default_rng(E)
+    lg = -np.abs(rng.standard_normal((T, E))).astype(np.float32)
+    lg[::4] = -lg[::4]
+    nan = np.array([0x7fc00000, 0xffc00000, 0x7f800001, 0xffffffff], np.uint32).view(np.float32)
+    for t in range(0, T, 3):
+        lg[t, 4 + rng.integers(0, E - 4, size=3)] = nan[t % 4]
+    lg[1, 5], lg[2, 4] = -np.inf, 3e38                    # (exp(inf - inf): a logit of +inf has no weight in the oracle either)
+    check_against_oracle(case, case.run(ext_logits=lg), check_logits=False)
