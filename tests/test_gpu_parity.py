@@ -724,8 +724,8 @@ def test_fp32_cta_pairs(monkeypatch, T, d, f, K, k, act, min_rows):
                                               (I.BF16, 300, 2, (True, False)), (I.F32, 257, 1, (False, True)),
                                               (I.BF16, 90, 1, (False, False))])
 def test_host_path_uses_pinned_buffers_in_place(dtype, T, k, pinned):
-    """swapmoe_forward_host with every mixture of pinned and pageable buffers, one of them a slice of a larger
-    allocation, from one row to more than a grid of the fetching kernel holds at once; and with one buffer for both."""
+    """swapmoe_forward_host with every mixture of pinned and pageable buffers, slices of larger allocations, from a few rows
+    to over a hundred CTAs of the fetching kernel; and with one buffer for both."""
     import torch
     from harness import Case, to_host_f32
     case = Case(_cfg(T=T, dtype=dtype, d=1024 if T > 2000 else 128, f=256, E=16, K=5, k=k, renorm=k > 1))
@@ -881,3 +881,93 @@ def test_general_gate_passes_over_nan_logits(T, E, k):
         lg[t, 4 + rng.integers(0, E - 4, size=3)] = nan[t % 4]
     lg[1, 5], lg[2, 4] = -np.inf, 3e38                    # (exp(inf - inf): a logit of +inf has no weight in the oracle either)
     check_against_oracle(case, case.run(ext_logits=lg), check_logits=False)
+
+
+@pytest.mark.parametrize("T,off,how", [(4607, 0, "pinned"), (4608, 0, "pinned"), (4609, 0, "pinned"),    # 9 MB at 1024 columns: in place up to it
+                                       (300, 1, "pinned"), (300, 8, "pinned"), (300, 0, "registered"), (300, 24, "registered")])
+def test_host_path_limits(T, off, how):
+    """Requests on both sides of the size from which the copies are used, buffers that start off a 16-byte boundary (off:
+    elements), and memory that the program has registered itself, whole or from somewhere inside."""
+    import torch
+    from harness import Case, to_host_f32
+    d = 1024 if T > 4000 else 128
+    case = Case(_cfg(T=T, d=d, f=256, E=16, K=5))
+    ref = case.run().copy()
+    bufs = [torch.zeros(T * d + 64, dtype=torch.bfloat16) for _ in range(2)]
+    if how == "pinned":
+        bufs = [b.pin_memory() for b in bufs]
+    else:
+        rt = torch.cuda.cudart()
+        assert all(int(rt.cudaHostRegister(b.data_ptr(), b.numel() * 2, 0)) == 0 for b in bufs)
+    try:
+        xh, oh = (b[off: off + T * d].view(T, d) for b in bufs)
+        xh.copy_(case.d_x.cpu())
+        for _ in range(2):
+            bufs[1].fill_(-1.0)
+            case.layer.forward_host(xh, oh)
+            assert np.array_equal(to_host_f32(oh), ref)
+            assert torch.all(bufs[1][:off] == -1.0) and torch.all(bufs[1][off + T * d:] == -1.0)
+    finally:
+        if how == "registered":
+            assert all(int(rt.cudaHostUnregister(b.data_ptr())) == 0 for b in bufs)
+
+
+@pytest.mark.parametrize("T,k,d", [(2, 1, 256), (40, 1, 256), (700, 2, 128)])
+def test_scores_between_forwards_without_a_wait(T, k, d):
+    """forward, read_scores_async with reset, forward, ... enqueued in one go: every snapshot holds the scores of the one
+    forward in front of it, as the waiting calls report them."""
+    import torch
+    from harness import Case
+    case = Case(_cfg(T=T, d=d, f=256, E=24, K=6, k=k, renorm=k > 1, zipf_s=1.0))
+    kinds = ("eq1", "count", "eq1_masked")
+    xs = [torch.roll(case.d_x, i, 1).contiguous() for i in range(6)]
+    want = []
+    for x in xs:
+        case.layer.forward(x, case.d_out)
+        want.append(np.stack([case.layer.read_score(n, reset=True) for n in kinds]))
+    snaps = [torch.full((3, 24), -1.0).pin_memory() for _ in range(24)]
+    for i, s in enumerate(snaps):
+        case.layer.forward(xs[i % 6], case.d_out)
+        case.layer.read_scores_async(kinds, s, reset=True)
+    torch.cuda.synchronize()
+    for i, s in enumerate(snaps):
+        assert np.array_equal(s.numpy(), want[i % 6]), i
+    assert len({w.tobytes() for w in want}) == 6
+
+
+@pytest.mark.parametrize("dtype,pairs", [(I.F32, None), (I.F32, "1"), (I.BF16, None)])
+def test_silu_over_its_range(monkeypatch, dtype, pairs):
+    """SwiGLU's activation from exp(-x) near 0 to infinite, on hidden units whose pre-activations are single exact products.
+    fp32: exp within 2 ulp, the sum and the two products half an ulp each, the reciprocal 1 ulp: 4.5 ulp of 2^-23 = 5.4e-7, and
+    bf16 half an ulp of 2^-8 on top (its exponential: 2 ulp + 1.2e-7 |x|, far below that)."""
+    import torch
+    from paper_2308_15030_b200 import binding
+    if pairs:
+        monkeypatch.setenv("SWAPMOE_PAIR32_MIN_ROWS", pairs)
+    d = f = 128
+    T = 160
+    dt = torch.float32 if dtype == I.F32 else torch.bfloat16
+    v = torch.cat([torch.linspace(-90, 90, 118), torch.tensor([-1e30, -2e2, -104.0, -88.5, -69.0, -1e-30, 0.0, 88.5, 2e2, 1e30])])
+    v = v.bfloat16().float()
+    scale = torch.linspace(-1.5, 1.5, T).bfloat16().float()
+    scale[0], scale[1] = 1.0, -1.0
+    a_in = torch.zeros(1, 2, f, d)
+    a_in[0, 0, :, 0] = v
+    a_in[0, 1, :, 1] = 1.0
+    x = torch.zeros(T, d)
+    x[:, 0], x[:, 1] = scale, 1.0
+    layer = binding.Layer(1, d, f, 1, 1, dtype, I.ACT_SWIGLU, 0, max_tokens=T)
+    layer.set_router(torch.zeros(1, d, dtype=dt, device="cuda"), np.ones(1, np.float32))
+    dev = [t.to(dt).cuda() for t in (x, a_in, torch.zeros(1, d, f))]
+    layer.set_resident(np.zeros(1, np.int32), dev[1], dev[2])
+    out = torch.empty_like(dev[0])
+    layer.forward(dev[0], out)
+    torch.cuda.synchronize()
+    h = layer.tap("h")
+    h = I.bits_to_f32(h) if dtype == I.BF16 else h
+    z = scale.double()[:, None] * v.double()[None, :]
+    ref = (z / (1.0 + torch.exp(-z))).numpy()
+    assert np.all(np.isfinite(h))
+    tol = 5.4e-7 if dtype == I.F32 else 2.0 ** -8
+    assert np.all(np.abs(h - ref) <= tol * np.abs(ref) + 1e-27)
+    assert layer.device_status() == (0, 0)
