@@ -90,13 +90,16 @@ static __device__ unsigned long long g_trace[kTraceKernels][kTraceCtas][kTraceSl
 // silu(x) = x / (1 + e) with e = exp(-x) given.  The division operator has a slow path behind a branch, which keeps the
 // compiler from interleaving the elements an epilogue thread works through: the epilogue of a 256 x 128 SwiGLU tile took
 // 22 us, more than its products (GEMM-1 alone at d_model 1024: 1400 rows, d_ff 3584 94.7 -> 35.5 us; 24044 rows, d_ff 512
-// 164 -> 69; d_model 4096, 8192 rows, d_ff 14336 1428 -> 1315).  Without a branch: the fast reciprocal, and one Newton-Raphson step for 1 / y
-// (r <- r + r (1 - y r)), which brings it from two ulp to one.  Beyond e = 1e30 the result is below 1e-28 and the step,
-// which would meet 0 x inf at the end of the range, is left out.
+// 164 -> 69; d_model 4096, 8192 rows, d_ff 14336 1428 -> 1315).  Without a branch: the fast reciprocal, one Newton-Raphson
+// step for 1 / y (r <- r + r (1 - y r)), and the quotient corrected by its remainder (q <- q + r (x - q y), Markstein 1990), which
+// leaves the error of the division operator (rms against 64 bits 4.34e-8 on either over x in [-3, 3], 5.00e-8 without the
+// correction).  From |x| = 69 on the steps, which would meet 0 x inf or inf - inf at the ends of the range, are left out: the
+// result is x there, or below 1e-28.
 __device__ __forceinline__ float silu_from_exp(float x, float e) {
   const float y = 1.f + e;
   const float r = __fdividef(1.f, y);
-  return x * (e < 1e30f ? fmaf(fmaf(-y, r, 1.f), r, r) : r);
+  const float r1 = fmaf(fmaf(-y, r, 1.f), r, r), q = x * r1;
+  return fabsf(x) < 69.f ? fmaf(fmaf(-q, y, x), r1, q) : x * r;
 }
 
 __device__ __forceinline__ float warp_sum(float v) {
