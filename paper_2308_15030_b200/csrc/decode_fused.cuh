@@ -816,9 +816,9 @@ decode_fused_kernel(const __grid_constant__ CUtensorMap tmWo, const DecodeArgs a
     const int gs = ti * n_jb + g_first;           // the group's first item, numbered over all items
     const int c_lo = gs / ipc, c_hi = (gs + g_size - 1) / ipc;
     const int n_sets = runs ? c_hi - c_lo + 1 : g_size;
-    // One thread publishes for the whole CTA: the block barrier above ordered everybody's stores
-    // before its fence (fences are cumulative), and its second fence orders the ticket before the
-    // reads of the other CTAs' rows (L2 loads below).
+    // One thread publishes for the whole CTA: the block barrier above orders everybody's stores before its ticket, whose
+    // release is cumulative, and the ticket's acquire with the barrier below orders the other CTAs' rows before their
+    // reads (L2 loads below).
     if (tid == 0) {
       R->last = dec_draw_ticket(&a.tickets[s * n_groups + grp]) == (unsigned)(n_sets - 1);
     }
