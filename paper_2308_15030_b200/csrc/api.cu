@@ -58,7 +58,7 @@ struct swapmoe_layer {
   int64_t launches;
   int32_t gemm_path;
   int32_t rows_pad_max;
-  int pair_min_rows;           // ... used when the slots hold at least this many rows on average (SWAPMOE_PAIR_MIN_ROWS)
+  int pair_min_rows;           // ... used when the slots hold at least this many rows on average (SWAPMOE_PAIR_MIN_ROWS, default 0)
   int gemm_pairs;              // CTA pairs available to the cta_group::2 grouped GEMM (0: not used; SWAPMOE_PAIR_GEMM=0)
   bool small_router_f32;       // fp32 layers: eight-token CTAs of the split-TF32 mma router (SWAPMOE_SMALL_ROUTER=0: never)
   bool small_router;           // eight-token mma router CTAs for batches of up to 64 tokens (bf16)
@@ -223,8 +223,9 @@ int32_t forward_impl(swapmoe_layer* L, const void* x, const float* ext_logits, v
   const int n_cta = (T + tok_tile - 1) / tok_tile;
   const int n_pairs = T * c.top_k;
   const bool use_tc = tc_selected(L->gemm_path, c, T);
-  const bool use_pairs = use_tc && tc_use_pairs(c, T, L->gemm_pairs, L->pair_min_rows);
-  const int mt = use_tc ? tc_row_subtiles(c, T, use_pairs) : 1;
+  // weight tiles per token tile of the grouped GEMMs on CTA pairs (0: one CTA per 128-row tile)
+  const int pc1 = use_tc && L->gemm_pairs > 0 ? tc_pair_cols(c, 1, n_pairs, L->pair_min_rows) : 0;
+  const int pc2 = use_tc && L->gemm_pairs > 0 ? tc_pair_cols(c, 2, n_pairs, L->pair_min_rows) : 0;
   const bool use_tc32 = !use_tc && L->tc32.enabled && L->tc32.arena_bound;
   // fp32 layers whose slots hold well under 128 rows on average: weights on the MMA's rows, the slot's tokens on its
   // columns (64-token tiles), so that no tensor time goes to empty rows (SWAPMOE_FP32_SWAP=0: never)
@@ -233,7 +234,7 @@ int32_t forward_impl(swapmoe_layer* L, const void* x, const float* ext_logits, v
   const bool pair32 = use_tc32 && !swap32 && L->tc32.n_pairs > 0 &&
                       (L->pair32_min_rows > 0 ? (long long)n_pairs >= (long long)L->pair32_min_rows * c.K
                                               : tc_f32_use_pairs(c, L->tc32.n_pairs, L->sm_count, n_pairs, L->y_copies));
-  const int tile_rows = use_tc ? kTcBM * mt : (use_tc32 ? (swap32 ? kF32SwapTok : pair32 ? 2 * kTcBM : kTcBM) : kMmaBM);
+  const int tile_rows = pc2 > 0 ? kPairMinTokens : use_tc ? kTcBM : (use_tc32 ? (swap32 ? kF32SwapTok : pair32 ? 2 * kTcBM : kTcBM) : kMmaBM);
   const int max_tiles = (n_pairs + tile_rows - 1) / tile_rows + c.K;
 
   RouterArgs ra;
@@ -256,9 +257,13 @@ int32_t forward_impl(swapmoe_layer* L, const void* x, const float* ext_logits, v
   sa.ticket = own_scan ? nullptr : L->ticket;
   sa.touched = L->touched;
   sa.n_cta = n_cta; sa.K = c.K; sa.E = c.E; sa.tile_rows = tile_rows;
-  // GEMM-2 with two row sub-tiles per CTA walks 256-row tiles; GEMM-1 then gets its own compact
-  // list of 128-row tiles (walking the 256-row list as pairs would leave holes in its schedule).
-  sa.tiles_b = mt == 2 ? L->tiles_b : nullptr; sa.n_tiles_b = L->n_tiles_b; sa.tile_rows_b = kTcBM;
+  sa.pair_cols = pc2; sa.inv_pairs = 1.f / (float)std::max(L->gemm_pairs, 1);
+  // GEMM-1 gets a list of its own where its tiles may be others
+  const int tile_rows1 = pc1 > 0 ? kPairMinTokens : use_tc ? kTcBM : tile_rows;
+  const bool two_lists = pc1 != pc2;
+  const int max_tiles1 = (n_pairs + tile_rows1 - 1) / tile_rows1 + c.K;
+  sa.tiles_b = two_lists ? L->tiles_b : nullptr; sa.n_tiles_b = L->n_tiles_b; sa.tile_rows_b = tile_rows1;
+  sa.pair_cols_b = pc1;
   ra.pf_base[0] = ra.pf_base[1] = nullptr;
   ra.pf_slot_bytes[0] = ra.pf_slot_bytes[1] = 16384;
   ra.pf_total_bytes[0] = ra.pf_total_bytes[1] = 0;
@@ -360,25 +365,33 @@ int32_t forward_impl(swapmoe_layer* L, const void* x, const float* ext_logits, v
   if (use_tc) {
     cudaEvent_t mid = L->stage_events ? static_cast<cudaEvent_t>(L->stage_events[4]) : nullptr;
     int32_t rc;
-    L->tc.only = rerun;
     if (L->small_path && n_pairs <= 64 && c.act == SWAPMOE_ACT_RELU) {
       if (rerun) return SWAPMOE_ERR_UNSUPPORTED;
       rc = tc_ffn_small(L->tc, L->small, c, L->xp, L->h, L->y, out, L->rows_pad_max, L->arena_in, L->arena_out,
                         L->tiles, L->n_tiles, L->row_pair, L->mgate, max_tiles, T, L->status, st, pdl,
                         &L->launches, &combined, mid);
-    } else if (mt == 2 && L->gemm_pairs > 0 && tc_wide_ok(c.d_ff)) {
-      // 256-row tiles: GEMM-1 always on CTA pairs (its one-CTA form pulls 48 KB per k-block); GEMM-2 on pairs for
-      // very large slots and where tc_gemm2_on_pairs says so, else on one CTA with two row sub-tiles (same bytes per
-      // flop, and a tile whose second half is empty costs half; cfg3: 128.6 -> 126.8 us)
-      rc = tc_ffn_pair(L->tc, L->gemm_pairs, c, L->h, L->y, out, L->tiles, L->n_tiles, L->row_pair, L->mgate, max_tiles,
-                       T, L->status, st, pdl, &L->launches, &combined, mid,
-                       use_pairs || tc_gemm2_on_pairs(c, T, L->gemm_pairs), L->row_group);
     } else {
-      rc = tc_ffn(L->tc, c, L->h, L->y, out, L->tiles, L->n_tiles, L->tiles_b, L->n_tiles_b, L->row_pair, L->mgate,
-                  max_tiles, mt, T,
-                  L->status, st, pdl, &L->launches, &combined, mid, L->row_group);
+      const TileDesc* tiles1 = two_lists ? L->tiles_b : L->tiles;
+      const int32_t* n_tiles1 = two_lists ? L->n_tiles_b : L->n_tiles;
+      const bool scatter = c.top_k == 1;
+      rc = SWAPMOE_OK;
+      if (rerun != 2) {
+        rc = pc1 > 0 ? tc_gemm_pair(L->tc, L->gemm_pairs, c, 1, L->h, tiles1, n_tiles1, max_tiles1, nullptr, nullptr, T,
+                                    L->status, st, pdl, L->row_group)
+                     : tc_gemm1(L->tc, c, L->h, tiles1, n_tiles1, max_tiles1, T, L->status, st, pdl, L->row_group);
+        L->launches++;
+      }
+      if (mid) cudaEventRecord(mid, st);
+      if (rc == SWAPMOE_OK && rerun != 1) {
+        void* dst = scatter ? out : static_cast<void*>(L->y);
+        rc = pc2 > 0 ? tc_gemm_pair(L->tc, L->gemm_pairs, c, 2, dst, L->tiles, L->n_tiles, max_tiles, L->row_pair,
+                                    L->mgate, T, L->status, st, pdl, L->row_group)
+                     : tc_gemm2(L->tc, c, dst, L->tiles, L->n_tiles, max_tiles, L->row_pair, L->mgate, T, L->status, st,
+                                pdl, L->row_group);
+        L->launches++;
+      }
+      combined = scatter;
     }
-    L->tc.only = 0;
     if (rc != SWAPMOE_OK) return rc;
   } else if (use_tc32) {
     cudaEvent_t mid = L->stage_events ? static_cast<cudaEvent_t>(L->stage_events[4]) : nullptr;
@@ -669,7 +682,7 @@ int32_t swapmoe_create(swapmoe_layer_t** out, const swapmoe_config_t* cfg) {
     const char* env = std::getenv("SWAPMOE_PAIR_GEMM");      // SWAPMOE_PAIR_GEMM=0: one CTA per tile for every shape
     L->gemm_pairs = (ok && L->tc.enabled && !(env && env[0] == '0')) ? tc_pair_init(L->sm_count) : 0;
     env = std::getenv("SWAPMOE_PAIR_MIN_ROWS");
-    L->pair_min_rows = env ? std::max(160, std::atoi(env)) : 1024;
+    L->pair_min_rows = env ? std::max(0, std::atoi(env)) : 0;
     if (std::getenv("SWAPMOE_DEBUG")) std::fprintf(stderr, "swapmoe: gemm_pairs=%d\n", L->gemm_pairs);
   }
   {

@@ -384,10 +384,9 @@ __device__ __forceinline__ void epi_store_tile(uint32_t taddr, unsigned char* st
   }
 }
 
-// MT = row sub-tiles of 128 rows that one CTA multiplies against the same weight tile.
-template <int BN, int MT = 1>
+template <int BN>
 struct TcSmem {
-  static constexpr int kABytes = MT * kTcBM * kTcBK * 2;
+  static constexpr int kABytes = kTcBM * kTcBK * 2;
   static constexpr int kBBytes = BN * kTcBK * 2;
   static constexpr int kStageBytes = kABytes + kBBytes;
   static constexpr int kStages = (kTcSmemBudget - 2048) / kStageBytes;
@@ -395,23 +394,17 @@ struct TcSmem {
   static constexpr int kBytes = kStages * kStageBytes + 2048 + kTcEpiStageBytes;
 };
 
-// C tile [128*MT, BN (or BN/2 for SwiGLU)] = epi(A[row0:row0+128*MT, :] * B[brow:brow+BN, :]^T).
-// With MT = 2 a slot's weight tile is loaded once for two 128-row sub-tiles (two TMEM
-// accumulators), which halves the weight bytes the SM has to ingest for slots with more
-// than 128 rows; a tile with <= 128 valid rows skips the second half entirely.
-template <int BN, int EPI, int MT = 1>
+// C tile [128, BN (or BN/2 for SwiGLU)] = epi(A[row0:row0+128, :] * B[brow:brow+BN, :]^T).
+template <int BN, int EPI>
 __global__ void __launch_bounds__(kTcThreads, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const TcGemmArgs a) {
-  using S = TcSmem<BN, MT>;
-  constexpr int kAccBufs = (2 * MT * BN <= 512) ? 2 : 1;   // TMEM accumulator sets
-  constexpr int kHalfBytes = kTcBM * kTcBK * 2;
+  using S = TcSmem<BN>;
   constexpr int kStages = S::kStages;
   constexpr int kNB = (EPI == kTcEpiSwigluBf16) ? 2 : 1;   // weight boxes per stage
   constexpr int kBoxRows = BN / kNB;
   constexpr int kOutCols = BN / kNB;                        // output columns per tile
-  constexpr uint32_t kTmemCols = kAccBufs * MT * BN <= 64 ? 64 : kAccBufs * MT * BN <= 128 ? 128
-                                 : kAccBufs * MT * BN <= 256 ? 256 : 512;      // a power of two
+  constexpr uint32_t kTmemCols = 2 * BN <= 64 ? 64 : 2 * BN <= 128 ? 128 : 2 * BN <= 256 ? 256 : 512;   // a power of two
   constexpr uint32_t kIdesc = make_idesc_bf16(kTcBM, BN);
 
   extern __shared__ unsigned char smem_raw[];
@@ -464,11 +457,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       const int4 raw = __ldcg(reinterpret_cast<const int4*>(a.tiles + rt));
       const TileDesc td = *reinterpret_cast<const TileDesc*>(&raw);
       const int brow = td.phys * a.b_rows_per_phys + ct * kBoxRows;
-      const int halves = (MT == 2 && td.rows > kTcBM) ? 2 : 1;
       pre = a.k_blocks < kStages ? a.k_blocks : kStages;
       for (int kb = 0; kb < pre; ++kb) {
         if (ptx::elect_one()) {
-          ptx::mbar_expect_tx(&full[kb], (uint32_t)(halves * a.a_box_bytes + S::kBBytes));
+          ptx::mbar_expect_tx(&full[kb], (uint32_t)(a.a_box_bytes + S::kBBytes));
 #pragma unroll
           for (int j = 0; j < kNB; ++j)
             ptx::tma_load_2d(sB + kb * S::kBBytes + j * kBoxRows * kTcBK * 2, &tmB, &full[kb], kb * kTcBK,
@@ -512,7 +504,6 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       const TileDesc td = (t == (int)blockIdx.x && rt == first_rt && rt < 32)
                               ? *reinterpret_cast<const TileDesc*>(&first_raw) : a.tiles[rt];
       const int brow = td.phys * a.b_rows_per_phys + ct * kBoxRows;
-      const int halves = (MT == 2 && td.rows > kTcBM) ? 2 : 1;
       for (int kb = 0; kb < a.k_blocks; ++kb) {
         const bool early = t == (int)blockIdx.x && kb < pre;   // armed and weights requested above
         if (!early) {
@@ -520,10 +511,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           if (!ok) break;
         }
         if (ptx::elect_one()) {
-          if (!early) ptx::mbar_expect_tx(&full[stage], (uint32_t)(halves * a.a_box_bytes + S::kBBytes));
-          for (int hf = 0; hf < halves; ++hf)
-            ptx::tma_load_2d(sA + stage * S::kABytes + hf * kHalfBytes, &tmA, &full[stage], kb * kTcBK,
-                             td.row0 + hf * kTcBM);
+          if (!early) ptx::mbar_expect_tx(&full[stage], (uint32_t)(a.a_box_bytes + S::kBBytes));
+          ptx::tma_load_2d(sA + stage * S::kABytes, &tmA, &full[stage], kb * kTcBK, td.row0);
           if (!early) {
 #pragma unroll
             for (int j = 0; j < kNB; ++j)
@@ -548,32 +537,22 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     uint32_t phase = 0, acc_phase = 0;
     bool ok = true;
     for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
-      int halves = 1;
-      {
-        int rt, ct_unused;
-        decode_tile(t, n_row_tiles, a.n_col_tiles, a.row_group, &rt, &ct_unused);
-        if (MT == 2) halves = a.tiles[rt].rows > kTcBM ? 2 : 1;
-      }
       ok = warp_wait(&acc_empty[acc], acc_phase ^ 1u, abort_flag, a.status, 2);
       if (!ok) break;
       ptx::tc_fence_after();
-      const uint32_t tmem_d = tmem_base + (uint32_t)(acc * MT * BN);
+      const uint32_t tmem_d = tmem_base + (uint32_t)(acc * BN);
       for (int kb = 0; kb < a.k_blocks; ++kb) {
         ok = warp_wait(&full[stage], phase, abort_flag, a.status, 3);
         if (!ok) break;
         if (first_full) { if (lane == 0) SWAPMOE_STAMP(kTr, 4); first_full = false; }
         ptx::tc_fence_after();
         const uint64_t db = make_kmajor_sw128_desc(ptx::smem_u32(sB + stage * S::kBBytes));
-        const uint64_t da0 = make_kmajor_sw128_desc(ptx::smem_u32(sA + stage * S::kABytes));
+        const uint64_t da = make_kmajor_sw128_desc(ptx::smem_u32(sA + stage * S::kABytes));
         if (ptx::elect_one()) {
-          for (int hf = 0; hf < halves; ++hf) {
-            const uint64_t da = da0 + (uint64_t)(hf * (kHalfBytes >> 4));
 #pragma unroll
-            for (int k = 0; k < kTcBK / kTcUmmaK; ++k) {
-              // advancing 16 elements along K inside the swizzled row = +32 bytes = +2 in the address field
-              ptx::umma_bf16(tmem_d + (uint32_t)(hf * BN), da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), kIdesc,
-                             (kb > 0 || k > 0) ? 1u : 0u);
-            }
+          for (int k = 0; k < kTcBK / kTcUmmaK; ++k) {
+            // advancing 16 elements along K inside the swizzled row = +32 bytes = +2 in the address field
+            ptx::umma_bf16(tmem_d, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), kIdesc, (kb > 0 || k > 0) ? 1u : 0u);
           }
           ptx::umma_commit(&empty[stage]);                             // frees the stage once these MMAs have read it
           if (kb + 1 == a.k_blocks) ptx::umma_commit(&acc_full[acc]);  // accumulator complete
@@ -582,7 +561,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         if (++stage == kStages) { stage = 0; phase ^= 1u; }
       }
       if (!ok) break;
-      if (++acc == kAccBufs) { acc = 0; acc_phase ^= 1u; }
+      if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
     }
     if (lane == 0) SWAPMOE_STAMP(kTr, 5);                  // last MMA issued
   } else if (warp >= 4) {
@@ -596,54 +575,42 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       int rt, ct;
       decode_tile(t, n_row_tiles, a.n_col_tiles, a.row_group, &rt, &ct);
       const TileDesc td = a.tiles[rt];
-      const int halves = (MT == 2 && td.rows > kTcBM) ? 2 : 1;
-      // where this thread's rows go (and, for the scatter epilogue, their gate values): two dependent
+      // where this thread's row goes (and, for the scatter epilogue, its gate value): two dependent
       // global loads, fetched while the tile's MMAs are still running
-      int drow_h[MT];                            // output row of C, -1: not stored
-      float gate_h[MT];
-#pragma unroll
-      for (int hf = 0; hf < MT; ++hf) {
-        const int rr = r + hf * kTcBM;           // row inside the (up to 256-row) tile
-        const bool valid = hf < halves && rr < td.rows;
-        drow_h[hf] = valid ? td.row0 + rr : -1;
-        gate_h[hf] = 1.f;
-        if (EPI == kTcEpiScatterBf16 && valid) {
-          const int p = a.row_pair[td.row0 + rr];
-          gate_h[hf] = a.gate[p];
-          drow_h[hf] = p / a.top_k;
-        }
+      int drow = r < td.rows ? td.row0 + r : -1;   // output row of C, -1: not stored
+      float gate = 1.f;
+      if (EPI == kTcEpiScatterBf16 && drow >= 0) {
+        const int p = a.row_pair[drow];
+        gate = a.gate[p];
+        drow = p / a.top_k;
       }
-      ok = bounded_wait(&acc_full[acc], acc_phase, abort_flag, a.status, 4);
+      ok = warp_wait(&acc_full[acc], acc_phase, abort_flag, a.status, 4);
       if (!ok) break;
       ptx::tc_fence_after();
-#pragma unroll
-      for (int hf = 0; hf < MT; ++hf) {
-        if (hf < halves) {
-          const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)((acc * MT + hf) * BN);
-          constexpr int kElem = (EPI == kTcEpiF32) ? 4 : 2;
-          if constexpr ((kOutCols * kElem) % 128 == 0) {
-            unsigned char* dst[8];
-            epi_row_pointers(dst, drow_h[hf], lane, a.C, (size_t)a.ldc, (size_t)ct * kOutCols, kElem);
-            epi_store_tile<EPI, kOutCols>(taddr, epi_stage + q * kTcEpiWarpStage, lane, gate_h[hf], dst, a.ldc - ct * kOutCols);
-          } else {
-            // tiles whose rows are no whole 128-byte chunks (the narrowest, and 80 columns): every thread stores its own
-            // row, sixteen columns at a time
-            bf16* dst = drow_h[hf] < 0 ? nullptr : static_cast<bf16*>(a.C) + (size_t)drow_h[hf] * a.ldc + (size_t)ct * kOutCols;
+      const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN);
+      constexpr int kElem = (EPI == kTcEpiF32) ? 4 : 2;
+      if constexpr ((kOutCols * kElem) % 128 == 0) {
+        unsigned char* dst[8];
+        epi_row_pointers(dst, drow, lane, a.C, (size_t)a.ldc, (size_t)ct * kOutCols, kElem);
+        epi_store_tile<EPI, kOutCols>(taddr, epi_stage + q * kTcEpiWarpStage, lane, gate, dst, a.ldc - ct * kOutCols);
+      } else {
+        // tiles whose rows are no whole 128-byte chunks (the narrowest, and 80 columns): every thread stores its own
+        // row, sixteen columns at a time
+        bf16* dst = drow < 0 ? nullptr : static_cast<bf16*>(a.C) + (size_t)drow * a.ldc + (size_t)ct * kOutCols;
 #pragma unroll 1
-            for (int c0 = 0; c0 < min(kOutCols, a.ldc - ct * kOutCols); c0 += 16) {
-              uint4 pc[2];
-              epi_load_pieces16<EPI>(taddr, c0, kOutCols, gate_h[hf], pc);
-              if (dst != nullptr) {
-                reinterpret_cast<uint4*>(dst + c0)[0] = pc[0];
-                reinterpret_cast<uint4*>(dst + c0)[1] = pc[1];
-              }
-            }
+        for (int c0 = 0; c0 < min(kOutCols, a.ldc - ct * kOutCols); c0 += 16) {
+          uint4 pc[2];
+          __syncwarp();
+          epi_load_pieces16<EPI>(taddr, c0, kOutCols, gate, pc);
+          if (dst != nullptr) {
+            reinterpret_cast<uint4*>(dst + c0)[0] = pc[0];
+            reinterpret_cast<uint4*>(dst + c0)[1] = pc[1];
           }
         }
       }
       ptx::tc_fence_before();
       ptx::mbar_arrive(&acc_empty[acc]);       // 128 arrivals hand the buffer back to the MMA warp
-      if (++acc == kAccBufs) { acc = 0; acc_phase ^= 1u; }
+      if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
     }
     if (threadIdx.x == 128) SWAPMOE_STAMP(kTr, 6);   // this CTA's last epilogue done
   }
@@ -674,10 +641,11 @@ struct TcState {
   CUtensorMap map_xp[4], map_h[4];    // activations [rows_pad, d] / [rows_pad, f]; box rows 128, 64, 32, 16
   CUtensorMap map_win[4];             // W_in flattened to 2D, one map per entry of kBn1Options
   CUtensorMap map_wout[4];            // W_out flattened to 2D, one map per entry of kBn2Options
+  CUtensorMap map_h_out, map_y_out;   // stores of h [rows_pad, f] (box 32 x 32; SwiGLU 16 x 32) and y [rows_pad, d] fp32 (32 x 32)
+  CUtensorMap map_win_gated;          // SwiGLU: W_in as sixteen rows of W1, the same sixteen of W3, ... (gemm_tc_pair.cuh)
   CUtensorMap map_wr;                 // router matrix [E, d], box 64 x Epad
   bool arena_bound;
   bool router_ok;                     // tensor-core router usable (bf16 layer)
-  int only;                           // 0: both grouped GEMMs; 1 / 2: launch only GEMM-1 / GEMM-2 (measurement re-runs)
 };
 
 // Every bf16 layer: d_model and d_ff are multiples of 64, so k-blocks are whole, and the last column tile may be ragged.
@@ -689,32 +657,6 @@ inline bool tc_supported(const swapmoe_config_t& c) {
 
 // Whether 256-column tiles suit a matrix of n columns: at most a fifth of the last tiles' width empty.
 inline bool tc_wide_ok(int n) { return (long long)(n + 255) / 256 * 256 * 4 <= 5ll * n; }
-
-// Row sub-tiles per CTA for a forward of T tokens: two when the average slot has well over
-// 128 rows (weight tiles are then shared by two sub-tiles), one for small slots (nothing to
-// share) and for very large ones (tensor-bound: keep the double-buffered accumulators).
-inline int tc_row_subtiles(const swapmoe_config_t& c, int T, bool cta_pairs = false) {
-  const long long rows_per_slot = (long long)T * c.top_k / c.K;
-  // CTA pairs (tc_gemm_pair_kernel) keep two accumulator sets, so they take the very large slots
-  if (cta_pairs && rows_per_slot >= 1024) return 2;
-  return (rows_per_slot >= 160 && rows_per_slot < 1024 && tc_wide_ok(c.d_model)) ? 2 : 1;
-}
-// Whether a forward with 256-row tiles runs on CTA pairs: slots of at least `min_rows` rows on average (a
-// 256-row tile with <= 128 valid rows leaves one SM of the pair idle, so ragged small slots stay with one CTA per tile).
-inline bool tc_use_pairs(const swapmoe_config_t& c, int T, int n_pairs, int min_rows) {
-  return n_pairs > 0 && (long long)T * c.top_k / c.K >= min_rows && tc_wide_ok(c.d_model) && tc_wide_ok(c.d_ff);
-}
-
-// Whether GEMM-2 of such a forward runs on CTA pairs although its slots are smaller than that.  One CTA with two row
-// sub-tiles fills tensor memory with one accumulator set, so a tile's epilogue is not overlapped, but a tile whose second
-// half is empty costs it half.  Alone, one CTA / pairs, us: short contractions, d_ff 512 59 / 49, 768 22.5 / 20.9,
-// 1024 117 / 95, 2048 29 / 24.5; long ones, 3072 46 / 51, 4096 113 / 123; and where the tiles fit one round of pairs two
-// SMs work on each instead of one: d_ff 3584, 32 tiles 44 / 27.
-inline bool tc_gemm2_on_pairs(const swapmoe_config_t& c, int T, int n_pairs) {
-  const long long rows = (long long)T * c.top_k;
-  const long long tiles = (rows / (2 * kTcBM) + (rows < c.K ? rows : c.K) / 2 + 1) * ((c.d_model + 255) / 256);
-  return c.d_ff <= 2048 || tiles <= n_pairs;
-}
 
 // Automatic choice: tensor cores whenever the shape allows it.
 inline bool tc_selected(int path, const swapmoe_config_t& c, int /*T*/) {
@@ -745,17 +687,16 @@ inline bool tc_encode_2d_box(PFN_encodeTiled enc, CUtensorMap* m, const void* ba
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int BN, int EPI, int MT = 1>
+template <int BN, int EPI>
 inline bool tc_set_smem_attr() {
-  return cudaFuncSetAttribute(tc_gemm_kernel<BN, EPI, MT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              TcSmem<BN, MT>::kBytes) == cudaSuccess;
+  return cudaFuncSetAttribute(tc_gemm_kernel<BN, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              TcSmem<BN>::kBytes) == cudaSuccess;
 }
 
-inline int32_t tc_init(TcState& s, const swapmoe_config_t& c, void* xp, void* h, float* /*y*/, int rows_pad) {
+inline int32_t tc_init(TcState& s, const swapmoe_config_t& c, void* xp, void* h, float* y, int rows_pad) {
   s.enabled = false;
   s.arena_bound = false;
   s.router_ok = false;
-  s.only = 0;
   if (c.dtype != SWAPMOE_BF16) return SWAPMOE_OK;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return SWAPMOE_ERR_CUDA;
@@ -774,14 +715,24 @@ inline int32_t tc_init(TcState& s, const swapmoe_config_t& c, void* xp, void* h,
     if (!tc_encode_2d(s.encode, &s.map_h[i], h, (uint64_t)rows_pad, (uint64_t)c.d_ff, (uint32_t)(kTcBM >> i)))
       return SWAPMOE_ERR_CUDA;
   }
+  if (!tc_encode_2d_box(s.encode, &s.map_h_out, h, (uint64_t)rows_pad, (uint64_t)c.d_ff, c.act == SWAPMOE_ACT_SWIGLU ? 16 : 32, 32,
+                        CU_TENSOR_MAP_SWIZZLE_NONE))
+    return SWAPMOE_ERR_CUDA;
+  {
+    const cuuint64_t dims[2] = {(cuuint64_t)c.d_model, (cuuint64_t)rows_pad};
+    const cuuint64_t strides[1] = {(cuuint64_t)c.d_model * 4};
+    const cuuint32_t box[2] = {32, 32}, estr[2] = {1, 1};
+    if (s.encode(&s.map_y_out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, y, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                 CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+      return SWAPMOE_ERR_CUDA;
+  }
   bool ok = tc_set_smem_attr<256, kTcEpiReluBf16>() && tc_set_smem_attr<128, kTcEpiReluBf16>() &&
             tc_set_smem_attr<64, kTcEpiReluBf16>() && tc_set_smem_attr<256, kTcEpiSwigluBf16>() &&
             tc_set_smem_attr<128, kTcEpiSwigluBf16>() && tc_set_smem_attr<64, kTcEpiSwigluBf16>() && tc_set_smem_attr<160, kTcEpiSwigluBf16>() &&
             tc_set_smem_attr<256, kTcEpiF32>() && tc_set_smem_attr<128, kTcEpiF32>() &&
             tc_set_smem_attr<64, kTcEpiF32>() && tc_set_smem_attr<32, kTcEpiF32>() &&
             tc_set_smem_attr<256, kTcEpiScatterBf16>() && tc_set_smem_attr<128, kTcEpiScatterBf16>() &&
-            tc_set_smem_attr<64, kTcEpiScatterBf16>() && tc_set_smem_attr<32, kTcEpiScatterBf16>() &&
-            tc_set_smem_attr<256, kTcEpiF32, 2>() && tc_set_smem_attr<256, kTcEpiScatterBf16, 2>();
+            tc_set_smem_attr<64, kTcEpiScatterBf16>() && tc_set_smem_attr<32, kTcEpiScatterBf16>();
   if (!ok) return SWAPMOE_ERR_CUDA;
   s.enabled = true;
   return SWAPMOE_OK;
@@ -799,6 +750,17 @@ inline int32_t tc_bind_arena(TcState& s, const swapmoe_config_t& c, const void* 
     if (!tc_encode_2d(s.encode, &s.map_wout[i], arena_out, (uint64_t)P * c.d_model, (uint64_t)c.d_ff,
                       (uint32_t)kBn2Options[i]))
       return SWAPMOE_ERR_CUDA;
+  if (nin == 2) {
+    const cuuint64_t d = (cuuint64_t)c.d_model, f = (cuuint64_t)c.d_ff;
+    const cuuint64_t dims[5] = {d, 16, 2, f / 16, (cuuint64_t)P};
+    const cuuint64_t strides[4] = {d * 2, f * d * 2, 16 * d * 2, 2 * f * d * 2};
+    const cuuint32_t box[5] = {(cuuint32_t)kTcBK, 16, 2, 4, 1};
+    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    if (s.encode(&s.map_win_gated, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(arena_in), dims, strides, box, estr,
+                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+      return SWAPMOE_ERR_CUDA;
+  }
   s.arena_bound = true;
   return SWAPMOE_OK;
 }

@@ -88,6 +88,7 @@ tc_gemm_f32_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
     ptx::prefetch_tmap(&tmA);
     ptx::prefetch_tmap(&tmB);
   }
+  ptx::cluster_start_sync();
   if (warp == 2) {
     ptx::tmem_alloc_pair(tmem_slot, 512);
     ptx::tmem_relinquish_pair();

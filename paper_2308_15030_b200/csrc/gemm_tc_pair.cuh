@@ -1,35 +1,37 @@
-// Grouped expert GEMM on CTA pairs (SwapMoE Section 2: the experts' FFN restricted to the
-// resident slots): two SMs share one 256-row x 256-column tile through tcgen05 `cta_group::2`.
+// Grouped expert GEMM on CTA pairs (SwapMoE Section 2: the experts' FFN restricted to the resident slots): two SMs share
+// one tile of 256 WEIGHT rows x up to 256 TOKENS through tcgen05 `cta_group::2`.
 //
-// Why a pair: with one SM per 128 x 256 tile every k-block of 64 costs 48 KB of operands (16 KB of
-// activations, 32 KB of weights) for 512 tensor-core clocks, which is more than an SM can ingest
-// while the tensor pipe runs at full rate.  In a pair each CTA stages its own 128 activation rows
-// and HALF of the weight tile (128 of the 256 weight rows); the MMA, issued by the even CTA for
-// both, reads the two halves from both shared memories and every CTA's tensor core fills the
-// accumulator of its own 128 rows (all 256 columns) in its own TMEM.  That is 32 KB per CTA and
-// k-block: the weight bytes an SM pulls are halved, a stage is 32 KB so six stages fit, and the
-// accumulator (256 columns) still fits twice, so the epilogue of one tile overlaps the next tile's
-// MMAs.
+// Why a pair: each CTA stages its own 128 weight rows and half of the tile's tokens; the MMA, issued by the even CTA for
+// both, reads the halves from both shared memories and every CTA's tensor core fills the accumulator of its own 128 weight
+// rows (all tokens) in its own TMEM.  That is at most 32 KB per CTA and 64-column k-block for 512 tensor clocks (one CTA
+// alone: 48 KB), and two accumulator sets fit tensor memory, so the epilogue of one tile overlaps the next tile's MMAs.
+// Why the weights are the MMA's rows: its columns then are tokens, whose number is free in steps of 32, so a slot costs
+// neither operand bytes nor tensor time for rows it does not have.  A slot's n rows are cut into tiles of equal height
+// (slot_layout_warp), and the ring holds more stages where the tiles are small: what a pair pulls per second is bytes in
+// flight over the latency of a load (2 us under load).
 //
-// Roles in each CTA (256 threads): warp 0 = TMA producer (own activation rows, own half of the
-// weight tile; completion is signalled on the EVEN CTA's `full` barrier, which expects the bytes
-// of both CTAs), warp 1 = MMA issuer (even CTA only), warp 2 = TMEM allocation, warps 4-7 =
-// epilogue for the CTA's own 128 rows.  `tcgen05.commit` with a two-CTA mask hands the stage back
-// to both producers and announces a finished accumulator to both epilogues; the epilogue warps of
-// both CTAs arrive on the even CTA's `acc_empty` barrier.  No load uses cluster multicast.  Every
-// wait is bounded as in tc_gemm_kernel.
+// Roles in each CTA (384 threads): warp 0 = TMA producer (completion is signalled on the EVEN CTA's `full` barrier, which
+// expects the bytes of both CTAs), warp 1 = MMA issuer (even CTA only), warp 2 = TMEM allocation, warps 4-11 =
+// epilogue of the CTA's own 128 weight rows.  `tcgen05.commit` with a two-CTA mask hands the stage back to both producers
+// and announces a finished accumulator to both epilogues; the epilogue warps of both CTAs arrive on the even CTA's
+// `acc_empty` barrier.  No load uses cluster multicast.  Every wait is bounded as in tc_gemm_kernel.
 #pragma once
 #include "gemm_tc.cuh"
 
 namespace swapmoe {
 
-constexpr int kPairBN = 256;                                  // accumulator columns of the pair's tile
-constexpr int kPairHalfRows = kPairBN / 2;                    // weight rows each CTA stages
-constexpr int kPairABytes = kTcBM * kTcBK * 2;                // 16 KB
-constexpr int kPairBBytes = kPairHalfRows * kTcBK * 2;        // 16 KB
-constexpr int kPairStageBytes = kPairABytes + kPairBBytes;
-constexpr int kPairStages = (kTcSmemBudget - 2048) / kPairStageBytes;
-constexpr int kPairSmemBytes = kPairStages * kPairStageBytes + 2048 + kTcEpiStageBytes;
+constexpr int kPairTokens = 256;                              // most tokens of a tile
+constexpr int kPairMinTokens = 64;                            // ... and the least that pick_tile_height allows it
+constexpr int kPairTokenStep = 32;                            // their number is a multiple of this
+constexpr int kPairThreads = 384;
+constexpr int kPairABytes = kTcBM * kTcBK * 2;                // 16 KB: the CTA's weight rows of a k-block
+constexpr int kPairBBytes = kPairTokens / 2 * kTcBK * 2;      // at most 16 KB: its tokens
+constexpr int kPairStageArea = 6 * (kPairABytes + kPairBBytes);   // 6 stages of 256 tokens, 8 of 128, 9 of 64
+constexpr int kPairMaxStages = 9;
+__device__ __forceinline__ int pair_stages(int max_tokens) { return max_tokens > 128 ? 6 : max_tokens > 64 ? 8 : 9; }
+constexpr int kPairWarpBytes = 4096;                          // staging of each epilogue warp
+// + alignment slack and barriers (1 KB each)
+constexpr int kPairSmemBytes = kPairStageArea + 2048 + 8 * kPairWarpBytes;
 
 namespace ptx {
 
@@ -47,6 +49,13 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t smem_addr, uint32_t rank
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// tcgen05.alloc.cta_group::2 takes columns in both SMs, so neither CTA may issue it before the other one has started: without
+// this a pair was seen waiting for ever in its allocation (8192 tokens, top-4 of 256 experts, where CTAs of the
+// permutation in front still occupy a part of the SMs when the pairs come up).
+__device__ __forceinline__ void cluster_start_sync() {
+  __syncthreads();
+  cluster_sync_all();
+}
 // Tile load whose completion bytes are credited to a barrier that may live in the peer CTA.
 __device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* map, uint32_t bar_cluster_addr, int c0,
                                                  int c1) {
@@ -55,6 +64,26 @@ __device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* m
       ::"r"(smem_u32(dst)), "l"(map), "r"(bar_cluster_addr), "r"(c0), "r"(c1)
       : "memory");
 }
+// The same for a box of five dimensions.
+__device__ __forceinline__ void tma_load_5d_pair(void* dst, const CUtensorMap* map, uint32_t bar_cluster_addr, int c0,
+                                                 int c1, int c2, int c3, int c4) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6, %7}], [%2];"
+      ::"r"(smem_u32(dst)), "l"(map), "r"(bar_cluster_addr), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4)
+      : "memory");
+}
+// A box of shared memory to global memory; columns and rows outside the matrix are left out.
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, const void* src, int c0, int c1) {
+  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];\ncp.async.bulk.commit_group;" ::"l"(map),
+               "r"(smem_u32(src)), "r"(c0), "r"(c1)
+               : "memory");
+}
+// At most N of this thread's stores still read their shared memory.
+template <int N>
+__device__ __forceinline__ void tma_store_wait_read() {
+  asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 // Arrival on a barrier that the peer CTA's threads wait on (mbar_try_wait_cluster).  Relaxed at cluster scope: with the tcgen05
 // fences on either side it orders this warp's tcgen05 accesses (the accumulator has been read, tcgen05.wait::ld has
 // returned) before the waiter's, and nothing else is handed over: nobody in this kernel reads the stores of the epilogue.  With
@@ -93,32 +122,44 @@ __device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
 
 }  // namespace ptx
 
-// C tile [256, 256 (128 for SwiGLU)] = epi(A[row0 : row0 + 256, :] * B^T); rows row0 + 128 r .. + 127 belong to
-// CTA r of the pair.  `a.tiles` lists 256-row tiles; a tile with <= 128 valid rows leaves the odd CTA without
-// activation rows to fetch or results to store (its tensor core multiplies stale shared memory into TMEM columns
-// nobody reads).
+struct TcPairArgs {
+  void* C;                  // [rows, ldc]
+  const TileDesc* tiles;    // token tiles: up to 256 rows, multiples of 32 but for a slot's last one
+  const int32_t* n_tiles;   // [0] their number, [1] what they hold at most (256, 128 or 64 tokens)
+  int32_t* status;
+  int32_t ldc;              // columns of C
+  int32_t n_col_tiles;      // weight tiles per slot (256 rows; SwiGLU 128 of either matrix)
+  int32_t k_blocks;
+  int32_t w_rows;           // weight rows per arena entry
+  int32_t row_group;        // token tiles per scheduling group (see decode_tile)
+  const int32_t* row_pair;  // [rows] pair index of each padded row (scatter epilogue)
+  const float* gate;        // [T*k] masked gate values (scatter epilogue)
+  int32_t early_w;          // 1: the tile list is final when the CTAs start: weights are requested early
+};
+
+// C[token, 256 (128 for SwiGLU) weight rows] = epi(W[256 rows, :] * x[tokens, :]^T); weight rows 128 r .. + 127 of the tile
+// belong to CTA r of the pair.  The even CTA stages the first half of the tile's tokens, the odd CTA the second.
+// SwiGLU: the 128 lanes hold sixteen rows of W1, the same sixteen of W3, the next sixteen of W1 ... (one 5-D TMA box), so the
+// two products of a hidden unit sit in lanes l and l + 16 of one epilogue warp.
 template <int EPI>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTcThreads, 1)
-tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                    const TcGemmArgs a) {
-  constexpr int kStages = kPairStages;
-  constexpr int kOutCols = (EPI == kTcEpiSwigluBf16) ? kPairBN / 2 : kPairBN;
-  constexpr uint32_t kTmemCols = 2 * kPairBN;                 // two accumulator sets
-  constexpr uint32_t kIdesc = make_idesc_bf16(2 * kTcBM, kPairBN);
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
+tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX128,
+                    const __grid_constant__ CUtensorMap tmX64, const __grid_constant__ CUtensorMap tmX32,
+                    const __grid_constant__ CUtensorMap tmX16, const __grid_constant__ CUtensorMap tmC, const TcPairArgs a) {
+  constexpr bool kSwiglu = EPI == kTcEpiSwigluBf16;
+  constexpr uint32_t kTmemCols = 2 * kPairTokens;             // two accumulator sets
 
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  unsigned char* sA = smem;                                   // [stages][128][64] bf16
-  unsigned char* sB = smem + kStages * kPairABytes;           // [stages][128][64] bf16
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kStages * kPairStageBytes);
+  unsigned char* sW = smem;                                   // [stages][128][64] bf16
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kPairStageArea);
   uint64_t* full = bars;                    // [stages]  used in the even CTA
-  uint64_t* empty = bars + kStages;         // [stages]  one in each CTA (the commit reaches both)
-  uint64_t* acc_full = bars + 2 * kStages;  // [2]       one in each CTA
+  uint64_t* empty = bars + kPairMaxStages;  // [stages]  one in each CTA (the commit reaches both)
+  uint64_t* acc_full = bars + 2 * kPairMaxStages;  // [2]  one in each CTA
   uint64_t* acc_empty = acc_full + 2;       // [2]       used in the even CTA
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  unsigned char* epi_stage = smem + kStages * kPairStageBytes + 1024;   // [4 warps][32 rows][128 bytes]
 
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp-uniform
   const uint32_t rank = ptx::cluster_ctarank();               // 0: issues the MMAs
@@ -128,13 +169,14 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   (void)kTr;
   if (threadIdx.x == 0) {
     SWAPMOE_STAMP(kTr, 0);
-    for (int s = 0; s < kStages; ++s) { ptx::mbar_init(&full[s], 1); ptx::mbar_init(&empty[s], 1); }
-    for (int b = 0; b < 2; ++b) { ptx::mbar_init(&acc_full[b], 1); ptx::mbar_init(&acc_empty[b], 8); }
+    for (int s = 0; s < kPairMaxStages; ++s) { ptx::mbar_init(&full[s], 1); ptx::mbar_init(&empty[s], 1); }
+    for (int b = 0; b < 2; ++b) { ptx::mbar_init(&acc_full[b], 1); ptx::mbar_init(&acc_empty[b], 16); }
     *abort_flag = 0;
     ptx::fence_barrier_init();
-    ptx::prefetch_tmap(&tmA);
-    ptx::prefetch_tmap(&tmB);
+    ptx::prefetch_tmap(&tmW);
+    ptx::prefetch_tmap(&tmX128);
   }
+  ptx::cluster_start_sync();                                  // before the first access to the peer's tensor memory
   if (warp == 2) {
     ptx::tmem_alloc_pair(tmem_slot, kTmemCols);               // issued in both CTAs: one allocation for the pair
     ptx::tmem_relinquish_pair();
@@ -145,26 +187,34 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   ptx::tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
-  // As in tc_gemm_kernel: with `early_b` each producer requests the weight boxes of its first stages before the
+  // tokens of a tile in the MMA's columns; each CTA stages half of them
+  auto tile_cols = [](int rows) { return (rows + kPairTokenStep - 1) & ~(kPairTokenStep - 1); };
+  const uint32_t full0 = ptx::map_to_cta(ptx::smem_u32(full), 0u);
+  auto load_w = [&](int stage, int kb, int phys, int ct) {
+    const uint32_t bar = full0 + 8u * (uint32_t)stage;
+    if (kSwiglu)
+      ptx::tma_load_5d_pair(sW + stage * kPairABytes, &tmW, bar, kb * kTcBK, 0, 0, ct * 8 + (int)rank * 4, phys);
+    else
+      ptx::tma_load_2d_pair(sW + stage * kPairABytes, &tmW, bar, kb * kTcBK,
+                            phys * a.w_rows + ct * 2 * kTcBM + (int)rank * kTcBM);
+  };
+
+  // As in tc_gemm_kernel: with `early_w` each producer requests the weight boxes of its first stages before the
   // dependent-launch wait.
   int pre = 0;
-  if (warp == 0 && a.early_b) {
-    const int n_rt = __ldcg(a.n_tiles);
+  if (warp == 0 && a.early_w) {
+    const int n_rt = __ldcg(a.n_tiles), early_stages = pair_stages(__ldcg(a.n_tiles + 1));
     if (pair < n_rt * a.n_col_tiles) {
       int rt, ct;
       decode_tile(pair, n_rt, a.n_col_tiles, a.row_group, &rt, &ct);
       const int4 raw = __ldcg(reinterpret_cast<const int4*>(a.tiles + rt));
       const TileDesc td = *reinterpret_cast<const TileDesc*>(&raw);
-      const int brow = td.phys * a.b_rows_per_phys +
-                       (EPI == kTcEpiSwigluBf16 ? ct * kPairHalfRows + (int)rank * a.b_rows_gate
-                                                : ct * kPairBN + (int)rank * kPairHalfRows);
-      pre = a.k_blocks < kStages ? a.k_blocks : kStages;
-      const uint32_t full0 = ptx::map_to_cta(ptx::smem_u32(full), 0u);
+      const uint32_t bytes = (uint32_t)(2 * kPairABytes + tile_cols(td.rows) * kTcBK * 2);
+      pre = a.k_blocks < early_stages ? a.k_blocks : early_stages;
       for (int kb = 0; kb < pre; ++kb) {
         if (ptx::elect_one()) {
-          if (rank == 0)
-            ptx::mbar_expect_tx(&full[kb], (uint32_t)((td.rows > kTcBM ? 2 : 1) * kPairABytes + 2 * kPairBBytes));
-          ptx::tma_load_2d_pair(sB + kb * kPairBBytes, &tmB, full0 + 8u * (uint32_t)kb, kb * kTcBK, brow);
+          if (rank == 0) ptx::mbar_expect_tx(&full[kb], bytes);
+          load_w(kb, kb, td.phys, ct);
         }
         __syncwarp();
       }
@@ -174,12 +224,13 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
   pdl_wait();      // the activations come from the preceding kernel
   pdl_trigger();
   if (threadIdx.x == 0) SWAPMOE_STAMP(kTr, 2);
-  const int n_row_tiles = *a.n_tiles;
+  const int n_row_tiles = a.n_tiles[0], max_tokens = a.n_tiles[1];
   const int total = n_row_tiles * a.n_col_tiles;
+  const int n_stages = pair_stages(max_tokens), x_bytes = max_tokens / 2 * kTcBK * 2;
+  unsigned char* sX = smem + n_stages * kPairABytes;          // [stages][max_tokens / 2][64] bf16
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer (both CTAs)
-    const uint32_t full0 = ptx::map_to_cta(ptx::smem_u32(full), 0u);
     int stage = 0;
     uint32_t phase = 0;
     bool ok = true;
@@ -187,29 +238,30 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       int rt, ct;
       decode_tile(t, n_row_tiles, a.n_col_tiles, a.row_group, &rt, &ct);
       const TileDesc td = a.tiles[rt];
-      const bool two_halves = td.rows > kTcBM;
-      // ReLU / plain: the pair's 256 weight rows are consecutive; SwiGLU: 128 rows of W1 (even CTA) and the
-      // same 128 rows of W3 (odd CTA)
-      const int brow = td.phys * a.b_rows_per_phys +
-                       (EPI == kTcEpiSwigluBf16 ? ct * kPairHalfRows + (int)rank * a.b_rows_gate
-                                                : ct * kPairBN + (int)rank * kPairHalfRows);
-      const int arow = td.row0 + (int)rank * kTcBM;
-      const bool load_a = rank == 0 || two_halves;
-      const uint32_t bytes = (uint32_t)((two_halves ? 2 : 1) * kPairABytes + 2 * kPairBBytes);
+      const int cols = tile_cols(td.rows), half = cols / 2;     // half: a multiple of 16, at most 128
+      const int xrow = td.row0 + (int)rank * half;
+      const uint32_t bytes = (uint32_t)(2 * kPairABytes + cols * kTcBK * 2);
       for (int kb = 0; kb < a.k_blocks; ++kb) {
         const bool early = t == pair && kb < pre;          // armed and weights requested above
         if (!early) {
           ok = warp_wait<true>(&empty[stage], phase ^ 1u, abort_flag, a.status, 11);
           if (!ok) break;
         }
-        const uint32_t bar = full0 + 8u * (uint32_t)stage;
         if (ptx::elect_one()) {
           if (rank == 0 && !early) ptx::mbar_expect_tx(&full[stage], bytes);
-          if (load_a) ptx::tma_load_2d_pair(sA + stage * kPairABytes, &tmA, bar, kb * kTcBK, arow);
-          if (!early) ptx::tma_load_2d_pair(sB + stage * kPairBBytes, &tmB, bar, kb * kTcBK, brow);
+          const uint32_t bar = full0 + 8u * (uint32_t)stage;
+          unsigned char* dst = sX + stage * x_bytes;
+          if (half == 128) {
+            ptx::tma_load_2d_pair(dst, &tmX128, bar, kb * kTcBK, xrow);
+          } else {                                             // boxes of 64, 32 and 16 rows
+            if (half & 64) ptx::tma_load_2d_pair(dst, &tmX64, bar, kb * kTcBK, xrow);
+            if (half & 32) ptx::tma_load_2d_pair(dst + (half & 64) * 128, &tmX32, bar, kb * kTcBK, xrow + (half & 64));
+            if (half & 16) ptx::tma_load_2d_pair(dst + (half & 96) * 128, &tmX16, bar, kb * kTcBK, xrow + (half & 96));
+          }
+          if (!early) load_w(stage, kb, td.phys, ct);
         }
         __syncwarp();
-        if (++stage == kStages) { stage = 0; phase ^= 1u; }
+        if (++stage == n_stages) { stage = 0; phase ^= 1u; }
       }
       if (lane == 0) SWAPMOE_STAMP(kTr, 3);
     }
@@ -225,26 +277,29 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       uint32_t phase = 0, acc_phase = 0;
       bool ok = true;
       for (int t = pair; t < total && ok; t += n_pairs) {
+        int rt, ct_unused;
+        decode_tile(t, n_row_tiles, a.n_col_tiles, a.row_group, &rt, &ct_unused);
+        const uint32_t idesc = make_idesc_bf16(2 * kTcBM, tile_cols(a.tiles[rt].rows));
         ok = warp_wait<true>(&acc_empty[acc], acc_phase ^ 1u, abort_flag, a.status, 12);
         if (!ok) break;
         ptx::tc_fence_after();
-        const uint32_t tmem_d = tmem_base + (uint32_t)(acc * kPairBN);
+        const uint32_t tmem_d = tmem_base + (uint32_t)(acc * kPairTokens);
         for (int kb = 0; kb < a.k_blocks; ++kb) {
           ok = warp_wait<true>(&full[stage], phase, abort_flag, a.status, 13);
           if (!ok) break;
           ptx::tc_fence_after();
           if (lane == 0 && t == pair && kb == 0) SWAPMOE_STAMP(kTr, 4);
-          const uint64_t da = make_kmajor_sw128_desc(ptx::smem_u32(sA + stage * kPairABytes));
-          const uint64_t db = make_kmajor_sw128_desc(ptx::smem_u32(sB + stage * kPairBBytes));
+          const uint64_t dw = make_kmajor_sw128_desc(ptx::smem_u32(sW + stage * kPairABytes));
+          const uint64_t dx = make_kmajor_sw128_desc(ptx::smem_u32(sX + stage * x_bytes));
           if (ptx::elect_one()) {
 #pragma unroll
             for (int k = 0; k < kTcBK / kTcUmmaK; ++k)
-              ptx::umma_bf16_pair(tmem_d, da + (uint64_t)(2 * k), db + (uint64_t)(2 * k), kIdesc, (kb > 0 || k > 0) ? 1u : 0u);
+              ptx::umma_bf16_pair(tmem_d, dw + (uint64_t)(2 * k), dx + (uint64_t)(2 * k), idesc, (kb > 0 || k > 0) ? 1u : 0u);
             ptx::umma_commit_pair(&empty[stage]);   // frees the stage in both CTAs once these MMAs have read it
             if (kb + 1 == a.k_blocks) ptx::umma_commit_pair(&acc_full[acc]);    // accumulator complete, in both CTAs
           }
           __syncwarp();
-          if (++stage == kStages) { stage = 0; phase ^= 1u; }
+          if (++stage == n_stages) { stage = 0; phase ^= 1u; }
         }
         if (!ok) break;
         if (lane == 0) SWAPMOE_STAMP(kTr, 5);
@@ -252,10 +307,15 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       }
     }
   } else if (warp >= 4) {
-    // -------------------------------------------------------------------- epilogue (own 128 rows)
-    const int q = warp - 4;                    // TMEM lane quarter this warp may read
-    const int r = q * 32 + lane;               // row of the CTA's half owned by this thread
-    const int rr = (int)rank * kTcBM + r;      // row inside the 256-row tile
+    // -------------------------------------------------------------------- epilogue (own 128 weight rows)
+    const int q = warp & 3;                    // TMEM lane quarter this warp may read
+    const int part = (warp - 4) >> 2;          // two warps per quarter take turns with the chunks of 32 tokens
+    const int odd = lane & 1, hi = lane >> 4;
+    // the warp's 4 KB: a box on its way to global memory (bf16: two), or output row and gate value of its 128 tokens
+    unsigned char* s_stage = smem + kPairStageArea + 1024 + (warp - 4) * kPairWarpBytes;
+    int2* s_dest = reinterpret_cast<int2*>(s_stage);
+    int buf = 0;
+    const uint32_t acc_empty0 = ptx::map_to_cta(ptx::smem_u32(acc_empty), 0u);
     int acc = 0;
     uint32_t acc_phase = 0;
     bool ok = true;
@@ -263,32 +323,104 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
       int rt, ct;
       decode_tile(t, n_row_tiles, a.n_col_tiles, a.row_group, &rt, &ct);
       const TileDesc td = a.tiles[rt];
-      const bool row_ok = rr < td.rows;
-      // where this thread's row goes (and, for the scatter epilogue, its gate value): two dependent
-      // global loads, fetched while the tile's MMAs are still running
-      int drow = row_ok ? td.row0 + rr : -1;     // output row of C, -1: not stored
-      float gate = 1.f;
-      if (EPI == kTcEpiScatterBf16 && row_ok) {
-        const int p = a.row_pair[td.row0 + rr];
-        gate = a.gate[p];
-        drow = p / a.top_k;
+      // first of this warp's output columns (32; SwiGLU 16), all of them in the matrix or none
+      const int col0 = kSwiglu ? (ct * 8 + (int)rank * 4 + q) * 16 : ct * 2 * kTcBM + (int)rank * kTcBM + q * 32;
+      const bool col_ok = col0 < a.ldc;
+      if (EPI == kTcEpiScatterBf16) {
+        // where the tokens of this warp's chunks go and their gate values: two dependent global loads that the tile's MMAs
+        // hide (fetched a chunk ahead they set the pace: d_model 1536, d_ff 1088, 10000 tokens, GEMM-2 61 us)
+        __syncwarp();                                          // the tile before has been read out
+#pragma unroll
+        for (int i = 0; i < kPairTokens / 64; ++i) {
+          const int token = (2 * i + part) * 32 + lane;
+          const int p = token < td.rows ? a.row_pair[td.row0 + token] : 0;      // top-1: the pair is the token
+          s_dest[i * 32 + lane] = make_int2(p, token < td.rows ? __float_as_int(a.gate[p]) : 0);
+        }
       }
-      ok = bounded_wait<true>(&acc_full[acc], acc_phase, abort_flag, a.status, 14);
+      ok = warp_wait<true>(&acc_full[acc], acc_phase, abort_flag, a.status, 14);
       if (!ok) break;
       ptx::tc_fence_after();
-      if (rank == 0 || td.rows > kTcBM) {      // the odd CTA has nothing to read for a tile of <= 128 rows
-        const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * kPairBN);
-        unsigned char* dst[8];
-        epi_row_pointers(dst, drow, lane, a.C, (size_t)a.ldc, (size_t)ct * kOutCols, EPI == kTcEpiF32 ? 4 : 2);
-        epi_store_tile<EPI, kOutCols>(taddr, epi_stage + q * kTcEpiWarpStage, lane, gate, dst, a.ldc - ct * kOutCols);
+      const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * kPairTokens);
+      const int last = (td.rows - 1) >> 5;                   // the tile's last chunk
+      const int my_last = last - ((last ^ part) & 1);        // this warp's last one (-1: none)
+      if (my_last < 0 && lane == 0) ptx::mbar_arrive_cluster(acc_empty0 + 8u * (uint32_t)acc);
+#pragma unroll 1
+      for (int c = part; c <= last; c += 2) {
+        const int t0 = 32 * c, left = td.rows - t0;          // valid tokens of this chunk (may exceed 32)
+        uint32_t v[32];
+        __syncwarp();                                        // the tensor-memory load is one of the whole warp
+        ptx::tmem_ld32(taddr + (uint32_t)t0, v);
+        ptx::tmem_ld_wait();
+        if (c == my_last) {
+          // last read of this accumulator: one arrival per warp on the even CTA's barrier, 16 hand it back to the MMA issuer
+          ptx::tc_fence_before();
+          __syncwarp();
+          if (lane == 0) ptx::mbar_arrive_cluster(acc_empty0 + 8u * (uint32_t)acc);
+        }
+        if (!col_ok) continue;
+        // Boxes of 32 tokens leave through the TMA unit (stored by the lanes themselves, eight warps' stores held up the
+        // operand loads: fp32 y, 24044 rows of 1024, GEMM-2 45.7 us against 41.2).  Rows up to the next multiple of 32 are
+        // stored with the valid ones: they lie in the slot's own segment, and nobody reads a row that no pair occupies.
+        unsigned char* stg = s_stage;
+        if (EPI != kTcEpiScatterBf16) {
+          if (EPI != kTcEpiF32) stg += (buf ^= 2048);
+          if (lane == 0) {
+            if (EPI == kTcEpiF32) ptx::tma_store_wait_read<0>();
+            else ptx::tma_store_wait_read<1>();
+          }
+          __syncwarp();
+        }
+        if (EPI == kTcEpiF32) {
+          float* w = reinterpret_cast<float*>(stg) + lane;     // [32 tokens][32 columns]
+#pragma unroll
+          for (int j = 0; j < 32; ++j) w[32 * j] = __uint_as_float(v[j]);
+        } else if (EPI == kTcEpiSwigluBf16) {
+          // lanes l and l + 16 hold the two products of hidden unit l & 15: the lower one finishes token 2 i, the upper one
+          // token 2 i + 1; then neighbours trade, so that each has two units of one token
+          uint32_t* w = reinterpret_cast<uint32_t*>(stg) + (2 * odd + hi) * 8 + ((lane & 14) >> 1);    // [32 tokens][16 units]
+          float o[16];
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            const float v0 = __uint_as_float(v[2 * i]), v1 = __uint_as_float(v[2 * i + 1]);
+            const float r = __shfl_xor_sync(0xffffffffu, hi ? v0 : v1, 16);
+            const float x1 = hi ? r : v0, x3 = hi ? v1 : r;
+            o[i] = silu_from_exp(x1, __expf(-x1)) * x3;
+          }
+#pragma unroll
+          for (int m = 0; m < 8; ++m) {
+            const float r = __shfl_xor_sync(0xffffffffu, odd ? o[2 * m] : o[2 * m + 1], 1);
+            w[32 * m] = odd ? pack_bf16x2(r, o[2 * m + 1]) : pack_bf16x2(o[2 * m], r);
+          }
+        } else {
+          // neighbouring lanes trade, so that each holds two output columns of one token (scatter: 64 contiguous bytes of
+          // two tokens per instruction)
+          uint32_t* w = reinterpret_cast<uint32_t*>(stg) + odd * 16 + (lane >> 1);      // [32 tokens][32 columns]
+          bf16* dst = static_cast<bf16*>(a.C) + col0 + (lane & 30);
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            const float v0 = __uint_as_float(v[2 * i]), v1 = __uint_as_float(v[2 * i + 1]);
+            const float r = __shfl_xor_sync(0xffffffffu, odd ? v0 : v1, 1);
+            const float lo = odd ? r : v0, up = odd ? v1 : r;
+            if (EPI == kTcEpiReluBf16) {
+              w[32 * i] = pack_bf16x2(fmaxf(lo, 0.f), fmaxf(up, 0.f));
+            } else {
+              const int j = 2 * i + odd;
+              const int2 to = s_dest[(c >> 1) * 32 + j];
+              const float g = __int_as_float(to.y);
+              if (j < left) *reinterpret_cast<uint32_t*>(dst + (size_t)to.x * a.ldc) = pack_bf16x2(lo * g, up * g);
+            }
+          }
+        }
+        if (EPI != kTcEpiScatterBf16) {
+          ptx::fence_proxy_async();                            // the staged box is read by the TMA unit
+          __syncwarp();
+          if (lane == 0) ptx::tma_store_2d(&tmC, stg, col0, td.row0 + t0);
+        }
       }
-      ptx::tc_fence_before();
-      __syncwarp();
-      // one arrival per warp, on the even CTA's barrier: 8 arrivals hand the buffer back to the MMA issuer
-      if (lane == 0) ptx::mbar_arrive_cluster(ptx::map_to_cta(ptx::smem_u32(&acc_empty[acc]), 0u));
-      if (r == 0) SWAPMOE_STAMP(kTr, 6);
+      if (q == 0 && lane == 0) SWAPMOE_STAMP(kTr, 6);
       if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
     }
+    if (EPI != kTcEpiScatterBf16 && lane == 0) ptx::tma_store_wait_all();
   }
   ptx::tc_fence_before();
   __syncthreads();
@@ -298,6 +430,9 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_consta
     ptx::tmem_dealloc_pair(tmem_base, kTmemCols);
   }
 }
+
+typedef void (*TcPairKernel)(const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap, const CUtensorMap,
+                             const CUtensorMap, const TcPairArgs);
 
 template <int EPI>
 inline bool tc_pair_set_smem_attr() {
@@ -313,7 +448,7 @@ inline int tc_pair_init(int sm_count) {
     return 0;
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(2 * (sm_count / 2)); cfg.blockDim = dim3(kTcThreads); cfg.dynamicSmemBytes = kPairSmemBytes;
+  cfg.gridDim = dim3(2 * (sm_count / 2)); cfg.blockDim = dim3(kPairThreads); cfg.dynamicSmemBytes = kPairSmemBytes;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
@@ -326,85 +461,41 @@ inline int tc_pair_init(int sm_count) {
   return n < sm_count / 2 ? n : sm_count / 2;
 }
 
-// Runs both grouped GEMMs on CTA pairs over the list of 256-row tiles.  With top_k == 1 the second
-// GEMM writes gate * y straight into `out` (*combined = true) and no combine kernel is needed.
-inline int32_t tc_ffn_pair(TcState& s, int n_pairs, const swapmoe_config_t& c, void* h, float* y, void* out,
-                           const TileDesc* tiles, const int32_t* n_tiles, const int32_t* row_pair, const float* mgate,
-                           int max_tiles, int n_tokens, int32_t* status, cudaStream_t st, bool pdl, int64_t* launches,
-                           bool* combined, cudaEvent_t between = nullptr, bool gemm2_pairs = true,
-                           int row_group_forced = 0) {
+// Launches GEMM-1 (which = 1) or GEMM-2 (2) of a layer on CTA pairs over its list of token tiles.  With top_k == 1 the second
+// GEMM writes gate * y straight into `out` and no combine kernel is needed.
+inline int32_t tc_gemm_pair(TcState& s, int n_pairs, const swapmoe_config_t& c, int which, void* out, const TileDesc* tiles,
+                            const int32_t* n_tiles, int max_tiles, const int32_t* row_pair, const float* mgate,
+                            int n_tokens, int32_t* status, cudaStream_t st, bool pdl, int row_group_forced) {
   if (!s.enabled || !s.arena_bound || n_pairs < 1) return SWAPMOE_ERR_NOT_READY;
-  const bool swiglu = c.act == SWAPMOE_ACT_SWIGLU;
-  const bool scatter = c.top_k == 1;
-  const int out1 = swiglu ? kPairBN / 2 : kPairBN;
+  const bool swiglu = c.act == SWAPMOE_ACT_SWIGLU, scatter = c.top_k == 1;
   const long long pairs = (long long)n_tokens * c.top_k;
-  int row_group = 1 << 30;
-  if (row_group_forced > 0) row_group = row_group_forced;
+  TcPairArgs g;
+  g.C = out; g.status = status; g.tiles = tiles; g.n_tiles = n_tiles; g.row_pair = row_pair; g.gate = mgate;
+  g.row_group = 1 << 30;
+  if (row_group_forced > 0) g.row_group = row_group_forced;
   else if (pairs * (long long)c.d_model * 2 > (48ll << 20)) {
     // groups of about 20 MB of token rows (Mixtral shape, 4096 tokens: 8-12 tiles of 256 rows measure 2.58-2.70 ms
     // per forward, 16 tiles 2.68-2.80, 32 tiles 2.86-3.01, 4 tiles 2.68-2.72, 1 tile 3.0)
-    row_group = (int)((20ll << 20) / (2ll * kTcBM * c.d_model * 2));
-    if (row_group < 4) row_group = 4;
+    g.row_group = (int)((20ll << 20) / (2ll * kTcBM * c.d_model * 2));
+    if (g.row_group < 4) g.row_group = 4;
   }
-  TcGemmArgs g1;
-  g1.C = h; g1.status = status; g1.ldc = c.d_ff;
-  g1.tiles = tiles; g1.n_tiles = n_tiles;
-  g1.n_col_tiles = (c.d_ff + out1 - 1) / out1;
-  g1.k_blocks = c.d_model / kTcBK;
-  g1.b_rows_per_phys = swiglu ? 2 * c.d_ff : c.d_ff;
-  g1.b_rows_gate = swiglu ? c.d_ff : 0;
-  g1.row_pair = nullptr; g1.gate = nullptr; g1.top_k = c.top_k;
-  g1.row_group = row_group;
-  g1.a_box_bytes = kPairABytes;
-  g1.early_b = 0;
-  long long work = (long long)max_tiles * g1.n_col_tiles;
-  int grid = 2 * (work > n_pairs ? n_pairs : (int)work);
-  // weight boxes of 128 rows: kBn1Options[1] for one input matrix, kBn1Options[0] / 2 for SwiGLU's two
-  cudaError_t e = s.only == 2 ? cudaSuccess :
-      swiglu ? launch_kernel(tc_gemm_pair_kernel<kTcEpiSwigluBf16>, dim3(grid), dim3(kTcThreads), kPairSmemBytes, st, pdl,
-                             s.map_xp[0], s.map_win[0], g1)
-             : launch_kernel(tc_gemm_pair_kernel<kTcEpiReluBf16>, dim3(grid), dim3(kTcThreads), kPairSmemBytes, st, pdl,
-                             s.map_xp[0], s.map_win[1], g1);
-  if (e != cudaSuccess) return SWAPMOE_ERR_CUDA;
-  if (s.only != 2) ++*launches;
-  if (between) cudaEventRecord(between, st);
-  if (s.only == 1) { *combined = scatter; return SWAPMOE_OK; }
-
-  TcGemmArgs g2;
-  g2.C = scatter ? out : static_cast<void*>(y);
-  g2.tiles = tiles; g2.n_tiles = n_tiles; g2.status = status; g2.ldc = c.d_model;
-  g2.n_col_tiles = (c.d_model + kPairBN - 1) / kPairBN;
-  g2.k_blocks = c.d_ff / kTcBK;
-  g2.b_rows_per_phys = c.d_model;
-  g2.b_rows_gate = 0;
-  g2.row_pair = row_pair; g2.gate = mgate; g2.top_k = c.top_k;
-  g2.row_group = row_group;
-  g2.a_box_bytes = kPairABytes;
-  g2.early_b = 1;
-  work = (long long)max_tiles * g2.n_col_tiles;
-  grid = 2 * (work > n_pairs ? n_pairs : (int)work);
-  const bool pdl2 = pdl && between == nullptr;
-  if (!gemm2_pairs) {
-    // one CTA per 256-row tile with two row sub-tiles: the same operand bytes per flop as a pair, and a tile whose
-    // second half is empty costs half
-    g2.a_box_bytes = kTcBM * kTcBK * 2;
-    grid = work > s.sm_count ? s.sm_count : (int)work;
-    const TcGemmKernel k = scatter ? tc_gemm_kernel<256, kTcEpiScatterBf16, 2> : tc_gemm_kernel<256, kTcEpiF32, 2>;
-    if (launch_kernel(k, dim3(grid), dim3(kTcThreads), TcSmem<256, 2>::kBytes, st, pdl2, s.map_h[0], s.map_wout[0], g2) !=
-        cudaSuccess)
-      return SWAPMOE_ERR_CUDA;
-    ++*launches;
-    *combined = scatter;
-    return SWAPMOE_OK;
+  const CUtensorMap *mw, *mx, *mc;
+  TcPairKernel k;
+  if (which == 1) {
+    const int out1 = swiglu ? kTcBM : 2 * kTcBM;
+    g.ldc = c.d_ff; g.n_col_tiles = (c.d_ff + out1 - 1) / out1; g.k_blocks = c.d_model / kTcBK;
+    g.w_rows = c.d_ff; g.early_w = 0;
+    k = swiglu ? tc_gemm_pair_kernel<kTcEpiSwigluBf16> : tc_gemm_pair_kernel<kTcEpiReluBf16>;
+    mw = swiglu ? &s.map_win_gated : &s.map_win[1]; mx = s.map_xp; mc = &s.map_h_out;
+  } else {
+    g.ldc = c.d_model; g.n_col_tiles = (c.d_model + 2 * kTcBM - 1) / (2 * kTcBM); g.k_blocks = c.d_ff / kTcBK;
+    g.w_rows = c.d_model; g.early_w = 1;
+    k = scatter ? tc_gemm_pair_kernel<kTcEpiScatterBf16> : tc_gemm_pair_kernel<kTcEpiF32>;
+    mw = &s.map_wout[1]; mx = s.map_h; mc = &s.map_y_out;
   }
-  e = scatter ? launch_kernel(tc_gemm_pair_kernel<kTcEpiScatterBf16>, dim3(grid), dim3(kTcThreads), kPairSmemBytes, st, pdl2,
-                              s.map_h[0], s.map_wout[1], g2)
-              : launch_kernel(tc_gemm_pair_kernel<kTcEpiF32>, dim3(grid), dim3(kTcThreads), kPairSmemBytes, st, pdl2,
-                              s.map_h[0], s.map_wout[1], g2);
-  if (e != cudaSuccess) return SWAPMOE_ERR_CUDA;
-  ++*launches;
-  *combined = scatter;
-  return SWAPMOE_OK;
+  const long long work = (long long)max_tiles * g.n_col_tiles;
+  return launch_kernel(k, dim3(2 * (work > n_pairs ? n_pairs : (int)work)), dim3(kPairThreads), kPairSmemBytes, st, pdl, *mw,
+                       mx[0], mx[1], mx[2], mx[3], *mc, g) == cudaSuccess ? SWAPMOE_OK : SWAPMOE_ERR_CUDA;
 }
 
 }  // namespace swapmoe

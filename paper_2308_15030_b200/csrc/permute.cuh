@@ -19,7 +19,7 @@ struct ScanArgs {
   int32_t* offset;           // [K+1]  exclusive scan of count
   int32_t* pad_offset;       // [K+1]  same with every segment rounded up to kSegAlign rows
   TileDesc* tiles;           // GEMM work list
-  int32_t* n_tiles;          // [1]
+  int32_t* n_tiles;          // [2] their number, the most rows one may hold
   float* imp;                // [E] accumulator of Eq. (1)
   unsigned* ticket;          // [1] router CTAs finished so far (returns to 0); nullptr: the router CTAs do not
                              // scan at all - the permute kernel sums the histograms itself (see below)
@@ -27,6 +27,10 @@ struct ScanArgs {
   int32_t* n_tiles_b;
   unsigned long long* touched;   // [1] running total of slots that received at least one pair, or nullptr
   int32_t n_cta, K, E, tile_rows, tile_rows_b;
+  // > 0: a list of token tiles for CTA pairs, which take this many weight tiles per token tile (see pick_tile_height); 0: tiles
+  // of tile_rows rows
+  int32_t pair_cols, pair_cols_b;
+  float inv_pairs;           // 1 / CTA pairs that share the work
 };
 
 // Eq. (1) partial sums are added with ONE association wherever they are reduced: the router CTAs
@@ -47,6 +51,48 @@ __device__ __forceinline__ float reduce_column_serial(const float* src, int n_ro
   return total;
 }
 
+// Height of the tiles that `count` rows are cut into when none may hold more than 2^shift of them: all the same, rounded up
+// to a multiple of 32.
+__device__ __forceinline__ int even_tile_rows(int count, int shift) {
+  const int n = (count + (1 << shift) - 1) >> shift;
+  return n == 0 ? 0 : ((count + n - 1) / n + 31) & ~31;
+}
+
+// log2 of the most tokens a tile of a CTA-pair GEMM may hold, 6 to 8, for the slots of this warp's lanes (two each).  Large tiles
+// pull each weight less often; small ones are more, which fills the pairs, and their ring holds more stages.  A k-block of a
+// tile of h tokens takes 0.19 us + h ns (d_model 1024, d_ff 4096, eight slots, 12000 tokens, GEMM-1 alone, us, 64 / 128 / 256
+// tokens: 175 / 115 / 86), tiles are dealt out in turn, and of the two bounds on the longest share the lower one is
+// taken.  us for both GEMMs alone, 64 / 128 / 256: 768 x 3072, 16 slots, 400 tokens 36.6 / 36.7 / 37.5, 2048 55 / 41.6 / 44.1,
+// 4096 83 / 60 / 50; one CTA per tile, the kernel before, 40.1 / 41.4 / 69.4 there.
+__device__ __forceinline__ int pick_tile_height(const int (&count)[2], int cols, float inv_pairs) {
+  int best = 8;
+  float best_cost = 3.0e38f;
+#pragma unroll 1
+  for (int sh = 8; sh >= 6; --sh) {                          // (cold code on the way to GEMM-1: no divisions, not unrolled)
+    const int cap = 1 << sh;
+    const int n0 = (count[0] + cap - 1) >> sh, n1 = (count[1] + cap - 1) >> sh;
+    const int h0 = min(count[0], cap), h1 = min(count[1], cap);
+    const float n = (float)(__reduce_add_sync(0xffffffffu, n0 + n1) * cols) * inv_pairs;
+    const float sum = (float)__reduce_add_sync(0xffffffffu, n0 * (190 + h0) + n1 * (190 + h1)) * ((float)cols * inv_pairs);
+    const float longest = (float)(190 + __reduce_max_sync(0xffffffffu, max(h0, h1)));
+    const float cost = fminf(ceilf(n - 1e-3f) * longest, sum + longest);
+    if (cost < best_cost) { best_cost = cost; best = sh; }
+  }
+  return best;
+}
+
+// Tiles of one slot.
+__device__ __forceinline__ void write_slot_tiles(TileDesc* tiles, int count, int n_tiles, int rows, int phys, int row0, int slot) {
+  for (int i = 0; i < n_tiles; ++i) {
+    TileDesc td;
+    td.phys = phys;
+    td.row0 = row0 + i * rows;
+    td.rows = min(rows, count - i * rows);
+    td.slot = slot;
+    tiles[i] = td;
+  }
+}
+
 // Slot layout by one warp from the per-slot counts in shared memory: lane l owns slots l and l + 32
 // (K <= 64); offsets, padded offsets and first-tile indices are exclusive prefix sums over the slots,
 // taken with warp scans (tile heights are powers of two: shifts, no divisions - this code runs once,
@@ -55,19 +101,21 @@ __device__ __forceinline__ float reduce_column_serial(const float* src, int n_ro
 __device__ __forceinline__ void slot_layout_warp(const ScanArgs& a, const int32_t* s_count, int32_t* s_off,
                                                  int32_t* s_pad, bool write_global) {
   const int lane = threadIdx.x & 31;
-  const int sh_a = 31 - __clz(a.tile_rows);
   const bool two_lists = write_global && a.tiles_b != nullptr;
-  const int sh_b = two_lists ? 31 - __clz(a.tile_rows_b) : 0;
   int c[2], off[2], pad[2], ta[2], tb[2], ph[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) c[h] = lane + 32 * h < a.K ? s_count[lane + 32 * h] : 0;
+  int sh_a = 31 - __clz(a.tile_rows), sh_b = two_lists ? 31 - __clz(a.tile_rows_b) : 0;
+  if (write_global && a.pair_cols > 0) sh_a = pick_tile_height(c, a.pair_cols, a.inv_pairs);
+  if (two_lists && a.pair_cols_b > 0) sh_b = pick_tile_height(c, a.pair_cols_b, a.inv_pairs);
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const int s = lane + 32 * h;
-    c[h] = s < a.K ? s_count[s] : 0;
     ph[h] = (write_global && s < a.K) ? a.phys_slot[s] : 0;     // issued early: its latency hides behind the scans
     off[h] = c[h];
     pad[h] = (c[h] + kSegAlign - 1) & ~(kSegAlign - 1);
-    ta[h] = (c[h] + a.tile_rows - 1) >> sh_a;
-    tb[h] = two_lists ? (c[h] + a.tile_rows_b - 1) >> sh_b : 0;
+    ta[h] = (c[h] + (1 << sh_a) - 1) >> sh_a;
+    tb[h] = two_lists ? (c[h] + (1 << sh_b) - 1) >> sh_b : 0;
   }
   {
     // slots whose weights this forward reads: the algorithmic weight traffic of the layer
@@ -95,38 +143,25 @@ __device__ __forceinline__ void slot_layout_warp(const ScanArgs& a, const int32_
     if (s < a.K) {
       const int cnt = c[h];
       const int padded = (cnt + kSegAlign - 1) & ~(kSegAlign - 1);
-      const int nt = (cnt + a.tile_rows - 1) >> sh_a;
+      const int nt = (cnt + (1 << sh_a) - 1) >> sh_a;
       const int o_excl = off[h] - cnt, p_excl = pad[h] - padded, t_excl = ta[h] - nt;
       if (s_off != nullptr) { s_off[s] = o_excl; s_pad[s] = p_excl; }
       if (!write_global) continue;
       a.count[s] = cnt;
       a.offset[s] = o_excl;
       a.pad_offset[s] = p_excl;
-      for (int i = 0; i < nt; ++i) {
-        TileDesc td;
-        td.phys = ph[h];
-        td.row0 = p_excl + i * a.tile_rows;
-        td.rows = min(a.tile_rows, cnt - i * a.tile_rows);
-        td.slot = s;
-        a.tiles[t_excl + i] = td;
-      }
+      write_slot_tiles(a.tiles + t_excl, cnt, nt, a.pair_cols > 0 ? even_tile_rows(cnt, sh_a) : a.tile_rows, ph[h], p_excl, s);
       if (s == a.K - 1) {
         a.offset[a.K] = off[h];
         a.pad_offset[a.K] = pad[h];
-        *a.n_tiles = ta[h];
+        a.n_tiles[0] = ta[h];
+        a.n_tiles[1] = 1 << sh_a;
       }
       if (two_lists) {                         // same segments cut into tiles of another height
-        const int ntb = (cnt + a.tile_rows_b - 1) >> sh_b;
+        const int ntb = (cnt + (1 << sh_b) - 1) >> sh_b;
         const int tb_excl = tb[h] - ntb;
-        for (int i = 0; i < ntb; ++i) {
-          TileDesc td;
-          td.phys = ph[h];
-          td.row0 = p_excl + i * a.tile_rows_b;
-          td.rows = min(a.tile_rows_b, cnt - i * a.tile_rows_b);
-          td.slot = s;
-          a.tiles_b[tb_excl + i] = td;
-        }
-        if (s == a.K - 1) *a.n_tiles_b = tb[h];
+        write_slot_tiles(a.tiles_b + tb_excl, cnt, ntb, a.pair_cols_b > 0 ? even_tile_rows(cnt, sh_b) : a.tile_rows_b, ph[h], p_excl, s);
+        if (s == a.K - 1) { a.n_tiles_b[0] = tb[h]; a.n_tiles_b[1] = 1 << sh_b; }
       }
     }
   }

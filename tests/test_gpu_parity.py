@@ -980,3 +980,24 @@ def test_silu_over_its_range(monkeypatch, dtype, pairs):
         sel = (np.abs(z.numpy()) < 20.0) & (ref != 0.0)
         assert np.sqrt(np.mean(((h - ref)[sel] / ref[sel]) ** 2)) <= 4.65e-8
     assert layer.device_status() == (0, 0)
+
+
+@pytest.mark.parametrize("counts", [(1, 31, 32, 33, 0, 2), (63, 64, 65, 0, 127, 128), (129, 255, 256, 257, 0, 513),
+                                    (1025, 3, 0, 97, 64, 1)])
+@pytest.mark.parametrize("k,act,renorm", [(1, I.ACT_RELU, 0), (2, I.ACT_SWIGLU, 1)])
+def test_token_tiles_of_cta_pairs(counts, k, act, renorm):
+    """Slots whose row counts lie around the token tiles of the CTA-pair GEMMs (steps of 32, caps of 64, 128 and 256, equal
+    heights beyond) and empty ones, with a ragged last weight tile (d_ff 448: 256 + 192 rows, SwiGLU 3.5 tiles of 128): external
+    logits send token t to a prescribed slot.  Tolerance: the layer's (bf16 h and out)."""
+    from harness import Case, check_against_oracle
+    K, E, T = len(counts), 8, sum(counts)
+    cfg = _cfg(T=T, d=256, f=448, E=E, K=K, k=k, act=act, renorm=renorm)
+    case = Case(cfg, s2e=np.arange(K))
+    first = np.random.default_rng(7).permutation(np.repeat(np.arange(K), counts))
+    logits = np.random.default_rng(8).standard_normal((T, E)).astype(np.float32)
+    logits[np.arange(T), first] += 40.0
+    if k == 2:                                  # the second choice: the slot before, so every count is a sum of two
+        logits[np.arange(T), (first + K - 1) % K] += 30.0
+    res = check_against_oracle(case, case.run(ext_logits=logits), check_logits=False)
+    want = np.bincount(first, minlength=K) + (np.bincount((first + K - 1) % K, minlength=K) if k == 2 else 0)
+    assert np.array_equal(res["oracle"]["count"], want)
