@@ -47,7 +47,7 @@ struct swapmoe_layer {
   bool small_path;             // small-batch GEMM kernels for <= 64 pairs
   TcSmallCache small;
   TileDesc* tiles;
-  TileDesc* tiles_b;           // 128-row work list kept beside a 256-row one (see forward_impl)
+  TileDesc* tiles_b;           // second work list (see forward_impl)
   int32_t* n_tiles_b;
   void *xp, *h, *x_stage, *out_stage;
   // host state
@@ -234,8 +234,9 @@ int32_t forward_impl(swapmoe_layer* L, const void* x, const float* ext_logits, v
   const bool pair32 = use_tc32 && !swap32 && L->tc32.n_pairs > 0 &&
                       (L->pair32_min_rows > 0 ? (long long)n_pairs >= (long long)L->pair32_min_rows * c.K
                                               : tc_f32_use_pairs(c, L->tc32.n_pairs, L->sm_count, n_pairs, L->y_copies));
-  const int tile_rows = pc2 > 0 ? kPairMinTokens : use_tc ? kTcBM : (use_tc32 ? (swap32 ? kF32SwapTok : pair32 ? 2 * kTcBM : kTcBM) : kMmaBM);
-  const int max_tiles = (n_pairs + tile_rows - 1) / tile_rows + c.K;
+  const int tile_rows = pc1 > 0 && pc2 > 0 ? 0 : use_tc ? kTcBM : (use_tc32 ? (swap32 ? kF32SwapTok : pair32 ? 2 * kTcBM : kTcBM) : kMmaBM);
+  const int max_tiles = tile_rows > 0 ? (n_pairs + tile_rows - 1) / tile_rows + c.K : 0;
+  const int max_pair_tiles = (n_pairs + kPairMinTokens - 1) / kPairMinTokens + c.K;
 
   RouterArgs ra;
   ra.x = x; ra.Wr = L->Wr; ra.ext_logits = ext_logits; ra.e2s = L->e2s; ra.enorm = L->enorm;
@@ -257,13 +258,12 @@ int32_t forward_impl(swapmoe_layer* L, const void* x, const float* ext_logits, v
   sa.ticket = own_scan ? nullptr : L->ticket;
   sa.touched = L->touched;
   sa.n_cta = n_cta; sa.K = c.K; sa.E = c.E; sa.tile_rows = tile_rows;
-  sa.pair_cols = pc2; sa.inv_pairs = 1.f / (float)std::max(L->gemm_pairs, 1);
-  // GEMM-1 gets a list of its own where its tiles may be others
-  const int tile_rows1 = pc1 > 0 ? kPairMinTokens : use_tc ? kTcBM : tile_rows;
-  const bool two_lists = pc1 != pc2;
-  const int max_tiles1 = (n_pairs + tile_rows1 - 1) / tile_rows1 + c.K;
-  sa.tiles_b = two_lists ? L->tiles_b : nullptr; sa.n_tiles_b = L->n_tiles_b; sa.tile_rows_b = tile_rows1;
-  sa.pair_cols_b = pc1;
+  // token tiles for CTA pairs: one list where the two GEMMs have the same number of weight tiles, else one each
+  PairList list1 = {}, list2 = {};
+  if (pc1 > 0) list1 = {L->tiles_b, L->n_tiles_b, pc1};
+  if (pc2 > 0) list2 = pc1 == 0 ? PairList{L->tiles_b, L->n_tiles_b, pc2} : pc1 == pc2 ? list1 : PairList{L->tiles, L->n_tiles, pc2};
+  sa.pair[0] = list1; sa.pair[1] = pc1 == pc2 ? PairList{} : list2;
+  sa.inv_pairs = 1.f / (float)std::max(L->gemm_pairs, 1);
   ra.pf_base[0] = ra.pf_base[1] = nullptr;
   ra.pf_slot_bytes[0] = ra.pf_slot_bytes[1] = 16384;
   ra.pf_total_bytes[0] = ra.pf_total_bytes[1] = 0;
@@ -371,20 +371,18 @@ int32_t forward_impl(swapmoe_layer* L, const void* x, const float* ext_logits, v
                         L->tiles, L->n_tiles, L->row_pair, L->mgate, max_tiles, T, L->status, st, pdl,
                         &L->launches, &combined, mid);
     } else {
-      const TileDesc* tiles1 = two_lists ? L->tiles_b : L->tiles;
-      const int32_t* n_tiles1 = two_lists ? L->n_tiles_b : L->n_tiles;
       const bool scatter = c.top_k == 1;
       rc = SWAPMOE_OK;
       if (rerun != 2) {
-        rc = pc1 > 0 ? tc_gemm_pair(L->tc, L->gemm_pairs, c, 1, L->h, tiles1, n_tiles1, max_tiles1, nullptr, nullptr, T,
+        rc = pc1 > 0 ? tc_gemm_pair(L->tc, L->gemm_pairs, c, 1, L->h, list1.tiles, list1.n_tiles, max_pair_tiles, nullptr, nullptr, T,
                                     L->status, st, pdl, L->row_group)
-                     : tc_gemm1(L->tc, c, L->h, tiles1, n_tiles1, max_tiles1, T, L->status, st, pdl, L->row_group);
+                     : tc_gemm1(L->tc, c, L->h, L->tiles, L->n_tiles, max_tiles, T, L->status, st, pdl, L->row_group);
         L->launches++;
       }
       if (mid) cudaEventRecord(mid, st);
       if (rc == SWAPMOE_OK && rerun != 1) {
         void* dst = scatter ? out : static_cast<void*>(L->y);
-        rc = pc2 > 0 ? tc_gemm_pair(L->tc, L->gemm_pairs, c, 2, dst, L->tiles, L->n_tiles, max_tiles, L->row_pair,
+        rc = pc2 > 0 ? tc_gemm_pair(L->tc, L->gemm_pairs, c, 2, dst, list2.tiles, list2.n_tiles, max_pair_tiles, L->row_pair,
                                     L->mgate, T, L->status, st, pdl, L->row_group)
                      : tc_gemm2(L->tc, c, dst, L->tiles, L->n_tiles, max_tiles, L->row_pair, L->mgate, T, L->status, st,
                                 pdl, L->row_group);

@@ -187,7 +187,7 @@ tc_gemm_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
         gate = a.gate[p];
         crow = (size_t)(p / a.top_k) * a.ldc + (size_t)ct * BN;
       }
-      ok = bounded_wait(&acc_full[acc], acc_phase, abort_flag, a.status, 34);
+      ok = warp_wait(&acc_full[acc], acc_phase, abort_flag, a.status, 34);
       if (!ok) break;
       ptx::tc_fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN);

@@ -5,6 +5,12 @@
 
 namespace swapmoe {
 
+struct PairList {
+  TileDesc* tiles;           // or nullptr
+  int32_t* n_tiles;          // [2] their number, the most rows one may hold
+  int32_t cols;              // weight tiles per token tile
+};
+
 struct ScanArgs {
   const int32_t* cta_hist;   // [n_cta, K]
   const float* cta_imp;      // [n_cta, E]
@@ -19,17 +25,14 @@ struct ScanArgs {
   int32_t* offset;           // [K+1]  exclusive scan of count
   int32_t* pad_offset;       // [K+1]  same with every segment rounded up to kSegAlign rows
   TileDesc* tiles;           // GEMM work list
-  int32_t* n_tiles;          // [2] their number, the most rows one may hold
+  int32_t* n_tiles;          // [1]
   float* imp;                // [E] accumulator of Eq. (1)
   unsigned* ticket;          // [1] router CTAs finished so far (returns to 0); nullptr: the router CTAs do not
                              // scan at all - the permute kernel sums the histograms itself (see below)
-  TileDesc* tiles_b;         // optional second work list with tile_rows_b rows per tile (or nullptr)
-  int32_t* n_tiles_b;
   unsigned long long* touched;   // [1] running total of slots that received at least one pair, or nullptr
-  int32_t n_cta, K, E, tile_rows, tile_rows_b;
-  // > 0: a list of token tiles for CTA pairs, which take this many weight tiles per token tile (see pick_tile_height); 0: tiles
-  // of tile_rows rows
-  int32_t pair_cols, pair_cols_b;
+  int32_t n_cta, K, E;
+  int32_t tile_rows;         // rows per tile of `tiles` (a power of two), 0: no such list
+  PairList pair[2];          // lists of token tiles for CTA pairs
   float inv_pairs;           // 1 / CTA pairs that share the work
 };
 
@@ -81,61 +84,78 @@ __device__ __forceinline__ int pick_tile_height(const int (&count)[2], int cols,
   return best;
 }
 
-// Tiles of one slot.
-__device__ __forceinline__ void write_slot_tiles(TileDesc* tiles, int count, int n_tiles, int rows, int phys, int row0, int slot) {
-  for (int i = 0; i < n_tiles; ++i) {
-    TileDesc td;
-    td.phys = phys;
-    td.row0 = row0 + i * rows;
-    td.rows = min(rows, count - i * rows);
-    td.slot = slot;
-    tiles[i] = td;
+// The list of token tiles for CTA pairs, by one warp whose lanes own slots l and l + 32: `row0` = first row of a slot's segment.
+// Out of line: small batches run slot_layout_warp once per forward, through cold code, and have no such list (twelve layers of
+// 1024 x 4096 at 29 tokens: 1.5 us per layer when this was part of it).
+static __device__ __noinline__ void write_pair_tiles(const PairList l, float inv_pairs, int count0, int count1, int phys0,
+                                              int phys1, int row0, int row1) {
+  const int lane = threadIdx.x & 31;
+  const int count[2] = {count0, count1};
+  const int sh = pick_tile_height(count, l.cols, inv_pairs);
+  int base = 0;
+#pragma unroll 1
+  for (int h = 0; h < 2; ++h) {
+    const int cnt = h == 0 ? count0 : count1, phys = h == 0 ? phys0 : phys1, first = h == 0 ? row0 : row1;
+    const int nt = (cnt + (1 << sh) - 1) >> sh, rows = even_tile_rows(cnt, sh);
+    int incl = nt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += u;
+    }
+    TileDesc* dst = l.tiles + base + incl - nt;
+    for (int i = 0; i < nt; ++i) {
+      TileDesc td;
+      td.phys = phys;
+      td.row0 = first + i * rows;
+      td.rows = min(rows, cnt - i * rows);
+      td.slot = lane + 32 * h;
+      dst[i] = td;
+    }
+    base += __shfl_sync(0xffffffffu, incl, 31);
   }
+  if (lane == 0) { l.n_tiles[0] = base; l.n_tiles[1] = 1 << sh; }
 }
 
 // Slot layout by one warp from the per-slot counts in shared memory: lane l owns slots l and l + 32
 // (K <= 64); offsets, padded offsets and first-tile indices are exclusive prefix sums over the slots,
-// taken with warp scans (tile heights are powers of two: shifts, no divisions - this code runs once,
+// taken with warp scans (the heights of `tiles` are powers of two: shifts, no divisions - this code runs once,
 // every dependent instruction counts).  s_off / s_pad (shared, may be nullptr) receive the exclusive
 // offsets; with `write_global` the warp also writes count / offset / pad_offset and the tile lists.
 __device__ __forceinline__ void slot_layout_warp(const ScanArgs& a, const int32_t* s_count, int32_t* s_off,
                                                  int32_t* s_pad, bool write_global) {
   const int lane = threadIdx.x & 31;
-  const bool two_lists = write_global && a.tiles_b != nullptr;
-  int c[2], off[2], pad[2], ta[2], tb[2], ph[2];
-#pragma unroll
-  for (int h = 0; h < 2; ++h) c[h] = lane + 32 * h < a.K ? s_count[lane + 32 * h] : 0;
-  int sh_a = 31 - __clz(a.tile_rows), sh_b = two_lists ? 31 - __clz(a.tile_rows_b) : 0;
-  if (write_global && a.pair_cols > 0) sh_a = pick_tile_height(c, a.pair_cols, a.inv_pairs);
-  if (two_lists && a.pair_cols_b > 0) sh_b = pick_tile_height(c, a.pair_cols_b, a.inv_pairs);
+  const int sh = a.tile_rows > 0 ? 31 - __clz(a.tile_rows) : 31;      // 31: no tiles
+  const int round = a.tile_rows > 0 ? a.tile_rows - 1 : 0;
+  int c[2], off[2], pad[2], ta[2], ph[2];
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const int s = lane + 32 * h;
+    c[h] = s < a.K ? s_count[s] : 0;
     ph[h] = (write_global && s < a.K) ? a.phys_slot[s] : 0;     // issued early: its latency hides behind the scans
     off[h] = c[h];
     pad[h] = (c[h] + kSegAlign - 1) & ~(kSegAlign - 1);
-    ta[h] = (c[h] + (1 << sh_a) - 1) >> sh_a;
-    tb[h] = two_lists ? (c[h] + (1 << sh_b) - 1) >> sh_b : 0;
+    ta[h] = (c[h] + round) >> sh;
   }
   {
     // slots whose weights this forward reads: the algorithmic weight traffic of the layer
     const int nz = __popc(__ballot_sync(0xffffffffu, c[0] > 0)) + __popc(__ballot_sync(0xffffffffu, c[1] > 0));
     if (write_global && lane == 0 && a.touched != nullptr) atomicAdd(a.touched, (unsigned long long)nz);
   }
-  // inclusive scans of the four quantities over 64 slots
+  // inclusive scans of the three quantities over 64 slots
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int u0 = __shfl_up_sync(0xffffffffu, off[h], o), u1 = __shfl_up_sync(0xffffffffu, pad[h], o);
-      const int u2 = __shfl_up_sync(0xffffffffu, ta[h], o), u3 = __shfl_up_sync(0xffffffffu, tb[h], o);
-      if (lane >= o) { off[h] += u0; pad[h] += u1; ta[h] += u2; tb[h] += u3; }
+      const int u2 = __shfl_up_sync(0xffffffffu, ta[h], o);
+      if (lane >= o) { off[h] += u0; pad[h] += u1; ta[h] += u2; }
     }
   }
   {
     const int t0 = __shfl_sync(0xffffffffu, off[0], 31), t1 = __shfl_sync(0xffffffffu, pad[0], 31);
-    const int t2 = __shfl_sync(0xffffffffu, ta[0], 31), t3 = __shfl_sync(0xffffffffu, tb[0], 31);
-    off[1] += t0; pad[1] += t1; ta[1] += t2; tb[1] += t3;
+    const int t2 = __shfl_sync(0xffffffffu, ta[0], 31);
+    off[1] += t0; pad[1] += t1; ta[1] += t2;
   }
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
@@ -143,27 +163,33 @@ __device__ __forceinline__ void slot_layout_warp(const ScanArgs& a, const int32_
     if (s < a.K) {
       const int cnt = c[h];
       const int padded = (cnt + kSegAlign - 1) & ~(kSegAlign - 1);
-      const int nt = (cnt + (1 << sh_a) - 1) >> sh_a;
+      const int nt = (cnt + round) >> sh;
       const int o_excl = off[h] - cnt, p_excl = pad[h] - padded, t_excl = ta[h] - nt;
       if (s_off != nullptr) { s_off[s] = o_excl; s_pad[s] = p_excl; }
       if (!write_global) continue;
       a.count[s] = cnt;
       a.offset[s] = o_excl;
       a.pad_offset[s] = p_excl;
-      write_slot_tiles(a.tiles + t_excl, cnt, nt, a.pair_cols > 0 ? even_tile_rows(cnt, sh_a) : a.tile_rows, ph[h], p_excl, s);
+      for (int i = 0; i < nt; ++i) {
+        TileDesc td;
+        td.phys = ph[h];
+        td.row0 = p_excl + i * a.tile_rows;
+        td.rows = min(a.tile_rows, cnt - i * a.tile_rows);
+        td.slot = s;
+        a.tiles[t_excl + i] = td;
+      }
       if (s == a.K - 1) {
         a.offset[a.K] = off[h];
         a.pad_offset[a.K] = pad[h];
-        a.n_tiles[0] = ta[h];
-        a.n_tiles[1] = 1 << sh_a;
-      }
-      if (two_lists) {                         // same segments cut into tiles of another height
-        const int ntb = (cnt + (1 << sh_b) - 1) >> sh_b;
-        const int tb_excl = tb[h] - ntb;
-        write_slot_tiles(a.tiles_b + tb_excl, cnt, ntb, a.pair_cols_b > 0 ? even_tile_rows(cnt, sh_b) : a.tile_rows_b, ph[h], p_excl, s);
-        if (s == a.K - 1) { a.n_tiles_b[0] = tb[h]; a.n_tiles_b[1] = 1 << sh_b; }
+        if (a.tile_rows > 0) *a.n_tiles = ta[h];
       }
     }
+  }
+  if (write_global) {
+    const int first0 = pad[0] - ((c[0] + kSegAlign - 1) & ~(kSegAlign - 1));
+    const int first1 = pad[1] - ((c[1] + kSegAlign - 1) & ~(kSegAlign - 1));
+    if (a.pair[0].tiles != nullptr) write_pair_tiles(a.pair[0], a.inv_pairs, c[0], c[1], ph[0], ph[1], first0, first1);
+    if (a.pair[1].tiles != nullptr) write_pair_tiles(a.pair[1], a.inv_pairs, c[0], c[1], ph[0], ph[1], first0, first1);
   }
 }
 
@@ -331,7 +357,7 @@ __device__ __forceinline__ float reduce_columns_parallel(const float* src, int n
 // kTop1: one pair per token, in code of its own: the kernel runs once through cold code, and the loops of the general form
 // cost a twelve-layer step of 29 tokens 2 %.
 template <typename T, bool kTop1>
-__global__ void __launch_bounds__(kPermThreads) permute_gather_kernel(const PermuteArgs a) {
+__global__ void __launch_bounds__(kPermThreads, 2) permute_gather_kernel(const PermuteArgs a) {
   // 11 KB of shared memory, so that these CTAs fit beside a router CTA (over 210 KB) and are already
   // waiting when the router finishes.  The reducing CTAs use the same bytes for their shares.
   constexpr int kRawBytes = (kPermThreads / 32) * kMaxSlots * 4 + kPermThreads * 4 + 4 * kMaxSlots * 4 + 2 * kPermThreads * 4;

@@ -104,10 +104,10 @@ extern "C" int32_t swapmoe_route_static(const void* x_dev, const void* Wr_dev, c
   sa.n_tiles = reinterpret_cast<int32_t*>(s + kOffNTiles);
   sa.imp = imp_dev;
   sa.ticket = reinterpret_cast<unsigned*>(s + kOffTicket);
-  sa.tiles_b = nullptr; sa.n_tiles_b = nullptr; sa.tile_rows_b = 0; sa.touched = nullptr;
+  sa.touched = nullptr;
   sa.cta_cnt = nullptr; sa.cta_mimp = nullptr; sa.s2e = nullptr; sa.cnt = nullptr; sa.mimp = nullptr;
   sa.n_cta = n_cta; sa.K = K; sa.E = E; sa.tile_rows = kStaticTileRows;
-  sa.pair_cols = sa.pair_cols_b = 0; sa.inv_pairs = 1.f;
+  sa.pair[0].tiles = sa.pair[1].tiles = nullptr; sa.inv_pairs = 1.f;
   if (dtype == SWAPMOE_BF16)
     router_gate_fn<bf16>(E)<<<n_cta, 256, router_smem_bytes(E), st>>>(ra);
   else
