@@ -365,11 +365,11 @@ int32_t forward_impl(swapmoe_layer* L, const void* x, const float* ext_logits, v
   if (use_tc) {
     cudaEvent_t mid = L->stage_events ? static_cast<cudaEvent_t>(L->stage_events[4]) : nullptr;
     int32_t rc;
-    if (L->small_path && n_pairs <= 64 && c.act == SWAPMOE_ACT_RELU) {
-      if (rerun) return SWAPMOE_ERR_UNSUPPORTED;
+    if (L->small_path && n_pairs <= 64) {
+      if (rerun && c.act == SWAPMOE_ACT_RELU) return SWAPMOE_ERR_UNSUPPORTED;
       rc = tc_ffn_small(L->tc, L->small, c, L->xp, L->h, L->y, out, L->rows_pad_max, L->arena_in, L->arena_out,
                         L->tiles, L->n_tiles, L->row_pair, L->mgate, max_tiles, T, L->status, st, pdl,
-                        &L->launches, &combined, mid);
+                        &L->launches, &combined, rerun, mid);
     } else {
       const bool scatter = c.top_k == 1;
       rc = SWAPMOE_OK;

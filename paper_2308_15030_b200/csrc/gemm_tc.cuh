@@ -594,7 +594,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         epi_row_pointers(dst, drow, lane, a.C, (size_t)a.ldc, (size_t)ct * kOutCols, kElem);
         epi_store_tile<EPI, kOutCols>(taddr, epi_stage + q * kTcEpiWarpStage, lane, gate, dst, a.ldc - ct * kOutCols);
       } else {
-        // tiles whose rows are no whole 128-byte chunks (the narrowest, and 80 columns): every thread stores its own
+        // tiles whose rows are no whole 128-byte chunks (the narrowest): every thread stores its own
         // row, sixteen columns at a time
         bf16* dst = drow < 0 ? nullptr : static_cast<bf16*>(a.C) + (size_t)drow * a.ldc + (size_t)ct * kOutCols;
 #pragma unroll 1
@@ -630,8 +630,7 @@ typedef CUresult (*PFN_encodeTiled)(CUtensorMap*, CUtensorMapDataType, cuuint32_
 
 // Column-tile widths the kernels are built for.  Narrow tiles exist for small batches
 // (decode): with few row tiles, wide column tiles would leave most SMs without work.
-// (the last of GEMM-1's: SwiGLU layers at up to 64 pairs, see tc_plan_gemm1)
-constexpr int kBn1Options[4] = {256, 128, 64, 160};
+constexpr int kBn1Options[3] = {256, 128, 64};
 constexpr int kBn2Options[4] = {256, 128, 64, 32};
 
 struct TcState {
@@ -639,7 +638,7 @@ struct TcState {
   int sm_count;
   PFN_encodeTiled encode;
   CUtensorMap map_xp[4], map_h[4];    // activations [rows_pad, d] / [rows_pad, f]; box rows 128, 64, 32, 16
-  CUtensorMap map_win[4];             // W_in flattened to 2D, one map per entry of kBn1Options
+  CUtensorMap map_win[3];             // W_in flattened to 2D, one map per entry of kBn1Options
   CUtensorMap map_wout[4];            // W_out flattened to 2D, one map per entry of kBn2Options
   CUtensorMap map_h_out, map_y_out;   // stores of h [rows_pad, f] (box 32 x 32; SwiGLU 16 x 32) and y [rows_pad, d] fp32 (32 x 32)
   CUtensorMap map_win_gated;          // SwiGLU: W_in as sixteen rows of W1, the same sixteen of W3, ... (gemm_tc_pair.cuh)
@@ -728,7 +727,7 @@ inline int32_t tc_init(TcState& s, const swapmoe_config_t& c, void* xp, void* h,
   }
   bool ok = tc_set_smem_attr<256, kTcEpiReluBf16>() && tc_set_smem_attr<128, kTcEpiReluBf16>() &&
             tc_set_smem_attr<64, kTcEpiReluBf16>() && tc_set_smem_attr<256, kTcEpiSwigluBf16>() &&
-            tc_set_smem_attr<128, kTcEpiSwigluBf16>() && tc_set_smem_attr<64, kTcEpiSwigluBf16>() && tc_set_smem_attr<160, kTcEpiSwigluBf16>() &&
+            tc_set_smem_attr<128, kTcEpiSwigluBf16>() && tc_set_smem_attr<64, kTcEpiSwigluBf16>() &&
             tc_set_smem_attr<256, kTcEpiF32>() && tc_set_smem_attr<128, kTcEpiF32>() &&
             tc_set_smem_attr<64, kTcEpiF32>() && tc_set_smem_attr<32, kTcEpiF32>() &&
             tc_set_smem_attr<256, kTcEpiScatterBf16>() && tc_set_smem_attr<128, kTcEpiScatterBf16>() &&
@@ -742,7 +741,7 @@ inline int32_t tc_bind_arena(TcState& s, const swapmoe_config_t& c, const void* 
   if (!s.enabled) return SWAPMOE_OK;
   const int P = c.K + c.spare_slots;
   const int nin = c.act == SWAPMOE_ACT_SWIGLU ? 2 : 1;
-  for (int i = 0; i < 4; ++i)     // SwiGLU loads W1 and W3 as two boxes of half the tile width
+  for (int i = 0; i < 3; ++i)     // SwiGLU loads W1 and W3 as two boxes of half the tile width
     if (!tc_encode_2d(s.encode, &s.map_win[i], arena_in, (uint64_t)P * nin * c.d_ff, (uint64_t)c.d_model,
                       (uint32_t)(kBn1Options[i] / nin)))
       return SWAPMOE_ERR_CUDA;

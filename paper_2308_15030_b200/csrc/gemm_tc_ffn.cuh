@@ -7,8 +7,8 @@
 namespace swapmoe {
 
 // Weight tiles per token tile where a grouped GEMM (which = 1 or 2) runs on CTA pairs, 0: one CTA per tile.  Pairs take
-// every forward of more than 64 (token, expert) pairs (up to there the small-batch kernel, and for SwiGLU the tiles between
-// the powers of two, fill the SMs better: 960 x 2624, four slots, 13 tokens 35.5 us per forward against 39.6) whose matrices
+// every forward of more than 64 (token, expert) pairs (up to there the small-batch kernel fills the SMs better: SwiGLU 960 x
+// 2624, four slots, 13 tokens 31.0 us per forward against 39.6) whose matrices
 // leave at most a fifth of the last weight tile empty.  us per forward, one CTA per tile / pairs: 768 x 3072, 16 slots, 70
 // tokens 48.4 / 45.5, 800 53.1 / 48.7, 2048 52.4 / 52.2, 4096 81.4 / 64.8; 1024 x 512 top-4 of 256, 64 slots, 2500 95.6 / 85.7;
 // SwiGLU top-2, four slots, 1024 x 3584, 700 76.5 / 62.0, 4096 x 14336, 200 318.9 / 296.0.
@@ -48,15 +48,11 @@ struct TcGemm1Plan : TcRowPlan {
 inline bool tc_plan_gemm1(const TcState& s, const swapmoe_config_t& c, int n_tokens, int max_tiles, int row_group_forced,
                           TcGemm1Plan* p) {
   const bool swiglu = c.act == SWAPMOE_ACT_SWIGLU;
-  const long long pairs = (long long)n_tokens * c.top_k;
   tc_plan_rows(c, n_tokens, row_group_forced, p);
   // (SwiGLU counts the rows of both matrices; with one matrix's the model saw half the tiles: 13 tokens, d_model 4096,
   // d_ff 14336, four slots, GEMM-1 alone 187 us at 448 tiles on 148 SMs, 174 at 896 narrower ones)
-  // With few rows the weights are all there is to pull, and what counts is how evenly the column tiles fill the last round:
-  // SwiGLU at up to 64 pairs may also take 160 weight rows (80 outputs), whose epilogue is only good for few rows.
-  // us per forward without / with, four slots: 4096 x 14336 at 13 tokens 258 / 245, 2048 x 5632 at 6 85 / 72, 960 x 2624 at
-  // 20 41 / 36; 1024 x 3584, where 256 rows are one round, keeps them.
-  p->i1 = tc_pick_bn(kBn1Options, swiglu && pairs <= 64 ? 4 : 3, swiglu ? 2 * c.d_ff : c.d_ff, p->row_tiles_est, s.sm_count, p->a_box_bytes, swiglu ? 64 : 32);
+  p->i1 = tc_pick_bn(kBn1Options, 3, swiglu ? 2 * c.d_ff : c.d_ff, p->row_tiles_est, s.sm_count, p->a_box_bytes,
+                     swiglu ? 64 : 32);
   if (p->i1 < 0) return false;
   p->bn1 = kBn1Options[p->i1];
   const int out1 = swiglu ? p->bn1 / 2 : p->bn1;
@@ -84,11 +80,11 @@ inline int32_t tc_gemm1(TcState& s, const swapmoe_config_t& c, void* h, const Ti
   g.row_group = plan.row_group;
   g.a_box_bytes = plan.a_box_bytes;
   g.early_b = 0;
-  static const TcGemmKernel kernels[2][4] = {
-      {tc_gemm_kernel<256, kTcEpiReluBf16>, tc_gemm_kernel<128, kTcEpiReluBf16>, tc_gemm_kernel<64, kTcEpiReluBf16>, nullptr},
+  static const TcGemmKernel kernels[2][3] = {
+      {tc_gemm_kernel<256, kTcEpiReluBf16>, tc_gemm_kernel<128, kTcEpiReluBf16>, tc_gemm_kernel<64, kTcEpiReluBf16>},
       {tc_gemm_kernel<256, kTcEpiSwigluBf16>, tc_gemm_kernel<128, kTcEpiSwigluBf16>,
-       tc_gemm_kernel<64, kTcEpiSwigluBf16>, tc_gemm_kernel<160, kTcEpiSwigluBf16>}};
-  static const int smem[4] = {TcSmem<256>::kBytes, TcSmem<128>::kBytes, TcSmem<64>::kBytes, TcSmem<160>::kBytes};
+       tc_gemm_kernel<64, kTcEpiSwigluBf16>}};
+  static const int smem[3] = {TcSmem<256>::kBytes, TcSmem<128>::kBytes, TcSmem<64>::kBytes};
   return launch_kernel(kernels[swiglu ? 1 : 0][plan.i1], dim3(plan.grid), dim3(kTcThreads), smem[plan.i1], st, pdl,
                        s.map_xp[plan.ia], s.map_win[plan.i1], g) == cudaSuccess ? SWAPMOE_OK : SWAPMOE_ERR_CUDA;
 }

@@ -13,8 +13,8 @@
 //     128 rows, the rest is whatever lies behind in shared memory and only feeds accumulator
 //     lanes whose rows are never stored;
 //   - takes the stage count at run time (up to 16).
-// Every mbarrier wait is bounded as in tc_gemm_kernel.  ReLU / fp32 / scatter epilogues only
-// (a SwiGLU layer uses the general kernel for its first GEMM).
+// Every mbarrier wait is bounded as in tc_gemm_kernel.  SwiGLU: a 4-D map brings the same BN / 2 rows of W1 and W3 side by
+// side, so a stage of several k-blocks is one box there too.
 #pragma once
 #include "gemm_tc.cuh"
 
@@ -37,11 +37,20 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, u
       : "memory");
 }
 
+__device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, uint64_t* bar, int c0, int c1, int c2, int c3) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
+      ::"r"(ptx::smem_u32(dst)), "l"(map), "r"(ptx::smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+      : "memory");
+}
+
 template <int BN, int EPI>
 __global__ void __launch_bounds__(kTcThreads, 1)
 tc_gemm_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                      const TcSmallArgs sa) {
   const TcGemmArgs& a = sa.g;
+  constexpr bool kSwiglu = EPI == kTcEpiSwigluBf16;
+  constexpr int kOutCols = kSwiglu ? BN / 2 : BN;
   constexpr int kBTile = BN * kTcBK * 2;                    // one k-block of the weight box
   constexpr uint32_t kTmemCols = 2 * BN <= 64 ? 64 : 2 * BN <= 128 ? 128 : 2 * BN <= 256 ? 256 : 512;   // a power of two
   constexpr uint32_t kIdesc = make_idesc_bf16(kTcBM, BN);
@@ -81,6 +90,10 @@ tc_gemm_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
   const uint32_t tmem_base = *tmem_slot;
 
   const int n_chunks = (a.k_blocks + kps - 1) / kps;
+  auto load_w = [&](void* dst, uint64_t* bar, int brow, int k0) {
+    if constexpr (kSwiglu) tma_load_4d(dst, &tmB, bar, 0, brow, 0, k0);
+    else tma_load_3d(dst, &tmB, bar, 0, brow, k0);
+  };
   // As in tc_gemm_kernel: with `early_b` the producer requests the weight boxes of its first stages before the
   // dependent-launch wait.
   int pre = 0;
@@ -90,12 +103,12 @@ tc_gemm_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
       const int ct = (int)blockIdx.x / n_rt, rt = (int)blockIdx.x - ct * n_rt;
       const int4 rawd = __ldcg(reinterpret_cast<const int4*>(a.tiles + rt));
       const TileDesc td = *reinterpret_cast<const TileDesc*>(&rawd);
-      const int brow = td.phys * a.b_rows_per_phys + ct * BN;
+      const int brow = td.phys * a.b_rows_per_phys + ct * kOutCols;
       pre = n_chunks < n_stages ? n_chunks : n_stages;
       for (int c = 0; c < pre; ++c) {
         if (ptx::elect_one()) {
           ptx::mbar_expect_tx(&full[c], (uint32_t)(stage_a + stage_b));
-          tma_load_3d(sB + c * stage_b, &tmB, &full[c], 0, brow, c * kps);
+          load_w(sB + c * stage_b, &full[c], brow, c * kps);
         }
         __syncwarp();
       }
@@ -114,7 +127,7 @@ tc_gemm_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     for (int t = blockIdx.x; t < total && ok; t += gridDim.x) {
       const int ct = t / n_row_tiles, rt = t - ct * n_row_tiles;
       const TileDesc td = a.tiles[rt];
-      const int brow = td.phys * a.b_rows_per_phys + ct * BN;
+      const int brow = td.phys * a.b_rows_per_phys + ct * kOutCols;
       for (int c = 0; c < n_chunks; ++c) {
         const bool early = t == (int)blockIdx.x && c < pre;    // armed and weights requested above
         if (!early) {
@@ -124,7 +137,7 @@ tc_gemm_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
         if (ptx::elect_one()) {
           if (!early) ptx::mbar_expect_tx(&full[stage], (uint32_t)(stage_a + stage_b));
           tma_load_3d(sA + stage * stage_a, &tmA, &full[stage], 0, td.row0, c * kps);
-          if (!early) tma_load_3d(sB + stage * stage_b, &tmB, &full[stage], 0, brow, c * kps);
+          if (!early) load_w(sB + stage * stage_b, &full[stage], brow, c * kps);
         }
         __syncwarp();
         if (++stage == n_stages) { stage = 0; phase ^= 1u; }
@@ -180,7 +193,7 @@ tc_gemm_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
       // the row's destination and gate value (two dependent global loads) are fetched while the
       // tile's MMAs are still running
       const bool row_ok = r < td.rows;
-      size_t crow = (size_t)(td.row0 + r) * a.ldc + (size_t)ct * BN;
+      size_t crow = (size_t)(td.row0 + r) * a.ldc + (size_t)ct * kOutCols;
       float gate = 1.f;
       if (EPI == kTcEpiScatterBf16 && row_ok) {
         const int p = a.row_pair[td.row0 + r];
@@ -191,6 +204,20 @@ tc_gemm_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
       if (!ok) break;
       ptx::tc_fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN);
+      if constexpr (kSwiglu) {
+        if (q * 32 < td.rows) {
+#pragma unroll 1
+          for (int c0 = 0; c0 < min(kOutCols, a.ldc - ct * kOutCols); c0 += 16) {
+            uint4 pc[2];
+            __syncwarp();
+            epi_load_pieces16<EPI>(taddr, c0, kOutCols, 1.f, pc);
+            if (row_ok) {
+              uint4* dst = reinterpret_cast<uint4*>(static_cast<bf16*>(a.C) + crow + c0);
+              dst[0] = pc[0]; dst[1] = pc[1];
+            }
+          }
+        }
+      } else {
 #pragma unroll 1
       for (int c0 = 0; c0 < min(BN, a.ldc - ct * BN); c0 += 32) {
         uint32_t v[32];
@@ -219,6 +246,7 @@ tc_gemm_small_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
             }
           }
         }
+      }
       }
       ptx::tc_fence_before();
       ptx::mbar_arrive(&acc_empty[acc]);
@@ -249,6 +277,8 @@ inline bool tc_encode_3d(PFN_encodeTiled enc, CUtensorMap* m, const void* base, 
 // powers of two let the column tiles fill the last round.  us, powers of two
 // only / all: 768 x 3072, 16 slots, 12 tokens 29.3 / 27.8, 40 tokens 36.4 / 34.2; 704 x 2240 at 40 31.5 / 30.5; twelve layers
 // of 1024 x 4096 at 29 726 / 715; 1536 x 1088, 48 slots, 60 tokens 80.6 / 81.1.
+// SwiGLU layers (half a tile of either matrix), which ran on the general kernel before, us per forward there / here, four slots, 13
+// tokens: 4096 x 14336 254 / 243, 1024 x 3584 50.3 / 36.4, 2048 x 5632 70.6 / 63.5, 960 x 2624 34.8 / 31.0.
 constexpr int kSmallBn[8] = {256, 224, 192, 160, 128, 96, 64, 32};
 
 // As tc_pick_bn (bytes the busiest SM pulls over all k-blocks), plus the epilogue of its last tile, which nothing overlaps:
@@ -319,6 +349,8 @@ inline bool tc_small_set_attrs() {
   for (int i = 0; i < 8; ++i) {
     ok = ok && cudaFuncSetAttribute(tc_small_kernel_for<kTcEpiReluBf16>(i), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     kSmSmemBudget) == cudaSuccess;
+    ok = ok && cudaFuncSetAttribute(tc_small_kernel_for<kTcEpiSwigluBf16>(i),
+                                    cudaFuncAttributeMaxDynamicSharedMemorySize, kSmSmemBudget) == cudaSuccess;
     ok = ok && cudaFuncSetAttribute(tc_small_kernel_for<kTcEpiF32>(i), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     kSmSmemBudget) == cudaSuccess;
     ok = ok && cudaFuncSetAttribute(tc_small_kernel_for<kTcEpiScatterBf16>(i),
@@ -327,26 +359,46 @@ inline bool tc_small_set_attrs() {
   return ok;
 }
 
-// Both grouped GEMMs of a ReLU layer for a small batch (pairs <= 64).  Same contract as tc_ffn.
+// The same rows of W1 and W3 as a box of two: the third dimension is the step from one matrix to the other (rows from the last
+// W3 on are outside the map and read as zeros).
+inline bool tc_encode_gated(PFN_encodeTiled enc, CUtensorMap* m, const void* arena_in, const swapmoe_config_t& c, uint32_t box_rows,
+                            uint32_t box_k) {
+  const cuuint64_t d = (cuuint64_t)c.d_model, f = (cuuint64_t)c.d_ff;
+  const cuuint64_t dims[4] = {(cuuint64_t)kTcBK, (cuuint64_t)(2 * (c.K + c.spare_slots) - 1) * f, 2, d / kTcBK};
+  const cuuint64_t strides[3] = {d * 2, f * d * 2, (cuuint64_t)kTcBK * 2};
+  const cuuint32_t box[4] = {(cuuint32_t)kTcBK, box_rows, 2, box_k};
+  const cuuint32_t estr[4] = {1, 1, 1, 1};
+  return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(arena_in), dims, strides, box, estr,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// The grouped GEMMs of a small batch (pairs <= 64): both, or with only = 1 / 2 one of them.  With top_k == 1 the second writes
+// gate * y straight into `out` (*combined = true).
 inline int32_t tc_ffn_small(TcState& s, TcSmallCache& cache, const swapmoe_config_t& c, const void* xp, void* h,
                             float* y, void* out, int rows_pad, const void* arena_in, const void* arena_out,
                             const TileDesc* tiles, const int32_t* n_tiles, const int32_t* row_pair,
                             const float* mgate, int max_tiles, int n_tokens, int32_t* status, cudaStream_t st,
-                            bool pdl, int64_t* launches, bool* combined, cudaEvent_t between = nullptr) {
+                            bool pdl, int64_t* launches, bool* combined, int only, cudaEvent_t between = nullptr) {
   if (!s.enabled || !s.arena_bound) return SWAPMOE_ERR_NOT_READY;
+  const bool swiglu = c.act == SWAPMOE_ACT_SWIGLU;
+  const int mats = swiglu ? 2 : 1;
   const long long pairs = (long long)n_tokens * c.top_k;
   int a_rows = 16;
   while (a_rows < pairs) a_rows <<= 1;                       // 16, 32 or 64
   const int a_tile = a_rows * kTcBK * 2;
-  const long long row_tiles = pairs < c.K ? pairs : c.K;     // one row tile per touched slot
+  // one row tile per slot that may be touched (for those a batch likely touches the widths come out wide, and a batch that
+  // spreads further pays a whole round: 1024 x 4096, 16 slots, 16 tokens 54.3 -> 61.1 us per forward)
+  const long long row_tiles = pairs < c.K ? pairs : c.K;
   if (!cache.valid || cache.a_rows != a_rows || cache.n_tokens != n_tokens) {
     const int P = c.K + c.spare_slots;
-    if (!tc_small_geometry(c.d_ff, c.d_model / kTcBK, row_tiles, s.sm_count, a_tile, &cache.g1) ||
+    if (!tc_small_geometry(mats * c.d_ff, c.d_model / kTcBK, row_tiles, s.sm_count, a_tile, &cache.g1) ||
         !tc_small_geometry(c.d_model, c.d_ff / kTcBK, row_tiles, s.sm_count, a_tile, &cache.g2))
       return SWAPMOE_ERR_UNSUPPORTED;
     if (!tc_encode_3d(s.encode, &cache.mA1, xp, (uint64_t)rows_pad, (uint64_t)c.d_model, a_rows, cache.g1.kps) ||
-        !tc_encode_3d(s.encode, &cache.mB1, arena_in, (uint64_t)P * c.d_ff, (uint64_t)c.d_model, cache.g1.bn,
-                      cache.g1.kps) ||
+        !(swiglu ? tc_encode_gated(s.encode, &cache.mB1, arena_in, c, cache.g1.bn / 2, cache.g1.kps)
+                 : tc_encode_3d(s.encode, &cache.mB1, arena_in, (uint64_t)P * c.d_ff, (uint64_t)c.d_model, cache.g1.bn,
+                                cache.g1.kps)) ||
         !tc_encode_3d(s.encode, &cache.mA2, h, (uint64_t)rows_pad, (uint64_t)c.d_ff, a_rows, cache.g2.kps) ||
         !tc_encode_3d(s.encode, &cache.mB2, arena_out, (uint64_t)P * c.d_model, (uint64_t)c.d_ff, cache.g2.bn,
                       cache.g2.kps))
@@ -358,17 +410,22 @@ inline int32_t tc_ffn_small(TcState& s, TcSmallCache& cache, const swapmoe_confi
   const bool scatter = c.top_k == 1;
   TcSmallArgs a1;
   a1.g.C = h; a1.g.tiles = tiles; a1.g.n_tiles = n_tiles; a1.g.status = status; a1.g.ldc = c.d_ff;
-  a1.g.n_col_tiles = (c.d_ff + cache.g1.bn - 1) / cache.g1.bn; a1.g.k_blocks = c.d_model / kTcBK;
-  a1.g.b_rows_per_phys = c.d_ff; a1.g.b_rows_gate = 0; a1.g.a_box_bytes = a_tile; a1.g.row_group = 1 << 30;
+  a1.g.n_col_tiles = (mats * c.d_ff + cache.g1.bn - 1) / cache.g1.bn; a1.g.k_blocks = c.d_model / kTcBK;
+  a1.g.b_rows_per_phys = mats * c.d_ff; a1.g.b_rows_gate = 0; a1.g.a_box_bytes = a_tile; a1.g.row_group = 1 << 30;
   a1.g.row_pair = nullptr; a1.g.gate = nullptr; a1.g.top_k = c.top_k; a1.g.early_b = 0;
   a1.kps = cache.g1.kps; a1.n_stages = cache.g1.n_stages; a1.a_tile_bytes = a_tile;
   long long work = (long long)max_tiles * a1.g.n_col_tiles;
   int grid = work > s.sm_count ? s.sm_count : (int)work;
-  if (launch_kernel(tc_small_kernel_for<kTcEpiReluBf16>(cache.g1.bn_index), dim3(grid), dim3(kTcThreads),
-                    cache.g1.smem_bytes, st, pdl, cache.mA1, cache.mB1, a1) != cudaSuccess)
-    return SWAPMOE_ERR_CUDA;
-  ++*launches;
+  if (only != 2) {
+    if (launch_kernel(swiglu ? tc_small_kernel_for<kTcEpiSwigluBf16>(cache.g1.bn_index)
+                             : tc_small_kernel_for<kTcEpiReluBf16>(cache.g1.bn_index),
+                      dim3(grid), dim3(kTcThreads), cache.g1.smem_bytes, st, pdl, cache.mA1, cache.mB1, a1) != cudaSuccess)
+      return SWAPMOE_ERR_CUDA;
+    ++*launches;
+  }
   if (between) cudaEventRecord(between, st);
+  *combined = c.top_k == 1;
+  if (only == 1) return SWAPMOE_OK;
 
   TcSmallArgs a2;
   a2.g.C = scatter ? out : static_cast<void*>(y);
