@@ -352,10 +352,10 @@ int32_t forward_impl(swapmoe_layer* L, const void* x, const float* ext_logits, v
   pa.scan = sa;
   mark(L, 2, st);
   const int groups = groups_planned;
-  // own_scan: three extra columns of CTAs, whose first CTAs reduce the three per-expert scores
+  // own_scan: four extra columns of CTAs, whose first CTAs reduce the three per-expert scores and lay out the slots
   if (!rerun) {
     if (launch_kernel(c.top_k == 1 ? permute_gather_kernel<DT, true> : permute_gather_kernel<DT, false>,
-                      dim3(n_cta + (own_scan ? 3 : 0), groups), dim3(kPermThreads), 0, st, pdl, pa) != cudaSuccess)
+                      dim3(n_cta + (own_scan ? 4 : 0), groups), dim3(kPermThreads), 0, st, pdl, pa) != cudaSuccess)
       return SWAPMOE_ERR_CUDA;
     L->launches++;
   }

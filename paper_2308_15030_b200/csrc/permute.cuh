@@ -302,9 +302,9 @@ struct PermuteArgs {
   int32_t* row_pair;          // [rows_pad] flat pair index stored in each occupied padded row
   void* xp;                   // [rows_pad, d]
   int32_t T, d, k, K, tok_tile;
-  int32_t own_scan;           // 1: this kernel sums the router's per-CTA histograms itself (scan.*), CTA (0, 0)
-                              // publishes count / offset / pad_offset / tile lists, and the extra CTA column
-                              // blockIdx.x == scan.n_cta reduces the Eq. (1) partials
+  int32_t own_scan;           // 1: this kernel sums the router's per-CTA histograms itself (scan.*); of four extra CTA columns
+                              // from blockIdx.x == scan.n_cta on, three reduce the per-expert scores and the fourth
+                              // publishes count / offset / pad_offset / tile lists
   ScanArgs scan;
 };
 
@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(kPermThreads, 2) permute_gather_kernel(const P
   // the next kernel's CTAs may be scheduled at once: they stop at their own wait, and until then they
   // touch nothing this kernel or the router writes
   pdl_trigger();
-  if (a.own_scan && (int)blockIdx.x >= a.scan.n_cta) {
+  if (a.own_scan && (int)blockIdx.x >= a.scan.n_cta && (int)blockIdx.x < a.scan.n_cta + 3) {
     // ---- the three extra columns of CTAs: the first CTA of column n_cta + w reduces score w of {Eq. (1), token
     // counts, Eq. (1) over the masked routing}: each is done before the copying CTAs are, none delays the grid
     if (blockIdx.y != 0) return;
@@ -396,6 +396,11 @@ __global__ void __launch_bounds__(kPermThreads, 2) permute_gather_kernel(const P
     }
     return;
   }
+  // The CTA of one more column has no tokens: it lays the slots out for everybody else (counts, offsets, tile lists), which takes
+  // 2 to 5 us longer than the offsets alone and held up the whole grid when the first token tile's CTA did it (2048 tokens of
+  // 768 x 3072: rows placed 2.2 us after the other CTAs' ones, 6011 tokens top-4 5 us).
+  const bool publish = a.own_scan && (int)blockIdx.x == a.scan.n_cta + 3;
+  if (publish && blockIdx.y != 0) return;
   if (tid == 0 && blockIdx.y == 0) SWAPMOE_STAMP(1, 0);
   const int npair = a.tok_tile * a.k;          // <= 512
   const int nwarp_p = (npair + 31) >> 5;
@@ -462,7 +467,8 @@ __global__ void __launch_bounds__(kPermThreads, 2) permute_gather_kernel(const P
       s_base[tid] = before;
     }
     __syncthreads();
-    if (warp == 0) slot_layout_warp(a.scan, s_tot, s_off, s_pad, blockIdx.x == 0 && blockIdx.y == 0);
+    if (warp == 0) slot_layout_warp(a.scan, s_tot, s_off, s_pad, publish);
+    if (publish) return;
   } else {
     if (tid < a.K) {
       s_base[tid] = a.cta_base[(size_t)blockIdx.x * a.K + tid];
