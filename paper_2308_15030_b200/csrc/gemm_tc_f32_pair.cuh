@@ -88,16 +88,20 @@ tc_gemm_f32_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_co
     ptx::prefetch_tmap(&tmA);
     ptx::prefetch_tmap(&tmB);
   }
-  ptx::cluster_start_sync();
-  if (warp == 2) {
-    ptx::tmem_alloc_pair(tmem_slot, 512);
-    ptx::tmem_relinquish_pair();
+  ptx::cluster_start_sync();                      // both CTAs run and their barriers are initialised
+  // Who needs tensor memory waits for this CTA's allocation (the MMA issuer learns of the peer's by its converters' first
+  // arrivals); the producers go on.
+  uint32_t tmem_base = 0;
+  if (warp != 0 && warp != 3) {
+    if (warp == 2) {
+      ptx::tmem_alloc_pair(tmem_slot, 512);
+      ptx::tmem_relinquish_pair();
+    }
+    ptx::tc_fence_before();
+    asm volatile("bar.sync 1, %0;" ::"n"(kF32PairThreads - 64) : "memory");
+    ptx::tc_fence_after();
+    tmem_base = *tmem_slot;
   }
-  ptx::tc_fence_before();
-  __syncthreads();
-  ptx::cluster_sync_all();                        // the peer's barriers are initialised before anyone signals them
-  ptx::tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
 
   // weight rows of column tile ct that this CTA stages
   auto weight_row = [&](const TileDesc& td, int ct) {

@@ -29,9 +29,12 @@ constexpr int kPairBBytes = kPairTokens / 2 * kTcBK * 2;      // at most 16 KB: 
 constexpr int kPairStageArea = 6 * (kPairABytes + kPairBBytes);   // 6 stages of 256 tokens, 8 of 128, 9 of 64
 constexpr int kPairMaxStages = 9;
 __device__ __forceinline__ int pair_stages(int max_tokens) { return max_tokens > 128 ? 6 : max_tokens > 64 ? 8 : 9; }
-constexpr int kPairWarpBytes = 4096;                          // staging of each epilogue warp
-// + alignment slack and barriers (1 KB each)
-constexpr int kPairSmemBytes = kPairStageArea + 2048 + 8 * kPairWarpBytes;
+// staging of an epilogue warp: a box of 32 tokens x 32 columns (SwiGLU 16), or output row and gate value of its 128 tokens
+__host__ __device__ constexpr int pair_warp_bytes(int epi) { return epi == kTcEpiF32 ? 4096 : epi == kTcEpiScatterBf16 ? 1024 : 2048; }
+// + alignment slack and barriers (1 KB each).  GEMM-1's leave room for a CTA of the permutation (12 KB), so that its CTAs may come
+// up while the permutation still runs.
+__host__ __device__ constexpr int pair_smem_bytes(int epi) { return kPairStageArea + 2048 + 8 * pair_warp_bytes(epi); }
+static_assert(pair_smem_bytes(kTcEpiReluBf16) + 1024 + 12288 <= 228 * 1024, "beside a CTA of the permutation");
 
 namespace ptx {
 
@@ -72,17 +75,18 @@ __device__ __forceinline__ void tma_load_5d_pair(void* dst, const CUtensorMap* m
       ::"r"(smem_u32(dst)), "l"(map), "r"(bar_cluster_addr), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4)
       : "memory");
 }
+// The same, releasing what this thread has done before.
+__device__ __forceinline__ void mbar_arrive_release_cluster(uint32_t bar_cluster_addr) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr) : "memory");
+}
 // A box of shared memory to global memory; columns and rows outside the matrix are left out.
 __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, const void* src, int c0, int c1) {
   asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];\ncp.async.bulk.commit_group;" ::"l"(map),
                "r"(smem_u32(src)), "r"(c0), "r"(c1)
                : "memory");
 }
-// At most N of this thread's stores still read their shared memory.
-template <int N>
-__device__ __forceinline__ void tma_store_wait_read() {
-  asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
-}
+// This thread's stores have read their shared memory.
+__device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 // Arrival on a barrier that the peer CTA's threads wait on (mbar_try_wait_cluster).  Relaxed at cluster scope: with the tcgen05
 // fences on either side it orders this warp's tcgen05 accesses (the accumulator has been read, tcgen05.wait::ld has
@@ -158,7 +162,8 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
   uint64_t* empty = bars + kPairMaxStages;  // [stages]  one in each CTA (the commit reaches both)
   uint64_t* acc_full = bars + 2 * kPairMaxStages;  // [2]  one in each CTA
   uint64_t* acc_empty = acc_full + 2;       // [2]       used in the even CTA
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
+  uint64_t* tmem_ready = acc_empty + 2;     // used in the even CTA: the odd one has allocated its half
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tmem_ready + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;   // warp-uniform
@@ -167,8 +172,25 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
 
   constexpr int kTr = (EPI == kTcEpiReluBf16 || EPI == kTcEpiSwigluBf16) ? 2 : 3;   // trace id: GEMM-1 or GEMM-2
   (void)kTr;
+  // The producer's first tile: the number of tiles and the first 32 descriptors (the list holds at least so many) in one round
+  // trip, for GEMM-2 underneath the barriers below.
+  int4 first_raw = make_int4(0, 0, 0, 0);
+  int2 first_n = make_int2(0, 0);
+  auto fetch_list = [&]() {
+    first_raw = __ldcg(reinterpret_cast<const int4*>(a.tiles + lane));
+    first_n = __ldcg(reinterpret_cast<const int2*>(a.n_tiles));
+  };
+  auto tile_at = [&](int rt) -> TileDesc {                   // by the whole producer warp
+    const int src = rt & 31;
+    const int4 raw = rt < 32 ? make_int4(__shfl_sync(0xffffffffu, first_raw.x, src), __shfl_sync(0xffffffffu, first_raw.y, src),
+                                         __shfl_sync(0xffffffffu, first_raw.z, src), __shfl_sync(0xffffffffu, first_raw.w, src))
+                             : __ldcg(reinterpret_cast<const int4*>(a.tiles + rt));
+    return *reinterpret_cast<const TileDesc*>(&raw);
+  };
+  if (warp == 0 && a.early_w) fetch_list();
   if (threadIdx.x == 0) {
     SWAPMOE_STAMP(kTr, 0);
+    ptx::mbar_init(tmem_ready, 1);
     for (int s = 0; s < kPairMaxStages; ++s) { ptx::mbar_init(&full[s], 1); ptx::mbar_init(&empty[s], 1); }
     for (int b = 0; b < 2; ++b) { ptx::mbar_init(&acc_full[b], 1); ptx::mbar_init(&acc_empty[b], 16); }
     *abort_flag = 0;
@@ -176,16 +198,20 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
     ptx::prefetch_tmap(&tmW);
     ptx::prefetch_tmap(&tmX128);
   }
-  ptx::cluster_start_sync();                                  // before the first access to the peer's tensor memory
-  if (warp == 2) {
-    ptx::tmem_alloc_pair(tmem_slot, kTmemCols);               // issued in both CTAs: one allocation for the pair
-    ptx::tmem_relinquish_pair();
+  ptx::cluster_start_sync();                                  // both CTAs run and their barriers are initialised
+  // Tensor memory: who needs it waits for this CTA's allocation, the MMA issuer also for the peer's; the producers go on.
+  uint32_t tmem_base = 0;
+  if (warp != 0 && warp != 3) {
+    if (warp == 2) {
+      ptx::tmem_alloc_pair(tmem_slot, kTmemCols);             // issued in both CTAs: one allocation for the pair
+      ptx::tmem_relinquish_pair();
+      if (rank == 1 && lane == 0) ptx::mbar_arrive_release_cluster(ptx::map_to_cta(ptx::smem_u32(tmem_ready), 0u));
+    }
+    ptx::tc_fence_before();
+    asm volatile("bar.sync 1, %0;" ::"n"(kPairThreads - 64) : "memory");
+    ptx::tc_fence_after();
+    tmem_base = *tmem_slot;
   }
-  ptx::tc_fence_before();
-  __syncthreads();
-  ptx::cluster_sync_all();                                    // the peer's barriers are initialised before anyone signals them
-  ptx::tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
 
   // tokens of a tile in the MMA's columns; each CTA stages half of them
   auto tile_cols = [](int rows) { return (rows + kPairTokenStep - 1) & ~(kPairTokenStep - 1); };
@@ -203,12 +229,11 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
   // dependent-launch wait.
   int pre = 0;
   if (warp == 0 && a.early_w) {
-    const int n_rt = __ldcg(a.n_tiles), early_stages = pair_stages(__ldcg(a.n_tiles + 1));
+    const int n_rt = first_n.x, early_stages = pair_stages(first_n.y);
     if (pair < n_rt * a.n_col_tiles) {
       int rt, ct;
       decode_tile(pair, n_rt, a.n_col_tiles, a.row_group, &rt, &ct);
-      const int4 raw = __ldcg(reinterpret_cast<const int4*>(a.tiles + rt));
-      const TileDesc td = *reinterpret_cast<const TileDesc*>(&raw);
+      const TileDesc td = tile_at(rt);
       const uint32_t bytes = (uint32_t)(2 * kPairABytes + tile_cols(td.rows) * kTcBK * 2);
       pre = a.k_blocks < early_stages ? a.k_blocks : early_stages;
       for (int kb = 0; kb < pre; ++kb) {
@@ -224,7 +249,9 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
   pdl_wait();      // the activations come from the preceding kernel
   pdl_trigger();
   if (threadIdx.x == 0) SWAPMOE_STAMP(kTr, 2);
-  const int n_row_tiles = a.n_tiles[0], max_tokens = a.n_tiles[1];
+  if (warp == 0 && !a.early_w) fetch_list();
+  else if (warp != 0) first_n = __ldcg(reinterpret_cast<const int2*>(a.n_tiles));
+  const int n_row_tiles = first_n.x, max_tokens = first_n.y;
   const int total = n_row_tiles * a.n_col_tiles;
   const int n_stages = pair_stages(max_tokens), x_bytes = max_tokens / 2 * kTcBK * 2;
   unsigned char* sX = smem + n_stages * kPairABytes;          // [stages][max_tokens / 2][64] bf16
@@ -237,7 +264,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
     for (int t = pair; t < total && ok; t += n_pairs) {
       int rt, ct;
       decode_tile(t, n_row_tiles, a.n_col_tiles, a.row_group, &rt, &ct);
-      const TileDesc td = a.tiles[rt];
+      const TileDesc td = t == pair ? tile_at(rt) : a.tiles[rt];
       const int cols = tile_cols(td.rows), half = cols / 2;     // half: a multiple of 16, at most 128
       const int xrow = td.row0 + (int)rank * half;
       const uint32_t bytes = (uint32_t)(2 * kPairABytes + cols * kTcBK * 2);
@@ -275,7 +302,8 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
       // ------------------------------------------------------------------ MMA issuer (even CTA, for the pair)
       int stage = 0, acc = 0;
       uint32_t phase = 0, acc_phase = 0;
-      bool ok = true;
+      bool ok = warp_wait<true>(tmem_ready, 0u, abort_flag, a.status, 15);
+      ptx::tc_fence_after();
       for (int t = pair; t < total && ok; t += n_pairs) {
         int rt, ct_unused;
         decode_tile(t, n_row_tiles, a.n_col_tiles, a.row_group, &rt, &ct_unused);
@@ -311,10 +339,8 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
     const int q = warp & 3;                    // TMEM lane quarter this warp may read
     const int part = (warp - 4) >> 2;          // two warps per quarter take turns with the chunks of 32 tokens
     const int odd = lane & 1, hi = lane >> 4;
-    // the warp's 4 KB: a box on its way to global memory (bf16: two), or output row and gate value of its 128 tokens
-    unsigned char* s_stage = smem + kPairStageArea + 1024 + (warp - 4) * kPairWarpBytes;
+    unsigned char* s_stage = smem + kPairStageArea + 1024 + (warp - 4) * pair_warp_bytes(EPI);
     int2* s_dest = reinterpret_cast<int2*>(s_stage);
-    int buf = 0;
     const uint32_t acc_empty0 = ptx::map_to_cta(ptx::smem_u32(acc_empty), 0u);
     int acc = 0;
     uint32_t acc_phase = 0;
@@ -363,11 +389,7 @@ tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
         // stored with the valid ones: they lie in the slot's own segment, and nobody reads a row that no pair occupies.
         unsigned char* stg = s_stage;
         if (EPI != kTcEpiScatterBf16) {
-          if (EPI != kTcEpiF32) stg += (buf ^= 2048);
-          if (lane == 0) {
-            if (EPI == kTcEpiF32) ptx::tma_store_wait_read<0>();
-            else ptx::tma_store_wait_read<1>();
-          }
+          if (lane == 0) ptx::tma_store_wait_read();
           __syncwarp();
         }
         if (EPI == kTcEpiF32) {
@@ -436,7 +458,7 @@ typedef void (*TcPairKernel)(const CUtensorMap, const CUtensorMap, const CUtenso
 
 template <int EPI>
 inline bool tc_pair_set_smem_attr() {
-  return cudaFuncSetAttribute(tc_gemm_pair_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmemBytes) ==
+  return cudaFuncSetAttribute(tc_gemm_pair_kernel<EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, pair_smem_bytes(EPI)) ==
          cudaSuccess;
 }
 
@@ -448,7 +470,7 @@ inline int tc_pair_init(int sm_count) {
     return 0;
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(2 * (sm_count / 2)); cfg.blockDim = dim3(kPairThreads); cfg.dynamicSmemBytes = kPairSmemBytes;
+  cfg.gridDim = dim3(2 * (sm_count / 2)); cfg.blockDim = dim3(kPairThreads); cfg.dynamicSmemBytes = pair_smem_bytes(kTcEpiF32);
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
@@ -481,20 +503,23 @@ inline int32_t tc_gemm_pair(TcState& s, int n_pairs, const swapmoe_config_t& c, 
   }
   const CUtensorMap *mw, *mx, *mc;
   TcPairKernel k;
+  int epi;
   if (which == 1) {
     const int out1 = swiglu ? kTcBM : 2 * kTcBM;
     g.ldc = c.d_ff; g.n_col_tiles = (c.d_ff + out1 - 1) / out1; g.k_blocks = c.d_model / kTcBK;
     g.w_rows = c.d_ff; g.early_w = 0;
+    epi = swiglu ? kTcEpiSwigluBf16 : kTcEpiReluBf16;
     k = swiglu ? tc_gemm_pair_kernel<kTcEpiSwigluBf16> : tc_gemm_pair_kernel<kTcEpiReluBf16>;
     mw = swiglu ? &s.map_win_gated : &s.map_win[1]; mx = s.map_xp; mc = &s.map_h_out;
   } else {
     g.ldc = c.d_model; g.n_col_tiles = (c.d_model + 2 * kTcBM - 1) / (2 * kTcBM); g.k_blocks = c.d_ff / kTcBK;
     g.w_rows = c.d_model; g.early_w = 1;
+    epi = scatter ? kTcEpiScatterBf16 : kTcEpiF32;
     k = scatter ? tc_gemm_pair_kernel<kTcEpiScatterBf16> : tc_gemm_pair_kernel<kTcEpiF32>;
     mw = &s.map_wout[1]; mx = s.map_h; mc = &s.map_y_out;
   }
   const long long work = (long long)max_tiles * g.n_col_tiles;
-  return launch_kernel(k, dim3(2 * (work > n_pairs ? n_pairs : (int)work)), dim3(kPairThreads), kPairSmemBytes, st, pdl, *mw,
+  return launch_kernel(k, dim3(2 * (work > n_pairs ? n_pairs : (int)work)), dim3(kPairThreads), pair_smem_bytes(epi), st, pdl, *mw,
                        mx[0], mx[1], mx[2], mx[3], *mc, g) == cudaSuccess ? SWAPMOE_OK : SWAPMOE_ERR_CUDA;
 }
 
