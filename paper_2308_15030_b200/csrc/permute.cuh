@@ -121,9 +121,10 @@ static __device__ __noinline__ void write_pair_tiles(const PairList l, float inv
 // (K <= 64); offsets, padded offsets and first-tile indices are exclusive prefix sums over the slots,
 // taken with warp scans (the heights of `tiles` are powers of two: shifts, no divisions - this code runs once,
 // every dependent instruction counts).  s_off / s_pad (shared, may be nullptr) receive the exclusive
-// offsets; with `write_global` the warp also writes count / offset / pad_offset and the tile lists.
+// offsets; with kPublish the warp also writes count / offset / pad_offset and the tile lists.
+template <bool kPublish>
 __device__ __forceinline__ void slot_layout_warp(const ScanArgs& a, const int32_t* s_count, int32_t* s_off,
-                                                 int32_t* s_pad, bool write_global) {
+                                                 int32_t* s_pad) {
   const int lane = threadIdx.x & 31;
   const int sh = a.tile_rows > 0 ? 31 - __clz(a.tile_rows) : 31;      // 31: no tiles
   const int round = a.tile_rows > 0 ? a.tile_rows - 1 : 0;
@@ -132,15 +133,15 @@ __device__ __forceinline__ void slot_layout_warp(const ScanArgs& a, const int32_
   for (int h = 0; h < 2; ++h) {
     const int s = lane + 32 * h;
     c[h] = s < a.K ? s_count[s] : 0;
-    ph[h] = (write_global && s < a.K) ? a.phys_slot[s] : 0;     // issued early: its latency hides behind the scans
+    ph[h] = (kPublish && s < a.K) ? a.phys_slot[s] : 0;         // issued early: its latency hides behind the scans
     off[h] = c[h];
     pad[h] = (c[h] + kSegAlign - 1) & ~(kSegAlign - 1);
-    ta[h] = (c[h] + round) >> sh;
+    ta[h] = kPublish ? (c[h] + round) >> sh : 0;
   }
-  {
+  if constexpr (kPublish) {
     // slots whose weights this forward reads: the algorithmic weight traffic of the layer
     const int nz = __popc(__ballot_sync(0xffffffffu, c[0] > 0)) + __popc(__ballot_sync(0xffffffffu, c[1] > 0));
-    if (write_global && lane == 0 && a.touched != nullptr) atomicAdd(a.touched, (unsigned long long)nz);
+    if (lane == 0 && a.touched != nullptr) atomicAdd(a.touched, (unsigned long long)nz);
   }
   // inclusive scans of the three quantities over 64 slots
 #pragma unroll
@@ -148,13 +149,13 @@ __device__ __forceinline__ void slot_layout_warp(const ScanArgs& a, const int32_
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int u0 = __shfl_up_sync(0xffffffffu, off[h], o), u1 = __shfl_up_sync(0xffffffffu, pad[h], o);
-      const int u2 = __shfl_up_sync(0xffffffffu, ta[h], o);
+      const int u2 = kPublish ? __shfl_up_sync(0xffffffffu, ta[h], o) : 0;
       if (lane >= o) { off[h] += u0; pad[h] += u1; ta[h] += u2; }
     }
   }
   {
     const int t0 = __shfl_sync(0xffffffffu, off[0], 31), t1 = __shfl_sync(0xffffffffu, pad[0], 31);
-    const int t2 = __shfl_sync(0xffffffffu, ta[0], 31);
+    const int t2 = kPublish ? __shfl_sync(0xffffffffu, ta[0], 31) : 0;
     off[1] += t0; pad[1] += t1; ta[1] += t2;
   }
 #pragma unroll
@@ -163,29 +164,30 @@ __device__ __forceinline__ void slot_layout_warp(const ScanArgs& a, const int32_
     if (s < a.K) {
       const int cnt = c[h];
       const int padded = (cnt + kSegAlign - 1) & ~(kSegAlign - 1);
-      const int nt = (cnt + round) >> sh;
-      const int o_excl = off[h] - cnt, p_excl = pad[h] - padded, t_excl = ta[h] - nt;
+      const int o_excl = off[h] - cnt, p_excl = pad[h] - padded;
       if (s_off != nullptr) { s_off[s] = o_excl; s_pad[s] = p_excl; }
-      if (!write_global) continue;
-      a.count[s] = cnt;
-      a.offset[s] = o_excl;
-      a.pad_offset[s] = p_excl;
-      for (int i = 0; i < nt; ++i) {
-        TileDesc td;
-        td.phys = ph[h];
-        td.row0 = p_excl + i * a.tile_rows;
-        td.rows = min(a.tile_rows, cnt - i * a.tile_rows);
-        td.slot = s;
-        a.tiles[t_excl + i] = td;
-      }
-      if (s == a.K - 1) {
-        a.offset[a.K] = off[h];
-        a.pad_offset[a.K] = pad[h];
-        if (a.tile_rows > 0) *a.n_tiles = ta[h];
+      if constexpr (kPublish) {
+        const int nt = (cnt + round) >> sh, t_excl = ta[h] - nt;
+        a.count[s] = cnt;
+        a.offset[s] = o_excl;
+        a.pad_offset[s] = p_excl;
+        for (int i = 0; i < nt; ++i) {
+          TileDesc td;
+          td.phys = ph[h];
+          td.row0 = p_excl + i * a.tile_rows;
+          td.rows = min(a.tile_rows, cnt - i * a.tile_rows);
+          td.slot = s;
+          a.tiles[t_excl + i] = td;
+        }
+        if (s == a.K - 1) {
+          a.offset[a.K] = off[h];
+          a.pad_offset[a.K] = pad[h];
+          if (a.tile_rows > 0) *a.n_tiles = ta[h];
+        }
       }
     }
   }
-  if (write_global) {
+  if constexpr (kPublish) {
     const int first0 = pad[0] - ((c[0] + kSegAlign - 1) & ~(kSegAlign - 1));
     const int first1 = pad[1] - ((c[1] + kSegAlign - 1) & ~(kSegAlign - 1));
     if (a.pair[0].tiles != nullptr) write_pair_tiles(a.pair[0], a.inv_pairs, c[0], c[1], ph[0], ph[1], first0, first1);
@@ -265,7 +267,7 @@ __device__ __forceinline__ void scan_reduce_block(const ScanArgs& a, void* stage
   if (own_s && a.cta_mimp != nullptr)        // slots map to distinct experts: no two threads share a target
     a.mimp[my_expert] += reduce_column_serial(mimpp, a.n_cta, a.K, tid);
   __syncthreads();
-  if (tid < 32) slot_layout_warp(a, s_count, nullptr, nullptr, true);
+  if (tid < 32) slot_layout_warp<true>(a, s_count, nullptr, nullptr);
 }
 
 // Called by every thread of a router CTA after its partials are written.  With a ticket counter the
@@ -340,6 +342,40 @@ __device__ __forceinline__ float reduce_columns_parallel(const float* src, int n
   return total;
 }
 
+// Sums of the router CTAs' histograms, by all threads of a CTA.  Thread (share, slot) adds the rows of a contiguous share of the
+// router CTAs, all loads in flight together: the total and, with kBefore, the rows in front of router CTA `n_before`.
+template <bool kBefore>
+__device__ __forceinline__ void add_histogram_shares(const ScanArgs& a, int n_before, int32_t (*s_part)[kPermThreads]) {
+  const int tid = threadIdx.x, K = a.K, n_cta = a.n_cta;
+  const int PK = kPermThreads / K;                         // shares per slot
+  const int R = (n_cta + PK - 1) / PK;                     // router CTAs per share (<= 8 up to 256 CTAs, K = 16)
+  const int sh = tid / K, col = tid - sh * K;
+  if (sh >= PK) return;
+  int tot = 0, before = 0;
+  const int c0 = sh * R, c1 = min(n_cta, c0 + R);
+  for (int cb = c0; cb < c1; cb += 8) {
+    int v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = cb + u < c1 ? a.cta_hist[(size_t)(cb + u) * K + col] : 0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) { tot += v[u]; if (kBefore) before += cb + u < n_before ? v[u] : 0; }
+  }
+  s_part[0][tid] = tot;
+  if (kBefore) s_part[1][tid] = before;
+}
+// Behind a barrier: thread `slot` adds the shares.
+template <bool kBefore>
+__device__ __forceinline__ void fold_histogram_shares(const ScanArgs& a, const int32_t (*s_part)[kPermThreads], int32_t* s_tot,
+                                                      int32_t* s_base) {
+  const int tid = threadIdx.x, K = a.K, PK = kPermThreads / K;
+  if (tid >= K) return;
+  int tot = 0, before = 0;
+#pragma unroll 8
+  for (int q = 0; q < PK; ++q) { tot += s_part[0][q * K + tid]; if (kBefore) before += s_part[1][q * K + tid]; }
+  s_tot[tid] = tot;
+  if (kBefore) s_base[tid] = before;
+}
+
 // One CTA = the pairs of tok_tile (<= 128) tokens in flat order p = t*k + j.  The rank of a
 // pair among the pairs of the same slot is: pairs in earlier CTAs +
 // pairs in earlier warps of this CTA + earlier lanes of this warp (match + popc),
@@ -398,9 +434,20 @@ __global__ void __launch_bounds__(kPermThreads, 2) permute_gather_kernel(const P
   }
   // The CTA of one more column has no tokens: it lays the slots out for everybody else (counts, offsets, tile lists), which takes
   // 2 to 5 us longer than the offsets alone and held up the whole grid when the first token tile's CTA did it (2048 tokens of
-  // 768 x 3072: rows placed 2.2 us after the other CTAs' ones, 6011 tokens top-4 5 us).
-  const bool publish = a.own_scan && (int)blockIdx.x == a.scan.n_cta + 3;
-  if (publish && blockIdx.y != 0) return;
+  // 768 x 3072: rows placed 2.2 us after the other CTAs' ones, 6011 tokens top-4 5 us).  In a branch of its own: the copying
+  // CTAs hold token pieces in registers, and with the lists' code in their path (behind a run-time switch) the kernel spilled 76
+  // bytes a thread (us per forward with that code in line / here: 768 x 3072, 2048 tokens 55.7 / 54.8, 8192 tokens and 32 slots
+  // 132.3 / 131.5; twelve layers of 1024 x 4096 at 29 tokens 736.3 / 734.2).
+  if (a.own_scan && (int)blockIdx.x >= a.scan.n_cta + 3) {
+    if (blockIdx.y != 0) return;
+    pdl_wait();
+    add_histogram_shares<false>(a.scan, 0, s_part);
+    __syncthreads();
+    fold_histogram_shares<false>(a.scan, s_part, s_tot, nullptr);
+    __syncthreads();
+    if (warp == 0) slot_layout_warp<true>(a.scan, s_tot, nullptr, nullptr);
+    return;
+  }
   if (tid == 0 && blockIdx.y == 0) SWAPMOE_STAMP(1, 0);
   const int npair = a.tok_tile * a.k;          // <= 512
   const int nwarp_p = (npair + 31) >> 5;
@@ -435,40 +482,16 @@ __global__ void __launch_bounds__(kPermThreads, 2) permute_gather_kernel(const P
   const int p = p0 + tid;
   if (tid < npair && p < n_total) s = a.slot[p];
   if (a.own_scan) {
-    // thread (share, slot): the histogram rows of a contiguous share of the router CTAs, all loads in flight together
-    const int K = a.K, n_cta = a.scan.n_cta, n_before = (int)blockIdx.x;
-    const int PK = kPermThreads / K;                       // shares per slot
-    const int R = (n_cta + PK - 1) / PK;                   // router CTAs per share (<= 8 up to 256 CTAs, K = 16)
-    const int sh = tid / K, col = tid - sh * K;
-    if (sh < PK) {
-      int tot = 0, before = 0;
-      const int c0 = sh * R, c1 = min(n_cta, c0 + R);
-      for (int cb = c0; cb < c1; cb += 8) {
-        int v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) v[u] = cb + u < c1 ? a.scan.cta_hist[(size_t)(cb + u) * K + col] : 0;
-#pragma unroll
-        for (int u = 0; u < 8; ++u) { tot += v[u]; before += cb + u < n_before ? v[u] : 0; }
-      }
-      s_part[0][tid] = tot;
-      s_part[1][tid] = before;
-    }
+    add_histogram_shares<true>(a.scan, (int)blockIdx.x, s_part);
     if (warp < nwarp_p) {                      // ranks inside the warp need only the pairs' slots
       const uint32_t same = __match_any_sync(0xffffffffu, s);
       rank = __popc(same & ((1u << lane) - 1u));
       if (s >= 0 && rank == 0) wcount[warp][s] = __popc(same);
     }
     __syncthreads();
-    if (tid < K) {
-      int tot = 0, before = 0;
-#pragma unroll 8
-      for (int q = 0; q < PK; ++q) { tot += s_part[0][q * K + tid]; before += s_part[1][q * K + tid]; }
-      s_tot[tid] = tot;
-      s_base[tid] = before;
-    }
+    fold_histogram_shares<true>(a.scan, s_part, s_tot, s_base);
     __syncthreads();
-    if (warp == 0) slot_layout_warp(a.scan, s_tot, s_off, s_pad, publish);
-    if (publish) return;
+    if (warp == 0) slot_layout_warp<false>(a.scan, s_tot, s_off, s_pad);
   } else {
     if (tid < a.K) {
       s_base[tid] = a.cta_base[(size_t)blockIdx.x * a.K + tid];
