@@ -121,10 +121,12 @@ static __device__ __noinline__ void write_pair_tiles(const PairList l, float inv
 // (K <= 64); offsets, padded offsets and first-tile indices are exclusive prefix sums over the slots,
 // taken with warp scans (the heights of `tiles` are powers of two: shifts, no divisions - this code runs once,
 // every dependent instruction counts).  s_off / s_pad (shared, may be nullptr) receive the exclusive
-// offsets; with kPublish the warp also writes count / offset / pad_offset and the tile lists.
+// offsets.  With kPublish two warps publish what the GEMMs read, side by side: `which` = 0 writes count / offset / pad_offset,
+// `tiles` and the first list for CTA pairs, 1 the second one (GEMM-1 waits for both: us per forward by one warp / by two, 768 x
+// 3072, 2048 tokens 54.8 / 54.0, 512 x 2048 at 90 34.7 / 33.9, 1536 x 1088, 48 slots, 70 tokens 96.3 / 94.8).
 template <bool kPublish>
 __device__ __forceinline__ void slot_layout_warp(const ScanArgs& a, const int32_t* s_count, int32_t* s_off,
-                                                 int32_t* s_pad) {
+                                                 int32_t* s_pad, int which = 0) {
   const int lane = threadIdx.x & 31;
   const int sh = a.tile_rows > 0 ? 31 - __clz(a.tile_rows) : 31;      // 31: no tiles
   const int round = a.tile_rows > 0 ? a.tile_rows - 1 : 0;
@@ -141,7 +143,7 @@ __device__ __forceinline__ void slot_layout_warp(const ScanArgs& a, const int32_
   if constexpr (kPublish) {
     // slots whose weights this forward reads: the algorithmic weight traffic of the layer
     const int nz = __popc(__ballot_sync(0xffffffffu, c[0] > 0)) + __popc(__ballot_sync(0xffffffffu, c[1] > 0));
-    if (lane == 0 && a.touched != nullptr) atomicAdd(a.touched, (unsigned long long)nz);
+    if (which == 0 && lane == 0 && a.touched != nullptr) atomicAdd(a.touched, (unsigned long long)nz);
   }
   // inclusive scans of the three quantities over 64 slots
 #pragma unroll
@@ -166,7 +168,7 @@ __device__ __forceinline__ void slot_layout_warp(const ScanArgs& a, const int32_
       const int padded = (cnt + kSegAlign - 1) & ~(kSegAlign - 1);
       const int o_excl = off[h] - cnt, p_excl = pad[h] - padded;
       if (s_off != nullptr) { s_off[s] = o_excl; s_pad[s] = p_excl; }
-      if constexpr (kPublish) {
+      if (kPublish && which == 0) {
         const int nt = (cnt + round) >> sh, t_excl = ta[h] - nt;
         a.count[s] = cnt;
         a.offset[s] = o_excl;
@@ -190,8 +192,8 @@ __device__ __forceinline__ void slot_layout_warp(const ScanArgs& a, const int32_
   if constexpr (kPublish) {
     const int first0 = pad[0] - ((c[0] + kSegAlign - 1) & ~(kSegAlign - 1));
     const int first1 = pad[1] - ((c[1] + kSegAlign - 1) & ~(kSegAlign - 1));
-    if (a.pair[0].tiles != nullptr) write_pair_tiles(a.pair[0], a.inv_pairs, c[0], c[1], ph[0], ph[1], first0, first1);
-    if (a.pair[1].tiles != nullptr) write_pair_tiles(a.pair[1], a.inv_pairs, c[0], c[1], ph[0], ph[1], first0, first1);
+    if (a.pair[which].tiles != nullptr)
+      write_pair_tiles(a.pair[which], a.inv_pairs, c[0], c[1], ph[0], ph[1], first0, first1);
   }
 }
 
@@ -267,7 +269,7 @@ __device__ __forceinline__ void scan_reduce_block(const ScanArgs& a, void* stage
   if (own_s && a.cta_mimp != nullptr)        // slots map to distinct experts: no two threads share a target
     a.mimp[my_expert] += reduce_column_serial(mimpp, a.n_cta, a.K, tid);
   __syncthreads();
-  if (tid < 32) slot_layout_warp<true>(a, s_count, nullptr, nullptr);
+  if (tid < 64) slot_layout_warp<true>(a, s_count, nullptr, nullptr, tid >> 5);
 }
 
 // Called by every thread of a router CTA after its partials are written.  With a ticket counter the
@@ -445,7 +447,7 @@ __global__ void __launch_bounds__(kPermThreads, 2) permute_gather_kernel(const P
     __syncthreads();
     fold_histogram_shares<false>(a.scan, s_part, s_tot, nullptr);
     __syncthreads();
-    if (warp == 0) slot_layout_warp<true>(a.scan, s_tot, nullptr, nullptr);
+    if (warp < 2) slot_layout_warp<true>(a.scan, s_tot, nullptr, nullptr, warp);
     return;
   }
   if (tid == 0 && blockIdx.y == 0) SWAPMOE_STAMP(1, 0);

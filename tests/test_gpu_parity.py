@@ -1001,3 +1001,14 @@ def test_token_tiles_of_cta_pairs(counts, k, act, renorm):
     res = check_against_oracle(case, case.run(ext_logits=logits), check_logits=False)
     want = np.bincount(first, minlength=K) + (np.bincount((first + K - 1) % K, minlength=K) if k == 2 else 0)
     assert np.array_equal(res["oracle"]["count"], want)
+
+
+@pytest.mark.parametrize("k,act,renorm", [(1, I.ACT_RELU, 0), (2, I.ACT_SWIGLU, 1)])
+def test_tile_lists_of_both_products_from_the_last_router_cta(monkeypatch, k, act, renorm):
+    """Beyond 256 router CTAs the last one to finish lays out the slots; two of its warps write the lists of token tiles of the two
+    products (different numbers of weight tiles: a list each)."""
+    from harness import Case, check_against_oracle
+    monkeypatch.setenv("SWAPMOE_ROUTER_TOK", "32")
+    cfg = _cfg(T=8300, d=256, f=512, E=12, K=5, k=k, act=act, renorm=renorm, zipf_s=1.1)
+    case = Case(cfg)
+    check_against_oracle(case, case.run())
