@@ -91,7 +91,10 @@ enum {
    * unsliced contraction on the other paths (top-1 tensor-core layers fold gate * y into `out`).
    * Otherwise the call returns SWAPMOE_ERR_UNSUPPORTED. */
   SWAPMOE_TAP_H = 11,     /* layer dtype [T*k, d_ff]  act(W_in x) of every pair        */
-  SWAPMOE_TAP_Y = 12      /* fp32 [T*k, d_model]      W_out h of every pair            */
+  SWAPMOE_TAP_Y = 12,     /* fp32 [T*k, d_model]      W_out h of every pair            */
+  /* int32 [2, 2]: for grouped GEMM-1 and GEMM-2 of the last forward the number of token tiles it walked on CTA pairs and
+   * the most tokens one of them may hold (zeros: it ran on another kernel). */
+  SWAPMOE_TAP_TOKEN_TILES = 13
 };
 
 /*

@@ -27,6 +27,7 @@ TAPS = {
     "count": (6, np.int32), "offset": (7, np.int32), "perm": (8, np.int32),
     "inv": (9, np.int32), "xnorm": (10, np.float32),
     "h": (11, None), "y": (12, np.float32),       # h comes in the layer's dtype (bf16 as uint16 bit patterns)
+    "token_tiles": (13, np.int32),
 }
 
 EXPORTS = [
@@ -304,7 +305,7 @@ class Layer:
             dt = np.uint16 if c.dtype == BF16 else np.float32
         shape = {"logits": (T, c.E), "count": (c.K,), "offset": (c.K + 1,), "perm": (T * c.top_k,),
                  "inv": (T * c.top_k,), "xnorm": (T,), "h": (T * c.top_k, c.d_ff),
-                 "y": (T * c.top_k, c.d_model)}.get(name, (T, c.top_k))
+                 "y": (T * c.top_k, c.d_model), "token_tiles": (2, 2)}.get(name, (T, c.top_k))
         a = np.empty(shape, dtype=dt)
         _check(lib().swapmoe_debug_copy(self._h, which, _np_ptr(a), a.nbytes, _stream_ptr(stream)),
                "swapmoe_debug_copy")

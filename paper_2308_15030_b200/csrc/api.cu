@@ -68,6 +68,8 @@ struct swapmoe_layer {
   float* dec_ws;               // its partial-row workspace
   unsigned* dec_tickets;
   CUtensorMap dec_map_wo;      // W_out viewed for the decode kernel's column-slice loads
+  int tile_shift;              // log2 of the token-tile cap of the CTA-pair GEMMs (0: automatic; SWAPMOE_TILE_CAP)
+  const int32_t* pair_lists[2];   // {tiles, cap} of the token tiles GEMM-1 / GEMM-2 of the last forward walked on CTA pairs, or nullptr
   int row_group;               // row tiles per scheduling group of the grouped GEMMs (0: automatic; SWAPMOE_ROW_GROUP)
   bool h_valid, y_valid;       // whether the last forward left h / y in the workspace (debug taps)
   int32_t y_split_last;        // copies of y the last forward's GEMM-2 wrote (slices of its contraction)
@@ -206,6 +208,7 @@ int32_t forward_impl(swapmoe_layer* L, const void* x, const float* ext_logits, v
       return SWAPMOE_ERR_CUDA;
     L->launches++;
     L->h_valid = L->y_valid = false;          // the one-launch kernel keeps both in shared memory
+    L->pair_lists[0] = L->pair_lists[1] = nullptr;
     for (int i = 1; i <= 6; ++i) mark(L, i, st);
     return check_launch();
   }
@@ -260,8 +263,10 @@ int32_t forward_impl(swapmoe_layer* L, const void* x, const float* ext_logits, v
   sa.n_cta = n_cta; sa.K = c.K; sa.E = c.E; sa.tile_rows = tile_rows;
   // token tiles for CTA pairs: one list where the two GEMMs have the same number of weight tiles, else one each
   PairList list1 = {}, list2 = {};
-  if (pc1 > 0) list1 = {L->tiles_b, L->n_tiles_b, pc1};
-  if (pc2 > 0) list2 = pc1 == 0 ? PairList{L->tiles_b, L->n_tiles_b, pc2} : pc1 == pc2 ? list1 : PairList{L->tiles, L->n_tiles, pc2};
+  const int sh = L->tile_shift;
+  if (pc1 > 0) list1 = {L->tiles_b, L->n_tiles_b, pc1, sh};
+  if (pc2 > 0) list2 = pc1 == 0 ? PairList{L->tiles_b, L->n_tiles_b, pc2, sh} : pc1 == pc2 ? list1 : PairList{L->tiles, L->n_tiles, pc2, sh};
+  L->pair_lists[0] = list1.n_tiles; L->pair_lists[1] = list2.n_tiles;
   sa.pair[0] = list1; sa.pair[1] = pc1 == pc2 ? PairList{} : list2;
   sa.inv_pairs = 1.f / (float)std::max(L->gemm_pairs, 1);
   ra.pf_base[0] = ra.pf_base[1] = nullptr;
@@ -539,6 +544,8 @@ int32_t swapmoe_create(swapmoe_layer_t** out, const swapmoe_config_t* cfg) {
     L->small_path = !(env && env[0] == '0');
     env = std::getenv("SWAPMOE_ROW_GROUP");             // row tiles per scheduling group of the grouped GEMMs
     L->row_group = env && std::atoi(env) > 0 ? std::atoi(env) : 0;
+    env = std::getenv("SWAPMOE_TILE_CAP");              // most tokens per tile of the CTA-pair GEMMs: 64, 128 or 256 (else automatic)
+    L->tile_shift = env ? std::atoi(env) == 64 ? 6 : std::atoi(env) == 128 ? 7 : std::atoi(env) == 256 ? 8 : 0 : 0;
     // L2 weight prefetch from the router's idle blocks: budget in MB, 0 = off (default: by batch size, see forward_impl)
     env = std::getenv("SWAPMOE_PREFETCH_MB");
     L->l2_prefetch_bytes = env ? std::max(0ll, std::atoll(env)) << 20 : -1;
@@ -1017,6 +1024,16 @@ int32_t swapmoe_debug_copy(swapmoe_layer_t* L, int32_t which, void* host, size_t
     case SWAPMOE_TAP_PERM: src = L->perm; need = P * 4; break;
     case SWAPMOE_TAP_INV: src = L->inv; need = P * 4; break;
     case SWAPMOE_TAP_XNORM: src = L->xnorm; need = T * 4; break;
+    case SWAPMOE_TAP_TOKEN_TILES: {
+      if (bytes != 4 * sizeof(int32_t)) return SWAPMOE_ERR_INVALID_ARG;
+      int32_t* dst = static_cast<int32_t*>(host);
+      std::memset(dst, 0, bytes);
+      for (int g = 0; g < 2; ++g)
+        if (L->pair_lists[g] && !cuda_ok(cudaMemcpyAsync(dst + 2 * g, L->pair_lists[g], 2 * sizeof(int32_t), cudaMemcpyDeviceToHost,
+                                                         static_cast<cudaStream_t>(stream))))
+          return SWAPMOE_ERR_CUDA;
+      return cuda_ok(cudaStreamSynchronize(static_cast<cudaStream_t>(stream))) ? SWAPMOE_OK : SWAPMOE_ERR_CUDA;
+    }
     case SWAPMOE_TAP_H:
     case SWAPMOE_TAP_Y: return debug_copy_rows(L, which, host, bytes, static_cast<cudaStream_t>(stream));
     default: return SWAPMOE_ERR_INVALID_ARG;

@@ -9,6 +9,7 @@ struct PairList {
   TileDesc* tiles;           // or nullptr
   int32_t* n_tiles;          // [2] their number, the most rows one may hold
   int32_t cols;              // weight tiles per token tile
+  int32_t shift;             // log2 of the most rows a tile may hold, 0: picked from the row counts
 };
 
 struct ScanArgs {
@@ -91,7 +92,7 @@ static __device__ __noinline__ void write_pair_tiles(const PairList l, float inv
                                               int phys1, int row0, int row1) {
   const int lane = threadIdx.x & 31;
   const int count[2] = {count0, count1};
-  const int sh = pick_tile_height(count, l.cols, inv_pairs);
+  const int sh = l.shift > 0 ? l.shift : pick_tile_height(count, l.cols, inv_pairs);
   int base = 0;
 #pragma unroll 1
   for (int h = 0; h < 2; ++h) {

@@ -1012,3 +1012,41 @@ def test_tile_lists_of_both_products_from_the_last_router_cta(monkeypatch, k, ac
     cfg = _cfg(T=8300, d=256, f=512, E=12, K=5, k=k, act=act, renorm=renorm, zipf_s=1.1)
     case = Case(cfg)
     check_against_oracle(case, case.run())
+
+
+def _two_choices(counts):
+    """First and second slot of T = sum(counts) / 2 tokens such that slot s is chosen counts[s] times and no token chooses one twice."""
+    n = np.asarray(counts)
+    first, second = n // 2, n - n // 2
+    i = np.flatnonzero(n % 2)[::2]                       # odd counts in turn give their extra token to the first choice
+    first[i] += 1
+    second[i] -= 1
+    a, b = (np.repeat(np.arange(n.size), c) for c in (first, second))
+    assert a.size == b.size
+    b = np.roll(b, max(first.max(), second.max()) + n.size)
+    assert np.all(a != b)
+    return a, b
+
+
+@pytest.mark.parametrize("cap", [64, 128, 256])
+@pytest.mark.parametrize("counts", [(224, 240, 256, 257, 480, 513), (1, 31, 33, 96, 127, 129, 160, 191), (64, 65, 127, 385, 0, 513)])
+@pytest.mark.parametrize("k,act,renorm", [(1, I.ACT_RELU, 0), (2, I.ACT_SWIGLU, 1)])
+def test_token_tile_caps_of_cta_pairs(monkeypatch, cap, counts, k, act, renorm):
+    """All four epilogues of the CTA-pair GEMMs under each cap on a tile's tokens (rings of 9, 8 and 6 stages), with row counts
+    around the caps and tiles of every height a cap allows (activation boxes of 128 and of 64 + 32 + 16 rows, whole and in part): the
+    cap is forced, external logits send the tokens to prescribed slots, and the tile lists are read back.  d_ff 448 and d_model 256:
+    a ragged last weight tile, and a list each for the two products.  Tolerance: the layer's (bf16 h and out)."""
+    from harness import Case, check_against_oracle
+    monkeypatch.setenv("SWAPMOE_TILE_CAP", str(cap))
+    K, E = len(counts), 10
+    choices = [np.repeat(np.arange(K), counts)] if k == 1 else list(_two_choices(counts))
+    T = choices[0].size
+    order = np.random.default_rng(11).permutation(T)
+    logits = np.random.default_rng(12).standard_normal((T, E)).astype(np.float32)
+    for j, c in enumerate(choices):
+        logits[np.arange(T), c[order]] += 40.0 - 10.0 * j
+    case = Case(_cfg(T=T, d=256, f=448, E=E, K=K, k=k, act=act, renorm=renorm), s2e=np.arange(K))
+    res = check_against_oracle(case, case.run(ext_logits=logits), check_logits=False)
+    assert np.array_equal(res["oracle"]["count"], counts)
+    want = [int(np.sum(-(-np.asarray(counts) // cap))), cap]
+    assert case.layer.tap("token_tiles").tolist() == [want, want]
