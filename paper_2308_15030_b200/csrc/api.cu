@@ -704,7 +704,7 @@ int32_t swapmoe_create(swapmoe_layer_t** out, const swapmoe_config_t* cfg) {
     // sixteen-token CTAs: while the grid stays within one wave of CTAs and the shared memory fits
     L->small_router_max_t = 0;
     if (L->small_router && router_small_takes(c.d_model, c.E, 2)) {
-      L->small_router_max_t = 2 * kRsTok * L->sm_count;
+      L->small_router_max_t = 2 * kRsTok * std::min(L->sm_count, 256);
       const char* envm = std::getenv("SWAPMOE_SMALL_ROUTER_MAX_T");
       if (envm) L->small_router_max_t = std::min(std::atoi(envm), 2 * kRsTok * 256);
       ok = ok && cuda_ok(cudaFuncSetAttribute(router_small_fn(c.d_model, 2), cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -68,6 +68,9 @@ __device__ __forceinline__ int even_tile_rows(int count, int shift) {
 // tokens: 175 / 115 / 86), tiles are dealt out in turn, and of the two bounds on the longest share the lower one is
 // taken.  us for both GEMMs alone, 64 / 128 / 256: 768 x 3072, 16 slots, 400 tokens 36.6 / 36.7 / 37.5, 2048 55 / 41.6 / 44.1,
 // 4096 83 / 60 / 50; one CTA per tile, the kernel before, 40.1 / 41.4 / 69.4 there.
+// h is min(rows, cap) for all tiles of a slot, more than even_tile_rows gives just above a cap.  With its heights 1999 tokens of 768
+// x 3072 get GEMM-1 in tiles of 256 instead of 128, 17.9 us alone against 19.4, but the forward is level (53.6 / 53.7), and the
+// divisions on the way to GEMM-1 cost every mid-size batch 0.3 to 0.8 us (512 x 2048 at 700 35.0 / 35.7).
 __device__ __forceinline__ int pick_tile_height(const int (&count)[2], int cols, float inv_pairs) {
   int best = 8;
   float best_cost = 3.0e38f;
@@ -85,49 +88,55 @@ __device__ __forceinline__ int pick_tile_height(const int (&count)[2], int cols,
   return best;
 }
 
-// The list of token tiles for CTA pairs, by one warp whose lanes own slots l and l + 32: `row0` = first row of a slot's segment.
-// Out of line: small batches run slot_layout_warp once per forward, through cold code, and have no such list (twelve layers of
-// 1024 x 4096 at 29 tokens: 1.5 us per layer when this was part of it).
-static __device__ __noinline__ void write_pair_tiles(const PairList l, float inv_pairs, int count0, int count1, int phys0,
-                                              int phys1, int row0, int row1) {
+// A list of token tiles for CTA pairs, by one warp whose lanes own slots l and l + 32, from the slots' row counts in shared memory.
+// Out of line: two warps run it side by side for the two lists (GEMM-1 waits for both), once per forward and through cold code.  us
+// per forward, both by the warp that lays out the slots / here: 768 x 3072, 16 slots, 500 tokens 49.2 / 47.7, 2048 56.0 / 54.8;
+// 512 x 2048 at 90 34.9 / 33.0; 704 x 2240, 32 slots, 2600 tokens 71.5 / 69.4.
+static __device__ __noinline__ void write_pair_tiles(TileDesc* tiles, int32_t* n_tiles, int cols, int shift, float inv_pairs,
+                                                     const int32_t* s_count, const int32_t* phys_slot, int K) {
   const int lane = threadIdx.x & 31;
-  const int count[2] = {count0, count1};
-  const int sh = l.shift > 0 ? l.shift : pick_tile_height(count, l.cols, inv_pairs);
-  int base = 0;
+  int count[2], phys[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int s = lane + 32 * h;
+    count[h] = s < K ? s_count[s] : 0;
+    phys[h] = s < K ? phys_slot[s] : 0;          // issued early: its latency hides behind the rule
+  }
+  const int sh = shift > 0 ? shift : pick_tile_height(count, cols, inv_pairs);
+  int row0 = 0, tile0 = 0;                       // first row and first tile of the 32 slots at hand
 #pragma unroll 1
   for (int h = 0; h < 2; ++h) {
-    const int cnt = h == 0 ? count0 : count1, phys = h == 0 ? phys0 : phys1, first = h == 0 ? row0 : row1;
-    const int nt = (cnt + (1 << sh) - 1) >> sh, rows = even_tile_rows(cnt, sh);
-    int incl = nt;
+    const int cnt = h == 0 ? count[0] : count[1], ph = h == 0 ? phys[0] : phys[1];
+    const int padded = (cnt + kSegAlign - 1) & ~(kSegAlign - 1);
+    const int n = (cnt + (1 << sh) - 1) >> sh, rows = even_tile_rows(cnt, sh);
+    int rows_incl = padded, incl = n;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const int u = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += u;
+      const int u = __shfl_up_sync(0xffffffffu, rows_incl, o), v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) { rows_incl += u; incl += v; }
     }
-    TileDesc* dst = l.tiles + base + incl - nt;
-    for (int i = 0; i < nt; ++i) {
+    TileDesc* dst = tiles + tile0 + incl - n;
+    for (int i = 0; i < n; ++i) {
       TileDesc td;
-      td.phys = phys;
-      td.row0 = first + i * rows;
+      td.phys = ph;
+      td.row0 = row0 + rows_incl - padded + i * rows;
       td.rows = min(rows, cnt - i * rows);
       td.slot = lane + 32 * h;
       dst[i] = td;
     }
-    base += __shfl_sync(0xffffffffu, incl, 31);
+    row0 += __shfl_sync(0xffffffffu, rows_incl, 31);
+    tile0 += __shfl_sync(0xffffffffu, incl, 31);
   }
-  if (lane == 0) { l.n_tiles[0] = base; l.n_tiles[1] = 1 << sh; }
+  if (lane == 0) { n_tiles[0] = tile0; n_tiles[1] = 1 << sh; }
 }
 
 // Slot layout by one warp from the per-slot counts in shared memory: lane l owns slots l and l + 32
 // (K <= 64); offsets, padded offsets and first-tile indices are exclusive prefix sums over the slots,
 // taken with warp scans (the heights of `tiles` are powers of two: shifts, no divisions - this code runs once,
 // every dependent instruction counts).  s_off / s_pad (shared, may be nullptr) receive the exclusive
-// offsets.  With kPublish two warps publish what the GEMMs read, side by side: `which` = 0 writes count / offset / pad_offset,
-// `tiles` and the first list for CTA pairs, 1 the second one (GEMM-1 waits for both: us per forward by one warp / by two, 768 x
-// 3072, 2048 tokens 54.8 / 54.0, 512 x 2048 at 90 34.7 / 33.9, 1536 x 1088, 48 slots, 70 tokens 96.3 / 94.8).
-template <bool kPublish>
+// offsets; with `write_global` the warp also writes count / offset / pad_offset and `tiles`.
 __device__ __forceinline__ void slot_layout_warp(const ScanArgs& a, const int32_t* s_count, int32_t* s_off,
-                                                 int32_t* s_pad, int which = 0) {
+                                                 int32_t* s_pad, bool write_global) {
   const int lane = threadIdx.x & 31;
   const int sh = a.tile_rows > 0 ? 31 - __clz(a.tile_rows) : 31;      // 31: no tiles
   const int round = a.tile_rows > 0 ? a.tile_rows - 1 : 0;
@@ -136,15 +145,15 @@ __device__ __forceinline__ void slot_layout_warp(const ScanArgs& a, const int32_
   for (int h = 0; h < 2; ++h) {
     const int s = lane + 32 * h;
     c[h] = s < a.K ? s_count[s] : 0;
-    ph[h] = (kPublish && s < a.K) ? a.phys_slot[s] : 0;         // issued early: its latency hides behind the scans
+    ph[h] = (write_global && s < a.K) ? a.phys_slot[s] : 0;     // issued early: its latency hides behind the scans
     off[h] = c[h];
     pad[h] = (c[h] + kSegAlign - 1) & ~(kSegAlign - 1);
-    ta[h] = kPublish ? (c[h] + round) >> sh : 0;
+    ta[h] = (c[h] + round) >> sh;
   }
-  if constexpr (kPublish) {
+  {
     // slots whose weights this forward reads: the algorithmic weight traffic of the layer
     const int nz = __popc(__ballot_sync(0xffffffffu, c[0] > 0)) + __popc(__ballot_sync(0xffffffffu, c[1] > 0));
-    if (which == 0 && lane == 0 && a.touched != nullptr) atomicAdd(a.touched, (unsigned long long)nz);
+    if (write_global && lane == 0 && a.touched != nullptr) atomicAdd(a.touched, (unsigned long long)nz);
   }
   // inclusive scans of the three quantities over 64 slots
 #pragma unroll
@@ -152,13 +161,13 @@ __device__ __forceinline__ void slot_layout_warp(const ScanArgs& a, const int32_
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const int u0 = __shfl_up_sync(0xffffffffu, off[h], o), u1 = __shfl_up_sync(0xffffffffu, pad[h], o);
-      const int u2 = kPublish ? __shfl_up_sync(0xffffffffu, ta[h], o) : 0;
+      const int u2 = __shfl_up_sync(0xffffffffu, ta[h], o);
       if (lane >= o) { off[h] += u0; pad[h] += u1; ta[h] += u2; }
     }
   }
   {
     const int t0 = __shfl_sync(0xffffffffu, off[0], 31), t1 = __shfl_sync(0xffffffffu, pad[0], 31);
-    const int t2 = kPublish ? __shfl_sync(0xffffffffu, ta[0], 31) : 0;
+    const int t2 = __shfl_sync(0xffffffffu, ta[0], 31);
     off[1] += t0; pad[1] += t1; ta[1] += t2;
   }
 #pragma unroll
@@ -167,35 +176,36 @@ __device__ __forceinline__ void slot_layout_warp(const ScanArgs& a, const int32_
     if (s < a.K) {
       const int cnt = c[h];
       const int padded = (cnt + kSegAlign - 1) & ~(kSegAlign - 1);
-      const int o_excl = off[h] - cnt, p_excl = pad[h] - padded;
+      const int nt = (cnt + round) >> sh;
+      const int o_excl = off[h] - cnt, p_excl = pad[h] - padded, t_excl = ta[h] - nt;
       if (s_off != nullptr) { s_off[s] = o_excl; s_pad[s] = p_excl; }
-      if (kPublish && which == 0) {
-        const int nt = (cnt + round) >> sh, t_excl = ta[h] - nt;
-        a.count[s] = cnt;
-        a.offset[s] = o_excl;
-        a.pad_offset[s] = p_excl;
-        for (int i = 0; i < nt; ++i) {
-          TileDesc td;
-          td.phys = ph[h];
-          td.row0 = p_excl + i * a.tile_rows;
-          td.rows = min(a.tile_rows, cnt - i * a.tile_rows);
-          td.slot = s;
-          a.tiles[t_excl + i] = td;
-        }
-        if (s == a.K - 1) {
-          a.offset[a.K] = off[h];
-          a.pad_offset[a.K] = pad[h];
-          if (a.tile_rows > 0) *a.n_tiles = ta[h];
-        }
+      if (!write_global) continue;
+      a.count[s] = cnt;
+      a.offset[s] = o_excl;
+      a.pad_offset[s] = p_excl;
+      for (int i = 0; i < nt; ++i) {
+        TileDesc td;
+        td.phys = ph[h];
+        td.row0 = p_excl + i * a.tile_rows;
+        td.rows = min(a.tile_rows, cnt - i * a.tile_rows);
+        td.slot = s;
+        a.tiles[t_excl + i] = td;
+      }
+      if (s == a.K - 1) {
+        a.offset[a.K] = off[h];
+        a.pad_offset[a.K] = pad[h];
+        if (a.tile_rows > 0) *a.n_tiles = ta[h];
       }
     }
   }
-  if constexpr (kPublish) {
-    const int first0 = pad[0] - ((c[0] + kSegAlign - 1) & ~(kSegAlign - 1));
-    const int first1 = pad[1] - ((c[1] + kSegAlign - 1) & ~(kSegAlign - 1));
-    if (a.pair[which].tiles != nullptr)
-      write_pair_tiles(a.pair[which], a.inv_pairs, c[0], c[1], ph[0], ph[1], first0, first1);
-  }
+}
+
+// The lists of token tiles for CTA pairs, by warps 1 and 2 of a publishing CTA beside warp 0's slot_layout_warp.
+__device__ __forceinline__ void publish_pair_tiles(const ScanArgs& a, const int32_t* s_count) {
+  const int warp = threadIdx.x >> 5;
+  if (warp < 1 || warp > 2) return;
+  const PairList& l = a.pair[warp - 1];
+  if (l.tiles != nullptr) write_pair_tiles(l.tiles, l.n_tiles, l.cols, l.shift, a.inv_pairs, s_count, a.phys_slot, a.K);
 }
 
 // Last-CTA form of the scan (routing without a permutation: swapmoe_route_static; grids of more
@@ -270,7 +280,8 @@ __device__ __forceinline__ void scan_reduce_block(const ScanArgs& a, void* stage
   if (own_s && a.cta_mimp != nullptr)        // slots map to distinct experts: no two threads share a target
     a.mimp[my_expert] += reduce_column_serial(mimpp, a.n_cta, a.K, tid);
   __syncthreads();
-  if (tid < 64) slot_layout_warp<true>(a, s_count, nullptr, nullptr, tid >> 5);
+  if (tid < 32) slot_layout_warp(a, s_count, nullptr, nullptr, true);
+  publish_pair_tiles(a, s_count);
 }
 
 // Called by every thread of a router CTA after its partials are written.  With a ticket counter the
@@ -345,40 +356,6 @@ __device__ __forceinline__ float reduce_columns_parallel(const float* src, int n
   return total;
 }
 
-// Sums of the router CTAs' histograms, by all threads of a CTA.  Thread (share, slot) adds the rows of a contiguous share of the
-// router CTAs, all loads in flight together: the total and, with kBefore, the rows in front of router CTA `n_before`.
-template <bool kBefore>
-__device__ __forceinline__ void add_histogram_shares(const ScanArgs& a, int n_before, int32_t (*s_part)[kPermThreads]) {
-  const int tid = threadIdx.x, K = a.K, n_cta = a.n_cta;
-  const int PK = kPermThreads / K;                         // shares per slot
-  const int R = (n_cta + PK - 1) / PK;                     // router CTAs per share (<= 8 up to 256 CTAs, K = 16)
-  const int sh = tid / K, col = tid - sh * K;
-  if (sh >= PK) return;
-  int tot = 0, before = 0;
-  const int c0 = sh * R, c1 = min(n_cta, c0 + R);
-  for (int cb = c0; cb < c1; cb += 8) {
-    int v[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) v[u] = cb + u < c1 ? a.cta_hist[(size_t)(cb + u) * K + col] : 0;
-#pragma unroll
-    for (int u = 0; u < 8; ++u) { tot += v[u]; if (kBefore) before += cb + u < n_before ? v[u] : 0; }
-  }
-  s_part[0][tid] = tot;
-  if (kBefore) s_part[1][tid] = before;
-}
-// Behind a barrier: thread `slot` adds the shares.
-template <bool kBefore>
-__device__ __forceinline__ void fold_histogram_shares(const ScanArgs& a, const int32_t (*s_part)[kPermThreads], int32_t* s_tot,
-                                                      int32_t* s_base) {
-  const int tid = threadIdx.x, K = a.K, PK = kPermThreads / K;
-  if (tid >= K) return;
-  int tot = 0, before = 0;
-#pragma unroll 8
-  for (int q = 0; q < PK; ++q) { tot += s_part[0][q * K + tid]; if (kBefore) before += s_part[1][q * K + tid]; }
-  s_tot[tid] = tot;
-  if (kBefore) s_base[tid] = before;
-}
-
 // One CTA = the pairs of tok_tile (<= 128) tokens in flat order p = t*k + j.  The rank of a
 // pair among the pairs of the same slot is: pairs in earlier CTAs +
 // pairs in earlier warps of this CTA + earlier lanes of this warp (match + popc),
@@ -435,22 +412,13 @@ __global__ void __launch_bounds__(kPermThreads, 2) permute_gather_kernel(const P
     }
     return;
   }
-  // The CTA of one more column has no tokens: it lays the slots out for everybody else (counts, offsets, tile lists), which takes
+  // The CTA of one more column has no tokens: it publishes the layout of the slots (counts, offsets, tile lists), which takes
   // 2 to 5 us longer than the offsets alone and held up the whole grid when the first token tile's CTA did it (2048 tokens of
-  // 768 x 3072: rows placed 2.2 us after the other CTAs' ones, 6011 tokens top-4 5 us).  In a branch of its own: the copying
-  // CTAs hold token pieces in registers, and with the lists' code in their path (behind a run-time switch) the kernel spilled 76
-  // bytes a thread (us per forward with that code in line / here: 768 x 3072, 2048 tokens 55.7 / 54.8, 8192 tokens and 32 slots
-  // 132.3 / 131.5; twelve layers of 1024 x 4096 at 29 tokens 736.3 / 734.2).
-  if (a.own_scan && (int)blockIdx.x >= a.scan.n_cta + 3) {
-    if (blockIdx.y != 0) return;
-    pdl_wait();
-    add_histogram_shares<false>(a.scan, 0, s_part);
-    __syncthreads();
-    fold_histogram_shares<false>(a.scan, s_part, s_tot, nullptr);
-    __syncthreads();
-    if (warp < 2) slot_layout_warp<true>(a.scan, s_tot, nullptr, nullptr, warp);
-    return;
-  }
+  // 768 x 3072: rows placed 2.2 us after the other CTAs' ones, 6011 tokens top-4 5 us).  Up to the offsets it runs the code of the
+  // copying CTAs, which is warm (histogram sums of its own cost fp32 768 x 3072 at 256 tokens 0.7 us), and it writes the lists
+  // for CTA pairs behind them: in the layout itself that call made every copying CTA spill 76 bytes a thread.
+  const bool publish = a.own_scan && (int)blockIdx.x == a.scan.n_cta + 3;
+  if (publish && blockIdx.y != 0) return;
   if (tid == 0 && blockIdx.y == 0) SWAPMOE_STAMP(1, 0);
   const int npair = a.tok_tile * a.k;          // <= 512
   const int nwarp_p = (npair + 31) >> 5;
@@ -485,16 +453,43 @@ __global__ void __launch_bounds__(kPermThreads, 2) permute_gather_kernel(const P
   const int p = p0 + tid;
   if (tid < npair && p < n_total) s = a.slot[p];
   if (a.own_scan) {
-    add_histogram_shares<true>(a.scan, (int)blockIdx.x, s_part);
+    // thread (share, slot): the histogram rows of a contiguous share of the router CTAs, all loads in flight together
+    const int K = a.K, n_cta = a.scan.n_cta, n_before = (int)blockIdx.x;
+    const int PK = kPermThreads / K;                       // shares per slot
+    const int R = (n_cta + PK - 1) / PK;                   // router CTAs per share (<= 8 up to 256 CTAs, K = 16)
+    const int sh = tid / K, col = tid - sh * K;
+    if (sh < PK) {
+      int tot = 0, before = 0;
+      const int c0 = sh * R, c1 = min(n_cta, c0 + R);
+      for (int cb = c0; cb < c1; cb += 8) {
+        int v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = cb + u < c1 ? a.scan.cta_hist[(size_t)(cb + u) * K + col] : 0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) { tot += v[u]; before += cb + u < n_before ? v[u] : 0; }
+      }
+      s_part[0][tid] = tot;
+      s_part[1][tid] = before;
+    }
     if (warp < nwarp_p) {                      // ranks inside the warp need only the pairs' slots
       const uint32_t same = __match_any_sync(0xffffffffu, s);
       rank = __popc(same & ((1u << lane) - 1u));
       if (s >= 0 && rank == 0) wcount[warp][s] = __popc(same);
     }
     __syncthreads();
-    fold_histogram_shares<true>(a.scan, s_part, s_tot, s_base);
+    if (tid < K) {
+      int tot = 0, before = 0;
+#pragma unroll 8
+      for (int q = 0; q < PK; ++q) { tot += s_part[0][q * K + tid]; before += s_part[1][q * K + tid]; }
+      s_tot[tid] = tot;
+      s_base[tid] = before;
+    }
     __syncthreads();
-    if (warp == 0) slot_layout_warp<false>(a.scan, s_tot, s_off, s_pad);
+    if (warp == 0) slot_layout_warp(a.scan, s_tot, s_off, s_pad, publish);
+    if (publish) {
+      publish_pair_tiles(a.scan, s_tot);
+      return;
+    }
   } else {
     if (tid < a.K) {
       s_base[tid] = a.cta_base[(size_t)blockIdx.x * a.K + tid];

@@ -359,8 +359,9 @@ __global__ void __launch_bounds__(kDecThreads, 1) router_small_kernel(const Rout
     while (ptx::globaltimer_ns() - t0 < 2000000ull) __nanosleep(1000);
   }
   if (tid == 0) SWAPMOE_STAMP(0, 6);
-  finish_router_cta(a.scan, ring, 2 * half);                // the wave buffers are free: stage the scan inputs there
-  if (tid == 0) SWAPMOE_STAMP(0, 10);
+  // (Never more than 256 CTAs: the permutation sums the histograms.  The last-CTA scan of the other routers was compiled in here
+  // too, never ran, and its code changed the gate's: twelve layers of 1024 x 4096 at 29 tokens 739 us with it or 750, by what
+  // that scan calls.)
 }
 
 typedef void (*RouterSmallKernel)(const RouterArgs, int32_t*);

@@ -259,7 +259,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) router_small_f32_kernel(const 
     const uint64_t t0 = ptx::globaltimer_ns();
     while (ptx::globaltimer_ns() - t0 < 2000000ull) __nanosleep(1000);
   }
-  finish_router_cta(a.scan, ring, 2 * kRsfHalfBytes);       // the wave buffers are free: stage the scan inputs there
+  // (never more than 256 CTAs: the permutation sums the histograms)
 }
 
 }  // namespace swapmoe
