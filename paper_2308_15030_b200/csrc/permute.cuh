@@ -71,6 +71,9 @@ __device__ __forceinline__ int even_tile_rows(int count, int shift) {
 // h is min(rows, cap) for all tiles of a slot, more than even_tile_rows gives just above a cap.  With its heights 1999 tokens of 768
 // x 3072 get GEMM-1 in tiles of 256 instead of 128, 17.9 us alone against 19.4, but the forward is level (53.6 / 53.7), and the
 // divisions on the way to GEMM-1 cost every mid-size batch 0.3 to 0.8 us (512 x 2048 at 700 35.0 / 35.7).
+// Of caps that cost the same (half a percent: as a rule all slots fit the smallest one) the smallest, for its stages.  us per
+// forward, the largest / the smallest: 1024 x 4096, eight slots, 150 tokens 48.3 / 46.0, 768 x 3072 at 130 46.4 / 45.0, 1536 x
+// 1088, 48 slots, 1500 tokens 99.2 / 96.8; SwiGLU 4096 x 14336, 200 tokens 295 / 287; 768 x 768 top-3, 120 tokens level.
 __device__ __forceinline__ int pick_tile_height(const int (&count)[2], int cols, float inv_pairs) {
   int best = 8;
   float best_cost = 3.0e38f;
@@ -83,7 +86,7 @@ __device__ __forceinline__ int pick_tile_height(const int (&count)[2], int cols,
     const float sum = (float)__reduce_add_sync(0xffffffffu, n0 * (190 + h0) + n1 * (190 + h1)) * ((float)cols * inv_pairs);
     const float longest = (float)(190 + __reduce_max_sync(0xffffffffu, max(h0, h1)));
     const float cost = fminf(ceilf(n - 1e-3f) * longest, sum + longest);
-    if (cost < best_cost) { best_cost = cost; best = sh; }
+    if (cost < best_cost * 1.005f) { best_cost = cost; best = sh; }
   }
   return best;
 }

@@ -1050,3 +1050,18 @@ def test_token_tile_caps_of_cta_pairs(monkeypatch, cap, counts, k, act, renorm):
     assert np.array_equal(res["oracle"]["count"], counts)
     want = [int(np.sum(-(-np.asarray(counts) // cap))), cap]
     assert case.layer.tap("token_tiles").tolist() == [want, want]
+
+
+@pytest.mark.parametrize("k,act,renorm", [(1, I.ACT_RELU, 0), (2, I.ACT_SWIGLU, 1)])
+def test_slots_that_fit_the_smallest_cap_get_its_ring(k, act, renorm):
+    """Where no slot has more than 64 rows the three caps cut the same tiles, and the one whose ring has the most stages is taken."""
+    from harness import Case, check_against_oracle
+    counts = (60, 64, 2, 33, 0, 17)
+    first = np.repeat(np.arange(len(counts)), counts) if k == 1 else _two_choices(counts)[0]
+    logits = np.random.default_rng(13).standard_normal((first.size, 8)).astype(np.float32)
+    logits[np.arange(first.size), first] += 40.0
+    if k == 2:
+        logits[np.arange(first.size), _two_choices(counts)[1]] += 30.0
+    case = Case(_cfg(T=first.size, d=256, f=448, K=len(counts), k=k, act=act, renorm=renorm), s2e=np.arange(len(counts)))
+    check_against_oracle(case, case.run(ext_logits=logits), check_logits=False)
+    assert case.layer.tap("token_tiles").tolist() == [[5, 64], [5, 64]]
