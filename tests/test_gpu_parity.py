@@ -230,9 +230,8 @@ def test_cfg5_mixtral_shape_sampled():
 def test_grouped_tile_order_forced(monkeypatch, pair_gemm, k, act, renorm, T, K):
     """The grouped GEMMs walk large activation matrices in groups of row tiles (row tiles fastest inside a
     group, then column tiles, then the next group).  SWAPMOE_ROW_GROUP=2 forces that order on shapes the
-    oracle checks in full: 256-row tiles on CTA pairs (pairs for both GEMMs: SWAPMOE_PAIR_MIN_ROWS=160) and
-    on one CTA per tile (SWAPMOE_PAIR_GEMM=0), 128-row tiles (the third shape), an odd number of row tiles
-    (ragged last group)."""
+    oracle checks in full: token tiles of CTA pairs and 128-row tiles on one CTA each (SWAPMOE_PAIR_GEMM=0, and by
+    SWAPMOE_PAIR_MIN_ROWS=160 the third shape), several groups, the last one ragged where their number is odd."""
     from harness import Case, check_against_oracle
     monkeypatch.setenv("SWAPMOE_ROW_GROUP", "2")
     monkeypatch.setenv("SWAPMOE_PAIR_GEMM", pair_gemm)
@@ -241,8 +240,9 @@ def test_grouped_tile_order_forced(monkeypatch, pair_gemm, k, act, renorm, T, K)
     case = Case(cfg)
     res = check_against_oracle(case, case.run())
     cnt = res["oracle"]["count"]
-    tile = 256 if T * k // K >= 160 else 128
-    assert int(np.sum((cnt + tile - 1) // tile)) >= 5           # several groups of two row tiles
+    n, cap = case.layer.tap("token_tiles")[0].tolist()
+    assert (n > 0) == (pair_gemm == "1" and T * k // K >= 160)
+    assert (n if n > 0 else int(np.sum((cnt + 127) // 128))) >= 5           # several groups of two row tiles
 
 
 @pytest.mark.parametrize("dtype,k,act,renorm", [(I.BF16, 2, I.ACT_SWIGLU, 1), (I.BF16, 1, I.ACT_RELU, 0),
@@ -278,9 +278,8 @@ def test_hidden_and_expert_output_taps(monkeypatch, dtype, k, act, renorm):
 
 
 def test_two_row_subtiles_per_cta():
-    """Slots with 160..1023 rows on average run on 256-row tiles: GEMM-1 on CTA pairs, GEMM-2 on one CTA that
-    shares a weight tile between two 128-row sub-tiles; include slots above and below 128 rows and a ragged
-    last sub-tile."""
+    """Three popular experts and two rare ones in one batch of some hundred rows per slot: slots of one token tile beside slots
+    that are cut into several (the CTA-pair GEMMs; once one CTA held two sub-tiles of 128 rows here)."""
     import oracle
     from harness import Case, check_against_oracle
     for k, act, renorm in ((1, I.ACT_RELU, 0), (2, I.ACT_SWIGLU, 1)):
@@ -292,7 +291,7 @@ def test_two_row_subtiles_per_cta():
         case = Case(cfg, s2e=list(order[:3]) + list(order[-2:]))   # three popular and two rare experts
         res = check_against_oracle(case, case.run())
         cnt = res["oracle"]["count"]
-        # covered: entries with two full sub-tiles, and entries whose second sub-tile is absent
+        # covered: a slot that any cap cuts, and one that two tiles of 128 would not fill
         assert cnt.max() > 256 and any(0 < c % 256 <= 128 for c in cnt), cnt
 
 
@@ -325,10 +324,9 @@ def test_back_to_back_forwards_with_changing_batches(dtype):
 
 @pytest.mark.parametrize("min_rows", [None, "160"])
 def test_cta_pair_grouped_gemm(monkeypatch, min_rows):
-    """Slots of 1024+ rows on average run the grouped GEMMs on CTA pairs (one 256-row tile per two SMs,
-    cta_group::2): all four epilogues, tiles whose second half is full, ragged and absent.  With
-    SWAPMOE_PAIR_MIN_ROWS=160 the same kernels take the mid-size case of the test above; with
-    SWAPMOE_PAIR_GEMM=0 the one-CTA kernels must give the same routing and an output within tolerance."""
+    """The grouped GEMMs on CTA pairs (cta_group::2) with all four epilogues at 1300 and 300 rows per slot on average, the latter
+    with the least average that SWAPMOE_PAIR_MIN_ROWS admits set to 160; with SWAPMOE_PAIR_GEMM=0 the one-CTA kernels must
+    give the same routing and an output within tolerance."""
     import oracle
     from harness import Case, check_against_oracle
     if min_rows:
@@ -674,12 +672,12 @@ def test_general_gate_selects_in_expert_order(T, E, K, k, ext):
     (I.BF16, 90, 192, 320, 4, 2, I.ACT_SWIGLU),
     (I.BF16, 24, 704, 2240, 6, 1, I.ACT_RELU),      # small-batch kernels' widths between the powers of two
     (I.BF16, 20, 512, 3072, 8, 1, I.ACT_RELU),
-    (I.BF16, 20, 64, 2624, 4, 2, I.ACT_SWIGLU),     # few rows of a gated layer: 80-column tiles, the last one ragged
-    (I.BF16, 32, 128, 2560, 4, 2, I.ACT_SWIGLU),    # ... and whole ones, at the most pairs they take
-    (I.BF16, 1500, 704, 448, 5, 1, I.ACT_RELU),     # 256-row tiles: GEMM-1 on CTA pairs, GEMM-2 on two row sub-tiles
+    (I.BF16, 20, 64, 2624, 4, 2, I.ACT_SWIGLU),     # small-batch kernels, gated: 16-column tiles, one k-block
+    (I.BF16, 32, 128, 2560, 4, 2, I.ACT_SWIGLU),    # ... 48-column tiles, the last one ragged, at the most pairs they take
+    (I.BF16, 1500, 704, 448, 5, 1, I.ACT_RELU),     # both GEMMs on CTA pairs, the last weight tiles ragged
     (I.BF16, 900, 448, 704, 5, 2, I.ACT_SWIGLU),
-    (I.BF16, 900, 448, 320, 5, 2, I.ACT_RELU),      # 256-row tiles with a d_ff too narrow for wide column tiles
-    (I.BF16, 3000, 448, 960, 2, 1, I.ACT_RELU),     # both GEMMs on CTA pairs
+    (I.BF16, 900, 448, 320, 5, 2, I.ACT_RELU),      # a d_ff too narrow for CTA pairs: GEMM-1 on one CTA per tile
+    (I.BF16, 3000, 448, 960, 2, 1, I.ACT_RELU),
     (I.BF16, 1600, 960, 448, 2, 2, I.ACT_SWIGLU),
     (I.F32, 100, 192, 448, 5, 1, I.ACT_RELU),       # fp32, weights on the MMA rows
     (I.F32, 900, 320, 704, 4, 1, I.ACT_RELU),       # fp32, tokens on the MMA rows
@@ -1065,3 +1063,33 @@ def test_slots_that_fit_the_smallest_cap_get_its_ring(k, act, renorm):
     case = Case(_cfg(T=first.size, d=256, f=448, K=len(counts), k=k, act=act, renorm=renorm), s2e=np.arange(len(counts)))
     check_against_oracle(case, case.run(ext_logits=logits), check_logits=False)
     assert case.layer.tap("token_tiles").tolist() == [[5, 64], [5, 64]]
+
+
+# bf16 SwiGLU layers of 6 to 64 pairs: (T, d, f, K, k), then the rows of W1 and W3 together in a tile of GEMM-1 and its k-blocks per
+# stage on 148 SMs (test_kernel_resources_host.py).  Ragged last tiles (all but 128, which divides every 2 d_ff), rings that wrap,
+# and for two k-blocks per stage an odd number of them (a half-empty last stage).
+GATED_SMALL_BATCHES = [((20, 576, 1216, 4, 2), 96, 2), ((13, 576, 1792, 4, 2), 128, 2), ((13, 960, 2624, 4, 2), 160, 2),
+                       ((20, 448, 2432, 4, 2), 160, 1), ((20, 384, 256, 40, 2), 192, 1), ((20, 320, 3648, 4, 2), 224, 1),
+                       ((20, 448, 2752, 6, 2), 256, 1)]
+
+
+@pytest.mark.parametrize("shape", [g[0] for g in GATED_SMALL_BATCHES])
+def test_gated_small_batches_at_their_tile_widths(shape):
+    """GEMM-1 of a gated layer on the small-batch kernel: the same rows of W1 and W3 in one box, at each tile width its rule picks.
+    Unlike weights in the arena entries around a slot's own (slots in another order) would show rows taken from them."""
+    from harness import Case, check_against_oracle
+    T, d, f, K, k = shape
+    case = Case(_cfg(T=T, d=d, f=f, E=K + 4, K=K, k=k, act=I.ACT_SWIGLU, renorm=1), phys=list(range(1, K)) + [0])
+    check_against_oracle(case, case.run())
+    assert case.layer.tap("token_tiles").tolist() == [[0, 0], [0, 0]]
+
+
+@pytest.mark.parametrize("k,act,renorm", [(1, I.ACT_RELU, 0), (2, I.ACT_SWIGLU, 1)])
+@pytest.mark.parametrize("pairs", [6, 18, 34, 64])
+def test_general_kernel_with_few_rows(monkeypatch, pairs, k, act, renorm):
+    """SWAPMOE_SMALL_PATH=0: the one-CTA kernel with activation boxes of 16, 32 and 64 rows, which it fetches where a batch has no
+    more pairs than that."""
+    from harness import Case, check_against_oracle
+    monkeypatch.setenv("SWAPMOE_SMALL_PATH", "0")
+    case = Case(_cfg(T=pairs // k, d=192, f=320, k=k, act=act, renorm=renorm))
+    check_against_oracle(case, case.run())
