@@ -654,7 +654,11 @@ inline bool tc_supported(const swapmoe_config_t& c) {
   return c.dtype == SWAPMOE_BF16;
 }
 
-// Whether 256-column tiles suit a matrix of n columns: at most a fifth of the last tiles' width empty.
+// Whether tiles of 256 weight rows suit a matrix of n of them: at most a fifth of the width of all tiles empty, which the widths 64,
+// 128, 192, 320, 384 and 576 miss.  us per forward, 16 slots, one CTA per tile / CTA pairs there, at 300 and at 2500 tokens: 64 x 256
+// 17.4 / 18.7 and 21.5 / 23.2; 128 x 512 18.9 / 19.8 and 24.0 / 25.5; 192 x 768 20.7 / 21.1 and 27.5 / 27.5; 320 x 1280 27.2 / 26.3
+// and 32.6 / 33.5; 384 x 1536 29.9 / 29.2 and 37.0 / 36.7; 576 x 2304 37.0 / 36.6 and 47.1 / 49.6; 768 x 320 23.2 / 23.1 and 32.7 /
+// 33.3; SwiGLU top-2 of six slots, 150 and 1200: 1024 x 192 24.3 / 26.1 and 31.3 / 32.4, 320 x 960 25.3 / 25.1 and 32.5 / 33.3.
 inline bool tc_wide_ok(int n) { return (long long)(n + 255) / 256 * 256 * 4 <= 5ll * n; }
 
 // Automatic choice: tensor cores whenever the shape allows it.

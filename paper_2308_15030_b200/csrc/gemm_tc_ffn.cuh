@@ -8,10 +8,11 @@ namespace swapmoe {
 
 // Weight tiles per token tile where a grouped GEMM (which = 1 or 2) runs on CTA pairs, 0: one CTA per tile.  Pairs take
 // every forward of more than 64 (token, expert) pairs (up to there the small-batch kernel fills the SMs better: SwiGLU 960 x
-// 2624, four slots, 13 tokens 31.0 us per forward against 39.6) whose matrices
-// leave at most a fifth of the last weight tile empty.  us per forward, one CTA per tile / pairs: 768 x 3072, 16 slots, 70
-// tokens 48.4 / 45.5, 800 53.1 / 48.7, 2048 52.4 / 52.2, 4096 81.4 / 64.8; 1024 x 512 top-4 of 256, 64 slots, 2500 95.6 / 85.7;
-// SwiGLU top-2, four slots, 1024 x 3584, 700 76.5 / 62.0, 4096 x 14336, 200 318.9 / 296.0.
+// 2624, four slots, 13 tokens 31.0 us per forward against 39.6) whose matrices leave at most a fifth of the width of all
+// weight tiles together empty (tc_wide_ok).  us per forward, the tree in which they
+// took slots of 160 rows and more only / here: 768 x 3072, 16 slots, 70 tokens 48.6 / 42.7, 500 53.2 / 46.5, 2048 55.8 / 54.3, 5000
+// 92.8 / 83.7; 512 x 2048 at 90 33.8 / 31.7; 1536 x 1088, 48 slots, 110 tokens 95.7 / 93.5; 1024 x 512 top-4, 64 slots, 3000 92.4 /
+// 87.7; SwiGLU top-2, four slots, 1024 x 3584, 300 62.8 / 50.6, 4096 x 14336, 700 647 / 568.
 inline int tc_pair_cols(const swapmoe_config_t& c, int which, long long pairs, int min_rows) {
   const int width = which == 2 ? c.d_model : c.act == SWAPMOE_ACT_SWIGLU ? 2 * c.d_ff : c.d_ff;
   if (pairs <= 64 || pairs < (long long)min_rows * c.K || !tc_wide_ok(width)) return 0;

@@ -7,7 +7,7 @@
 // alone: 48 KB), and two accumulator sets fit tensor memory, so the epilogue of one tile overlaps the next tile's MMAs.
 // Why the weights are the MMA's rows: its columns then are tokens, whose number is free in steps of 32, so a slot costs
 // neither operand bytes nor tensor time for rows it does not have.  A slot's n rows are cut into tiles of equal height
-// (slot_layout_warp), and the ring holds more stages where the tiles are small: what a pair pulls per second is bytes in
+// (write_pair_tiles), and the ring holds more stages where the tiles are small: what a pair pulls per second is bytes in
 // flight over the latency of a load (2 us under load).
 //
 // Roles in each CTA (384 threads): warp 0 = TMA producer (completion is signalled on the EVEN CTA's `full` barrier, which
@@ -31,8 +31,9 @@ constexpr int kPairMaxStages = 9;
 __device__ __forceinline__ int pair_stages(int max_tokens) { return max_tokens > 128 ? 6 : max_tokens > 64 ? 8 : 9; }
 // staging of an epilogue warp: a box of 32 tokens x 32 columns (SwiGLU 16), or output row and gate value of its 128 tokens
 __host__ __device__ constexpr int pair_warp_bytes(int epi) { return epi == kTcEpiF32 ? 4096 : epi == kTcEpiScatterBf16 ? 1024 : 2048; }
-// + alignment slack and barriers (1 KB each).  GEMM-1's leave room for a CTA of the permutation (12 KB), so that its CTAs may come
-// up while the permutation still runs.
+// + alignment slack and barriers (1 KB each).  GEMM-1's leave room for a CTA of the permutation (12 KB).  The ReLU one comes up
+// beside it while the permutation still runs (72 registers of 384 threads and 64 of 512: 60416); the gated one does not (89, allocated
+// as 96: 69632 of the SM's 65536).
 __host__ __device__ constexpr int pair_smem_bytes(int epi) { return kPairStageArea + 2048 + 8 * pair_warp_bytes(epi); }
 static_assert(pair_smem_bytes(kTcEpiReluBf16) + 1024 + 12288 <= 228 * 1024, "beside a CTA of the permutation");
 
@@ -75,7 +76,7 @@ __device__ __forceinline__ void tma_load_5d_pair(void* dst, const CUtensorMap* m
       ::"r"(smem_u32(dst)), "l"(map), "r"(bar_cluster_addr), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4)
       : "memory");
 }
-// The same, releasing what this thread has done before.
+// Arrival on a barrier that may live in the peer CTA, releasing what this thread has done before.
 __device__ __forceinline__ void mbar_arrive_release_cluster(uint32_t bar_cluster_addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster_addr) : "memory");
 }
@@ -496,8 +497,11 @@ inline int32_t tc_gemm_pair(TcState& s, int n_pairs, const swapmoe_config_t& c, 
   g.row_group = 1 << 30;
   if (row_group_forced > 0) g.row_group = row_group_forced;
   else if (pairs * (long long)c.d_model * 2 > (48ll << 20)) {
-    // groups of about 20 MB of token rows (Mixtral shape, 4096 tokens: 8-12 tiles of 256 rows measure 2.58-2.70 ms
-    // per forward, 16 tiles 2.68-2.80, 32 tiles 2.86-3.01, 4 tiles 2.68-2.72, 1 tile 3.0)
+    // Token rows of a group stay in L2 across its weight tiles: as many tiles as make 20 MB when they hold 256 rows each (slots cut
+    // into lower tiles make smaller groups, down to half of that just above 256 rows a slot, a quarter under a cap of 64).  The
+    // optimum is flat: us per forward at 5 / 10 / 20 / 40 / all tiles per group, 1024 x 512 top-4, 64 slots, 16000 tokens 289 / 291
+    // / 290 / 295 / 322 (40 is what this rule gives); 2048 x 1024 top-2, 12000 tokens, slots of 330 to 420 rows 355 / 355 / 357 / 362 /
+    // 393 (20); SwiGLU 4096 x 14336, 4096 tokens, 4 / 10 / 16 / 32 / all 2592 / 2456 / 2469 / 2454 / 2490 (10).
     g.row_group = (int)((20ll << 20) / (2ll * kTcBM * c.d_model * 2));
     if (g.row_group < 4) g.row_group = 4;
   }
